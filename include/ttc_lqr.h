@@ -85,8 +85,9 @@ extern "C" {
 
 /* ids returned by TTC_QUERY_LAST_KERNEL */
 #define TTC_KERNEL_NONE           0
-#define TTC_KERNEL_RICCATI_CTA    1  /* generic: one CTA per instance, FFMA            */
-#define TTC_KERNEL_RICCATI_WARP   2  /* register-tiled FFMA, several instances per CTA */
+#define TTC_KERNEL_RICCATI_CTA    1  /* recursion on any shape, any mix of strides     */
+#define TTC_KERNEL_RICCATI_WARP   2  /* recursion at n = m = 16 / 32, A, B, R all per head or all per
+                                        token, rows of Q and Qf on 16-byte boundaries      */
 #define TTC_KERNEL_SCAN           4  /* symplectic-pair scan + gain/rollout kernel     */
 #define TTC_KERNEL_RICCATI_UMMA   5  /* tcgen05 contractions (tensor memory), n = m = 64 */
 #define TTC_KERNEL_LAYER          6  /* contextualised layer: parameters synthesised in-kernel */
@@ -96,11 +97,10 @@ typedef struct ttc_lqr_handle ttc_lqr_handle; /* opaque; owned by the library */
 
 /* One input operand.  `ptr` is owned by the caller and only read.  For ttc_lqr_solve it
  * is a DEVICE pointer (on the handle's device), for ttc_lqr_solve_host a HOST pointer.
- * It must be aligned to 16 bytes.  Strides are arbitrary non-negative element counts; the
- * fast kernels (tcgen05 for n = m = 64, the fp32 warp kernel for n = m = 16 / 32) read the
- * rows of Q and Qf with 16-byte loads and are chosen only when every batch and time stride
- * of those two operands is a multiple of 16 bytes (4 F32 or 8 BF16 elements); any other
- * stride is served, correctly but much more slowly, by the generic kernel. */
+ * It must be aligned to 16 bytes.  Strides are arbitrary non-negative element counts; vector
+ * loads are used when every batch and time stride of an operand is a multiple of 16 bytes
+ * (4 F32 or 8 BF16 elements).  Other strides are served with element-wise loads: somewhat
+ * slower for n, m <= 16, much slower (the generic kernel) above. */
 typedef struct {
     const void* ptr;
     int32_t     dtype;       /* TTC_F32 or TTC_BF16 (BF16 only for Q and x0)            */

@@ -1,0 +1,328 @@
+// Small dense matrices held by ONE WARP in the accumulator layout of mma.sync.m16n8k8, and the products, the blocked
+// Cholesky factorisation and the vector operations that the Riccati step needs on them, without shared memory.
+//
+// Layout: a matrix of 8 RB x 8 CB elements is cut into 16 x 8 tiles; lane = 4 g + t holds of tile (mt, cb)
+//     v[mt][cb][0], [1] = row 16 mt + g,     columns 8 cb + 2 t, + 1
+//     v[mt][cb][2], [3] = row 16 mt + 8 + g, the same columns          (absent rows are zero when RB is odd)
+// The instruction leaves the assignment of contraction indices to its k slots free as long as both operands agree.
+// With slot t <-> column 2 t and slot t + 4 <-> column 2 t + 1 of an 8-wide chunk, the registers of a matrix X are the A
+// operand of X as they stand, and also the B operand of X' (transposed).  So X * Y' needs no data movement, and the
+// Riccati step can be written with such products only (P symmetric):
+//     V = B'P = (B')(P)',  T = A'P,  S = R + (B')(V)',  Y' = (A')(V)',  A'PA = (A')(T)',  Z'Z = (Z')(Z')'
+// Every product keeps float32-grade accuracy: operands are split into a tf32 part rounded to nearest and the remainder,
+// three passes (lo*hi + hi*lo + hi*hi) accumulate in float32.  The dropped term and the truncation of the remainder are
+// both about 2^-23 of the product.
+#pragma once
+
+#include <stdint.h>
+
+namespace ttc {
+namespace frag {
+
+constexpr unsigned FULL = 0xffffffffu;
+
+template <int RB, int CB>
+struct Mat {
+    static constexpr int MT = (RB + 1) / 2;
+    float v[MT][CB][4];
+};
+// hi / lo parts of a matrix
+template <int RB, int CB>
+struct Split {
+    static constexpr int MT = (RB + 1) / 2;
+    uint32_t h[MT][CB][4], l[MT][CB][4];
+};
+
+__device__ __forceinline__ void split1(float x, uint32_t& h, uint32_t& l)
+{
+    h = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;      // nearest tf32 (ties away from zero)
+    l = __float_as_uint(x - __uint_as_float(h));           // exact; the tensor core ignores its lowest bits
+}
+
+__device__ __forceinline__ void mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// d = X Y' + c with c in other registers (or constant zero), which saves the copies that an in-place accumulation needs
+__device__ __forceinline__ void mma(float (&d)[4], const float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                    uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
+}
+
+template <int RB, int CB>
+__device__ __forceinline__ void split(Split<RB, CB>& s, const Mat<RB, CB>& m)
+{
+#pragma unroll
+    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (e >= 2 && 2 * mt + 1 >= RB) {           // rows that do not exist
+                    s.h[mt][cb][e] = 0u;
+                    s.l[mt][cb][e] = 0u;
+                } else {
+                    split1(m.v[mt][cb][e], s.h[mt][cb][e], s.l[mt][cb][e]);
+                }
+            }
+}
+
+// d = c + X * Y'   (X: 8 RB x 8 KB, Y: 8 CB x 8 KB; d: 8 RB x 8 CB; c null: zero; c may be d)
+template <int RB, int KB, int CB>
+__device__ __forceinline__ void product(Mat<RB, CB>& d, const Mat<RB, CB>* c, const Split<RB, KB>& x, const Split<CB, KB>& y)
+{
+    const float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb) {
+        // pass-major order: the tiles of a pass are independent of one another
+#pragma unroll
+        for (int pass = 0; pass < 3; ++pass)
+#pragma unroll
+            for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+                for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
+                    const uint32_t(&a)[4] = pass == 0 ? x.l[mt][kb] : x.h[mt][kb];
+                    const uint32_t(&b)[4] = pass == 1 ? y.l[cb / 2][kb] : y.h[cb / 2][kb];
+                    const uint32_t b0 = b[2 * (cb & 1)], b1 = b[2 * (cb & 1) + 1];
+                    if (kb || pass)
+                        mma(d.v[mt][cb], a[0], a[2], a[1], a[3], b0, b1);
+                    else if (c)
+                        mma(d.v[mt][cb], c->v[mt][cb], a[0], a[2], a[1], a[3], b0, b1);
+                    else
+                        mma(d.v[mt][cb], z, a[0], a[2], a[1], a[3], b0, b1);
+                }
+    }
+}
+
+__device__ __forceinline__ float rcp_fast(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Inverse of the Cholesky factor of one symmetric positive definite 8 x 8 block held as (a0, a1) = row g, columns 2 t,
+// 2 t + 1.  Eliminates below the diagonal in place, the vacated column taking the column of the (unit) inverse, then
+// scales row g by 1/sqrt(pivot g).  On return (a0, a1) = W = L^{-1} (lower triangular, exact zeros above the diagonal).
+// Returns 0 or 1 + the index of the first non-positive pivot (the same on every lane; the pivots up to it are those of
+// the elimination, what follows is meaningless).
+__device__ __forceinline__ int chol8_inverse(float& a0, float& a1, int lane)
+{
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+        const float sel = (j & 1) ? a1 : a0;
+        const float d = __shfl_sync(FULL, sel, 4 * j + (j >> 1));
+        const float col = __shfl_sync(FULL, sel, (lane & 28) | (j >> 1));
+        const float r0 = __shfl_sync(FULL, a0, 4 * j + t), r1 = __shfl_sync(FULL, a1, 4 * j + t);
+        const float f = (g > j) ? -col * rcp_fast(d) : 0.f;
+        a0 = fmaf(f, r0, a0);
+        a1 = fmaf(f, r1, a1);
+        if (g > j && t == (j >> 1)) {                      // column j is eliminated, the inverse's moves in
+            if (j & 1)
+                a1 = f;
+            else
+                a0 = f;
+        }
+    }
+    const float dg = __shfl_sync(FULL, (g & 1) ? a1 : a0, (lane & 28) | (g >> 1));
+    const unsigned bad = __ballot_sync(FULL, !(dg > 0.f));
+    const float rs = rsqrtf(dg);
+    a0 = 2 * t < g ? a0 * rs : 2 * t == g ? rs : 0.f;
+    a1 = 2 * t + 1 < g ? a1 * rs : 2 * t + 1 == g ? rs : 0.f;
+    return bad ? 1 + ((__ffs(bad) - 1) >> 2) : 0;
+}
+
+// transpose of an 8 x 8 block held as (row g, columns 2 t, 2 t + 1)
+__device__ __forceinline__ void transpose8(float& y0, float& y1, float x0, float x1, int lane)
+{
+    const int g = lane >> 2, t = lane & 3, src = 8 * t + (g >> 1);
+    const float p0 = __shfl_sync(FULL, x0, src), p1 = __shfl_sync(FULL, x1, src);
+    const float q0 = __shfl_sync(FULL, x0, src + 4), q1 = __shfl_sync(FULL, x1, src + 4);
+    y0 = (g & 1) ? p1 : p0;
+    y1 = (g & 1) ? q1 : q0;
+}
+
+// M <- (M + M')/2 on the diagonal blocks, and the blocks below the diagonal become the transposes of those above
+template <int NB>
+__device__ __forceinline__ void make_symmetric(Mat<NB, NB>& m, int lane)
+{
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        float y0, y1;
+        float& d0 = m.v[i / 2][i][2 * (i & 1)];
+        float& d1 = m.v[i / 2][i][2 * (i & 1) + 1];
+        transpose8(y0, y1, d0, d1, lane);
+        d0 = 0.5f * (d0 + y0);
+        d1 = 0.5f * (d1 + y1);
+#pragma unroll
+        for (int j = i + 1; j < NB; ++j)
+            transpose8(m.v[j / 2][i][2 * (j & 1)], m.v[j / 2][i][2 * (j & 1) + 1], m.v[i / 2][j][2 * (i & 1)],
+                       m.v[i / 2][j][2 * (i & 1) + 1], lane);
+    }
+}
+
+// vectors: "row form" = element 8 b + g in every lane of row g; "column form" = elements 8 b + 2 t, + 1 in lane (., t)
+__device__ __forceinline__ void row_to_col(float& c0, float& c1, float r, int lane)
+{
+    const int t = lane & 3;
+    c0 = __shfl_sync(FULL, r, 8 * t);
+    c1 = __shfl_sync(FULL, r, 8 * t + 4);
+}
+__device__ __forceinline__ float col_to_row(float c0, float c1, int lane)
+{
+    const int g = lane >> 2;
+    const float p0 = __shfl_sync(FULL, c0, g >> 1), p1 = __shfl_sync(FULL, c1, g >> 1);
+    return (g & 1) ? p1 : p0;
+}
+__device__ __forceinline__ float sum_over_t(float v)       // result in row form
+{
+    v += __shfl_xor_sync(FULL, v, 1);
+    v += __shfl_xor_sync(FULL, v, 2);
+    return v;
+}
+__device__ __forceinline__ float sum_over_g(float v)       // result in column form
+{
+    v += __shfl_xor_sync(FULL, v, 4);
+    v += __shfl_xor_sync(FULL, v, 8);
+    v += __shfl_xor_sync(FULL, v, 16);
+    return v;
+}
+
+// one 16 x 8 tile: d += X Y' over one 8-wide chunk (x: four registers of X's tile, y: the two registers of Y's block)
+struct Tile {
+    uint32_t h[4], l[4];
+};
+__device__ __forceinline__ void split_tile(Tile& s, const float (&v)[4])
+{
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        split1(v[e], s.h[e], s.l[e]);
+}
+__device__ __forceinline__ void mma3(float (&d)[4], const Tile& x, uint32_t yh0, uint32_t yh1, uint32_t yl0, uint32_t yl1,
+                                     bool from_zero = false)
+{
+    const float z[4] = {0.f, 0.f, 0.f, 0.f};
+    if (from_zero)
+        mma(d, z, x.l[0], x.l[2], x.l[1], x.l[3], yh0, yh1);
+    else
+        mma(d, x.l[0], x.l[2], x.l[1], x.l[3], yh0, yh1);
+    mma(d, x.h[0], x.h[2], x.h[1], x.h[3], yl0, yl1);
+    mma(d, x.h[0], x.h[2], x.h[1], x.h[3], yh0, yh1);
+}
+
+// Factorisation of S = L L' (nS = -S, 8 MB x 8 MB) together with Z' = Y'L^{-T} (nY = -Y', 8 NB x 8 MB), panel by panel
+// of eight columns: the diagonal block is factored and inverted in registers, everything else is a product with its
+// inverse.  On return nS holds L below the diagonal blocks, z the split of Z', w[p] = W_p = inverse of the p-th diagonal
+// block of L.  (Negated operands keep every update a plain accumulation.)  Returns 0 or 1 + the first bad pivot.
+template <int NB, int MB>
+__device__ __forceinline__ int factor(Mat<MB, MB>& nS, Mat<NB, MB>& nY, Split<NB, MB>& z, float (&w)[MB][2], int lane)
+{
+    int bad = 0;
+#pragma unroll
+    for (int p = 0; p < MB; ++p) {
+        float a0 = -nS.v[p / 2][p][2 * (p & 1)], a1 = -nS.v[p / 2][p][2 * (p & 1) + 1];
+        const int b = chol8_inverse(a0, a1, lane);
+        if (b && !bad)
+            bad = 8 * p + b;
+        w[p][0] = a0;
+        w[p][1] = a1;
+        uint32_t wh0, wh1, wl0, wl1;
+        split1(-a0, wh0, wl0);
+        split1(-a1, wh1, wl1);
+        Tile lt[Mat<MB, MB>::MT];
+#pragma unroll
+        for (int mt = p / 2; mt < Mat<MB, MB>::MT; ++mt) {
+            if (p + 1 < MB && 2 * mt + 1 > p) {            // the tile holds rows below the diagonal block
+                Tile x;
+                split_tile(x, nS.v[mt][p]);
+                float d[4];
+                mma3(d, x, wh0, wh1, wl0, wl1, true);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    nS.v[mt][p][e] = d[e];
+                split_tile(lt[mt], d);
+            }
+        }
+#pragma unroll
+        for (int mt = 0; mt < Mat<NB, MB>::MT; ++mt) {
+            Tile x;
+            split_tile(x, nY.v[mt][p]);
+            float d[4];
+            mma3(d, x, wh0, wh1, wl0, wl1, true);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                nY.v[mt][p][e] = d[e];                     // Z' (float32) replaces its column of -Y'
+                split1(d[e], z.h[mt][p][e], z.l[mt][p][e]);
+            }
+        }
+#pragma unroll
+        for (int q = p + 1; q < MB; ++q) {
+            const int e = 2 * (q & 1);
+            const Tile& y = lt[q / 2];
+#pragma unroll
+            for (int mt = q / 2; mt < Mat<MB, MB>::MT; ++mt)
+                mma3(nS.v[mt][q], lt[mt], y.h[e], y.h[e + 1], y.l[e], y.l[e + 1]);
+#pragma unroll
+            for (int mt = 0; mt < Mat<NB, MB>::MT; ++mt) {
+                Tile x;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    x.h[k] = z.h[mt][p][k];
+                    x.l[k] = z.l[mt][p][k];
+                }
+                mma3(nY.v[mt][q], x, y.h[e], y.h[e + 1], y.l[e], y.l[e + 1]);
+            }
+        }
+    }
+    return bad;
+}
+
+// K' = -Z'L^{-1} (8 NB x 8 MB) from the results of factor(); zt is Z' in float32 and becomes K'.
+// Block column p, last one first:  K'_p = (Z'_p + sum_{q > p} K'_q L_qp)(-W_p).
+template <int NB, int MB>
+__device__ __forceinline__ void gains(Mat<NB, MB>& zt, const Mat<MB, MB>& L, const float (&w)[MB][2], int lane)
+{
+    constexpr int MT = Mat<NB, MB>::MT;
+#pragma unroll
+    for (int p = MB - 1; p >= 0; --p) {
+#pragma unroll
+        for (int q = p + 1; q < MB; ++q) {
+            float y0, y1;
+            transpose8(y0, y1, L.v[q / 2][p][2 * (q & 1)], L.v[q / 2][p][2 * (q & 1) + 1], lane);
+            uint32_t h0, h1, l0, l1;
+            split1(y0, h0, l0);
+            split1(y1, h1, l1);
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                Tile x;
+                split_tile(x, zt.v[mt][q]);
+                mma3(zt.v[mt][p], x, h0, h1, l0, l1);
+            }
+        }
+        float y0, y1;
+        transpose8(y0, y1, -w[p][0], -w[p][1], lane);
+        uint32_t h0, h1, l0, l1;
+        split1(y0, h0, l0);
+        split1(y1, h1, l1);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            Tile x;
+            split_tile(x, zt.v[mt][p]);
+            float d[4];
+            mma3(d, x, h0, h1, l0, l1, true);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                zt.v[mt][p][e] = d[e];
+        }
+    }
+}
+
+} // namespace frag
+} // namespace ttc

@@ -12,6 +12,7 @@
 #include "common.cuh"
 #include "riccati_cta.cuh"
 #include "riccati_umma64.cuh"
+#include "riccati_frag.cuh"
 #include "riccati_warp.cuh"
 #include "ttc_layer.cuh"
 #include "sigma_product.cuh"
@@ -470,31 +471,35 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
             h->last_kernel = TTC_KERNEL_RICCATI_UMMA;
             return TTC_OK;
         }
-        // A, B, R either all per head or all per token (a mix goes to the generic kernel)
+        // A, B, R either all per head or all per token
         const bool per_token = A->bstride[2] != 0 && B->bstride[2] != 0 && R->bstride[2] != 0;
-        if ((head_shared || per_token) && n == m && (n == 16 || n == 32) && q_rows_aligned) {
-            // fp32 warp kernel: one instance per 16 / 32 lanes, chunks of tokens handed out by an atomic counter
+        const bool uniform = (head_shared || per_token) && n == m && (n == 16 || n == 32) && q_rows_aligned;
+        if (obf && !uniform)
+            return fail(TTC_STATUS_UNSUPPORTED, "bfloat16 outputs need n = m in {16, 32} or the tensor-core path at n = m = 64 "
+                                                "(per-head or per-token A, B, R; Q strides that keep 16-byte rows)");
+        if (n <= 16 && m <= 16) {
+            // one warp per instance, matrices in registers; the guarded variant takes any sizes and strides
+            const bool exact = q_rows_aligned && vector_rows_ok(p.A) && vector_rows_ok(p.B) && vector_rows_ok(p.R);
+            cudaError_t e = rfrag::launch_riccati_frag(p, time_varying, affine, exact, h->sm_count, st);
+            if (e != cudaSuccess)
+                return fail(TTC_STATUS_CUDA_ERROR, "riccati_frag launch: %s", cudaGetErrorString(e));
+            h->last_launches += 1;
+            h->total_launches += 1;
+            h->last_kernel = uniform ? TTC_KERNEL_RICCATI_WARP : TTC_KERNEL_RICCATI_CTA;
+            return TTC_OK;
+        }
+        if (uniform) {
+            // fp32 warp kernel: one instance per warp, chunks of tokens handed out by an atomic counter
             if ((s = ensure(h->ws_E, sizeof(int) * 4))) return s;
             int* counter = static_cast<int*>(h->ws_E.ptr);
             TTC_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), st));
-            void (*kern)(SolveParams, int*);
-            size_t smem;
-            long long chunks, grid;
-            if (n == 32) {
-                kern = per_token ? (affine ? rwarp::riccati_warp_kernel<32, true, true, true> : rwarp::riccati_warp_kernel<32, true, false, true>)
-                     : affine ? rwarp::riccati_warp_kernel<32, true, true>
-                     : time_varying ? rwarp::riccati_warp_kernel<32, true> : rwarp::riccati_warp_kernel<32, false>;
-                smem = rwarp::smem_bytes<32>(per_token);
-                chunks = p.b0 * p.b1 * ((tcount + rwarp::Shape<32>::SLOTS - 1) / rwarp::Shape<32>::SLOTS);
-                grid = (long long)h->sm_count * 3;
-            } else {
-                kern = per_token ? (affine ? rwarp::riccati_warp_kernel<16, true, true, true> : rwarp::riccati_warp_kernel<16, true, false, true>)
-                     : affine ? rwarp::riccati_warp_kernel<16, true, true>
-                     : time_varying ? rwarp::riccati_warp_kernel<16, true> : rwarp::riccati_warp_kernel<16, false>;
-                smem = rwarp::smem_bytes<16>(per_token);
-                chunks = p.b0 * p.b1 * ((tcount + rwarp::Shape<16>::SLOTS - 1) / rwarp::Shape<16>::SLOTS);
-                grid = (long long)h->sm_count * 4;
-            }
+            void (*kern)(SolveParams, int*) =
+                per_token ? (affine ? rwarp::riccati_warp_kernel<32, true, true, true> : rwarp::riccati_warp_kernel<32, true, false, true>)
+                : affine ? rwarp::riccati_warp_kernel<32, true, true>
+                : time_varying ? rwarp::riccati_warp_kernel<32, true> : rwarp::riccati_warp_kernel<32, false>;
+            const size_t smem = rwarp::smem_bytes<32>(per_token);
+            const long long chunks = p.b0 * p.b1 * ((tcount + rwarp::Shape<32>::SLOTS - 1) / rwarp::Shape<32>::SLOTS);
+            long long grid = (long long)h->sm_count * 3;
             TTC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             if (grid > chunks) grid = chunks;
             kern<<<(unsigned)grid, rwarp::THREADS, smem, st>>>(p, counter);
@@ -504,9 +509,6 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
             h->last_kernel = TTC_KERNEL_RICCATI_WARP;
             return TTC_OK;
         }
-        if (obf)
-            return fail(TTC_STATUS_UNSUPPORTED, "bfloat16 outputs need n = m in {16, 32} or the tensor-core path at n = m = 64 "
-                                                "(per-head or per-token A, B, R; Q strides that keep 16-byte rows)");
         const size_t smem = riccati_cta_smem_bytes(n, m);
         TTC_CUDA(cudaFuncSetAttribute(riccati_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         int per_sm = 1;
