@@ -100,11 +100,39 @@ __device__ __forceinline__ void product(Mat<RB, CB>& d, const Mat<RB, CB>* c, co
     }
 }
 
+// Value of another lane: lane (B | own bits under KEEP).  The segment mask of the instruction keeps any set of own lane
+// bits, so that the source needs no index register.
+template <int B, int KEEP>
+__device__ __forceinline__ float lane_value(float x)
+{
+    float r;
+    asm volatile("shfl.sync.idx.b32 %0, %1, %2, %3, 0xffffffff;" : "=f"(r) : "f"(x), "n"(B), "n"((KEEP << 8) | 0x1f));
+    return r;
+}
+
 __device__ __forceinline__ float rcp_fast(float x)
 {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
+}
+
+template <int J>
+__device__ __forceinline__ void pivot8(float& a0, float& a1, int g, int t)
+{
+    const float sel = (J & 1) ? a1 : a0;
+    const float d = lane_value<4 * J + (J >> 1), 0>(sel);
+    const float col = lane_value<(J >> 1), 28>(sel);
+    const float r0 = lane_value<4 * J, 3>(a0), r1 = lane_value<4 * J, 3>(a1);
+    const float f = (g > J) ? -col * rcp_fast(d) : 0.f;
+    a0 = fmaf(f, r0, a0);
+    a1 = fmaf(f, r1, a1);
+    if (g > J && t == (J >> 1)) {                          // column J is eliminated, the inverse's moves in
+        if (J & 1)
+            a1 = f;
+        else
+            a0 = f;
+    }
 }
 
 // Inverse of the Cholesky factor of one symmetric positive definite 8 x 8 block held as (a0, a1) = row g, columns 2 t,
@@ -115,22 +143,13 @@ __device__ __forceinline__ float rcp_fast(float x)
 __device__ __forceinline__ int chol8_inverse(float& a0, float& a1, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int j = 0; j < 7; ++j) {
-        const float sel = (j & 1) ? a1 : a0;
-        const float d = __shfl_sync(FULL, sel, 4 * j + (j >> 1));
-        const float col = __shfl_sync(FULL, sel, (lane & 28) | (j >> 1));
-        const float r0 = __shfl_sync(FULL, a0, 4 * j + t), r1 = __shfl_sync(FULL, a1, 4 * j + t);
-        const float f = (g > j) ? -col * rcp_fast(d) : 0.f;
-        a0 = fmaf(f, r0, a0);
-        a1 = fmaf(f, r1, a1);
-        if (g > j && t == (j >> 1)) {                      // column j is eliminated, the inverse's moves in
-            if (j & 1)
-                a1 = f;
-            else
-                a0 = f;
-        }
-    }
+    pivot8<0>(a0, a1, g, t);
+    pivot8<1>(a0, a1, g, t);
+    pivot8<2>(a0, a1, g, t);
+    pivot8<3>(a0, a1, g, t);
+    pivot8<4>(a0, a1, g, t);
+    pivot8<5>(a0, a1, g, t);
+    pivot8<6>(a0, a1, g, t);
     const float dg = __shfl_sync(FULL, (g & 1) ? a1 : a0, (lane & 28) | (g >> 1));
     const unsigned bad = __ballot_sync(FULL, !(dg > 0.f));
     const float rs = rsqrtf(dg);

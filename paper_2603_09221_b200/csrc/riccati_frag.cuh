@@ -43,9 +43,59 @@ __device__ __forceinline__ Place place(const SolveParams& p, unsigned w)
     return r;
 }
 
-// X = M' of a row-major M [rows k][cols i] (i < ni: row of X, k < nk: column of X); zero outside
-template <int RB, int CB, bool PAD>
-__device__ __forceinline__ void load_transposed(Mat<RB, CB>& x, const float* M, int nk, int ni, int lane)
+// ---- operands of one time step of one instance, staged in the warp's shared memory by asynchronous copies one step
+// ahead of their use: the registers they would occupy for a whole step go to a fifth CTA per SM instead.
+// A and B are read transposed (lane (g, t) takes row 2 t, column g): with rows of 8 NB + 4 floats the 32 lanes fall into
+// 32 banks.  Q and R are read as pairs along the rows (20 floats per row: five CTAs with two buffers each fit an SM).
+template <int NB, int MB>
+struct Operands {
+    static constexpr int LA = 8 * NB + 4, LB = 8 * MB + 4, LQ = NB == 1 ? 8 : 20, LR = MB == 1 ? 8 : 20;
+    float A[8 * NB * LA], B[8 * NB * LB], Q[8 * NB * LQ], R[8 * MB * LR];
+};
+
+__device__ __forceinline__ void copy16(float* dst, const float* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy4(float* dst, const float* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_landed()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+}
+// rows x cols row-major matrix (rows <= 8 RB, cols <= 8 CB) -> dst with row length LD; elements outside stay as they are
+template <int RB, int CB, int LD, bool PAD>
+__device__ __forceinline__ void stage(float* dst, const OperandDev& o, long long off, int rows, int cols, int lane)
+{
+    if (o.dtype == TTC_BF16) {
+#pragma unroll 4
+        for (int e = lane; e < 64 * RB * CB; e += 32) {
+            const int r = e / (8 * CB), c = e % (8 * CB);
+            if (!PAD || (r < rows && c < cols))
+                dst[r * LD + c] = load_elem(o, off + r * (PAD ? cols : 8 * CB) + c);
+        }
+        return;
+    }
+    const float* src = reinterpret_cast<const float*>(o.ptr) + off;
+    if (PAD) {
+#pragma unroll 4
+        for (int e = lane; e < 64 * RB * CB; e += 32) {
+            const int r = e / (8 * CB), c = e % (8 * CB);
+            if (r < rows && c < cols)
+                copy4(dst + r * LD + c, src + r * cols + c);
+        }
+    } else {
+#pragma unroll
+        for (int e = lane; e < 16 * RB * CB; e += 32)
+            copy16(dst + (e / (2 * CB)) * LD + 4 * (e % (2 * CB)), src + 4 * e);
+    }
+}
+// X = M' from shared memory
+template <int RB, int CB, int LD>
+__device__ __forceinline__ void load_transposed(Mat<RB, CB>& x, const float* M, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -53,20 +103,12 @@ __device__ __forceinline__ void load_transposed(Mat<RB, CB>& x, const float* M, 
 #pragma unroll
         for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int i = 16 * mt + g + ((e & 2) ? 8 : 0), k = 8 * cb + 2 * t + (e & 1);
-                if (e >= 2 && 2 * mt + 1 >= RB)
-                    x.v[mt][cb][e] = 0.f;
-                else if (PAD)
-                    x.v[mt][cb][e] = (i < ni && k < nk) ? __ldg(M + k * ni + i) : 0.f;
-                else
-                    x.v[mt][cb][e] = __ldg(M + k * (8 * RB) + i);
-            }
+            for (int e = 0; e < 4; ++e)
+                x.v[mt][cb][e] = e >= 2 && 2 * mt + 1 >= RB ? 0.f : M[(8 * cb + 2 * t + (e & 1)) * LD + 16 * mt + g + ((e & 2) ? 8 : 0)];
 }
-
-// x = -M of a square row-major float32 or bf16 matrix [d][d]; `pad` on the diagonal beyond d
-template <int RB, bool PAD>
-__device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const OperandDev& o, long long off, int d, float pad, int lane)
+// x = -M of a square matrix in shared memory
+template <int RB, int LD>
+__device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const float* M, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -75,26 +117,11 @@ __device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const OperandDev& o
         for (int cb = 0; cb < RB; ++cb)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int i = 16 * mt + 8 * h + g, k = 8 * cb + 2 * t;
-                float a = 0.f, b = 0.f;
-                if (h == 0 || 2 * mt + 1 < RB) {
-                    if (PAD) {
-                        a = i < d && k < d ? load_elem(o, off + i * d + k) : i == k ? pad : 0.f;
-                        b = i < d && k + 1 < d ? load_elem(o, off + i * d + k + 1) : i == k + 1 ? pad : 0.f;
-                    } else if (o.dtype == TTC_BF16) {
-                        const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(reinterpret_cast<const __nv_bfloat16*>(o.ptr) +
-                                                                                   off + i * (8 * RB) + k));
-                        a = __uint_as_float(w << 16);
-                        b = __uint_as_float(w & 0xffff0000u);
-                    } else {
-                        const float2 f = __ldg(reinterpret_cast<const float2*>(reinterpret_cast<const float*>(o.ptr) + off +
-                                                                               i * (8 * RB) + k));
-                        a = f.x;
-                        b = f.y;
-                    }
-                }
-                x.v[mt][cb][2 * h] = -a;
-                x.v[mt][cb][2 * h + 1] = -b;
+                float2 f = make_float2(0.f, 0.f);
+                if (h == 0 || 2 * mt + 1 < RB)
+                    f = *reinterpret_cast<const float2*>(M + (16 * mt + 8 * h + g) * LD + 8 * cb + 2 * t);
+                x.v[mt][cb][2 * h] = -f.x;
+                x.v[mt][cb][2 * h + 1] = -f.y;
             }
 }
 
@@ -175,9 +202,10 @@ struct Scratch {
 // PAD = n < 8 NB or m < 8 MB, or strides that do not keep the vector loads aligned: guarded element-wise accesses, the
 // missing part of R is the identity and everything else zero, which leaves the recursion of the existing part untouched.
 template <int NB, int MB, bool TV, bool AFF, bool PAD>
-__global__ void __launch_bounds__(32 * MAX_WARPS, 4) riccati_frag_kernel(SolveParams p)
+__global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_frag_kernel(SolveParams p)
 {
     __shared__ __align__(16) Scratch scratch[MAX_WARPS];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const long long widx = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (widx >= p.b0 * p.b1 * p.tcount)
@@ -192,23 +220,38 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 4) riccati_frag_kernel(SolvePa
     float* const Kbase = (p.K && !obf) ? p.K : p.Kws;       // float32 gains (the rollout reads them)
     const long long Koff = inst * (long long)H * m * n;
     const long long Poff = inst * (long long)(p.first_only ? 1 : H + 1) * n * n;
-    const float* Ag = reinterpret_cast<const float*>(p.A.ptr) + pl.off(p.A);
-    const float* Bg = reinterpret_cast<const float*>(p.B.ptr) + pl.off(p.B);
-    const long long oR = pl.off(p.R), oQ = pl.off(p.Q);
-
-    Mat<NB, NB> nP, At, nQ;
-    Mat<MB, NB> Bt;
-    Mat<MB, MB> nR;
+    using Ops = Operands<NB, MB>;
+    Ops* const ops = reinterpret_cast<Ops*>(smem_raw) + (threadIdx.x >> 5) * (TV ? 2 : 1);
+    const long long oA = pl.off(p.A), oB = pl.off(p.B), oR = pl.off(p.R), oQ = pl.off(p.Q);
+    Mat<NB, NB> nP;
     {
+        if (PAD) {                                          // what does not exist: R is the identity, the rest zero
+            for (int e = lane; e < (int)(sizeof(Ops) / sizeof(float)) * (TV ? 2 : 1); e += 32)
+                reinterpret_cast<float*>(ops)[e] = 0.f;
+            __syncwarp();
+            for (int i = m + lane; i < 8 * MB; i += 32) {
+                ops[0].R[i * Ops::LR + i] = 1.f;
+                if (TV)
+                    ops[1].R[i * Ops::LR + i] = 1.f;
+            }
+        }
         const long long last = TV ? H - 1 : 0;
-        load_transposed<NB, NB, PAD>(At, Ag + last * p.A.st, n, n, lane);
-        load_transposed<MB, NB, PAD>(Bt, Bg + last * p.B.st, n, m, lane);
-        load_negated<MB, PAD>(nR, p.R, oR + last * p.R.st, m, 1.f, lane);
-        load_negated<NB, PAD>(nQ, p.Q, oQ + last * p.Q.st, n, 0.f, lane);
-        if (TV && p.Qf.ptr)
-            load_negated<NB, PAD>(nP, p.Qf, pl.off(p.Qf), n, 0.f, lane);
-        else
-            nP = nQ;                                        // P_H = Q
+        if (TV && p.Qf.ptr) {                               // P_H = Q_f, by way of the second buffer
+            stage<NB, NB, Ops::LQ, PAD>(ops[TV].Q, p.Qf, pl.off(p.Qf), n, n, lane);
+            copies_landed();
+            load_negated<NB, Ops::LQ>(nP, ops[TV].Q, lane);
+            __syncwarp();
+        }
+#pragma unroll
+        for (int b = 0; b < (TV ? 2 : 1); ++b) {            // the second buffer: what does not change with time
+            if (b == 0 || !p.A.st) stage<NB, NB, Ops::LA, PAD>(ops[b].A, p.A, oA + last * p.A.st, n, n, lane);
+            if (b == 0 || !p.B.st) stage<NB, MB, Ops::LB, PAD>(ops[b].B, p.B, oB + last * p.B.st, n, m, lane);
+            if (b == 0 || !p.R.st) stage<MB, MB, Ops::LR, PAD>(ops[b].R, p.R, oR + last * p.R.st, m, m, lane);
+            if (b == 0 || !p.Q.st) stage<NB, NB, Ops::LQ, PAD>(ops[b].Q, p.Q, oQ + last * p.Q.st, n, n, lane);
+        }
+        copies_landed();
+        if (!(TV && p.Qf.ptr))
+            load_negated<NB, Ops::LQ>(nP, ops[0].Q, lane);  // P_H = Q
     }
     if (p.P && !p.first_only)
         store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, n, obf, lane);
@@ -232,10 +275,23 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 4) riccati_frag_kernel(SolvePa
     int fail = 0;
 #pragma unroll 1
     for (int ts = H - 1; ts >= 0; --ts) {
-        Mat<MB, NB> V;
-        Mat<NB, NB> T;
+        const Ops& op = ops[TV ? (H - 1 - ts) & 1 : 0];
+        if (TV && ts < H - 1)
+            copies_landed();                                // also: every lane is done with the other buffer
+        if (TV && ts > 0) {                                 // operands of the next step
+            Ops& nx = ops[(H - ts) & 1];
+            if (p.A.st) stage<NB, NB, Ops::LA, PAD>(nx.A, p.A, oA + (ts - 1) * p.A.st, n, n, lane);
+            if (p.B.st) stage<NB, MB, Ops::LB, PAD>(nx.B, p.B, oB + (ts - 1) * p.B.st, n, m, lane);
+            if (p.R.st) stage<MB, MB, Ops::LR, PAD>(nx.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
+            if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(nx.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
+        }
+        Mat<NB, NB> At, T;
+        Mat<MB, NB> Bt, V;
         Mat<NB, MB> Zt;
-        Mat<MB, MB> S;
+        Mat<MB, MB> S, nR;
+        load_transposed<NB, NB, Ops::LA>(At, op.A, lane);
+        load_transposed<MB, NB, Ops::LB>(Bt, op.B, lane);
+        load_negated<MB, Ops::LR>(nR, op.R, lane);
         Split<NB, NB> as, ps;
         Split<MB, NB> bs, vs;
         split(as, At);
@@ -247,7 +303,8 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 4) riccati_frag_kernel(SolvePa
         product<MB, NB, MB>(S, &nR, bs, vs);                // -S = -R + B' V'
         product<NB, NB, MB>(Zt, nullptr, as, vs);           // -Y' = A' V'
         split(ps, T);
-        product<NB, NB, NB>(nP, &nQ, as, ps);               // -Q - A'P A
+        load_negated<NB, Ops::LQ>(nP, op.Q, lane);
+        product<NB, NB, NB>(nP, &nP, as, ps);               // -Q - A'P A
         float gr[MB], ap[NB];                               // affine: B'p + r and A'p in row form
         if (AFF && ts < p.r_count) {
             float pc[NB][2];
@@ -271,19 +328,6 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 4) riccati_frag_kernel(SolvePa
                     s = fmaf(At.v[b / 2][k][2 * (b & 1)], pc[k][0], fmaf(At.v[b / 2][k][2 * (b & 1) + 1], pc[k][1], s));
                 ap[b] = sum_over_t(s);
             }
-        }
-        if (TV && ts > 1 && p.Q.st) {
-            // Q_t comes from HBM: one request per warp brings the matrix of the step after next to L2
-            const long long bytes = (oQ + (ts - 2) * p.Q.st) * (p.Q.dtype == TTC_BF16 ? 2 : 4);
-            if (lane * 32 < n * n * (p.Q.dtype == TTC_BF16 ? 2 : 4))
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p.Q.ptr) + bytes + lane * 32));
-        }
-        if (TV && ts > 0) {
-            // operands of the next step: in flight while this step is factored
-            if (p.A.st) load_transposed<NB, NB, PAD>(At, Ag + (ts - 1) * p.A.st, n, n, lane);
-            if (p.B.st) load_transposed<MB, NB, PAD>(Bt, Bg + (ts - 1) * p.B.st, n, m, lane);
-            if (p.R.st) load_negated<MB, PAD>(nR, p.R, oR + (ts - 1) * p.R.st, m, 1.f, lane);
-            if (p.Q.st) load_negated<NB, PAD>(nQ, p.Q, oQ + (ts - 1) * p.Q.st, n, 0.f, lane);
         }
         Split<NB, MB> zs;
         float w[MB][2];
@@ -416,6 +460,8 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, 4) riccati_frag_kernel(SolvePa
 
     // ---- forward loop of Alg. 1: two lanes per row, the vectors in the warp's scratch; the rows of K_{t+1} (and of
     // A_{t+1}, B_{t+1}) are in flight while step t is summed
+    const float* Ag = reinterpret_cast<const float*>(p.A.ptr) + oA;
+    const float* Bg = reinterpret_cast<const float*>(p.B.ptr) + oB;
     const int i = lane >> 1, c0n = (lane & 1) * 4 * NB, c0m = (lane & 1) * 4 * MB;
     if ((lane & 1) == 0) {
         sc.x[i] = (i < n && p.x0.ptr) ? load_elem(p.x0, pl.off(p.x0) + i) : 0.f;
@@ -487,20 +533,26 @@ inline cudaError_t launch_riccati_frag(const SolveParams& p, bool time_varying, 
 {
     const long long nwin = p.b0 * p.b1 * p.tcount;
     void (*kern)(SolveParams);
+    size_t per_warp = sizeof(Operands<2, 2>);
     const bool sq8 = p.n <= 8 && p.m <= 8, m8 = p.m <= 8;
     const bool pad8 = !(exact && p.n == 8 && p.m == 8), pad16 = !(exact && p.n == 16 && p.m == 16);
-    if (affine)
-        kern = pad16 ? riccati_frag_kernel<2, 2, true, true, true> : riccati_frag_kernel<2, 2, true, true, false>;
-    else if (time_varying)
-        kern = pad16 ? riccati_frag_kernel<2, 2, true, false, true> : riccati_frag_kernel<2, 2, true, false, false>;
-    else if (sq8)
+    if (affine || time_varying) {
+        per_warp *= 2;
+        if (affine)
+            kern = pad16 ? riccati_frag_kernel<2, 2, true, true, true> : riccati_frag_kernel<2, 2, true, true, false>;
+        else
+            kern = pad16 ? riccati_frag_kernel<2, 2, true, false, true> : riccati_frag_kernel<2, 2, true, false, false>;
+    } else if (sq8) {
         kern = pad8 ? riccati_frag_kernel<1, 1, false, false, true> : riccati_frag_kernel<1, 1, false, false, false>;
-    else if (m8)
+        per_warp = sizeof(Operands<1, 1>);
+    } else if (m8) {
         kern = riccati_frag_kernel<2, 1, false, false, true>;
-    else
+        per_warp = sizeof(Operands<2, 1>);
+    } else {
         kern = pad16 ? riccati_frag_kernel<2, 2, false, false, true> : riccati_frag_kernel<2, 2, false, false, false>;
+    }
     const int warps = nwin <= 4ll * sm_count ? 1 : MAX_WARPS;
-    kern<<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, 0, st>>>(p);
+    kern<<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, warps * per_warp, st>>>(p);
     return cudaGetLastError();
 }
 
