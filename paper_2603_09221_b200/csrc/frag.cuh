@@ -39,6 +39,12 @@ __device__ __forceinline__ void split1(float x, uint32_t& h, uint32_t& l)
     l = __float_as_uint(x - __uint_as_float(h));           // exact; the tensor core ignores its lowest bits
 }
 
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t& h0, uint32_t& h1, uint32_t& l0, uint32_t& l1)
+{
+    split1(x0, h0, l0);
+    split1(x1, h1, l1);
+}
+
 __device__ __forceinline__ void mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
     asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -63,12 +69,13 @@ __device__ __forceinline__ void split(Split<RB, CB>& s, const Mat<RB, CB>& m)
 #pragma unroll
         for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
+            for (int e = 0; e < 4; e += 2) {
                 if (e >= 2 && 2 * mt + 1 >= RB) {           // rows that do not exist
-                    s.h[mt][cb][e] = 0u;
-                    s.l[mt][cb][e] = 0u;
+                    s.h[mt][cb][e] = s.h[mt][cb][e + 1] = 0u;
+                    s.l[mt][cb][e] = s.l[mt][cb][e + 1] = 0u;
                 } else {
-                    split1(m.v[mt][cb][e], s.h[mt][cb][e], s.l[mt][cb][e]);
+                    split2(m.v[mt][cb][e], m.v[mt][cb][e + 1], s.h[mt][cb][e], s.h[mt][cb][e + 1], s.l[mt][cb][e],
+                           s.l[mt][cb][e + 1]);
                 }
             }
 }
@@ -152,9 +159,10 @@ __device__ __forceinline__ int chol8_inverse(float& a0, float& a1, int lane)
     pivot8<6>(a0, a1, g, t);
     const float dg = __shfl_sync(FULL, (g & 1) ? a1 : a0, (lane & 28) | (g >> 1));
     const unsigned bad = __ballot_sync(FULL, !(dg > 0.f));
-    const float rs = rsqrtf(dg);
-    a0 = 2 * t < g ? a0 * rs : 2 * t == g ? rs : 0.f;
-    a1 = 2 * t + 1 < g ? a1 * rs : 2 * t + 1 == g ? rs : 0.f;
+    float rs;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(dg));
+    a0 = (2 * t < g ? a0 : 2 * t == g ? 1.f : 0.f) * rs;
+    a1 = (2 * t + 1 < g ? a1 : 2 * t + 1 == g ? 1.f : 0.f) * rs;
     return bad ? 1 + ((__ffs(bad) - 1) >> 2) : 0;
 }
 
@@ -221,8 +229,8 @@ struct Tile {
 __device__ __forceinline__ void split_tile(Tile& s, const float (&v)[4])
 {
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-        split1(v[e], s.h[e], s.l[e]);
+    for (int e = 0; e < 4; e += 2)
+        split2(v[e], v[e + 1], s.h[e], s.h[e + 1], s.l[e], s.l[e + 1]);
 }
 __device__ __forceinline__ void mma3(float (&d)[4], const Tile& x, uint32_t yh0, uint32_t yh1, uint32_t yl0, uint32_t yl1,
                                      bool from_zero = false)
@@ -253,8 +261,7 @@ __device__ __forceinline__ int factor(Mat<MB, MB>& nS, Mat<NB, MB>& nY, Split<NB
         w[p][0] = a0;
         w[p][1] = a1;
         uint32_t wh0, wh1, wl0, wl1;
-        split1(-a0, wh0, wl0);
-        split1(-a1, wh1, wl1);
+        split2(-a0, -a1, wh0, wh1, wl0, wl1);
         Tile lt[Mat<MB, MB>::MT];
 #pragma unroll
         for (int mt = p / 2; mt < Mat<MB, MB>::MT; ++mt) {
@@ -276,9 +283,10 @@ __device__ __forceinline__ int factor(Mat<MB, MB>& nS, Mat<NB, MB>& nY, Split<NB
             float d[4];
             mma3(d, x, wh0, wh1, wl0, wl1, true);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
+            for (int e = 0; e < 4; e += 2) {
                 nY.v[mt][p][e] = d[e];                     // Z' (float32) replaces its column of -Y'
-                split1(d[e], z.h[mt][p][e], z.l[mt][p][e]);
+                nY.v[mt][p][e + 1] = d[e + 1];
+                split2(d[e], d[e + 1], z.h[mt][p][e], z.h[mt][p][e + 1], z.l[mt][p][e], z.l[mt][p][e + 1]);
             }
         }
 #pragma unroll
@@ -316,8 +324,7 @@ __device__ __forceinline__ void gains(Mat<NB, MB>& zt, const Mat<MB, MB>& L, con
             float y0, y1;
             transpose8(y0, y1, L.v[q / 2][p][2 * (q & 1)], L.v[q / 2][p][2 * (q & 1) + 1], lane);
             uint32_t h0, h1, l0, l1;
-            split1(y0, h0, l0);
-            split1(y1, h1, l1);
+            split2(y0, y1, h0, h1, l0, l1);
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt) {
                 Tile x;
@@ -328,8 +335,7 @@ __device__ __forceinline__ void gains(Mat<NB, MB>& zt, const Mat<MB, MB>& L, con
         float y0, y1;
         transpose8(y0, y1, -w[p][0], -w[p][1], lane);
         uint32_t h0, h1, l0, l1;
-        split1(y0, h0, l0);
-        split1(y1, h1, l1);
+        split2(y0, y1, h0, h1, l0, l1);
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
             Tile x;
@@ -341,6 +347,92 @@ __device__ __forceinline__ void gains(Mat<NB, MB>& zt, const Mat<MB, MB>& L, con
                 zt.v[mt][p][e] = d[e];
         }
     }
+}
+
+// ---- operands that stay the same over many products: their split parts in shared memory in register order, one
+// 16-byte word per lane, tile and part, so that a product reads them without arithmetic
+template <int RB, int CB>
+struct Stored {
+    static constexpr int MT = (RB + 1) / 2;
+    uint4 q[MT][CB][2][32];
+};
+template <int RB, int CB>
+__device__ __forceinline__ void keep(Stored<RB, CB>& st, const Mat<RB, CB>& m, int lane)
+{
+    Split<RB, CB> s;
+    split(s, m);
+#pragma unroll
+    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb) {
+            // in the order of the instruction's A registers, so that the loaded group is used as it is
+            st.q[mt][cb][0][lane] = make_uint4(s.h[mt][cb][0], s.h[mt][cb][2], s.h[mt][cb][1], s.h[mt][cb][3]);
+            st.q[mt][cb][1][lane] = make_uint4(s.l[mt][cb][0], s.l[mt][cb][2], s.l[mt][cb][1], s.l[mt][cb][3]);
+        }
+}
+// d = c + X * Y' with X stored
+template <int RB, int KB, int CB>
+__device__ __forceinline__ void product(Mat<RB, CB>& d, const Mat<RB, CB>* c, const Stored<RB, KB>& x, const Split<CB, KB>& y, int lane)
+{
+    const float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb) {
+        uint4 a[Mat<RB, CB>::MT][2];
+#pragma unroll
+        for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
+            a[mt][0] = x.q[mt][kb][0][lane];
+            a[mt][1] = x.q[mt][kb][1][lane];
+        }
+#pragma unroll
+        for (int pass = 0; pass < 3; ++pass)
+#pragma unroll
+            for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+                for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
+                    const uint4 v = a[mt][pass == 0];
+                    const uint32_t(&b)[4] = pass == 1 ? y.l[cb / 2][kb] : y.h[cb / 2][kb];
+                    const uint32_t b0 = b[2 * (cb & 1)], b1 = b[2 * (cb & 1) + 1];
+                    if (kb || pass)
+                        mma(d.v[mt][cb], v.x, v.y, v.z, v.w, b0, b1);
+                    else if (c)
+                        mma(d.v[mt][cb], c->v[mt][cb], v.x, v.y, v.z, v.w, b0, b1);
+                    else
+                        mma(d.v[mt][cb], z, v.x, v.y, v.z, v.w, b0, b1);
+                }
+    }
+}
+// d = c + X X' with a result that is symmetric bit for bit when c is: lo*hi and hi*lo start from zero, so that one is the
+// transpose of the other, and are added to each other first
+template <int NB, int KB>
+__device__ __forceinline__ void product_symmetric(Mat<NB, NB>& d, const Split<NB, KB>& x)
+{
+    const float z[4] = {0.f, 0.f, 0.f, 0.f};
+    constexpr int MT = Mat<NB, NB>::MT;
+#pragma unroll
+    for (int cb = 0; cb < NB; ++cb)
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            float e1[4], e2[4];
+#pragma unroll
+            for (int kb = 0; kb < KB; ++kb) {
+                const uint32_t(&xh)[4] = x.h[mt][kb];
+                const uint32_t(&xl)[4] = x.l[mt][kb];
+                const uint32_t(&yh)[4] = x.h[cb / 2][kb];
+                const uint32_t(&yl)[4] = x.l[cb / 2][kb];
+                const int i = 2 * (cb & 1);
+                if (kb == 0) {
+                    mma(e1, z, xl[0], xl[2], xl[1], xl[3], yh[i], yh[i + 1]);
+                    mma(e2, z, xh[0], xh[2], xh[1], xh[3], yl[i], yl[i + 1]);
+                } else {
+                    mma(e1, xl[0], xl[2], xl[1], xl[3], yh[i], yh[i + 1]);
+                    mma(e2, xh[0], xh[2], xh[1], xh[3], yl[i], yl[i + 1]);
+                }
+                mma(d.v[mt][cb], xh[0], xh[2], xh[1], xh[3], yh[i], yh[i + 1]);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                d.v[mt][cb][e] += e1[e] + e2[e];
+        }
 }
 
 } // namespace frag

@@ -52,6 +52,22 @@ struct Operands {
     static constexpr int LA = 8 * NB + 4, LB = 8 * MB + 4, LQ = NB == 1 ? 8 : 20, LR = MB == 1 ? 8 : 20;
     float A[8 * NB * LA], B[8 * NB * LB], Q[8 * NB * LQ], R[8 * MB * LR];
 };
+// time-invariant form: A' and B' once more, split and in register order
+template <int NB, int MB>
+struct Fixed {
+    Stored<NB, NB> A;
+    Stored<MB, NB> B;
+};
+// what a warp keeps in shared memory
+template <int NB, int MB, bool TV>
+struct WarpMem {
+    Operands<NB, MB> op[2];
+};
+template <int NB, int MB>
+struct WarpMem<NB, MB, false> {
+    Operands<NB, MB> op[1];
+    Fixed<NB, MB> fixed;
+};
 
 __device__ __forceinline__ void copy16(float* dst, const float* src)
 {
@@ -221,37 +237,46 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_fr
     const long long Koff = inst * (long long)H * m * n;
     const long long Poff = inst * (long long)(p.first_only ? 1 : H + 1) * n * n;
     using Ops = Operands<NB, MB>;
-    Ops* const ops = reinterpret_cast<Ops*>(smem_raw) + (threadIdx.x >> 5) * (TV ? 2 : 1);
+    WarpMem<NB, MB, TV>* const ops = reinterpret_cast<WarpMem<NB, MB, TV>*>(smem_raw) + (threadIdx.x >> 5);
     const long long oA = pl.off(p.A), oB = pl.off(p.B), oR = pl.off(p.R), oQ = pl.off(p.Q);
     Mat<NB, NB> nP;
     {
         if (PAD) {                                          // what does not exist: R is the identity, the rest zero
             for (int e = lane; e < (int)(sizeof(Ops) / sizeof(float)) * (TV ? 2 : 1); e += 32)
-                reinterpret_cast<float*>(ops)[e] = 0.f;
+                reinterpret_cast<float*>(ops->op)[e] = 0.f;
             __syncwarp();
             for (int i = m + lane; i < 8 * MB; i += 32) {
-                ops[0].R[i * Ops::LR + i] = 1.f;
+                ops->op[0].R[i * Ops::LR + i] = 1.f;
                 if (TV)
-                    ops[1].R[i * Ops::LR + i] = 1.f;
+                    ops->op[1].R[i * Ops::LR + i] = 1.f;
             }
         }
         const long long last = TV ? H - 1 : 0;
         if (TV && p.Qf.ptr) {                               // P_H = Q_f, by way of the second buffer
-            stage<NB, NB, Ops::LQ, PAD>(ops[TV].Q, p.Qf, pl.off(p.Qf), n, n, lane);
+            stage<NB, NB, Ops::LQ, PAD>(ops->op[TV].Q, p.Qf, pl.off(p.Qf), n, n, lane);
             copies_landed();
-            load_negated<NB, Ops::LQ>(nP, ops[TV].Q, lane);
+            load_negated<NB, Ops::LQ>(nP, ops->op[TV].Q, lane);
             __syncwarp();
         }
 #pragma unroll
         for (int b = 0; b < (TV ? 2 : 1); ++b) {            // the second buffer: what does not change with time
-            if (b == 0 || !p.A.st) stage<NB, NB, Ops::LA, PAD>(ops[b].A, p.A, oA + last * p.A.st, n, n, lane);
-            if (b == 0 || !p.B.st) stage<NB, MB, Ops::LB, PAD>(ops[b].B, p.B, oB + last * p.B.st, n, m, lane);
-            if (b == 0 || !p.R.st) stage<MB, MB, Ops::LR, PAD>(ops[b].R, p.R, oR + last * p.R.st, m, m, lane);
-            if (b == 0 || !p.Q.st) stage<NB, NB, Ops::LQ, PAD>(ops[b].Q, p.Q, oQ + last * p.Q.st, n, n, lane);
+            if (b == 0 || !p.A.st) stage<NB, NB, Ops::LA, PAD>(ops->op[b].A, p.A, oA + last * p.A.st, n, n, lane);
+            if (b == 0 || !p.B.st) stage<NB, MB, Ops::LB, PAD>(ops->op[b].B, p.B, oB + last * p.B.st, n, m, lane);
+            if (b == 0 || !p.R.st) stage<MB, MB, Ops::LR, PAD>(ops->op[b].R, p.R, oR + last * p.R.st, m, m, lane);
+            if (b == 0 || !p.Q.st) stage<NB, NB, Ops::LQ, PAD>(ops->op[b].Q, p.Q, oQ + last * p.Q.st, n, n, lane);
         }
         copies_landed();
+        if constexpr (!TV) {
+            Mat<NB, NB> At;
+            Mat<MB, NB> Bt;
+            load_transposed<NB, NB, Ops::LA>(At, ops->op[0].A, lane);
+            load_transposed<MB, NB, Ops::LB>(Bt, ops->op[0].B, lane);
+            keep(ops->fixed.A, At, lane);
+            keep(ops->fixed.B, Bt, lane);
+            __syncwarp();
+        }
         if (!(TV && p.Qf.ptr))
-            load_negated<NB, Ops::LQ>(nP, ops[0].Q, lane);  // P_H = Q
+            load_negated<NB, Ops::LQ>(nP, ops->op[0].Q, lane);  // P_H = Q
     }
     if (p.P && !p.first_only)
         store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, n, obf, lane);
@@ -275,11 +300,11 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_fr
     int fail = 0;
 #pragma unroll 1
     for (int ts = H - 1; ts >= 0; --ts) {
-        const Ops& op = ops[TV ? (H - 1 - ts) & 1 : 0];
+        const Ops& op = ops->op[TV ? (H - 1 - ts) & 1 : 0];
         if (TV && ts < H - 1)
             copies_landed();                                // also: every lane is done with the other buffer
         if (TV && ts > 0) {                                 // operands of the next step
-            Ops& nx = ops[(H - ts) & 1];
+            Ops& nx = ops->op[(H - ts) & 1];
             if (p.A.st) stage<NB, NB, Ops::LA, PAD>(nx.A, p.A, oA + (ts - 1) * p.A.st, n, n, lane);
             if (p.B.st) stage<NB, MB, Ops::LB, PAD>(nx.B, p.B, oB + (ts - 1) * p.B.st, n, m, lane);
             if (p.R.st) stage<MB, MB, Ops::LR, PAD>(nx.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
@@ -289,22 +314,36 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_fr
         Mat<MB, NB> Bt, V;
         Mat<NB, MB> Zt;
         Mat<MB, MB> S, nR;
-        load_transposed<NB, NB, Ops::LA>(At, op.A, lane);
-        load_transposed<MB, NB, Ops::LB>(Bt, op.B, lane);
         load_negated<MB, Ops::LR>(nR, op.R, lane);
-        Split<NB, NB> as, ps;
-        Split<MB, NB> bs, vs;
-        split(as, At);
-        split(bs, Bt);
+        Split<NB, NB> ps;
+        Split<MB, NB> vs;
         split(ps, nP);
-        product<MB, NB, NB>(V, nullptr, bs, ps);            // V = B' nP
-        product<NB, NB, NB>(T, nullptr, as, ps);            // T = A' nP
-        split(vs, V);
-        product<MB, NB, MB>(S, &nR, bs, vs);                // -S = -R + B' V'
-        product<NB, NB, MB>(Zt, nullptr, as, vs);           // -Y' = A' V'
-        split(ps, T);
-        load_negated<NB, Ops::LQ>(nP, op.Q, lane);
-        product<NB, NB, NB>(nP, &nP, as, ps);               // -Q - A'P A
+        if constexpr (TV) {
+            load_transposed<NB, NB, Ops::LA>(At, op.A, lane);
+            load_transposed<MB, NB, Ops::LB>(Bt, op.B, lane);
+            Split<NB, NB> as;
+            Split<MB, NB> bs;
+            split(as, At);
+            split(bs, Bt);
+            product<MB, NB, NB>(V, nullptr, bs, ps);        // V = B' nP
+            product<NB, NB, NB>(T, nullptr, as, ps);        // T = A' nP
+            split(vs, V);
+            product<MB, NB, MB>(S, &nR, bs, vs);            // -S = -R + B' V'
+            product<NB, NB, MB>(Zt, nullptr, as, vs);       // -Y' = A' V'
+            split(ps, T);
+            load_negated<NB, Ops::LQ>(nP, op.Q, lane);
+            product<NB, NB, NB>(nP, &nP, as, ps);           // -Q - A'P A
+        } else {
+            const Fixed<NB, MB>& fx = ops->fixed;
+            product<MB, NB, NB>(V, nullptr, fx.B, ps, lane);
+            product<NB, NB, NB>(T, nullptr, fx.A, ps, lane);
+            split(vs, V);
+            product<MB, NB, MB>(S, &nR, fx.B, vs, lane);
+            product<NB, NB, MB>(Zt, nullptr, fx.A, vs, lane);
+            split(ps, T);
+            load_negated<NB, Ops::LQ>(nP, op.Q, lane);
+            product<NB, NB, NB>(nP, &nP, fx.A, ps, lane);
+        }
         float gr[MB], ap[NB];                               // affine: B'p + r and A'p in row form
         if (AFF && ts < p.r_count) {
             float pc[NB][2];
@@ -533,21 +572,21 @@ inline cudaError_t launch_riccati_frag(const SolveParams& p, bool time_varying, 
 {
     const long long nwin = p.b0 * p.b1 * p.tcount;
     void (*kern)(SolveParams);
-    size_t per_warp = sizeof(Operands<2, 2>);
+    size_t per_warp = sizeof(WarpMem<2, 2, false>);
     const bool sq8 = p.n <= 8 && p.m <= 8, m8 = p.m <= 8;
     const bool pad8 = !(exact && p.n == 8 && p.m == 8), pad16 = !(exact && p.n == 16 && p.m == 16);
     if (affine || time_varying) {
-        per_warp *= 2;
+        per_warp = sizeof(WarpMem<2, 2, true>);
         if (affine)
             kern = pad16 ? riccati_frag_kernel<2, 2, true, true, true> : riccati_frag_kernel<2, 2, true, true, false>;
         else
             kern = pad16 ? riccati_frag_kernel<2, 2, true, false, true> : riccati_frag_kernel<2, 2, true, false, false>;
     } else if (sq8) {
         kern = pad8 ? riccati_frag_kernel<1, 1, false, false, true> : riccati_frag_kernel<1, 1, false, false, false>;
-        per_warp = sizeof(Operands<1, 1>);
+        per_warp = sizeof(WarpMem<1, 1, false>);
     } else if (m8) {
         kern = riccati_frag_kernel<2, 1, false, false, true>;
-        per_warp = sizeof(Operands<2, 1>);
+        per_warp = sizeof(WarpMem<2, 1, false>);
     } else {
         kern = pad16 ? riccati_frag_kernel<2, 2, false, false, true> : riccati_frag_kernel<2, 2, false, false, false>;
     }

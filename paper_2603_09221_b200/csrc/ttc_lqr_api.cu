@@ -15,6 +15,7 @@
 #include "riccati_frag.cuh"
 #include "riccati_warp.cuh"
 #include "ttc_layer.cuh"
+#include "layer_frag.cuh"
 #include "sigma_product.cuh"
 #include "layer_grad.cuh"
 #include "lqr_grad.cuh"
@@ -255,19 +256,23 @@ int ttc_lqr_create(const ttc_lqr_config* cfg, ttc_lqr_handle** out)
     TTC_CUDA(cudaGetDeviceCount(&ndev));
     if (cfg->device < 0 || cfg->device >= ndev)
         return fail(TTC_STATUS_CUDA_ERROR, "device %d not present (%d devices)", cfg->device, ndev);
-    cudaDeviceProp prop;
-    TTC_CUDA(cudaGetDeviceProperties(&prop, cfg->device));
-    if (prop.major != 10)
+    // single attributes: cudaGetDeviceProperties collects everything about the device and takes 3 to 20 ms
+    int major = 0, minor = 0, sms = 0, pitch = 0;
+    TTC_CUDA(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cfg->device));
+    TTC_CUDA(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, cfg->device));
+    TTC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cfg->device));
+    TTC_CUDA(cudaDeviceGetAttribute(&pitch, cudaDevAttrMaxPitch, cfg->device));
+    if (major != 10)
         return fail(TTC_STATUS_CUDA_ERROR, "device %d is sm_%d%d; this library is built for sm_100a only",
-                    cfg->device, prop.major, prop.minor);
+                    cfg->device, major, minor);
     TTC_CUDA(cudaSetDevice(cfg->device));
     ttc_lqr_handle* h = new (std::nothrow) ttc_lqr_handle();
     if (!h)
         return fail(TTC_STATUS_ALLOC_FAILED, "host allocation failed");
     h->cfg = *cfg;
     h->N = N;
-    h->sm_count = prop.multiProcessorCount;
-    h->max_pitch = prop.memPitch;
+    h->sm_count = sms;
+    h->max_pitch = (size_t)pitch;
     h->host_stream = nullptr;
     h->in_stream = h->out_stream = nullptr;
     h->host_pipeline_ready = false;
@@ -788,10 +793,6 @@ static int launch_layer(ttc_lqr_handle* h, const ttc_layer_inputs* in, int32_t T
                         cudaStream_t st, long long i0 = 0, long long cnt = -1)
 {
     const int n = h->cfg.n;
-    int s;
-    if ((s = ensure(h->ws_E, sizeof(int) * 4))) return s;
-    int* counter = static_cast<int*>(h->ws_E.ptr);
-    TTC_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), st));
     layer::LayerParams p;
     p.N = cnt < 0 ? h->N : cnt;
     p.T = T;
@@ -803,30 +804,9 @@ static int launch_layer(ttc_lqr_handle* h, const ttc_layer_inputs* in, int32_t T
     p.B_basis = in->B_basis; p.Q_basis = in->Q_basis;
     p.u1 = u1 ? u1 + on : nullptr; p.P0 = P0 ? P0 + on * n : nullptr; p.info = info ? info + i0 : nullptr;
     p.Kws = nullptr; p.Pws = nullptr; p.g = nullptr; p.k0 = nullptr;
-    void (*kern)(layer::LayerParams, int*);
-    size_t smem;
-    long long chunks, grid;
-    if (n == 32) {
-        kern = layer::ttc_layer_kernel<32>;
-        smem = layer::smem_bytes<32>();
-        chunks = (p.N + rwarp::Shape<32>::SLOTS - 1) / rwarp::Shape<32>::SLOTS;
-        grid = (long long)h->sm_count * 3;
-    } else if (p.N <= (long long)h->sm_count * 2 * rwarp::Shape<16>::SLOTS) {
-        // the machine is less than half full: 16 lanes per instance walk the chain faster than 8 lanes with two columns each
-        kern = layer::ttc_layer_kernel<16>;
-        smem = layer::smem_bytes<16>();
-        chunks = (p.N + rwarp::Shape<16>::SLOTS - 1) / rwarp::Shape<16>::SLOTS;
-        grid = (long long)h->sm_count * 4;
-    } else {
-        kern = layer::ttc_layer_kernel_c2<16>;
-        smem = layer::smem_bytes_c2<16>();
-        chunks = (p.N + layer::Shape2<16>::SLOTS - 1) / layer::Shape2<16>::SLOTS;
-        grid = (long long)h->sm_count * 2;
-    }
-    TTC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (grid > chunks) grid = chunks;
-    kern<<<(unsigned)grid, rwarp::THREADS, smem, st>>>(p, counter);
-    TTC_CUDA(cudaGetLastError());
+    const cudaError_t e = n == 32 ? lfrag::launch_layer_frag<4>(p, h->sm_count, st) : lfrag::launch_layer_frag<2>(p, h->sm_count, st);
+    if (e != cudaSuccess)
+        return fail(TTC_STATUS_CUDA_ERROR, "layer launch: %s", cudaGetErrorString(e));
     h->last_launches += 1;
     h->total_launches += 1;
     h->last_kernel = TTC_KERNEL_LAYER;
