@@ -80,8 +80,9 @@ __device__ __forceinline__ void split(Split<RB, CB>& s, const Mat<RB, CB>& m)
             }
 }
 
-// d = c + X * Y'   (X: 8 RB x 8 KB, Y: 8 CB x 8 KB; d: 8 RB x 8 CB; c null: zero; c may be d)
-template <int RB, int KB, int CB>
+// d = c + X * Y'   (X: 8 RB x 8 KB, Y: 8 CB x 8 KB; d: 8 RB x 8 CB; c null: zero; c may be d).  LOWER: only the tiles that
+// touch the lower triangle, of a result whose upper one is not needed or follows from it.
+template <int RB, int KB, int CB, bool LOWER = false>
 __device__ __forceinline__ void product(Mat<RB, CB>& d, const Mat<RB, CB>* c, const Split<RB, KB>& x, const Split<CB, KB>& y)
 {
     const float z[4] = {0.f, 0.f, 0.f, 0.f};
@@ -94,6 +95,8 @@ __device__ __forceinline__ void product(Mat<RB, CB>& d, const Mat<RB, CB>* c, co
             for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
                 for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
+                    if (LOWER && cb > 2 * mt + 1)
+                        continue;
                     const uint32_t(&a)[4] = pass == 0 ? x.l[mt][kb] : x.h[mt][kb];
                     const uint32_t(&b)[4] = pass == 1 ? y.l[cb / 2][kb] : y.h[cb / 2][kb];
                     const uint32_t b0 = b[2 * (cb & 1)], b1 = b[2 * (cb & 1) + 1];
@@ -176,7 +179,19 @@ __device__ __forceinline__ void transpose8(float& y0, float& y1, float x0, float
     y1 = (g & 1) ? q1 : q0;
 }
 
-// M <- (M + M')/2 on the diagonal blocks, and the blocks below the diagonal become the transposes of those above
+// the tiles above the diagonal that LOWER products leave out: transposes of those below
+template <int NB>
+__device__ __forceinline__ void mirror(Mat<NB, NB>& m, int lane)
+{
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+#pragma unroll
+        for (int j = 2; j < NB; ++j)
+            if (j >= 2 * (i / 2) + 2)
+                transpose8(m.v[i / 2][j][2 * (i & 1)], m.v[i / 2][j][2 * (i & 1) + 1], m.v[j / 2][i][2 * (j & 1)],
+                       m.v[j / 2][i][2 * (j & 1) + 1], lane);
+}
+// M <- (M + M')/2 on the diagonal blocks, and the blocks above the diagonal become the transposes of those below
 template <int NB>
 __device__ __forceinline__ void make_symmetric(Mat<NB, NB>& m, int lane)
 {
@@ -189,9 +204,10 @@ __device__ __forceinline__ void make_symmetric(Mat<NB, NB>& m, int lane)
         d0 = 0.5f * (d0 + y0);
         d1 = 0.5f * (d1 + y1);
 #pragma unroll
-        for (int j = i + 1; j < NB; ++j)
-            transpose8(m.v[j / 2][i][2 * (j & 1)], m.v[j / 2][i][2 * (j & 1) + 1], m.v[i / 2][j][2 * (i & 1)],
-                       m.v[i / 2][j][2 * (i & 1) + 1], lane);
+        for (int j = 1; j < NB; ++j)
+            if (j > i)
+                transpose8(m.v[i / 2][j][2 * (i & 1)], m.v[i / 2][j][2 * (i & 1) + 1], m.v[j / 2][i][2 * (j & 1)],
+                       m.v[j / 2][i][2 * (j & 1) + 1], lane);
     }
 }
 
@@ -264,8 +280,8 @@ __device__ __forceinline__ int factor(Mat<MB, MB>& nS, Mat<NB, MB>& nY, Split<NB
         split2(-a0, -a1, wh0, wh1, wl0, wl1);
         Tile lt[Mat<MB, MB>::MT];
 #pragma unroll
-        for (int mt = p / 2; mt < Mat<MB, MB>::MT; ++mt) {
-            if (p + 1 < MB && 2 * mt + 1 > p) {            // the tile holds rows below the diagonal block
+        for (int mt = 0; mt < Mat<MB, MB>::MT; ++mt) {
+            if (mt >= p / 2 && p + 1 < MB && 2 * mt + 1 > p) {            // the tile holds rows below the diagonal block
                 Tile x;
                 split_tile(x, nS.v[mt][p]);
                 float d[4];
@@ -290,12 +306,15 @@ __device__ __forceinline__ int factor(Mat<MB, MB>& nS, Mat<NB, MB>& nY, Split<NB
             }
         }
 #pragma unroll
-        for (int q = p + 1; q < MB; ++q) {
+        for (int q = 1; q < MB; ++q) {
+            if (q <= p)
+                continue;
             const int e = 2 * (q & 1);
-            const Tile& y = lt[q / 2];
+            const Tile y = lt[q / 2];
 #pragma unroll
-            for (int mt = q / 2; mt < Mat<MB, MB>::MT; ++mt)
-                mma3(nS.v[mt][q], lt[mt], y.h[e], y.h[e + 1], y.l[e], y.l[e + 1]);
+            for (int mt = 0; mt < Mat<MB, MB>::MT; ++mt)
+                if (mt >= q / 2)
+                    mma3(nS.v[mt][q], lt[mt], y.h[e], y.h[e + 1], y.l[e], y.l[e + 1]);
 #pragma unroll
             for (int mt = 0; mt < Mat<NB, MB>::MT; ++mt) {
                 Tile x;
@@ -320,7 +339,9 @@ __device__ __forceinline__ void gains(Mat<NB, MB>& zt, const Mat<MB, MB>& L, con
 #pragma unroll
     for (int p = MB - 1; p >= 0; --p) {
 #pragma unroll
-        for (int q = p + 1; q < MB; ++q) {
+        for (int q = 1; q < MB; ++q) {
+            if (q <= p)
+                continue;
             float y0, y1;
             transpose8(y0, y1, L.v[q / 2][p][2 * (q & 1)], L.v[q / 2][p][2 * (q & 1) + 1], lane);
             uint32_t h0, h1, l0, l1;
@@ -371,7 +392,7 @@ __device__ __forceinline__ void keep(Stored<RB, CB>& st, const Mat<RB, CB>& m, i
         }
 }
 // d = c + X * Y' with X stored
-template <int RB, int KB, int CB>
+template <int RB, int KB, int CB, bool LOWER = false>
 __device__ __forceinline__ void product(Mat<RB, CB>& d, const Mat<RB, CB>* c, const Stored<RB, KB>& x, const Split<CB, KB>& y, int lane)
 {
     const float z[4] = {0.f, 0.f, 0.f, 0.f};
@@ -389,6 +410,8 @@ __device__ __forceinline__ void product(Mat<RB, CB>& d, const Mat<RB, CB>* c, co
             for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
                 for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
+                    if (LOWER && cb > 2 * mt + 1)
+                        continue;
                     const uint4 v = a[mt][pass == 0];
                     const uint32_t(&b)[4] = pass == 1 ? y.l[cb / 2][kb] : y.h[cb / 2][kb];
                     const uint32_t b0 = b[2 * (cb & 1)], b1 = b[2 * (cb & 1) + 1];
@@ -401,6 +424,21 @@ __device__ __forceinline__ void product(Mat<RB, CB>& d, const Mat<RB, CB>* c, co
                 }
     }
 }
+// the float32 matrix back from its parts (exact)
+template <int RB, int CB>
+__device__ __forceinline__ void unkeep(Mat<RB, CB>& m, const Stored<RB, CB>& st, int lane)
+{
+#pragma unroll
+    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb) {
+            const uint4 h = st.q[mt][cb][0][lane], l = st.q[mt][cb][1][lane];
+            m.v[mt][cb][0] = __uint_as_float(h.x) + __uint_as_float(l.x);
+            m.v[mt][cb][2] = __uint_as_float(h.y) + __uint_as_float(l.y);
+            m.v[mt][cb][1] = __uint_as_float(h.z) + __uint_as_float(l.z);
+            m.v[mt][cb][3] = __uint_as_float(h.w) + __uint_as_float(l.w);
+        }
+}
 // d = c + X X' with a result that is symmetric bit for bit when c is: lo*hi and hi*lo start from zero, so that one is the
 // transpose of the other, and are added to each other first
 template <int NB, int KB>
@@ -412,6 +450,8 @@ __device__ __forceinline__ void product_symmetric(Mat<NB, NB>& d, const Split<NB
     for (int cb = 0; cb < NB; ++cb)
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
+            if (cb > 2 * mt + 1)
+                continue;                                  // lower tiles only: mirror() fills the rest
             float e1[4], e2[4];
 #pragma unroll
             for (int kb = 0; kb < KB; ++kb) {

@@ -171,7 +171,7 @@ __device__ __forceinline__ int backward(Mat<NB, NB>& nP, Slot<NB>& sl, const Rat
         {
             Split<NB, NB> vs;
             split(vs, V);
-            product<NB, NB, NB>(S, nullptr, sl.B, vs, lane);         // Bbar' V'
+            product<NB, NB, NB, true>(S, nullptr, sl.B, vs, lane);         // Bbar' V'
         }
         transpose<NB>(Zt, V, lane);
 #pragma unroll
@@ -182,7 +182,9 @@ __device__ __forceinline__ int backward(Mat<NB, NB>& nP, Slot<NB>& sl, const Rat
                 for (int e = 0; e < 4; ++e) {
                     const int b = 2 * mt + (e >> 1);
                     Zt.v[mt][cb][e] *= ar[b];               // -Y' = A V'
-                    // -S = G Bbar' V' - R
+                    // -S = G Bbar' V' - R (lower tiles)
+                    if (cb > 2 * mt + 1)
+                        continue;
                     if (cb == b)
                         S.v[mt][cb][e] = fmaf(S.v[mt][cb][e], gr[b], t == (g >> 1) && (e & 1) == (g & 1) ? -rd[b] : 0.f);
                     else
@@ -217,6 +219,7 @@ __device__ __forceinline__ int backward(Mat<NB, NB>& nP, Slot<NB>& sl, const Rat
         if (bad && !fail)
             fail = s * N + bad;
         product_symmetric<NB, NB>(nP, zs);
+        mirror<NB>(nP, lane);
         on_step(s, Zt, S, w);
     }
     return fail;

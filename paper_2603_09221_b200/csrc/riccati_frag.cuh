@@ -1,17 +1,21 @@
-// Riccati-backward + rollout kernel for n, m <= 16, float32: one WARP per instance, every matrix of the step in registers
-// in the mma.sync accumulator layout (frag.cuh), so that a step is a chain of tensor-core products, two or one
-// eight-column factorisation panels and a few shuffles, without shared memory and without barriers.
+// Riccati-backward + rollout kernel, float32, for n, m up to 32 (any request) or 48 (time-invariant): one WARP per
+// instance, every matrix of the step in registers in the mma.sync accumulator layout (frag.cuh), so that a step is a
+// chain of tensor-core products, one eight-column factorisation panel per block of controls and a few shuffles, without
+// barriers.  Other sizes than whole blocks are padded: R with the identity, everything else with zero.
 //
 // The recursion is carried in negated variables (nP = -P etc.): every update is then a plain accumulation.
 //   V = B' nP,  T = A' nP,  nS = -R + B' V',  nY' = A' V',  nP_t = -Q + A' T' + Z' Z     (Prop. 3.1; Alg. 1)
 // with S = L L', Z = L^{-1} Y and, when gains are wanted, K' = -Z' L^{-1} from the inverses of L's diagonal blocks.
 //
-// What bounds it: a step is 87 tensor-core instructions (8 cycles each on a scheduler's pipe) in about 830, and four
-// warps per scheduler (128 registers) hide most of the chain of five products and sixteen pivots.  Columns of the
-// matrices spread over the lanes of a warp with rows broadcast from shared memory (the form this replaced) ran at 88 %
-// of the load/store pipe and 4.3 us per step for a single instance; this one takes about 2 us.
-// 65536 instances, H = 32, operands from memory: 4.26 -> 2.84 ms (tensor pipe 46 %, issue slots 55 %); 4096 instances,
-// H = 16, all outputs: 188 -> 109 us; 64 instances of n = m = 8, H = 8: 107 -> 22 us (generic kernel before).
+// What bounds it: at n = 16 a step is 87 tensor-core instructions (8 cycles on a scheduler's pipe, about 4 of its issue
+// slots) in about 830, and four or five warps per scheduler hide most of the chain of five products and sixteen pivots.
+// At n = 32 it is 670 tensor-core instructions, two warps per scheduler (all 255 registers); above, registers spill to
+// local memory (0.3 KB per lane at 40 x 16, 2.6 KB at 40 x 40), which the first-level cache absorbs.
+// The forms this replaced: rows broadcast from shared memory at n = 16 (load/store pipe at 88 %), products through shared
+// memory at n = 32 (74 %), one CTA per instance with two barriers per pivot elsewhere.  Measured before -> now:
+//   65536 instances n = 16, H = 32, operands from memory  4.26 -> 2.65 ms     4096, n = 16, H = 16, all outputs 188 -> 107 us
+//   16384 instances n = 32, H = 64, all outputs           14.2 -> 8.5 ms      1155, n = 40, m = 12, H = 20     2428 -> 232 us
+//   64 instances n = 8, H = 8, own dynamics               107 -> 23 us
 #pragma once
 
 #include "common.cuh"
@@ -43,30 +47,31 @@ __device__ __forceinline__ Place place(const SolveParams& p, unsigned w)
     return r;
 }
 
-// ---- operands of one time step of one instance, staged in the warp's shared memory by asynchronous copies one step
-// ahead of their use: the registers they would occupy for a whole step go to a fifth CTA per SM instead.
-// A and B are read transposed (lane (g, t) takes row 2 t, column g): with rows of 8 NB + 4 floats the 32 lanes fall into
-// 32 banks.  Q and R are read as pairs along the rows (20 floats per row: five CTAs with two buffers each fit an SM).
+// ---- operands of one time step of one instance, staged in the warp's shared memory by asynchronous copies ahead of
+// their use.  A and B are read transposed (lane (g, t) takes row 2 t, column g): with rows of 8 k + 4 floats the 32 lanes
+// fall into 32 banks.  Q and R are read as pairs along the rows.
+constexpr int pair_stride(int blocks) { return 8 * blocks + (blocks == 2 ? 4 : blocks % 2 ? 0 : 8); }
 template <int NB, int MB>
 struct Operands {
-    static constexpr int LA = 8 * NB + 4, LB = 8 * MB + 4, LQ = NB == 1 ? 8 : 20, LR = MB == 1 ? 8 : 20;
+    static constexpr int LA = 8 * NB + 4, LB = 8 * MB + 4, LQ = pair_stride(NB), LR = pair_stride(MB);
     float A[8 * NB * LA], B[8 * NB * LB], Q[8 * NB * LQ], R[8 * MB * LR];
 };
-// time-invariant form: A' and B' once more, split and in register order
-template <int NB, int MB>
-struct Fixed {
-    Stored<NB, NB> A;
-    Stored<MB, NB> B;
-};
-// what a warp keeps in shared memory
-template <int NB, int MB, bool TV>
+// What a warp keeps in shared memory.  Time-varying and n <= 16: two buffers in turn, A and B split in registers in every
+// step.  Otherwise A' and B' are split once per change and kept in register order; the raw matrices pass through the same
+// place.  (For n = 32 a second buffer does not fit, and the splits of five products cost more than storing them.)
+template <int NB, int MB, bool TWO>
 struct WarpMem {
     Operands<NB, MB> op[2];
 };
 template <int NB, int MB>
 struct WarpMem<NB, MB, false> {
-    Operands<NB, MB> op[1];
-    Fixed<NB, MB> fixed;
+    using Ops = Operands<NB, MB>;
+    Stored<NB, NB> A;
+    Stored<MB, NB> B;
+    float Q[8 * NB * Ops::LQ], R[8 * MB * Ops::LR];
+    __device__ __forceinline__ float* rawA() { return reinterpret_cast<float*>(&A); }
+    __device__ __forceinline__ float* rawB() { return reinterpret_cast<float*>(&B); }
+    static_assert(sizeof(Stored<NB, NB>) >= sizeof(Ops::A) && sizeof(Stored<MB, NB>) >= sizeof(Ops::B), "raw operand does not fit");
 };
 
 __device__ __forceinline__ void copy16(float* dst, const float* src)
@@ -109,9 +114,9 @@ __device__ __forceinline__ void stage(float* dst, const OperandDev& o, long long
             copy16(dst + (e / (2 * CB)) * LD + 4 * (e % (2 * CB)), src + 4 * e);
     }
 }
-// X = M' from shared memory
-template <int RB, int CB, int LD>
-__device__ __forceinline__ void load_transposed(Mat<RB, CB>& x, const float* M, int lane)
+// X = M' from shared memory (with PAD: zero outside the nk x ni matrix)
+template <int RB, int CB, int LD, bool PAD>
+__device__ __forceinline__ void load_transposed(Mat<RB, CB>& x, const float* M, int nk, int ni, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -119,8 +124,13 @@ __device__ __forceinline__ void load_transposed(Mat<RB, CB>& x, const float* M, 
 #pragma unroll
         for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                x.v[mt][cb][e] = e >= 2 && 2 * mt + 1 >= RB ? 0.f : M[(8 * cb + 2 * t + (e & 1)) * LD + 16 * mt + g + ((e & 2) ? 8 : 0)];
+            for (int e = 0; e < 4; ++e) {
+                const int i = 16 * mt + g + ((e & 2) ? 8 : 0), k = 8 * cb + 2 * t + (e & 1);
+                if (e >= 2 && 2 * mt + 1 >= RB)
+                    x.v[mt][cb][e] = 0.f;
+                else
+                    x.v[mt][cb][e] = PAD && !(i < ni && k < nk) ? 0.f : M[k * LD + i];
+            }
 }
 // x = -M of a square matrix in shared memory
 template <int RB, int LD>
@@ -192,41 +202,35 @@ __device__ __forceinline__ void store_gain(float* base, long long off, const Mat
             }
 }
 
-// `cnt` = 4 W consecutive elements of a row (16-byte loads), or with PAD element by element within [0, n)
+// W consecutive elements of a row (16-byte loads), or with PAD element by element within [0, n)
 template <int W, bool PAD>
-__device__ __forceinline__ void load_half_row(float (&v)[4 * W], const float* row, int c0, int n)
+__device__ __forceinline__ void load_part(float (&v)[W], const float* row, int c0, int n)
 {
     if (PAD) {
 #pragma unroll
-        for (int k = 0; k < 4 * W; ++k)
+        for (int k = 0; k < W; ++k)
             v[k] = c0 + k < n ? row[c0 + k] : 0.f;
     } else {
 #pragma unroll
-        for (int q = 0; q < W; ++q) {
+        for (int q = 0; q < W / 4; ++q) {
             const float4 f = *reinterpret_cast<const float4*>(row + c0 + 4 * q);
             v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
         }
     }
 }
 
-struct Scratch {
-    float x[16], u[16];
-};
-
 // NB, MB: number of 8-blocks of the state and the control dimension.
 // TV = time-varying request (time strides or a terminal weight); AFF = linear control cost r_t'u_t (implies TV);
 // PAD = n < 8 NB or m < 8 MB, or strides that do not keep the vector loads aligned: guarded element-wise accesses, the
 // missing part of R is the identity and everything else zero, which leaves the recursion of the existing part untouched.
 template <int NB, int MB, bool TV, bool AFF, bool PAD>
-__global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_frag_kernel(SolveParams p)
+__global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 4) riccati_frag_kernel(SolveParams p)
 {
-    __shared__ __align__(16) Scratch scratch[MAX_WARPS];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const long long widx = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (widx >= p.b0 * p.b1 * p.tcount)
         return;
-    Scratch& sc = scratch[threadIdx.x >> 5];
     const Place pl = place(p, (unsigned)widx);
     const long long inst = pl.inst;
     const int n = PAD ? p.n : 8 * NB, m = PAD ? p.m : 8 * MB, H = p.H, obf = p.out_bf16;
@@ -237,46 +241,53 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_fr
     const long long Koff = inst * (long long)H * m * n;
     const long long Poff = inst * (long long)(p.first_only ? 1 : H + 1) * n * n;
     using Ops = Operands<NB, MB>;
-    WarpMem<NB, MB, TV>* const ops = reinterpret_cast<WarpMem<NB, MB, TV>*>(smem_raw) + (threadIdx.x >> 5);
+    constexpr bool TWO = TV && NB <= 2;
+    using Mem = WarpMem<NB, MB, TWO>;
+    Mem& mem = reinterpret_cast<Mem*>(smem_raw)[threadIdx.x >> 5];
     const long long oA = pl.off(p.A), oB = pl.off(p.B), oR = pl.off(p.R), oQ = pl.off(p.Q);
     Mat<NB, NB> nP;
+    if constexpr (PAD) {                                    // what does not exist: R is the identity, the rest zero
+        for (int e = lane; e < (int)(sizeof(Mem) / sizeof(float)); e += 32)
+            reinterpret_cast<float*>(&mem)[e] = 0.f;
+        __syncwarp();
+        for (int i = m + lane; i < 8 * MB; i += 32) {
+            if constexpr (TWO)
+                mem.op[0].R[i * Ops::LR + i] = mem.op[1].R[i * Ops::LR + i] = 1.f;
+            else
+                mem.R[i * Ops::LR + i] = 1.f;
+        }
+    }
     {
-        if (PAD) {                                          // what does not exist: R is the identity, the rest zero
-            for (int e = lane; e < (int)(sizeof(Ops) / sizeof(float)) * (TV ? 2 : 1); e += 32)
-                reinterpret_cast<float*>(ops->op)[e] = 0.f;
-            __syncwarp();
-            for (int i = m + lane; i < 8 * MB; i += 32) {
-                ops->op[0].R[i * Ops::LR + i] = 1.f;
-                if (TV)
-                    ops->op[1].R[i * Ops::LR + i] = 1.f;
+        const long long last = TV ? H - 1 : 0;
+        if constexpr (TWO) {
+            if (p.Qf.ptr) {                                 // P_H = Q_f, by way of the second buffer
+                stage<NB, NB, Ops::LQ, PAD>(mem.op[1].Q, p.Qf, pl.off(p.Qf), n, n, lane);
+                copies_landed();
+                load_negated<NB, Ops::LQ>(nP, mem.op[1].Q, lane);
+                __syncwarp();
+            }
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {                   // the second buffer: what does not change with time
+                if (b == 0 || !p.A.st) stage<NB, NB, Ops::LA, PAD>(mem.op[b].A, p.A, oA + last * p.A.st, n, n, lane);
+                if (b == 0 || !p.B.st) stage<NB, MB, Ops::LB, PAD>(mem.op[b].B, p.B, oB + last * p.B.st, n, m, lane);
+                if (b == 0 || !p.R.st) stage<MB, MB, Ops::LR, PAD>(mem.op[b].R, p.R, oR + last * p.R.st, m, m, lane);
+                if (b == 0 || !p.Q.st) stage<NB, NB, Ops::LQ, PAD>(mem.op[b].Q, p.Q, oQ + last * p.Q.st, n, n, lane);
+            }
+            copies_landed();
+            if (!p.Qf.ptr)
+                load_negated<NB, Ops::LQ>(nP, mem.op[0].Q, lane);
+        } else {
+            stage<NB, NB, Ops::LQ, PAD>(mem.Q, TV && p.Qf.ptr ? p.Qf : p.Q, TV && p.Qf.ptr ? pl.off(p.Qf) : oQ + last * p.Q.st, n, n, lane);
+            stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + last * p.A.st, n, n, lane);
+            stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + last * p.B.st, n, m, lane);
+            stage<MB, MB, Ops::LR, PAD>(mem.R, p.R, oR + last * p.R.st, m, m, lane);
+            copies_landed();
+            load_negated<NB, Ops::LQ>(nP, mem.Q, lane);     // P_H = Q_f or Q
+            if (TV && p.Qf.ptr) {
+                __syncwarp();
+                stage<NB, NB, Ops::LQ, PAD>(mem.Q, p.Q, oQ + last * p.Q.st, n, n, lane);
             }
         }
-        const long long last = TV ? H - 1 : 0;
-        if (TV && p.Qf.ptr) {                               // P_H = Q_f, by way of the second buffer
-            stage<NB, NB, Ops::LQ, PAD>(ops->op[TV].Q, p.Qf, pl.off(p.Qf), n, n, lane);
-            copies_landed();
-            load_negated<NB, Ops::LQ>(nP, ops->op[TV].Q, lane);
-            __syncwarp();
-        }
-#pragma unroll
-        for (int b = 0; b < (TV ? 2 : 1); ++b) {            // the second buffer: what does not change with time
-            if (b == 0 || !p.A.st) stage<NB, NB, Ops::LA, PAD>(ops->op[b].A, p.A, oA + last * p.A.st, n, n, lane);
-            if (b == 0 || !p.B.st) stage<NB, MB, Ops::LB, PAD>(ops->op[b].B, p.B, oB + last * p.B.st, n, m, lane);
-            if (b == 0 || !p.R.st) stage<MB, MB, Ops::LR, PAD>(ops->op[b].R, p.R, oR + last * p.R.st, m, m, lane);
-            if (b == 0 || !p.Q.st) stage<NB, NB, Ops::LQ, PAD>(ops->op[b].Q, p.Q, oQ + last * p.Q.st, n, n, lane);
-        }
-        copies_landed();
-        if constexpr (!TV) {
-            Mat<NB, NB> At;
-            Mat<MB, NB> Bt;
-            load_transposed<NB, NB, Ops::LA>(At, ops->op[0].A, lane);
-            load_transposed<MB, NB, Ops::LB>(Bt, ops->op[0].B, lane);
-            keep(ops->fixed.A, At, lane);
-            keep(ops->fixed.B, Bt, lane);
-            __syncwarp();
-        }
-        if (!(TV && p.Qf.ptr))
-            load_negated<NB, Ops::LQ>(nP, ops->op[0].Q, lane);  // P_H = Q
     }
     if (p.P && !p.first_only)
         store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, n, obf, lane);
@@ -300,49 +311,81 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_fr
     int fail = 0;
 #pragma unroll 1
     for (int ts = H - 1; ts >= 0; --ts) {
-        const Ops& op = ops->op[TV ? (H - 1 - ts) & 1 : 0];
-        if (TV && ts < H - 1)
-            copies_landed();                                // also: every lane is done with the other buffer
-        if (TV && ts > 0) {                                 // operands of the next step
-            Ops& nx = ops->op[(H - ts) & 1];
-            if (p.A.st) stage<NB, NB, Ops::LA, PAD>(nx.A, p.A, oA + (ts - 1) * p.A.st, n, n, lane);
-            if (p.B.st) stage<NB, MB, Ops::LB, PAD>(nx.B, p.B, oB + (ts - 1) * p.B.st, n, m, lane);
-            if (p.R.st) stage<MB, MB, Ops::LR, PAD>(nx.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
-            if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(nx.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
-        }
         Mat<NB, NB> At, T;
         Mat<MB, NB> Bt, V;
         Mat<NB, MB> Zt;
         Mat<MB, MB> S, nR;
-        load_negated<MB, Ops::LR>(nR, op.R, lane);
-        Split<NB, NB> ps;
-        Split<MB, NB> vs;
-        split(ps, nP);
-        if constexpr (TV) {
-            load_transposed<NB, NB, Ops::LA>(At, op.A, lane);
-            load_transposed<MB, NB, Ops::LB>(Bt, op.B, lane);
-            Split<NB, NB> as;
-            Split<MB, NB> bs;
+        if constexpr (TWO) {
+            const Ops& op = mem.op[(H - 1 - ts) & 1];
+            if (ts < H - 1)
+                copies_landed();                            // also: every lane is done with the other buffer
+            if (ts > 0) {                                   // operands of the next step
+                Ops& nx = mem.op[(H - ts) & 1];
+                if (p.A.st) stage<NB, NB, Ops::LA, PAD>(nx.A, p.A, oA + (ts - 1) * p.A.st, n, n, lane);
+                if (p.B.st) stage<NB, MB, Ops::LB, PAD>(nx.B, p.B, oB + (ts - 1) * p.B.st, n, m, lane);
+                if (p.R.st) stage<MB, MB, Ops::LR, PAD>(nx.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
+                if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(nx.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
+            }
+            load_negated<MB, Ops::LR>(nR, op.R, lane);
+            load_transposed<NB, NB, Ops::LA, false>(At, op.A, n, n, lane);
+            load_transposed<MB, NB, Ops::LB, false>(Bt, op.B, n, m, lane);
+            Split<NB, NB> as, ps;
+            Split<MB, NB> bs, vs;
+            split(ps, nP);
             split(as, At);
             split(bs, Bt);
             product<MB, NB, NB>(V, nullptr, bs, ps);        // V = B' nP
             product<NB, NB, NB>(T, nullptr, as, ps);        // T = A' nP
             split(vs, V);
-            product<MB, NB, MB>(S, &nR, bs, vs);            // -S = -R + B' V'
+            product<MB, NB, MB, true>(S, &nR, bs, vs);      // -S = -R + B' V'
             product<NB, NB, MB>(Zt, nullptr, as, vs);       // -Y' = A' V'
             split(ps, T);
             load_negated<NB, Ops::LQ>(nP, op.Q, lane);
-            product<NB, NB, NB>(nP, &nP, as, ps);           // -Q - A'P A
+            product<NB, NB, NB, true>(nP, &nP, as, ps);     // -Q - A'P A
         } else {
-            const Fixed<NB, MB>& fx = ops->fixed;
-            product<MB, NB, NB>(V, nullptr, fx.B, ps, lane);
-            product<NB, NB, NB>(T, nullptr, fx.A, ps, lane);
-            split(vs, V);
-            product<MB, NB, MB>(S, &nR, fx.B, vs, lane);
-            product<NB, NB, MB>(Zt, nullptr, fx.A, vs, lane);
-            split(ps, T);
-            load_negated<NB, Ops::LQ>(nP, op.Q, lane);
-            product<NB, NB, NB>(nP, &nP, fx.A, ps, lane);
+            if (TV || ts == H - 1)
+                copies_landed();
+            if (ts == H - 1 || (TV && p.A.st)) {            // raw -> split, in place
+                load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
+                __syncwarp();
+                keep(mem.A, At, lane);
+            }
+            if (ts == H - 1 || (TV && p.B.st)) {
+                load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
+                __syncwarp();
+                keep(mem.B, Bt, lane);
+            }
+            __syncwarp();
+            load_negated<MB, Ops::LR>(nR, mem.R, lane);
+            {
+                Split<NB, NB> ps;
+                split(ps, nP);
+                product<MB, NB, NB>(V, nullptr, mem.B, ps, lane);
+                product<NB, NB, NB>(T, nullptr, mem.A, ps, lane);
+            }
+            {
+                Split<MB, NB> vs;
+                split(vs, V);
+                product<MB, NB, MB, true>(S, &nR, mem.B, vs, lane);
+                product<NB, NB, MB>(Zt, nullptr, mem.A, vs, lane);
+            }
+            load_negated<NB, Ops::LQ>(nP, mem.Q, lane);
+            {
+                Split<NB, NB> tsp;
+                split(tsp, T);
+                product<NB, NB, NB, true>(nP, &nP, mem.A, tsp, lane);
+            }
+            if (AFF && ts < p.r_count) {                    // the float32 operands once more, for the vector recursion
+                unkeep(At, mem.A, lane);
+                unkeep(Bt, mem.B, lane);
+            }
+            if (TV && ts > 0) {                             // operands of the next step, in flight while this one is factored
+                __syncwarp();
+                if (p.A.st) stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + (ts - 1) * p.A.st, n, n, lane);
+                if (p.B.st) stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + (ts - 1) * p.B.st, n, m, lane);
+                if (p.R.st) stage<MB, MB, Ops::LR, PAD>(mem.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
+                if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(mem.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
+            }
         }
         float gr[MB], ap[NB];                               // affine: B'p + r and A'p in row form
         if (AFF && ts < p.r_count) {
@@ -373,7 +416,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_fr
         const int bad = factor<NB, MB>(S, Zt, zs, w, lane);  // Zt becomes Z', S the blocks of L
         if (bad && !fail)
             fail = ts * m + bad;
-        product<NB, MB, NB>(nP, &nP, zs, zs);                              // -P_t = -Q - A'PA + Z'Z
+        product<NB, MB, NB, true>(nP, &nP, zs, zs);                              // -P_t = -Q - A'PA + Z'Z
         const bool gain = need_K_all || need_k_all || (want_u0 && ts == 0);
         if (AFF) {
             // z = L^{-1}(B'p + r);  p_t = A'p - Z'z;  k_t = -L^{-T} z   (all zero while p and r are)
@@ -497,102 +540,181 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, TV && !AFF ? 5 : 4) riccati_fr
     if (want_u0 || !(p.x || p.u))
         return;
 
-    // ---- forward loop of Alg. 1: two lanes per row, the vectors in the warp's scratch; the rows of K_{t+1} (and of
-    // A_{t+1}, B_{t+1}) are in flight while step t is summed
+    // ---- forward loop of Alg. 1: LPR lanes per row and RPL rows per lane, the vectors in the warp's memory (whose
+    // operands are no longer needed); the rows of K_{t+1} (and of A_{t+1}, B_{t+1}) are in flight while step t is summed
+    constexpr int D = 8 * (NB > MB ? NB : MB), LPR = D <= 16 ? 2 : 1, RPL = D <= 32 ? 1 : 2, WN = 8 * NB / LPR, WM = 8 * MB / LPR;
+    static_assert(D <= 64, "rows");
     const float* Ag = reinterpret_cast<const float*>(p.A.ptr) + oA;
     const float* Bg = reinterpret_cast<const float*>(p.B.ptr) + oB;
-    const int i = lane >> 1, c0n = (lane & 1) * 4 * NB, c0m = (lane & 1) * 4 * MB;
-    if ((lane & 1) == 0) {
-        sc.x[i] = (i < n && p.x0.ptr) ? load_elem(p.x0, pl.off(p.x0) + i) : 0.f;
-        sc.u[i] = 0.f;
+    float* const sx = reinterpret_cast<float*>(&mem);
+    float* const su = sx + 64;
+    const int row0 = lane / LPR, c0n = (lane % LPR) * WN, c0m = (lane % LPR) * WM;
+    const bool writer = lane % LPR == 0;
+    float x0v[RPL];
+#pragma unroll
+    for (int q = 0; q < RPL; ++q) {
+        const int i = row0 + 32 * q;
+        x0v[q] = (i < n && p.x0.ptr) ? load_elem(p.x0, pl.off(p.x0) + i) : 0.f;
     }
     __syncwarp();                                           // also: K_t stored by the other lanes are visible
-    const bool xo = p.x && (lane & 1) == 0 && i < n, uo = p.u && (lane & 1) == 0 && i < m;
-    const long long xoff = inst * (long long)(H + 1) * n + i, uoff = inst * (long long)(p.first_only ? m : H * m) + i;
-    const int ri = i < n ? i : 0, rj = i < m ? i : 0;
-    const float* Kr = Kbase + Koff + (long long)rj * n;
-    float kr[4 * NB], ar[4 * NB], br[4 * MB], kt = 0.f;
-    load_half_row<NB, PAD>(kr, Kr, c0n, n);
-    load_half_row<NB, PAD>(ar, Ag + ri * n, c0n, n);
-    load_half_row<MB, PAD>(br, Bg + ri * m, c0m, m);
-    if (AFF && p.kff)
-        kt = p.kff[inst * (long long)H * m + rj];
-    else if (AFF) {                                         // only u_0 is wanted: k_0 is still in registers
 #pragma unroll
-        for (int b = 0; b < MB; ++b) {
-            const float e0 = __shfl_sync(FULL, kc0[b][0], (i & 7) >> 1), e1 = __shfl_sync(FULL, kc0[b][1], (i & 7) >> 1);
-            if (i / 8 == b)
-                kt = (i & 1) ? e1 : e0;
+    for (int q = 0; q < RPL; ++q)
+        if (writer) {
+            sx[row0 + 32 * q] = x0v[q];
+            su[row0 + 32 * q] = 0.f;
+        }
+    __syncwarp();
+    const float* Kr = Kbase + Koff;
+    float kr[RPL][WN], ar[RPL][WN], br[RPL][WM], kt[RPL];
+    auto load_rows = [&](int ts, bool dynamics) {
+#pragma unroll
+        for (int q = 0; q < RPL; ++q) {
+            const int i = row0 + 32 * q, ri = i < n ? i : 0, rj = i < m ? i : 0;
+            load_part<WN, PAD>(kr[q], Kr + ((long long)ts * m + rj) * n, c0n, n);
+            if (dynamics || (TV && p.A.st)) load_part<WN, PAD>(ar[q], Ag + ts * p.A.st + ri * n, c0n, n);
+            if (dynamics || (TV && p.B.st)) load_part<WM, PAD>(br[q], Bg + ts * p.B.st + ri * m, c0m, m);
+            if (AFF && p.kff)
+                kt[q] = p.kff[(inst * H + ts) * (long long)m + rj];
+        }
+    };
+    load_rows(0, true);
+    if (AFF && !p.kff) {                                    // only u_0 is wanted: k_0 is still in registers
+#pragma unroll
+        for (int q = 0; q < RPL; ++q) {
+            const int i = row0 + 32 * q;
+            kt[q] = 0.f;
+#pragma unroll
+            for (int b = 0; b < MB; ++b) {
+                const float e0 = __shfl_sync(FULL, kc0[b][0], (i & 7) >> 1), e1 = __shfl_sync(FULL, kc0[b][1], (i & 7) >> 1);
+                if (i / 8 == b)
+                    kt[q] = (i & 1) ? e1 : e0;
+            }
         }
     }
     const int steps = (p.x || !p.first_only) ? H : 1;
-    if (xo)
-        store_out(p.x, xoff, sc.x[i], obf);
+    const long long xoff = inst * (long long)(H + 1) * n, uoff = inst * (long long)(p.first_only ? m : H * m);
+#pragma unroll
+    for (int q = 0; q < RPL; ++q)
+        if (p.x && writer && row0 + 32 * q < n)
+            store_out(p.x, xoff + row0 + 32 * q, x0v[q], obf);
 #pragma unroll 1
     for (int ts = 0; ts < steps; ++ts) {
-        float xv[4 * NB], uv[4 * MB];
-        load_half_row<NB, false>(xv, sc.x, c0n, 16);
-        float us = 0.f, xs = 0.f;
+        float us[RPL], xs[RPL];
+        {
+            float xv[WN];
+            load_part<WN, false>(xv, sx, c0n, 64);
 #pragma unroll
-        for (int k = 0; k < 4 * NB; ++k) {
-            us = fmaf(kr[k], xv[k], us);
-            xs = fmaf(ar[k], xv[k], xs);
+            for (int q = 0; q < RPL; ++q) {
+                us[q] = xs[q] = 0.f;
+#pragma unroll
+                for (int k = 0; k < WN; ++k) {
+                    us[q] = fmaf(kr[q][k], xv[k], us[q]);
+                    xs[q] = fmaf(ar[q][k], xv[k], xs[q]);
+                }
+            }
         }
-        us += __shfl_xor_sync(FULL, us, 1);
-        if (AFF)
-            us += kt;
-        if ((lane & 1) == 0)
-            sc.u[i] = i < m ? us : 0.f;
-        if (uo && (!p.first_only || ts == 0))
-            store_out(p.u, uoff + (p.first_only ? 0 : (long long)ts * m), us, obf);
+#pragma unroll
+        for (int q = 0; q < RPL; ++q) {
+            const int i = row0 + 32 * q;
+            if (LPR == 2)
+                us[q] += __shfl_xor_sync(FULL, us[q], 1);
+            if (AFF)
+                us[q] += kt[q];
+            if (writer) {
+                su[i] = i < m ? us[q] : 0.f;
+                if (p.u && i < m && (!p.first_only || ts == 0))
+                    store_out(p.u, uoff + (p.first_only ? 0 : (long long)ts * m) + i, us[q], obf);
+            }
+        }
         __syncwarp();
-        load_half_row<MB, false>(uv, sc.u, c0m, 16);
+        {
+            float uv[WM];
+            load_part<WM, false>(uv, su, c0m, 64);
 #pragma unroll
-        for (int k = 0; k < 4 * MB; ++k)
-            xs = fmaf(br[k], uv[k], xs);
-        if (ts + 1 < steps) {
-            load_half_row<NB, PAD>(kr, Kr + (long long)(ts + 1) * m * n, c0n, n);
-            if (TV && p.A.st) load_half_row<NB, PAD>(ar, Ag + (ts + 1) * p.A.st + ri * n, c0n, n);
-            if (TV && p.B.st) load_half_row<MB, PAD>(br, Bg + (ts + 1) * p.B.st + ri * m, c0m, m);
-            if (AFF && p.kff)
-                kt = p.kff[(inst * H + ts + 1) * (long long)m + rj];
+            for (int q = 0; q < RPL; ++q)
+#pragma unroll
+                for (int k = 0; k < WM; ++k)
+                    xs[q] = fmaf(br[q][k], uv[k], xs[q]);
         }
-        xs += __shfl_xor_sync(FULL, xs, 1);
-        if ((lane & 1) == 0)
-            sc.x[i] = i < n ? xs : 0.f;
-        if (xo)
-            store_out(p.x, xoff + (long long)(ts + 1) * n, xs, obf);
+        if (ts + 1 < steps)
+            load_rows(ts + 1, false);
+#pragma unroll
+        for (int q = 0; q < RPL; ++q) {
+            const int i = row0 + 32 * q;
+            if (LPR == 2)
+                xs[q] += __shfl_xor_sync(FULL, xs[q], 1);
+            if (writer) {
+                sx[i] = i < n ? xs[q] : 0.f;
+                if (p.x && i < n)
+                    store_out(p.x, xoff + (long long)(ts + 1) * n + i, xs[q], obf);
+            }
+        }
         __syncwarp();
     }
 }
 
-// Launch for n, m <= 16.  `exact`: the strides keep the vector loads aligned (rows of Q, Qf, R and of K, A, B in the
-// rollout).  Few instances get a CTA each so that they spread over the SMs.
+template <int NB, int MB, bool TV, bool AFF, bool PAD>
+inline cudaError_t launch_one(const SolveParams& p, int sm_count, cudaStream_t st)
+{
+    // up to 16 states a CTA is four warps, unless the instances are so few that one warp each spreads them over more SMs;
+    // above, the operands of a warp fill 7 to 60 KB and CTAs of one warp pack best
+    const long long nwin = p.b0 * p.b1 * p.tcount;
+    const int warps = NB > 2 || nwin <= 4ll * sm_count ? 1 : MAX_WARPS;
+    const size_t smem = warps * sizeof(WarpMem<NB, MB, TV && NB <= 2>);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(riccati_frag_kernel<NB, MB, TV, AFF, PAD>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess)
+            return e;
+    }
+    riccati_frag_kernel<NB, MB, TV, AFF, PAD><<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, smem, st>>>(p);
+    return cudaGetLastError();
+}
+
+// Sizes this kernel serves: up to 32 x 32 for every request, up to 48 x 48 for time-invariant ones.
+inline bool riccati_frag_serves(int n, int m, bool time_varying)
+{
+    const int top = time_varying ? 32 : 48;
+    return n <= top && m <= top;
+}
+
+// `exact`: the strides keep the vector loads aligned (rows of Q, Qf, R and of K, A, B in the rollout).  The number of
+// control blocks is instantiated where it saves work (a step's products are linear in it) and registers allow.
 inline cudaError_t launch_riccati_frag(const SolveParams& p, bool time_varying, bool affine, bool exact, int sm_count, cudaStream_t st)
 {
-    const long long nwin = p.b0 * p.b1 * p.tcount;
-    void (*kern)(SolveParams);
-    size_t per_warp = sizeof(WarpMem<2, 2, false>);
-    const bool sq8 = p.n <= 8 && p.m <= 8, m8 = p.m <= 8;
-    const bool pad8 = !(exact && p.n == 8 && p.m == 8), pad16 = !(exact && p.n == 16 && p.m == 16);
-    if (affine || time_varying) {
-        per_warp = sizeof(WarpMem<2, 2, true>);
-        if (affine)
-            kern = pad16 ? riccati_frag_kernel<2, 2, true, true, true> : riccati_frag_kernel<2, 2, true, true, false>;
-        else
-            kern = pad16 ? riccati_frag_kernel<2, 2, true, false, true> : riccati_frag_kernel<2, 2, true, false, false>;
-    } else if (sq8) {
-        kern = pad8 ? riccati_frag_kernel<1, 1, false, false, true> : riccati_frag_kernel<1, 1, false, false, false>;
-        per_warp = sizeof(WarpMem<1, 1, false>);
-    } else if (m8) {
-        kern = riccati_frag_kernel<2, 1, false, false, true>;
-        per_warp = sizeof(WarpMem<2, 1, false>);
-    } else {
-        kern = pad16 ? riccati_frag_kernel<2, 2, false, false, true> : riccati_frag_kernel<2, 2, false, false, false>;
+    const int nb = (p.n + 7) / 8, mb = (p.m + 7) / 8, kb = nb > mb ? nb : mb;
+    const bool full16 = exact && p.n == 16 && p.m == 16, full32 = exact && p.n == 32 && p.m == 32;
+    if (affine) {
+        if (kb <= 2)
+            return full16 ? launch_one<2, 2, true, true, false>(p, sm_count, st) : launch_one<2, 2, true, true, true>(p, sm_count, st);
+        return full32 ? launch_one<4, 4, true, true, false>(p, sm_count, st) : launch_one<4, 4, true, true, true>(p, sm_count, st);
     }
-    const int warps = nwin <= 4ll * sm_count ? 1 : MAX_WARPS;
-    kern<<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, warps * per_warp, st>>>(p);
-    return cudaGetLastError();
+    if (time_varying) {
+        if (kb <= 2)
+            return full16 ? launch_one<2, 2, true, false, false>(p, sm_count, st) : launch_one<2, 2, true, false, true>(p, sm_count, st);
+        return full32 ? launch_one<4, 4, true, false, false>(p, sm_count, st) : launch_one<4, 4, true, false, true>(p, sm_count, st);
+    }
+    switch (kb) {
+    case 1:
+        return exact && p.n == 8 && p.m == 8 ? launch_one<1, 1, false, false, false>(p, sm_count, st)
+                                             : launch_one<1, 1, false, false, true>(p, sm_count, st);
+    case 2:
+        return full16 ? launch_one<2, 2, false, false, false>(p, sm_count, st)
+             : mb == 1 ? launch_one<2, 1, false, false, true>(p, sm_count, st) : launch_one<2, 2, false, false, true>(p, sm_count, st);
+    case 3:
+        return mb == 1 ? launch_one<3, 1, false, false, true>(p, sm_count, st) : launch_one<3, 3, false, false, true>(p, sm_count, st);
+    case 4:
+        return full32 ? launch_one<4, 4, false, false, false>(p, sm_count, st)
+             : mb == 1 ? launch_one<4, 1, false, false, true>(p, sm_count, st)
+             : mb == 2 ? launch_one<4, 2, false, false, true>(p, sm_count, st) : launch_one<4, 4, false, false, true>(p, sm_count, st);
+    case 5:
+        return mb == 1 ? launch_one<5, 1, false, false, true>(p, sm_count, st)
+             : mb == 2 ? launch_one<5, 2, false, false, true>(p, sm_count, st)
+             : mb == 3 ? launch_one<5, 3, false, false, true>(p, sm_count, st) : launch_one<5, 5, false, false, true>(p, sm_count, st);
+    default:
+        return mb <= 2 ? launch_one<6, 2, false, false, true>(p, sm_count, st)
+             : mb <= 4 ? launch_one<6, 4, false, false, true>(p, sm_count, st) : launch_one<6, 6, false, false, true>(p, sm_count, st);
+    }
 }
 
 } // namespace rfrag

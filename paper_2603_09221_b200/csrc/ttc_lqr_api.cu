@@ -482,8 +482,8 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
         if (obf && !uniform)
             return fail(TTC_STATUS_UNSUPPORTED, "bfloat16 outputs need n = m in {16, 32} or the tensor-core path at n = m = 64 "
                                                 "(per-head or per-token A, B, R; Q strides that keep 16-byte rows)");
-        if (n <= 16 && m <= 16) {
-            // one warp per instance, matrices in registers; the guarded variant takes any sizes and strides
+        if (rfrag::riccati_frag_serves(n, m, time_varying)) {
+            // one warp per instance, matrices in registers; the guarded variants take any sizes and strides
             const bool exact = q_rows_aligned && vector_rows_ok(p.A) && vector_rows_ok(p.B) && vector_rows_ok(p.R);
             cudaError_t e = rfrag::launch_riccati_frag(p, time_varying, affine, exact, h->sm_count, st);
             if (e != cudaSuccess)
@@ -491,27 +491,6 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
             h->last_launches += 1;
             h->total_launches += 1;
             h->last_kernel = uniform ? TTC_KERNEL_RICCATI_WARP : TTC_KERNEL_RICCATI_CTA;
-            return TTC_OK;
-        }
-        if (uniform) {
-            // fp32 warp kernel: one instance per warp, chunks of tokens handed out by an atomic counter
-            if ((s = ensure(h->ws_E, sizeof(int) * 4))) return s;
-            int* counter = static_cast<int*>(h->ws_E.ptr);
-            TTC_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), st));
-            void (*kern)(SolveParams, int*) =
-                per_token ? (affine ? rwarp::riccati_warp_kernel<32, true, true, true> : rwarp::riccati_warp_kernel<32, true, false, true>)
-                : affine ? rwarp::riccati_warp_kernel<32, true, true>
-                : time_varying ? rwarp::riccati_warp_kernel<32, true> : rwarp::riccati_warp_kernel<32, false>;
-            const size_t smem = rwarp::smem_bytes<32>(per_token);
-            const long long chunks = p.b0 * p.b1 * ((tcount + rwarp::Shape<32>::SLOTS - 1) / rwarp::Shape<32>::SLOTS);
-            long long grid = (long long)h->sm_count * 3;
-            TTC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            if (grid > chunks) grid = chunks;
-            kern<<<(unsigned)grid, rwarp::THREADS, smem, st>>>(p, counter);
-            TTC_CUDA(cudaGetLastError());
-            h->last_launches += 1;
-            h->total_launches += 1;
-            h->last_kernel = TTC_KERNEL_RICCATI_WARP;
             return TTC_OK;
         }
         const size_t smem = riccati_cta_smem_bytes(n, m);

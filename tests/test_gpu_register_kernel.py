@@ -10,7 +10,8 @@ from tests.test_gpu_affine import affine_workload, check, run_both
 from tests.test_gpu_parity import small_workload
 
 pytestmark = pytest.mark.gpu
-SIZES = [(1, 1), (2, 7), (7, 8), (8, 7), (8, 9), (9, 8), (15, 1), (16, 8), (15, 16), (16, 15)]
+SIZES = [(1, 1), (2, 7), (7, 8), (8, 7), (8, 9), (9, 8), (15, 1), (16, 8), (15, 16), (16, 15), (17, 5), (24, 24), (25, 8),
+         (31, 32), (32, 16), (20, 30), (33, 7), (40, 16), (39, 24), (33, 40), (41, 9), (48, 32), (47, 48)]
 
 
 @pytest.mark.parametrize("n,m", SIZES)
@@ -25,14 +26,14 @@ def test_block_edges_time_invariant(n, m):
     pu.compare(f, pu.run_oracle(w, first_only=True), idx, 1e-4, names=("P", "u"))
 
 
-@pytest.mark.parametrize("n,m", [(1, 2), (8, 9), (9, 8), (15, 16)])
+@pytest.mark.parametrize("n,m", [(1, 2), (8, 9), (9, 8), (15, 16), (17, 31), (32, 24)])
 def test_block_edges_time_varying_with_linear_term(n, m):
     w = affine_workload(n, m, 5, (1, 2, 4), seed=90 + 17 * n + m)
     check(*run_both(w), False)
     check(*run_both(w, first_only=True, want=("P", "pvec", "u", "info")), True)
 
 
-@pytest.mark.parametrize("n,m", [(5, 4), (8, 8), (12, 5), (16, 16)])
+@pytest.mark.parametrize("n,m", [(5, 4), (8, 8), (12, 5), (16, 16), (21, 20), (32, 32), (40, 12)])
 def test_odd_strides_and_failed_instances(n, m):
     """Operands whose matrices start at odd element offsets, and an instance whose R is not positive definite at the last
     pivot: reported with that pivot, filled with NaN, its neighbours untouched."""
