@@ -35,6 +35,12 @@ struct SolveParams {
     float* pvec;   // p_t [N][H+1][n] ([N][n] when first_only) or null
     int first_only;
     int out_bf16;  // K, P, x, u are bfloat16 arrays (round to nearest even) instead of float32
+    // chunked form (scan over the horizon): the horizon of an instance is cut into pieces of chunk_len steps (the last one
+    // shorter) that are solved independently from the value matrix at their end and the state at their start
+    int chunk_len, chunks;       // pieces that this launch solves per instance
+    int coarse;                  // number of boundaries behind t = 0: P_{k chunk_len} and x_{k chunk_len}, k = 0..coarse
+    const float *Pc, *xc;        // [N][coarse + 1][n][n], [N][coarse + 1][n] (xc null: no states)
+    int* piece_info;             // [N * chunks]
 };
 
 __device__ __forceinline__ long long operand_offset(const OperandDev& o, long long i, long long b1,

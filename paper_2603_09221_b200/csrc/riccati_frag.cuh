@@ -223,23 +223,28 @@ __device__ __forceinline__ void load_part(float (&v)[W], const float* row, int c
 // TV = time-varying request (time strides or a terminal weight); AFF = linear control cost r_t'u_t (implies TV);
 // PAD = n < 8 NB or m < 8 MB, or strides that do not keep the vector loads aligned: guarded element-wise accesses, the
 // missing part of R is the identity and everything else zero, which leaves the recursion of the existing part untouched.
-template <int NB, int MB, bool TV, bool AFF, bool PAD>
+// CH = one piece of the horizon of an instance (see SolveParams; time-invariant): it starts from the value matrix and the
+// state at the piece's ends, writes its part of the outputs and leaves failures to the caller.
+template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false>
 __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 4) riccati_frag_kernel(SolveParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const long long widx = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (widx >= p.b0 * p.b1 * p.tcount)
+    if (widx >= p.b0 * p.b1 * p.tcount * (CH ? p.chunks : 1))
         return;
-    const Place pl = place(p, (unsigned)widx);
+    const int chunk = CH ? (int)(widx % p.chunks) : 0;
+    const Place pl = place(p, (unsigned)(CH ? widx / p.chunks : widx));
     const long long inst = pl.inst;
-    const int n = PAD ? p.n : 8 * NB, m = PAD ? p.m : 8 * MB, H = p.H, obf = p.out_bf16;
+    const int n = PAD ? p.n : 8 * NB, m = PAD ? p.m : 8 * MB, obf = p.out_bf16;
+    const int Ht = p.H, tb = CH ? chunk * p.chunk_len : 0, H = CH ? min(p.chunk_len, Ht - tb) : Ht;      // steps tb .. tb + H - 1 of Ht
+    const bool last_piece = tb + H == Ht, first_ok = chunk == 0 || !p.first_only;
     const bool need_K_all = p.K != nullptr || p.x != nullptr || (p.u != nullptr && !p.first_only);
     const bool want_u0 = p.u != nullptr && p.first_only && !need_K_all;
     const bool need_k_all = AFF && p.kff != nullptr;
     float* const Kbase = (p.K && !obf) ? p.K : p.Kws;       // float32 gains (the rollout reads them)
-    const long long Koff = inst * (long long)H * m * n;
-    const long long Poff = inst * (long long)(p.first_only ? 1 : H + 1) * n * n;
+    const long long Koff = (inst * (long long)Ht + tb) * m * n;
+    const long long Poff = (inst * (long long)(p.first_only ? 1 : Ht + 1) + (p.first_only ? 0 : tb)) * n * n;
     using Ops = Operands<NB, MB>;
     constexpr bool TWO = TV && NB <= 2;
     using Mem = WarpMem<NB, MB, TWO>;
@@ -277,25 +282,38 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
             if (!p.Qf.ptr)
                 load_negated<NB, Ops::LQ>(nP, mem.op[0].Q, lane);
         } else {
-            stage<NB, NB, Ops::LQ, PAD>(mem.Q, TV && p.Qf.ptr ? p.Qf : p.Q, TV && p.Qf.ptr ? pl.off(p.Qf) : oQ + last * p.Q.st, n, n, lane);
+            OperandDev end = TV && p.Qf.ptr ? p.Qf : p.Q;   // P_H
+            long long oend = TV && p.Qf.ptr ? pl.off(p.Qf) : oQ + last * p.Q.st;
+            const bool inner = CH && chunk < p.coarse;
+            if (inner) {
+                end.ptr = p.Pc;
+                end.dtype = TTC_F32;
+                oend = (inst * (p.coarse + 1) + chunk + 1) * (long long)n * n;
+            }
+            stage<NB, NB, Ops::LQ, PAD>(mem.Q, end, oend, n, n, lane);
             stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + last * p.A.st, n, n, lane);
             stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + last * p.B.st, n, m, lane);
             stage<MB, MB, Ops::LR, PAD>(mem.R, p.R, oR + last * p.R.st, m, m, lane);
             copies_landed();
-            load_negated<NB, Ops::LQ>(nP, mem.Q, lane);     // P_H = Q_f or Q
-            if (TV && p.Qf.ptr) {
+            load_negated<NB, Ops::LQ>(nP, mem.Q, lane);
+            if ((TV && p.Qf.ptr) || inner) {
                 __syncwarp();
                 stage<NB, NB, Ops::LQ, PAD>(mem.Q, p.Q, oQ + last * p.Q.st, n, n, lane);
             }
         }
     }
-    if (p.P && !p.first_only)
+    if (p.P && !p.first_only && last_piece)
         store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, n, obf, lane);
 
+    auto start_state = [&](int i) {
+        if (CH && p.xc)
+            return p.xc[(inst * (p.coarse + 1) + chunk) * (long long)n + i];
+        return p.x0.ptr ? load_elem(p.x0, pl.off(p.x0) + i) : 0.f;
+    };
     float xr[NB];                                           // x_0 in row form
 #pragma unroll
     for (int b = 0; b < NB; ++b)
-        xr[b] = (p.x0.ptr && 8 * b + g < n) ? load_elem(p.x0, pl.off(p.x0) + 8 * b + g) : 0.f;
+        xr[b] = 8 * b + g < n ? start_state(8 * b + g) : 0.f;
 
     float pr[NB];                                           // affine term: p_{t+1} in row form
     float kc0[MB][2];                                       // k_t in column form
@@ -343,7 +361,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
             load_negated<NB, Ops::LQ>(nP, op.Q, lane);
             product<NB, NB, NB, true>(nP, &nP, as, ps);     // -Q - A'P A
         } else {
-            if (TV || ts == H - 1)
+            if (TV || ts == H - 1)                          // (what CH stages for P_H is followed by Q)
                 copies_landed();
             if (ts == H - 1 || (TV && p.A.st)) {            // raw -> split, in place
                 load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
@@ -503,11 +521,17 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
         // orientation only, the antisymmetric part E obeys E <- -A'E A: it grows along an open-loop unstable A however
         // well the closed loop is damped.
         make_symmetric<NB>(nP, lane);
-        if (p.P && (!p.first_only || ts == 0))
+        if (p.P && first_ok && (!p.first_only || ts == 0))
             store_negated<NB, PAD>(p.P, Poff + (long long)(p.first_only ? 0 : ts) * n * n, nP, n, obf, lane);
     }
-    if (p.info && lane == 0)
+    if (CH) {
+        if (lane == 0)
+            p.piece_info[widx] = fail;
+    } else if (p.info && lane == 0) {
         p.info[inst] = fail;
+    }
+    if (CH && fail)
+        return;
     if (fail) {                                             // uniform over the warp
         const float qn = quiet_nan();
         __syncwarp();
@@ -554,7 +578,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
 #pragma unroll
     for (int q = 0; q < RPL; ++q) {
         const int i = row0 + 32 * q;
-        x0v[q] = (i < n && p.x0.ptr) ? load_elem(p.x0, pl.off(p.x0) + i) : 0.f;
+        x0v[q] = i < n ? start_state(i) : 0.f;
     }
     __syncwarp();                                           // also: K_t stored by the other lanes are visible
 #pragma unroll
@@ -592,7 +616,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
         }
     }
     const int steps = (p.x || !p.first_only) ? H : 1;
-    const long long xoff = inst * (long long)(H + 1) * n, uoff = inst * (long long)(p.first_only ? m : H * m);
+    const long long xoff = (inst * (long long)(Ht + 1) + tb) * n, uoff = p.first_only ? inst * m : (inst * (long long)Ht + tb) * m;
 #pragma unroll
     for (int q = 0; q < RPL; ++q)
         if (p.x && writer && row0 + 32 * q < n)
@@ -622,7 +646,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
                 us[q] += kt[q];
             if (writer) {
                 su[i] = i < m ? us[q] : 0.f;
-                if (p.u && i < m && (!p.first_only || ts == 0))
+                if (p.u && i < m && first_ok && (!p.first_only || ts == 0))
                     store_out(p.u, uoff + (p.first_only ? 0 : (long long)ts * m) + i, us[q], obf);
             }
         }
@@ -645,7 +669,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
                 xs[q] += __shfl_xor_sync(FULL, xs[q], 1);
             if (writer) {
                 sx[i] = i < n ? xs[q] : 0.f;
-                if (p.x && i < n)
+                if (p.x && i < n && (!CH || last_piece || ts + 1 < H))
                     store_out(p.x, xoff + (long long)(ts + 1) * n + i, xs[q], obf);
             }
         }
@@ -653,21 +677,21 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     }
 }
 
-template <int NB, int MB, bool TV, bool AFF, bool PAD>
+template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false>
 inline cudaError_t launch_one(const SolveParams& p, int sm_count, cudaStream_t st)
 {
     // up to 16 states a CTA is four warps, unless the instances are so few that one warp each spreads them over more SMs;
     // above, the operands of a warp fill 7 to 60 KB and CTAs of one warp pack best
-    const long long nwin = p.b0 * p.b1 * p.tcount;
+    const long long nwin = p.b0 * p.b1 * p.tcount * (CH ? p.chunks : 1);
     const int warps = NB > 2 || nwin <= 4ll * sm_count ? 1 : MAX_WARPS;
     const size_t smem = warps * sizeof(WarpMem<NB, MB, TV && NB <= 2>);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(riccati_frag_kernel<NB, MB, TV, AFF, PAD>,
+        const cudaError_t e = cudaFuncSetAttribute(riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
     }
-    riccati_frag_kernel<NB, MB, TV, AFF, PAD><<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, smem, st>>>(p);
+    riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH><<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, smem, st>>>(p);
     return cudaGetLastError();
 }
 

@@ -195,5 +195,21 @@ __device__ __forceinline__ void mma32_store(float* Dm, const float (&acc)[2][4][
         }
 }
 
+// out[:] += sum_k coef[k] * row_k(M)      (M row-major in shared memory, row stride LD)
+template <int N>
+__device__ __forceinline__ void mix(f32x2 (&out)[N / 2], const float (&coef)[N], const float* M)
+{
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        axpy_row<N>(out, coef[k], M + k * Shape<N>::LD);
+}
+template <int N>
+__device__ __forceinline__ void zero2(f32x2 (&v)[N / 2])
+{
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i)
+        v[i] = 0ull;
+}
+
 } // namespace rwarp
 } // namespace ttc

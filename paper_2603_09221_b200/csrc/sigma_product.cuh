@@ -14,7 +14,6 @@
 #pragma once
 
 #include "ttc_layer.cuh"
-#include "scan_warp.cuh"
 
 namespace ttc {
 namespace sigma {
@@ -24,8 +23,8 @@ using rwarp::THREADS;
 using rwarp::f32x2;
 using rwarp::pack_row;
 using rwarp::unpack_row;
-using scanw::mix;
-using scanw::zero2;
+using rwarp::mix;
+using rwarp::zero2;
 
 template <int N>
 struct Slot {

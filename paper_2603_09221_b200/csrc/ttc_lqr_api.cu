@@ -20,7 +20,7 @@
 #include "layer_grad.cuh"
 #include "lqr_grad.cuh"
 #include "scan_pair.cuh"
-#include "scan_warp.cuh"
+#include "scan_frag.cuh"
 #include "peak_probe.cuh"
 
 using namespace ttc;
@@ -183,9 +183,12 @@ bool vector_rows_ok(const OperandDev& o)
     return ((o.s0 | o.s1 | o.s2 | o.st) % q) == 0;
 }
 
-// Start of an API call: make sure the small workspace exists and clear the device error word (word 1) on `st`.
+// Start of an API call that may run the tensor-memory kernel (n = m = 64): make sure the small workspace exists and clear
+// the device error word (word 1) on `st`.  No other kernel has bounded waits.
 int clear_device_error(ttc_lqr_handle* h, cudaStream_t st)
 {
+    if (h->cfg.n != 64 || h->cfg.m != 64)
+        return TTC_OK;
     int s = ensure(h->ws_E, sizeof(int) * 4);
     if (s)
         return s;
@@ -390,35 +393,33 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
     if (obf && (method == TTC_SCAN || time_varying))
         return fail(TTC_STATUS_UNSUPPORTED, "bfloat16 outputs are served by the sequential recursion of ttc_lqr_solve only");
     if (method == TTC_SCAN) {
-        // n = m = 16 / 32: the scan that is parallel in time; it keeps every P_t (in the caller's P or in the
-        // workspace).  Other shapes: the generic scan, which keeps every P_t, or a single value matrix (P_1) per
-        // instance when only P_0 / u_0 are wanted.
-        const bool warp_scan = n == m && (n == 16 || n == 32);
-        const int pfull = warp_scan || !(p.first_only && !K && !x);
-        float* Pbuf;
-        if (pfull && P && !p.first_only) {
-            Pbuf = P;
-        } else {
-            const size_t per = pfull ? (size_t)(H + 1) * n * n : (size_t)n * n;
-            if ((s = ensure(h->ws_P, sizeof(float) * (size_t)h->N * per))) return s;
-            Pbuf = static_cast<float*>(h->ws_P.ptr);
-        }
-        if ((s = ensure(h->ws_E, sizeof(int) * (size_t)h->N))) return s;
+        // n = m = 16 / 32: pieces of the horizon in parallel.  Other shapes: the generic scan, which keeps every P_t (in
+        // the caller's P or in the workspace), or a single value matrix (P_1) per instance when only P_0 / u_0 are wanted.
         int launches = 0;
         cudaError_t e;
-        if (warp_scan) {
-            // parallel in time: per doubling round one launch over every (instance, application) and one over the
-            // squarings, then one over every (instance, t) for the gains, then the rollout
-            if ((s = ensure(h->ws_elem, sizeof(float) * (size_t)h->N * scanw::ELEM_MATS * n * n))) return s;
-            if (!K && (x || u)) {
+        if (n == m && (n == 16 || n == 32)) {
+            if ((s = ensure(h->ws_E, sizeof(int) * scanf::flag_words(h->N, H)))) return s;
+            if ((s = ensure(h->ws_elem, sizeof(float) * scanf::workspace_floats(h->N, n, H)))) return s;
+            if (!K && rollout_needs_all_K) {
                 if ((s = ensure(h->ws_K, sizeof(float) * (size_t)h->N * H * m * n))) return s;
                 p.Kws = static_cast<float*>(h->ws_K.ptr);
             }
-            float* elem = static_cast<float*>(h->ws_elem.ptr);
+            float* ws = static_cast<float*>(h->ws_elem.ptr);
             int* flags = static_cast<int*>(h->ws_E.ptr);
-            e = n == 16 ? scanw::launch_scan_warp<16>(p, Pbuf, elem, flags, h->sm_count, st, &launches)
-                        : scanw::launch_scan_warp<32>(p, Pbuf, elem, flags, h->sm_count, st, &launches);
+            const bool exact = vector_rows_ok(p.Q) && vector_rows_ok(p.A) && vector_rows_ok(p.B) && vector_rows_ok(p.R);
+            e = n == 16 ? scanf::launch_scan_frag<2>(p, ws, flags, exact, h->sm_count, st, &launches)
+                        : scanf::launch_scan_frag<4>(p, ws, flags, exact, h->sm_count, st, &launches);
         } else {
+            const int pfull = !(p.first_only && !K && !x);
+            float* Pbuf;
+            if (pfull && P && !p.first_only) {
+                Pbuf = P;
+            } else {
+                const size_t per = pfull ? (size_t)(H + 1) * n * n : (size_t)n * n;
+                if ((s = ensure(h->ws_P, sizeof(float) * (size_t)h->N * per))) return s;
+                Pbuf = static_cast<float*>(h->ws_P.ptr);
+            }
+            if ((s = ensure(h->ws_E, sizeof(int) * (size_t)h->N))) return s;
             e = launch_scan_path(p, Pbuf, static_cast<int*>(h->ws_E.ptr), pfull, h->sm_count, st, &launches);
         }
         if (e != cudaSuccess)
@@ -1113,8 +1114,8 @@ int ttc_lqr_solve_host(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operan
         // whose items do not fill a whole number of rounds of that grid leaves SMs idle in its last round (a slice
         // of 128 tokens x 32 heads is 128 items for 148 CTAs of the n = 64 kernel), so prefer the slice length that
         // fills its rounds best, among those that are at least 128 tokens and keep the slice count within the limit.
-        const int item_tokens = n == 64 ? 32 : n == 32 ? 4 : 8;
-        const long long grid = (long long)h->sm_count * (n == 64 ? 1 : n == 32 ? 3 : 4);
+        const int item_tokens = n == 64 ? 32 : n == 32 ? 1 : 4;
+        const long long grid = (long long)h->sm_count * (n == 64 ? 1 : n == 32 ? 8 : 4);
         const double round_tokens = (double)(grid * item_tokens) / (double)(b0 * b1);      // tokens per head in one round
         auto fill = [&](long long t) {
             const double rounds = std::ceil((double)((t + item_tokens - 1) / item_tokens * item_tokens) / round_tokens - 1e-9);
