@@ -41,6 +41,9 @@ struct SolveParams {
     int coarse;                  // number of boundaries behind t = 0: P_{k chunk_len} and x_{k chunk_len}, k = 0..coarse
     const float *Pc, *xc;        // [N][coarse + 1][n][n], [N][coarse + 1][n] (xc null: no states)
     int* piece_info;             // [N * chunks]
+    // gradients of the first control (Thm 3.2), in the form that one kernel computes whole: outputs [N][H][..] (each may be
+    // null) and the sequences x | xd | u | ud of every instance, [N][4][H + 1][max(n, m)]
+    float *dA, *dB, *dQ, *dQf, *dR, *dx0, *u0, *seq;
 };
 
 __device__ __forceinline__ long long operand_offset(const OperandDev& o, long long i, long long b1,

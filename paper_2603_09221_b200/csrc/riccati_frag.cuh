@@ -219,13 +219,200 @@ __device__ __forceinline__ void load_part(float (&v)[W], const float* row, int c
     }
 }
 
+// ---- gradients of a loss of u_0 (Thm 3.2), after the backward pass of the same instance --------------------------------
+// Both rollouts share every load of K_t, A_t, B_t, both co-state recursions every load of A_t, Q_t; the outer products
+//     dA_t = lam_{t+1} xd_t' + lamd_{t+1} x_t'      dB_t = lam_{t+1} ud_t' + lamd_{t+1} u_t'
+//     dQ_t = 1/2 (x_t xd_t' + xd_t x_t')            dR_t = 1/2 (u_t ud_t' + ud_t u_t')          lam_t = A_t'lam_{t+1} + Q_t x_t
+// leave the registers as soon as the co-states of their step are known.  Row i of a matrix belongs to LPR lanes.  The
+// gains and sequences that this warp wrote a moment ago come back from the second-level cache.
+template <int W>
+__device__ __forceinline__ void load_stream(float (&v)[W], const float* src)
+{
+#pragma unroll
+    for (int q = 0; q < W / 4; ++q) {
+        const float4 f = __ldg(reinterpret_cast<const float4*>(src) + q);
+        v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
+    }
+}
+// row segment a v' + b w' (scaled by half, products rounded before they are added, when symmetric)
+template <int W, bool SYM>
+__device__ __forceinline__ void store_outer(float* dst, float a, const float (&v)[W], float b, const float (&w)[W])
+{
+#pragma unroll
+    for (int q = 0; q < W / 4; ++q) {
+        float r[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            r[e] = SYM ? 0.5f * __fadd_rn(__fmul_rn(a, v[4 * q + e]), __fmul_rn(b, w[4 * q + e]))
+                       : fmaf(a, v[4 * q + e], b * w[4 * q + e]);
+        __stcs(reinterpret_cast<float4*>(dst) + q, make_float4(r[0], r[1], r[2], r[3]));
+    }
+}
+template <int NB>
+__device__ __forceinline__ void grad_tail(const SolveParams& p, const Place& pl, const float (&xr)[NB], const float (&k0)[NB][2],
+                                          float* sm, int lane)
+{
+    constexpr int N = 8 * NB, LPR = N <= 16 ? 2 : 1, W = N / LPR;
+    const int H = p.H, i = lane / LPR, c0 = (lane % LPR) * W, g = lane >> 2, t = lane & 3;
+    const bool writer = lane % LPR == 0;
+    const long long inst = pl.inst;
+    const float* Ag = reinterpret_cast<const float*>(p.A.ptr) + pl.off(p.A);
+    const float* Bg = reinterpret_cast<const float*>(p.B.ptr) + pl.off(p.B);
+    const float* Qg = reinterpret_cast<const float*>(p.Q.ptr) + pl.off(p.Q);
+    const float* Qfg = p.Qf.ptr ? reinterpret_cast<const float*>(p.Qf.ptr) + pl.off(p.Qf) : Qg;
+    const float* Kg = p.K + inst * (long long)H * N * N;
+    float* X = p.seq + inst * (long long)(4 * (H + 1)) * N;
+    float* Xd = X + (long long)(H + 1) * N;
+    float* U = Xd + (long long)(H + 1) * N;
+    float* Ud = U + (long long)(H + 1) * N;
+    float *sx = sm, *sxd = sm + N, *su = sm + 2 * N, *sud = sm + 3 * N, *sk = sm + 4 * N;
+    __syncwarp();
+    if (g == 0)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            sk[8 * b + 2 * t] = k0[b][0];
+            sk[8 * b + 2 * t + 1] = k0[b][1];
+        }
+    if (t == 0)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            sx[8 * b + g] = xr[b];
+            sxd[8 * b + g] = 0.f;
+        }
+    __syncwarp();                                           // also: K_t stored by the other lanes are visible
+    auto sum = [](float v) { return LPR == 2 ? v + __shfl_xor_sync(FULL, v, 1) : v; };
+    if (writer) {
+        X[i] = sx[i];
+        Xd[i] = 0.f;
+    }
+    float kr[W], ar[W], br[W];
+    load_part<W, false>(kr, Kg + i * N, c0, N);
+    load_stream<W>(ar, Ag + i * N + c0);
+    load_stream<W>(br, Bg + i * N + c0);
+#pragma unroll 1
+    for (int ts = 0; ts < H; ++ts) {
+        float v[W], vd[W];
+        load_part<W, false>(v, sx, c0, N);
+        load_part<W, false>(vd, sxd, c0, N);
+        float us = 0.f, uds = 0.f, xs = 0.f, xds = 0.f;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            us = fmaf(kr[k], v[k], us);
+            uds = fmaf(kr[k], vd[k], uds);
+            xs = fmaf(ar[k], v[k], xs);
+            xds = fmaf(ar[k], vd[k], xds);
+        }
+        us = sum(us);
+        uds = sum(uds) + (ts == 0 ? sk[i] : 0.f);
+        if (writer) {
+            su[i] = us;
+            sud[i] = uds;
+            U[(long long)ts * N + i] = us;
+            Ud[(long long)ts * N + i] = uds;
+            if (ts == 0 && p.u0)
+                p.u0[inst * N + i] = us;
+        }
+        __syncwarp();
+        load_part<W, false>(v, su, c0, N);
+        load_part<W, false>(vd, sud, c0, N);
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            xs = fmaf(br[k], v[k], xs);
+            xds = fmaf(br[k], vd[k], xds);
+        }
+        if (ts + 1 < H) {
+            load_part<W, false>(kr, Kg + ((long long)(ts + 1) * N + i) * N, c0, N);
+            load_stream<W>(ar, Ag + (ts + 1) * p.A.st + i * N + c0);
+            load_stream<W>(br, Bg + (ts + 1) * p.B.st + i * N + c0);
+        }
+        xs = sum(xs);
+        xds = sum(xds);
+        if (writer) {
+            sx[i] = xs;
+            sxd[i] = xds;
+            X[(long long)(ts + 1) * N + i] = xs;
+            Xd[(long long)(ts + 1) * N + i] = xds;
+        }
+        __syncwarp();
+    }
+    // co-states of t = H, outer product of the terminal weight
+    float lam = 0.f, lamd = 0.f;
+    float *sl = su, *sld = sud;
+    {
+        float v[W], vd[W], q[W];
+        load_part<W, false>(v, sx, c0, N);
+        load_part<W, false>(vd, sxd, c0, N);
+        load_stream<W>(q, Qfg + i * N + c0);
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            lam = fmaf(q[k], v[k], lam);
+            lamd = fmaf(q[k], vd[k], lamd);
+        }
+        if (p.dQf)
+            store_outer<W, true>(p.dQf + (inst * N + i) * N + c0, sx[i], vd, sxd[i], v);
+    }
+    float qr[W];
+    load_stream<W>(qr, Qg + (H - 1) * p.Q.st + i * N + c0);
+#pragma unroll 1
+    for (int ts = H - 1; ts >= 0; --ts) {
+        lam = sum(lam);
+        lamd = sum(lamd);
+        __syncwarp();
+        if (writer) {
+            sl[i] = lam;
+            sld[i] = lamd;
+        }
+        float ac[W];                                        // column i of A_t, this lane's rows
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+            ac[k] = __ldg(Ag + ts * p.A.st + (c0 + k) * N + i);
+        const long long o = (inst * (long long)H + ts) * N * N + i * N + c0;
+        {
+            float u[W], ud[W];
+            load_part<W, false>(u, U + (long long)ts * N, c0, N);
+            load_part<W, false>(ud, Ud + (long long)ts * N, c0, N);
+            if (p.dB)
+                store_outer<W, false>(p.dB + o, lam, ud, lamd, u);
+            if (p.dR)
+                store_outer<W, true>(p.dR + o, U[(long long)ts * N + i], ud, Ud[(long long)ts * N + i], u);
+        }
+        float v[W], vd[W];
+        load_part<W, false>(v, X + (long long)ts * N, c0, N);
+        load_part<W, false>(vd, Xd + (long long)ts * N, c0, N);
+        if (p.dA)
+            store_outer<W, false>(p.dA + o, lam, vd, lamd, v);
+        if (p.dQ)
+            store_outer<W, true>(p.dQ + o, X[(long long)ts * N + i], vd, Xd[(long long)ts * N + i], v);
+        lam = lamd = 0.f;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            lam = fmaf(qr[k], v[k], lam);
+            lamd = fmaf(qr[k], vd[k], lamd);
+        }
+        if (ts > 0)
+            load_stream<W>(qr, Qg + (ts - 1) * p.Q.st + i * N + c0);
+        __syncwarp();
+        load_part<W, false>(v, sl, c0, N);
+        load_part<W, false>(vd, sld, c0, N);
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            lam = fmaf(ac[k], v[k], lam);
+            lamd = fmaf(ac[k], vd[k], lamd);
+        }
+    }
+    lamd = sum(lamd);
+    if (writer && p.dx0)
+        p.dx0[inst * N + i] = lamd;
+}
+
 // NB, MB: number of 8-blocks of the state and the control dimension.
 // TV = time-varying request (time strides or a terminal weight); AFF = linear control cost r_t'u_t (implies TV);
 // PAD = n < 8 NB or m < 8 MB, or strides that do not keep the vector loads aligned: guarded element-wise accesses, the
 // missing part of R is the identity and everything else zero, which leaves the recursion of the existing part untouched.
 // CH = one piece of the horizon of an instance (see SolveParams; time-invariant): it starts from the value matrix and the
 // state at the piece's ends, writes its part of the outputs and leaves failures to the caller.
-template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false>
+// GRAD = the gradients of the first control in the same kernel (n = m = 8 NB, float32 operands): see grad_tail().
+template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false, bool GRAD = false>
 __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 4) riccati_frag_kernel(SolveParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -556,9 +743,27 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
             for (long long e = lane; e < cnt; e += 32)
                 p.pvec[inst * cnt + e] = qn;
         }
+        if (GRAD) {
+            auto fill = [&](float* base, long long cnt) {
+                if (base)
+                    for (long long e = lane; e < cnt; e += 32)
+                        base[inst * cnt + e] = qn;
+            };
+            fill(p.dA, (long long)H * n * n);
+            fill(p.dB, (long long)H * n * m);
+            fill(p.dQ, (long long)H * n * n);
+            fill(p.dQf, (long long)n * n);
+            fill(p.dR, (long long)H * m * m);
+            fill(p.dx0, n);
+            fill(p.u0, m);
+        }
         if (need_k_all)
             for (long long e = lane; e < (long long)H * m; e += 32)
                 p.kff[inst * (long long)H * m + e] = qn;
+        return;
+    }
+    if constexpr (GRAD) {
+        grad_tail<NB>(p, pl, xr, kc0, reinterpret_cast<float*>(&mem), lane);
         return;
     }
     if (want_u0 || !(p.x || p.u))
@@ -677,7 +882,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     }
 }
 
-template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false>
+template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false, bool GRAD = false>
 inline cudaError_t launch_one(const SolveParams& p, int sm_count, cudaStream_t st)
 {
     // up to 16 states a CTA is four warps, unless the instances are so few that one warp each spreads them over more SMs;
@@ -686,12 +891,12 @@ inline cudaError_t launch_one(const SolveParams& p, int sm_count, cudaStream_t s
     const int warps = NB > 2 || nwin <= 4ll * sm_count ? 1 : MAX_WARPS;
     const size_t smem = warps * sizeof(WarpMem<NB, MB, TV && NB <= 2>);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH>,
+        const cudaError_t e = cudaFuncSetAttribute(riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH, GRAD>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
     }
-    riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH><<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, smem, st>>>(p);
+    riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH, GRAD><<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, smem, st>>>(p);
     return cudaGetLastError();
 }
 
@@ -739,6 +944,13 @@ inline cudaError_t launch_riccati_frag(const SolveParams& p, bool time_varying, 
         return mb <= 2 ? launch_one<6, 2, false, false, true>(p, sm_count, st)
              : mb <= 4 ? launch_one<6, 4, false, false, true>(p, sm_count, st) : launch_one<6, 6, false, false, true>(p, sm_count, st);
     }
+}
+
+// Gradients of the first control, everything in one kernel: n = m = 16 / 32, float32 operands with aligned strides.
+inline cudaError_t launch_grad_frag(const SolveParams& p, int sm_count, cudaStream_t st)
+{
+    return p.n == 16 ? launch_one<2, 2, true, true, false, false, true>(p, sm_count, st)
+                     : launch_one<4, 4, true, true, false, false, true>(p, sm_count, st);
 }
 
 } // namespace rfrag

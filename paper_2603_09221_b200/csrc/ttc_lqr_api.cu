@@ -645,6 +645,38 @@ int ttc_lqr_grad(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
     float* kws = static_cast<float*>(h->ws_k.ptr);
     h->last_launches = 0;
 
+    // Batches that fill the machine at n = m = 16 / 32: one kernel, whose warps carry an instance from the backward pass to
+    // the outer products (the gains come back from the second-level cache, and the writes of some warps overlap the
+    // arithmetic of others).  With few instances the separate kernels below spread the outer products over more SMs.
+    if (n == m && (n == 16 || n == 32) && h->N > 4ll * h->sm_count) {
+        SolveParams p = {};
+        p.n = n; p.m = m; p.H = H;
+        p.b0 = h->cfg.batch[0]; p.b1 = h->cfg.batch[1]; p.b2 = h->cfg.batch[2]; p.N = h->N;
+        p.t0 = 0; p.tcount = p.b2;
+        p.A = to_dev(A); p.B = to_dev(B); p.Q = to_dev(Q); p.R = to_dev(R); p.x0 = to_dev(x0);
+        p.Qf = to_dev((Qf && Qf->ptr) ? Qf : nullptr);
+        p.A.st = tstride[0]; p.B.st = tstride[1]; p.Q.st = tstride[2]; p.R.st = tstride[3];
+        if (p.Q.dtype == TTC_F32 && p.Qf.dtype == TTC_F32 && vector_rows_ok(p.A) && vector_rows_ok(p.B) && vector_rows_ok(p.Q) &&
+            vector_rows_ok(p.R) && vector_rows_ok(p.Qf)) {
+            p.r.ptr = g; p.r.dtype = TTC_F32;
+            p.r.s2 = m; p.r.s1 = m * p.b2; p.r.s0 = p.r.s1 * p.b1;
+            p.r_count = 1;
+            p.K = Kws;
+            p.info = info;
+            p.dA = dA; p.dB = dB; p.dQ = dQ; p.dQf = dQf; p.dR = dR; p.dx0 = dx0; p.u0 = u0;
+            p.seq = static_cast<float*>(h->ws_vec.ptr);
+            const cudaError_t e = rfrag::launch_grad_frag(p, h->sm_count, st);
+            if (e != cudaSuccess)
+                return fail(TTC_STATUS_CUDA_ERROR, "gradient launch: %s", cudaGetErrorString(e));
+            const bool head = A->bstride[2] == 0 && B->bstride[2] == 0 && R->bstride[2] == 0;
+            const bool token = A->bstride[2] != 0 && B->bstride[2] != 0 && R->bstride[2] != 0;
+            h->last_launches = 1;
+            h->total_launches += 1;
+            h->last_kernel = head || token ? TTC_KERNEL_RICCATI_WARP : TTC_KERNEL_RICCATI_CTA;
+            return TTC_OK;
+        }
+    }
+
     // Backward pass of the primal problem (K_t) with the dual problem's linear cost riding along: r_0 = g, r_t = 0
     // afterwards, so k_0 = -S_0^{-1} g is the dual's first control and every later k_t vanishes.
     ttc_operand r;
