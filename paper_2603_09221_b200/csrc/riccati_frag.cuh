@@ -225,6 +225,43 @@ __device__ __forceinline__ void load_part(float (&v)[W], const float* row, int c
 //     dQ_t = 1/2 (x_t xd_t' + xd_t x_t')            dR_t = 1/2 (u_t ud_t' + ud_t u_t')          lam_t = A_t'lam_{t+1} + Q_t x_t
 // leave the registers as soon as the co-states of their step are known.  Row i of a matrix belongs to LPR lanes.  The
 // gains and sequences that this warp wrote a moment ago come back from the second-level cache.
+// What a step reads comes through a ring of asynchronous copies several steps ahead: by the time the gains are read again
+// the stores of the other warps may have pushed them out to HBM.  Matrices keep rows of N floats with the 16-byte chunks
+// of a row exchanged (chunk q of row r at q ^ swizzle(r)), which makes row and column reads conflict-free.
+template <int N>
+struct GradRing {
+    static constexpr int FWD = 3 * N * N, BWD = 2 * N * N + 4 * N;         // floats per stage: K, A, B / A, Q, four vectors
+    static constexpr int FS = N == 16 ? 4 : 2, BS = N == 16 ? 5 : 2;       // stages
+    static constexpr int VEC = 8 * N;                                      // vectors in front of the stages
+    static constexpr size_t BYTES = sizeof(float) * (VEC + (FS * FWD > BS * BWD ? FS * FWD : BS * BWD));
+    static __device__ __forceinline__ int swizzle(int r) { return N == 16 ? (r >> 1) & 3 : r & 7; }
+    static __device__ __forceinline__ void copy(float* dst, const float* src, int lane)
+    {
+#pragma unroll
+        for (int e = lane; e < N * N / 4; e += 32) {
+            const int r = e / (N / 4), q = e % (N / 4);
+            copy16(dst + r * N + 4 * (q ^ swizzle(r)), src + 4 * e);
+        }
+    }
+    // W consecutive elements of row r from column c0
+    template <int W>
+    static __device__ __forceinline__ void row(float (&v)[W], const float* M, int r, int c0)
+    {
+#pragma unroll
+        for (int q = 0; q < W / 4; ++q) {
+            const float4 f = *reinterpret_cast<const float4*>(M + r * N + 4 * ((c0 / 4 + q) ^ swizzle(r)));
+            v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
+        }
+    }
+    static __device__ __forceinline__ float at(const float* M, int r, int c) { return M[r * N + 4 * ((c >> 2) ^ swizzle(r)) + (c & 3)]; }
+};
+__device__ __forceinline__ void commit_copies() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int K>
+__device__ __forceinline__ void wait_copies()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(K) : "memory");
+    __syncwarp();
+}
 template <int W>
 __device__ __forceinline__ void load_stream(float (&v)[W], const float* src)
 {
@@ -265,8 +302,22 @@ __device__ __forceinline__ void grad_tail(const SolveParams& p, const Place& pl,
     float* Xd = X + (long long)(H + 1) * N;
     float* U = Xd + (long long)(H + 1) * N;
     float* Ud = U + (long long)(H + 1) * N;
-    float *sx = sm, *sxd = sm + N, *su = sm + 2 * N, *sud = sm + 3 * N, *sk = sm + 4 * N;
-    __syncwarp();
+    using Ring = GradRing<N>;
+    constexpr int FS = Ring::FS, BS = Ring::BS;
+    float *sx = sm, *sxd = sm + N, *su = sm + 2 * N, *sud = sm + 3 * N, *sk = sm + 4 * N, *ring = sm + Ring::VEC;
+    __syncwarp();                                           // K_t stored by the other lanes are visible; the operands are done
+    auto stage_fwd = [&](int ts) {
+        if (ts < H) {
+            float* d = ring + (ts % FS) * Ring::FWD;
+            Ring::copy(d, Kg + (long long)ts * N * N, lane);
+            Ring::copy(d + N * N, Ag + ts * p.A.st, lane);
+            Ring::copy(d + 2 * N * N, Bg + ts * p.B.st, lane);
+        }
+        commit_copies();
+    };
+#pragma unroll
+    for (int k = 0; k < FS - 1; ++k)
+        stage_fwd(k);
     if (g == 0)
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
@@ -279,28 +330,32 @@ __device__ __forceinline__ void grad_tail(const SolveParams& p, const Place& pl,
             sx[8 * b + g] = xr[b];
             sxd[8 * b + g] = 0.f;
         }
-    __syncwarp();                                           // also: K_t stored by the other lanes are visible
+    __syncwarp();
     auto sum = [](float v) { return LPR == 2 ? v + __shfl_xor_sync(FULL, v, 1) : v; };
     if (writer) {
         X[i] = sx[i];
         Xd[i] = 0.f;
     }
-    float kr[W], ar[W], br[W];
-    load_part<W, false>(kr, Kg + i * N, c0, N);
-    load_stream<W>(ar, Ag + i * N + c0);
-    load_stream<W>(br, Bg + i * N + c0);
 #pragma unroll 1
     for (int ts = 0; ts < H; ++ts) {
-        float v[W], vd[W];
+        wait_copies<FS - 2>();
+        stage_fwd(ts + FS - 1);
+        const float* st = ring + (ts % FS) * Ring::FWD;
+        float v[W], vd[W], r[W];
         load_part<W, false>(v, sx, c0, N);
         load_part<W, false>(vd, sxd, c0, N);
         float us = 0.f, uds = 0.f, xs = 0.f, xds = 0.f;
+        Ring::template row<W>(r, st, i, c0);
 #pragma unroll
         for (int k = 0; k < W; ++k) {
-            us = fmaf(kr[k], v[k], us);
-            uds = fmaf(kr[k], vd[k], uds);
-            xs = fmaf(ar[k], v[k], xs);
-            xds = fmaf(ar[k], vd[k], xds);
+            us = fmaf(r[k], v[k], us);
+            uds = fmaf(r[k], vd[k], uds);
+        }
+        Ring::template row<W>(r, st + N * N, i, c0);
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            xs = fmaf(r[k], v[k], xs);
+            xds = fmaf(r[k], vd[k], xds);
         }
         us = sum(us);
         uds = sum(uds) + (ts == 0 ? sk[i] : 0.f);
@@ -315,15 +370,11 @@ __device__ __forceinline__ void grad_tail(const SolveParams& p, const Place& pl,
         __syncwarp();
         load_part<W, false>(v, su, c0, N);
         load_part<W, false>(vd, sud, c0, N);
+        Ring::template row<W>(r, st + 2 * N * N, i, c0);
 #pragma unroll
         for (int k = 0; k < W; ++k) {
-            xs = fmaf(br[k], v[k], xs);
-            xds = fmaf(br[k], vd[k], xds);
-        }
-        if (ts + 1 < H) {
-            load_part<W, false>(kr, Kg + ((long long)(ts + 1) * N + i) * N, c0, N);
-            load_stream<W>(ar, Ag + (ts + 1) * p.A.st + i * N + c0);
-            load_stream<W>(br, Bg + (ts + 1) * p.B.st + i * N + c0);
+            xs = fmaf(r[k], v[k], xs);
+            xds = fmaf(r[k], vd[k], xds);
         }
         xs = sum(xs);
         xds = sum(xds);
@@ -335,6 +386,21 @@ __device__ __forceinline__ void grad_tail(const SolveParams& p, const Place& pl,
         }
         __syncwarp();
     }
+    auto stage_bwd = [&](int k) {                           // k-th step backwards
+        const int ts = H - 1 - k;
+        if (ts >= 0) {
+            float* d = ring + (k % BS) * Ring::BWD;
+            Ring::copy(d, Ag + ts * p.A.st, lane);
+            Ring::copy(d + N * N, Qg + ts * p.Q.st, lane);
+            if (lane < N)                                   // x_t, xd_t, u_t, ud_t
+                copy16(d + 2 * N * N + 4 * lane, X + (long long)(lane / (N / 4)) * (H + 1) * N + (long long)ts * N + 4 * (lane % (N / 4)));
+        }
+        commit_copies();
+    };
+    wait_copies<0>();
+#pragma unroll
+    for (int k = 0; k < BS - 1; ++k)
+        stage_bwd(k);
     // co-states of t = H, outer product of the terminal weight
     float lam = 0.f, lamd = 0.f;
     float *sl = su, *sld = sud;
@@ -351,58 +417,62 @@ __device__ __forceinline__ void grad_tail(const SolveParams& p, const Place& pl,
         if (p.dQf)
             store_outer<W, true>(p.dQf + (inst * N + i) * N + c0, sx[i], vd, sxd[i], v);
     }
-    float qr[W];
-    load_stream<W>(qr, Qg + (H - 1) * p.Q.st + i * N + c0);
 #pragma unroll 1
     for (int ts = H - 1; ts >= 0; --ts) {
+        const int k0s = H - 1 - ts;
+        wait_copies<BS - 2>();
+        stage_bwd(k0s + BS - 1);
+        const float* st = ring + (k0s % BS) * Ring::BWD;
+        const float* vec = st + 2 * N * N;
         lam = sum(lam);
         lamd = sum(lamd);
-        __syncwarp();
         if (writer) {
             sl[i] = lam;
             sld[i] = lamd;
         }
-        float ac[W];                                        // column i of A_t, this lane's rows
-#pragma unroll
-        for (int k = 0; k < W; ++k)
-            ac[k] = __ldg(Ag + ts * p.A.st + (c0 + k) * N + i);
         const long long o = (inst * (long long)H + ts) * N * N + i * N + c0;
-        {
-            float u[W], ud[W];
-            load_part<W, false>(u, U + (long long)ts * N, c0, N);
-            load_part<W, false>(ud, Ud + (long long)ts * N, c0, N);
-            if (p.dB)
-                store_outer<W, false>(p.dB + o, lam, ud, lamd, u);
-            if (p.dR)
-                store_outer<W, true>(p.dR + o, U[(long long)ts * N + i], ud, Ud[(long long)ts * N + i], u);
-        }
         float v[W], vd[W];
-        load_part<W, false>(v, X + (long long)ts * N, c0, N);
-        load_part<W, false>(vd, Xd + (long long)ts * N, c0, N);
+        load_part<W, false>(v, vec + 2 * N, c0, N);
+        load_part<W, false>(vd, vec + 3 * N, c0, N);
+        if (p.dB)
+            store_outer<W, false>(p.dB + o, lam, vd, lamd, v);
+        if (p.dR)
+            store_outer<W, true>(p.dR + o, vec[2 * N + i], vd, vec[3 * N + i], v);
+        load_part<W, false>(v, vec, c0, N);
+        load_part<W, false>(vd, vec + N, c0, N);
         if (p.dA)
             store_outer<W, false>(p.dA + o, lam, vd, lamd, v);
         if (p.dQ)
-            store_outer<W, true>(p.dQ + o, X[(long long)ts * N + i], vd, Xd[(long long)ts * N + i], v);
+            store_outer<W, true>(p.dQ + o, vec[i], vd, vec[N + i], v);
         lam = lamd = 0.f;
+        float r[W];
+        Ring::template row<W>(r, st + N * N, i, c0);
 #pragma unroll
         for (int k = 0; k < W; ++k) {
-            lam = fmaf(qr[k], v[k], lam);
-            lamd = fmaf(qr[k], vd[k], lamd);
+            lam = fmaf(r[k], v[k], lam);
+            lamd = fmaf(r[k], vd[k], lamd);
         }
-        if (ts > 0)
-            load_stream<W>(qr, Qg + (ts - 1) * p.Q.st + i * N + c0);
         __syncwarp();
         load_part<W, false>(v, sl, c0, N);
         load_part<W, false>(vd, sld, c0, N);
 #pragma unroll
         for (int k = 0; k < W; ++k) {
-            lam = fmaf(ac[k], v[k], lam);
-            lamd = fmaf(ac[k], vd[k], lamd);
+            const float a = Ring::at(st, c0 + k, i);        // column i of A_t
+            lam = fmaf(a, v[k], lam);
+            lamd = fmaf(a, vd[k], lamd);
         }
     }
+    wait_copies<0>();
     lamd = sum(lamd);
     if (writer && p.dx0)
         p.dx0[inst * N + i] = lamd;
+}
+
+template <int NB, int MB, bool TV, bool GRAD>
+__host__ __device__ constexpr size_t warp_bytes()
+{
+    constexpr size_t a = sizeof(WarpMem<NB, MB, TV && NB <= 2>), b = GRAD ? GradRing<8 * NB>::BYTES : 0;
+    return ((a > b ? a : b) + 15) & ~size_t(15);
 }
 
 // NB, MB: number of 8-blocks of the state and the control dimension.
@@ -435,7 +505,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     using Ops = Operands<NB, MB>;
     constexpr bool TWO = TV && NB <= 2;
     using Mem = WarpMem<NB, MB, TWO>;
-    Mem& mem = reinterpret_cast<Mem*>(smem_raw)[threadIdx.x >> 5];
+    Mem& mem = *reinterpret_cast<Mem*>(smem_raw + (threadIdx.x >> 5) * warp_bytes<NB, MB, TV, GRAD>());
     const long long oA = pl.off(p.A), oB = pl.off(p.B), oR = pl.off(p.R), oQ = pl.off(p.Q);
     Mat<NB, NB> nP;
     if constexpr (PAD) {                                    // what does not exist: R is the identity, the rest zero
@@ -889,7 +959,7 @@ inline cudaError_t launch_one(const SolveParams& p, int sm_count, cudaStream_t s
     // above, the operands of a warp fill 7 to 60 KB and CTAs of one warp pack best
     const long long nwin = p.b0 * p.b1 * p.tcount * (CH ? p.chunks : 1);
     const int warps = NB > 2 || nwin <= 4ll * sm_count ? 1 : MAX_WARPS;
-    const size_t smem = warps * sizeof(WarpMem<NB, MB, TV && NB <= 2>);
+    const size_t smem = warps * warp_bytes<NB, MB, TV, GRAD>();
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH, GRAD>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
