@@ -42,7 +42,7 @@ struct SolveParams {
     const float *Pc, *xc;        // [N][coarse + 1][n][n], [N][coarse + 1][n] (xc null: no states)
     int* piece_info;             // [N * chunks]
     // gradients of the first control (Thm 3.2), in the form that one kernel computes whole: outputs [N][H][..] (each may be
-    // null) and the sequences x | xd | u | ud of every instance, [N][4][H + 1][max(n, m)]
+    // null) and the sequences x | xd | u | ud [N][4][H + 1][n]
     float *dA, *dB, *dQ, *dQf, *dR, *dx0, *u0, *seq;
 };
 

@@ -475,5 +475,41 @@ __device__ __forceinline__ void product_symmetric(Mat<NB, NB>& d, const Split<NB
         }
 }
 
+// z = L^{-1} v and k = -L^{-T} z for a vector in row form, from the results of factor(): z in column form, k in column form
+template <int MB>
+__device__ __forceinline__ void solve_vector(float (&zc)[MB][2], float (&kc)[MB][2], const float (&v)[MB], const Mat<MB, MB>& L,
+                                             const float (&w)[MB][2], int lane)
+{
+    float zr[MB], kr[MB];
+#pragma unroll
+    for (int b = 0; b < MB; ++b) {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < MB; ++k)
+            if (k < b)
+                s = fmaf(L.v[b / 2][k][2 * (b & 1)], zc[k][0], fmaf(L.v[b / 2][k][2 * (b & 1) + 1], zc[k][1], s));
+        float c0, c1;
+        row_to_col(c0, c1, b ? v[b] - sum_over_t(s) : v[b], lane);
+        zr[b] = sum_over_t(fmaf(w[b][0], c0, w[b][1] * c1));
+        row_to_col(zc[b][0], zc[b][1], zr[b], lane);
+    }
+#pragma unroll
+    for (int b = MB - 1; b >= 0; --b) {                     // last block first
+        float s0 = 0.f, s1 = 0.f;                           // (L_qb' k_q) in column form
+#pragma unroll
+        for (int q = 0; q < MB; ++q)
+            if (q > b) {
+                s0 = fmaf(L.v[q / 2][b][2 * (q & 1)], kr[q], s0);
+                s1 = fmaf(L.v[q / 2][b][2 * (q & 1) + 1], kr[q], s1);
+            }
+        float x = zr[b];
+        if (b + 1 < MB)
+            x += col_to_row(sum_over_g(s0), sum_over_g(s1), lane);
+        kc[b][0] = -sum_over_g(w[b][0] * x);
+        kc[b][1] = -sum_over_g(w[b][1] * x);
+        kr[b] = col_to_row(kc[b][0], kc[b][1], lane);
+    }
+}
+
 } // namespace frag
 } // namespace ttc

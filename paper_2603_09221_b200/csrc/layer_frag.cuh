@@ -131,6 +131,25 @@ struct Rates {
     }
 };
 
+// parameters of one instance: Bbar' and Qbar into the slot, nP = -P_T = -Q_T
+template <int NB>
+__device__ __forceinline__ void prepare(Slot<NB>& sl, Mat<NB, NB>& nP, const LayerParams& p, long long inst, int lane)
+{
+    Mat<NB, NB> B, Q, Bt;
+    synthesise<NB>(B, Q, nP, p, inst, lane);
+    transpose<NB>(Bt, B, lane);
+    keep(sl.B, Bt, lane);
+#pragma unroll
+    for (int mt = 0; mt < Mat<NB, NB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < NB; ++cb) {
+            sl.Q[mt][cb][lane] = make_float4(Q.v[mt][cb][0], Q.v[mt][cb][1], Q.v[mt][cb][2], Q.v[mt][cb][3]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                nP.v[mt][cb][e] = -nP.v[mt][cb][e];
+        }
+}
+
 // The backward recursion of one instance.  nP comes in as -P_T and goes out as -P_0; `on_step(s, Zt, S, w)` is called
 // with what gains() needs after each factorisation.  Returns 0 or s n + j + 1 for the first bad pivot.
 template <int NB, typename F>
@@ -236,21 +255,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB == 2 ? 5 : 2) layer_frag_ke
         return;
     Slot<NB>& sl = reinterpret_cast<Slot<NB>*>(smem_raw)[threadIdx.x >> 5];
     Mat<NB, NB> nP;
-    {
-        Mat<NB, NB> B, Q, Bt;
-        synthesise<NB>(B, Q, nP, p, inst, lane);
-        transpose<NB>(Bt, B, lane);
-        keep(sl.B, Bt, lane);
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-            for (int cb = 0; cb < NB; ++cb) {
-                sl.Q[mt][cb][lane] = make_float4(Q.v[mt][cb][0], Q.v[mt][cb][1], Q.v[mt][cb][2], Q.v[mt][cb][3]);
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    nP.v[mt][cb][e] = -nP.v[mt][cb][e];     // P_T = Q_T
-            }
-    }
+    prepare<NB>(sl, nP, p, inst, lane);
     Rates<NB> rates;
     rates.load(p, inst, lane);
     float rd[NB], hr[NB];

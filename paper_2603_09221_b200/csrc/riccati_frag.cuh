@@ -696,18 +696,8 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
         if (AFF) {
             // z = L^{-1}(B'p + r);  p_t = A'p - Z'z;  k_t = -L^{-T} z   (all zero while p and r are)
             if (ts < p.r_count) {
-                float zc[MB][2], zr[MB];
-#pragma unroll
-                for (int b = 0; b < MB; ++b) {
-                    float s = 0.f;
-#pragma unroll
-                    for (int k = 0; k < b; ++k)
-                        s = fmaf(S.v[b / 2][k][2 * (b & 1)], zc[k][0], fmaf(S.v[b / 2][k][2 * (b & 1) + 1], zc[k][1], s));
-                    float c0, c1;
-                    row_to_col(c0, c1, b ? gr[b] - sum_over_t(s) : gr[b], lane);
-                    zr[b] = sum_over_t(fmaf(w[b][0], c0, w[b][1] * c1));
-                    row_to_col(zc[b][0], zc[b][1], zr[b], lane);
-                }
+                float zc[MB][2];
+                solve_vector<MB>(zc, kc0, gr, S, w, lane);
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
                     float s = 0.f;
@@ -715,22 +705,6 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
                     for (int k = 0; k < MB; ++k)
                         s = fmaf(Zt.v[b / 2][k][2 * (b & 1)], zc[k][0], fmaf(Zt.v[b / 2][k][2 * (b & 1) + 1], zc[k][1], s));
                     pr[b] = ap[b] - sum_over_t(s);
-                }
-                float kr[MB];                               // k_t in row form, last block first
-#pragma unroll
-                for (int b = MB - 1; b >= 0; --b) {
-                    float s0 = 0.f, s1 = 0.f;               // (L_qb' k_q) in column form
-#pragma unroll
-                    for (int q = b + 1; q < MB; ++q) {
-                        s0 = fmaf(S.v[q / 2][b][2 * (q & 1)], kr[q], s0);
-                        s1 = fmaf(S.v[q / 2][b][2 * (q & 1) + 1], kr[q], s1);
-                    }
-                    float v = zr[b];
-                    if (b + 1 < MB)
-                        v += col_to_row(sum_over_g(s0), sum_over_g(s1), lane);
-                    kc0[b][0] = -sum_over_g(w[b][0] * v);
-                    kc0[b][1] = -sum_over_g(w[b][1] * v);
-                    kr[b] = col_to_row(kc0[b][0], kc0[b][1], lane);
                 }
             } else {
 #pragma unroll
@@ -792,7 +766,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     if (fail) {                                             // uniform over the warp
         const float qn = quiet_nan();
         __syncwarp();
-        if (p.K)
+        if (p.K && !GRAD)
             for (long long e = lane; e < (long long)H * m * n; e += 32)
                 store_out(p.K, Koff + e, qn, obf);
         if (p.P) {

@@ -1,6 +1,6 @@
 // BASELINE, not the solver: the reverse symplectic iteration of Thm 3.3 with row normalisation (the fused kernel the
 // paper describes in its hardware co-design appendix), restated for the contextualised layer's parameters so that it
-// can be timed and checked beside ttc_layer_kernel on the same inputs.
+// can be timed and checked beside layer_frag_kernel on the same inputs.
 //
 //     [Y1 Y2] = [I  Q_T] Sigma_T ... Sigma_1,      Sigma_t = [I 0; G_t I] diag(A_t^{-T}, A_t) [I Q_{t-1}; 0 I],
 //     G_t = B_t R_t^{-1} B_t',     P_0 = Y1^{-1} Y2,     lambda_0 = P_0 h_0,     u_1 = -R_1^{-1} B_1' A_1^{-T} lambda_0.
@@ -13,6 +13,7 @@
 // steps on inputs where the backward recursion stays at rounding level (measured in the tests and the sweep).
 #pragma once
 
+#include "riccati_warp.cuh"
 #include "ttc_layer.cuh"
 
 namespace ttc {

@@ -638,11 +638,6 @@ int ttc_lqr_grad(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int n = h->cfg.n, m = h->cfg.m;
     const int D = ((n > m ? n : m) + 3) & ~3;
-    if ((s = ensure(h->ws_K, sizeof(float) * (size_t)h->N * H * m * n))) return s;
-    if ((s = ensure(h->ws_k, sizeof(float) * (size_t)h->N * H * m))) return s;
-    if ((s = ensure(h->ws_vec, sizeof(float) * (size_t)h->N * 6 * (H + 1) * D))) return s;
-    float* Kws = static_cast<float*>(h->ws_K.ptr);
-    float* kws = static_cast<float*>(h->ws_k.ptr);
     h->last_launches = 0;
 
     // Batches that fill the machine at n = m = 16 / 32: one kernel, whose warps carry an instance from the backward pass to
@@ -661,7 +656,9 @@ int ttc_lqr_grad(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
             p.r.ptr = g; p.r.dtype = TTC_F32;
             p.r.s2 = m; p.r.s1 = m * p.b2; p.r.s0 = p.r.s1 * p.b1;
             p.r_count = 1;
-            p.K = Kws;
+            if ((s = ensure(h->ws_K, sizeof(float) * (size_t)h->N * H * m * n))) return s;
+            if ((s = ensure(h->ws_vec, sizeof(float) * (size_t)h->N * 4 * (H + 1) * n))) return s;
+            p.K = static_cast<float*>(h->ws_K.ptr);
             p.info = info;
             p.dA = dA; p.dB = dB; p.dQ = dQ; p.dQf = dQf; p.dR = dR; p.dx0 = dx0; p.u0 = u0;
             p.seq = static_cast<float*>(h->ws_vec.ptr);
@@ -677,6 +674,11 @@ int ttc_lqr_grad(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
         }
     }
 
+    if ((s = ensure(h->ws_K, sizeof(float) * (size_t)h->N * H * m * n))) return s;
+    if ((s = ensure(h->ws_k, sizeof(float) * (size_t)h->N * H * m))) return s;
+    if ((s = ensure(h->ws_vec, sizeof(float) * (size_t)h->N * 6 * (H + 1) * D))) return s;
+    float* Kws = static_cast<float*>(h->ws_K.ptr);
+    float* kws = static_cast<float*>(h->ws_k.ptr);
     // Backward pass of the primal problem (K_t) with the dual problem's linear cost riding along: r_0 = g, r_t = 0
     // afterwards, so k_0 = -S_0^{-1} g is the dual's first control and every later k_t vanishes.
     ttc_operand r;
@@ -815,7 +817,7 @@ static int launch_layer(ttc_lqr_handle* h, const ttc_layer_inputs* in, int32_t T
     p.r_inv = in->r_inv + on; p.h0 = in->h0 + on;
     p.B_basis = in->B_basis; p.Q_basis = in->Q_basis;
     p.u1 = u1 ? u1 + on : nullptr; p.P0 = P0 ? P0 + on * n : nullptr; p.info = info ? info + i0 : nullptr;
-    p.Kws = nullptr; p.Pws = nullptr; p.g = nullptr; p.k0 = nullptr;
+    p.Kws = nullptr; p.g = nullptr; p.k0 = nullptr;
     const cudaError_t e = n == 32 ? lfrag::launch_layer_frag<4>(p, h->sm_count, st) : lfrag::launch_layer_frag<2>(p, h->sm_count, st);
     if (e != cudaSuccess)
         return fail(TTC_STATUS_CUDA_ERROR, "layer launch: %s", cudaGetErrorString(e));
@@ -854,7 +856,7 @@ int ttc_lqr_solve_layer_sigma_baseline(ttc_lqr_handle* h, const ttc_layer_inputs
     p.r_inv = in->r_inv; p.h0 = in->h0;
     p.B_basis = in->B_basis; p.Q_basis = in->Q_basis;
     p.u1 = u1; p.P0 = P0; p.info = info;
-    p.Kws = nullptr; p.Pws = nullptr; p.g = nullptr; p.k0 = nullptr;
+    p.Kws = nullptr; p.g = nullptr; p.k0 = nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int slots = n == 32 ? rwarp::Shape<32>::SLOTS : rwarp::Shape<16>::SLOTS;
     long long grid = (p.N + slots - 1) / slots;
@@ -893,10 +895,9 @@ int ttc_lqr_layer_grad(ttc_lqr_handle* h, const ttc_layer_inputs* in, int32_t T,
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int n = h->cfg.n, r = in->r;
     const size_t N = (size_t)h->N, nn = (size_t)n * n;
-    if ((s = ensure(h->ws_K, sizeof(float) * 2 * N * T * nn))) return s;           // every K_s, then every P_s
+    if ((s = ensure(h->ws_K, sizeof(float) * N * T * nn))) return s;               // every K_s
     if ((s = ensure(h->ws_k, sizeof(float) * N * n))) return s;
     if ((s = ensure(h->ws_vec, sizeof(float) * N * 4 * (T + 1) * n))) return s;
-    if ((s = ensure(h->ws_E, sizeof(int) * 4))) return s;
     int* info_dev = info;
     if (!info_dev) {
         if ((s = ensure(h->ws_info, sizeof(int) * N))) return s;
@@ -906,8 +907,10 @@ int ttc_lqr_layer_grad(ttc_lqr_handle* h, const ttc_layer_inputs* in, int32_t T,
     if (bases && (s = ensure(h->ws_G, sizeof(float) * 3 * N * nn))) return s;
     h->last_launches = 0;
 
-    // (1) backward Riccati pass on the synthesised parameters; every gain and k_0 = -S_0^{-1} g are kept
-    layer::LayerParams p;
+    // (1) backward Riccati pass on the synthesised parameters, rollouts, co-states and the reductions of Thm 3.2's outer
+    // products onto the coefficients
+    lgrad::LayerGradParams q;
+    layer::LayerParams& p = q.lp;
     p.N = h->N; p.T = T; p.r = r;
     p.s_a = in->s_a; p.s_ga = in->s_gamma_a; p.s_gb = in->s_gamma_b; p.s_gq = in->s_gamma_q;
     p.s_b = in->s_b; p.s_q = in->s_q; p.s_qf = in->s_qf;
@@ -915,67 +918,31 @@ int ttc_lqr_layer_grad(ttc_lqr_handle* h, const ttc_layer_inputs* in, int32_t T,
     p.B_basis = in->B_basis; p.Q_basis = in->Q_basis;
     p.u1 = u1; p.P0 = nullptr; p.info = info_dev;
     p.Kws = static_cast<float*>(h->ws_K.ptr); p.g = g; p.k0 = static_cast<float*>(h->ws_k.ptr);
-    p.Pws = p.Kws + N * T * nn;
-    int* counter = static_cast<int*>(h->ws_E.ptr);
-    TTC_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), st));
-    {
-        // n = 16 with the machine at least half full: two columns per lane, as in the forward call
-        const bool c2 = n == 16 && p.N > (long long)h->sm_count * 2 * rwarp::Shape<16>::SLOTS;
-        void (*kern)(layer::LayerParams, int*) = n == 32 ? layer::ttc_layer_kernel<32, true>
-                                               : c2 ? layer::ttc_layer_kernel_c2<16, true> : layer::ttc_layer_kernel<16, true>;
-        const size_t smem = n == 32 ? layer::smem_bytes<32>() : c2 ? layer::smem_bytes_c2<16>() : layer::smem_bytes<16>();
-        const int slots = n == 32 ? rwarp::Shape<32>::SLOTS : c2 ? layer::Shape2<16>::SLOTS : rwarp::Shape<16>::SLOTS;
-        long long chunks = (p.N + slots - 1) / slots, grid = (long long)h->sm_count * (n == 32 ? 3 : c2 ? 2 : 4);
-        if (grid > chunks) grid = chunks;
-        TTC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kern<<<(unsigned)grid, rwarp::THREADS, smem, st>>>(p, counter);
-        TTC_CUDA(cudaGetLastError());
-    }
-    // (2) rollouts, co-states and the reductions of Thm 3.2's outer products onto the coefficients
-    lgrad::LayerGradParams q;
-    q.lp = p;
-    q.vec = static_cast<float*>(h->ws_vec.ptr);
+    q.seq = static_cast<float*>(h->ws_vec.ptr);
     q.info = info_dev;
     q.d_sa = out->s_a; q.d_ga = out->s_gamma_a; q.d_gb = out->s_gamma_b; q.d_gq = out->s_gamma_q;
     q.d_ri = out->r_inv; q.d_h0 = out->h0;
     q.d_sb = out->s_b; q.d_sq = out->s_q; q.d_sqf = out->s_qf;
     float* G = bases ? static_cast<float*>(h->ws_G.ptr) : nullptr;
     q.GB = G; q.GQ = G ? G + N * nn : nullptr; q.GF = G ? G + 2 * N * nn : nullptr;
-    {
-        const int slots = n == 32 ? rwarp::Shape<32>::SLOTS : rwarp::Shape<16>::SLOTS;
-        long long grid = (p.N + slots - 1) / slots;
-        const long long cap = (long long)h->sm_count * 8;
-        if (grid > cap) grid = cap;
-        if (n == 32) {
-            const size_t smem = sizeof(lgrad::Slot<32>) * slots;
-            TTC_CUDA(cudaFuncSetAttribute(lgrad::layer_grad_vectors_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            lgrad::layer_grad_vectors_kernel<32><<<(unsigned)grid, rwarp::THREADS, smem, st>>>(q);
-        } else {
-            const size_t smem = sizeof(lgrad::Slot<16>) * slots;
-            TTC_CUDA(cudaFuncSetAttribute(lgrad::layer_grad_vectors_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            lgrad::layer_grad_vectors_kernel<16><<<(unsigned)grid, rwarp::THREADS, smem, st>>>(q);
-        }
-        TTC_CUDA(cudaGetLastError());
+    int launches = 0;
+    cudaError_t e = n == 32 ? lgrad::launch_layer_grad<4>(q, h->sm_count, st, &launches)
+                            : lgrad::launch_layer_grad<2>(q, h->sm_count, st, &launches);
+    if (e != cudaSuccess)
+        return fail(TTC_STATUS_CUDA_ERROR, "layer gradient launch: %s", cudaGetErrorString(e));
+    // (2) the bases are shared by every instance: their gradients are sums over the instances
+    if (out->B_basis) {
+        TTC_CUDA(cudaMemsetAsync(out->B_basis, 0, sizeof(float) * (size_t)r * nn, st));
+        TTC_CUDA(lgrad::launch_basis_reduce(h->N, r, (int)nn, info_dev, in->s_b, q.GB, nullptr, nullptr, out->B_basis, h->sm_count, st));
+        ++launches;
     }
-    h->last_launches += 2;
-    h->total_launches += 2;
-    // (3) the bases are shared by every instance: their gradients are sums over the instances
-    if (bases) {
-        long long grid = (long long)h->sm_count * 4;
-        if (grid > (long long)N) grid = (long long)N;
-        if (out->B_basis) {
-            TTC_CUDA(cudaMemsetAsync(out->B_basis, 0, sizeof(float) * (size_t)r * nn, st));
-            lgrad::basis_reduce_kernel<<<(unsigned)grid, 256, 0, st>>>(h->N, r, (int)nn, info_dev, in->s_b, q.GB, nullptr, nullptr, out->B_basis);
-            TTC_CUDA(cudaGetLastError());
-            h->last_launches += 1; h->total_launches += 1;
-        }
-        if (out->Q_basis) {
-            TTC_CUDA(cudaMemsetAsync(out->Q_basis, 0, sizeof(float) * (size_t)r * nn, st));
-            lgrad::basis_reduce_kernel<<<(unsigned)grid, 256, 0, st>>>(h->N, r, (int)nn, info_dev, in->s_q, q.GQ, in->s_qf, q.GF, out->Q_basis);
-            TTC_CUDA(cudaGetLastError());
-            h->last_launches += 1; h->total_launches += 1;
-        }
+    if (out->Q_basis) {
+        TTC_CUDA(cudaMemsetAsync(out->Q_basis, 0, sizeof(float) * (size_t)r * nn, st));
+        TTC_CUDA(lgrad::launch_basis_reduce(h->N, r, (int)nn, info_dev, in->s_q, q.GQ, in->s_qf, q.GF, out->Q_basis, h->sm_count, st));
+        ++launches;
     }
+    h->last_launches += launches;
+    h->total_launches += launches;
     h->last_kernel = TTC_KERNEL_LAYER;
     return TTC_OK;
 }
