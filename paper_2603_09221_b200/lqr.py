@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import torch
 
@@ -44,6 +45,8 @@ class ttc_layer_inputs(ctypes.Structure):
                                                "r_inv", "h0", "B_basis", "Q_basis")] + [("r", ctypes.c_int32)]
 
 
+_LAYER_INPUTS = struct.Struct("11Pi")
+
 LAYER_GRAD_KEYS = ("s_a", "s_gamma_a", "s_gamma_b", "s_gamma_q", "s_b", "s_q", "s_qf", "r_inv", "h0", "B_basis", "Q_basis")
 
 
@@ -62,6 +65,7 @@ class TtcError(RuntimeError):
 
 
 _lib = None
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def library_path() -> str:
@@ -80,7 +84,7 @@ def load_library():
     P = ctypes.POINTER
     lib.ttc_lqr_create.restype = ctypes.c_int
     lib.ttc_lqr_create.argtypes = [P(ttc_lqr_config), P(ctypes.c_void_p)]
-    opp = P(ttc_operand)
+    opp = ctypes.c_void_p                                   # address of a ttc_operand
     lib.ttc_lqr_solve.restype = ctypes.c_int
     lib.ttc_lqr_solve.argtypes = [ctypes.c_void_p, opp, opp, opp, opp, opp, ctypes.c_int32] + \
         [ctypes.c_void_p] * 5 + [ctypes.c_uint32, ctypes.c_void_p]
@@ -170,6 +174,52 @@ def _operand(t, tail_ndim, batch):
     return op
 
 
+# Operands of one call, marshalled into one buffer of ttc_operand structures: filling ctypes fields one by one cost more
+# host time (19 us for five operands) than a small solve takes on the device.
+_DTYPES = {torch.float32: TTC_F32, torch.bfloat16: TTC_BF16}
+_OPERAND = struct.Struct("Piiqqq")
+_OPERAND_SIZE = _OPERAND.size
+assert _OPERAND_SIZE == ctypes.sizeof(ttc_operand)
+
+
+class _Operands:
+    """``count`` operand slots; ``put`` fills the next one and returns its address (None for a missing tensor)."""
+    __slots__ = ("buf", "base", "pos", "batch")
+
+    def __init__(self, count, batch):
+        self.buf = ctypes.create_string_buffer(count * _OPERAND_SIZE)
+        self.base = ctypes.addressof(self.buf)
+        self.pos = 0
+        self.batch = batch
+
+    def put(self, t, tail):
+        if t is None:
+            return None
+        pos = self.pos
+        dt = _DTYPES.get(t.dtype)
+        shape = t.shape
+        if dt is None or len(shape) != 3 + tail:
+            op = _operand(t, tail, self.batch)                 # the general form, and its errors
+            _OPERAND.pack_into(self.buf, pos, op.ptr or 0, op.dtype, 0, *op.bstride)
+        else:
+            b0, b1, b2 = self.batch
+            if tail == 2:
+                n0, n1, n2, rows, cols = shape
+                s0, s1, s2, sr, sc = t.stride()
+                dense = (sc == 1 or cols == 1) and (sr == cols or rows == 1)
+            else:
+                n0, n1, n2, cols = shape
+                s0, s1, s2, sc = t.stride()
+                dense = sc == 1 or cols == 1
+            # a dimension of length 1 is shared; anything else has to match the batch
+            if not dense or (n0 != 1 and n0 != b0) or (n1 != 1 and n1 != b1) or (n2 != 1 and n2 != b2):
+                _operand(t, tail, self.batch)                  # raises
+            _OPERAND.pack_into(self.buf, pos, t.data_ptr(), dt, 0, s0 if n0 != 1 else 0, s1 if n1 != 1 else 0,
+                               s2 if n2 != 1 else 0)
+        self.pos = pos + _OPERAND_SIZE
+        return self.base + pos
+
+
 class LqrSolver:
     """Owns one ``ttc_lqr_handle``.  ``batch`` is ``(seqs, heads, tokens)`` (shorter tuples are
     left-padded with 1)."""
@@ -205,91 +255,79 @@ class LqrSolver:
         return v.value
 
     def _ops(self, A, B, Q, R, x0):
-        ops = [_operand(A, 2, self.batch), _operand(B, 2, self.batch), _operand(Q, 2, self.batch),
-               _operand(R, 2, self.batch), _operand(x0, 1, self.batch)]
-        return [ctypes.byref(o) if o is not None else None for o in ops], ops
+        ops = _Operands(5, self.batch)
+        return (ops.put(A, 2), ops.put(B, 2), ops.put(Q, 2), ops.put(R, 2), ops.put(x0, 1)), ops
 
     @staticmethod
     def _ptr(t):
-        return None if t is None else ctypes.c_void_p(t.data_ptr())
+        return None if t is None else t.data_ptr()
+
+    def _stream(self, stream):
+        if stream is None:
+            # the raw handle directly where torch offers it: building a Stream object costs more than the rest of the call
+            return _raw_stream(self.device) if _raw_stream else torch.cuda.current_stream(self.device).cuda_stream
+        return stream.cuda_stream
 
     def solve(self, A, B, Q, R, x0, H, K=None, P=None, x=None, u=None, info=None, flags=0, stream=None):
         """Enqueue ``ttc_lqr_solve`` on ``stream`` (a ``torch.cuda.Stream``; default: current)."""
         refs, keep = self._ops(A, B, Q, R, x0)
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
-        _check(load_library().ttc_lqr_solve(
-            self._h, *refs, int(H), self._ptr(K), self._ptr(P), self._ptr(x), self._ptr(u), self._ptr(info),
-            int(flags), ctypes.c_void_p(stream.cuda_stream)))
+        ptr = self._ptr
+        status = _lib.ttc_lqr_solve(self._h, *refs, int(H), ptr(K), ptr(P), ptr(x), ptr(u), ptr(info), int(flags),
+                                    self._stream(stream))
+        if status:
+            _check(status)
 
     def solve_lowrank_q(self, A, B, U, d, scale, R, x0, H, K=None, P=None, x=None, u=None, info=None, flags=0, stream=None):
         """Enqueue ``ttc_lqr_solve_lowrank_q``: as :meth:`solve` with ``Q = scale * U U' + diag(d)`` handed over as
         ``U [..batch.., n, rank]`` and ``d [..batch.., n]``."""
-        ops = [_operand(A, 2, self.batch), _operand(B, 2, self.batch), _operand(U, 2, self.batch),
-               _operand(d, 1, self.batch), _operand(R, 2, self.batch), _operand(x0, 1, self.batch)]
-        ref = lambda o: ctypes.byref(o) if o is not None else None
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
+        ops = _Operands(6, self.batch)
+        a, b, uu, dd, rr, xx = ops.put(A, 2), ops.put(B, 2), ops.put(U, 2), ops.put(d, 1), ops.put(R, 2), ops.put(x0, 1)
+        ptr = self._ptr
         _check(load_library().ttc_lqr_solve_lowrank_q(
-            self._h, ref(ops[0]), ref(ops[1]), ref(ops[2]), ref(ops[3]), int(U.shape[-1]), ctypes.c_float(scale), ref(ops[4]),
-            ref(ops[5]), int(H), self._ptr(K), self._ptr(P), self._ptr(x), self._ptr(u), self._ptr(info), int(flags),
-            ctypes.c_void_p(stream.cuda_stream)))
+            self._h, a, b, uu, dd, int(U.shape[-1]), scale, rr, xx, int(H), ptr(K), ptr(P), ptr(x), ptr(u), ptr(info),
+            int(flags), self._stream(stream)))
+
+    def _tv_ops(self, A, B, Q, R, H, tv, ops):
+        """Addresses of A, B, Q, R and their time strides; operands named in ``tv`` carry a time axis."""
+        refs, tstride = [], (ctypes.c_int64 * 4)()
+        for i, (name, t) in enumerate((("A", A), ("B", B), ("Q", Q), ("R", R))):
+            if name in tv:
+                if t.shape[-3] < H:
+                    raise ValueError("operand %s has %d time steps, H = %d" % (name, t.shape[-3], H))
+                tstride[i] = t.stride(-3)
+                t = t.select(-3, 0)
+            refs.append(ops.put(t, 2))
+        return refs, tstride
 
     def solve_tv(self, A, B, Q, R, Qf, x0, H, tv=("A", "B", "Q", "R"), K=None, P=None, x=None, u=None, info=None,
                  flags=0, stream=None):
         """Enqueue ``ttc_lqr_solve_tv``.  Operands named in ``tv`` carry a time axis of length >= H right after
         their batch dimensions (``A [..batch.., H, n, n]``); the others are as for :meth:`solve`.  ``Qf`` is the
         terminal weight (may be None when Q is not time-varying)."""
-        ops, tstride = [], (ctypes.c_int64 * 4)()
-        for i, (name, t, tail) in enumerate((("A", A, 2), ("B", B, 2), ("Q", Q, 2), ("R", R, 2))):
-            if name in tv:
-                if t.shape[-3] < H:
-                    raise ValueError("operand %s has %d time steps, H = %d" % (name, t.shape[-3], H))
-                ops.append(_operand(t[..., 0, :, :], 2, self.batch))
-                tstride[i] = t.stride(-3)
-            else:
-                ops.append(_operand(t, 2, self.batch))
-                tstride[i] = 0
-        oqf = _operand(Qf, 2, self.batch) if Qf is not None else None      # NULL: Q_f = Q (Q constant in time)
-        ox = _operand(x0, 1, self.batch)
-        ref = lambda o: ctypes.byref(o) if o is not None else None
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
-        _check(load_library().ttc_lqr_solve_tv(
-            self._h, ref(ops[0]), ref(ops[1]), ref(ops[2]), ref(ops[3]), tstride, ref(oqf), ref(ox), int(H),
-            self._ptr(K), self._ptr(P), self._ptr(x), self._ptr(u), self._ptr(info), int(flags),
-            ctypes.c_void_p(stream.cuda_stream)))
+        ops = _Operands(6, self.batch)
+        refs, tstride = self._tv_ops(A, B, Q, R, H, tv, ops)
+        qf, xx = ops.put(Qf, 2), ops.put(x0, 1)                # Qf None: Q_f = Q (Q constant in time)
+        ptr = self._ptr
+        _check(load_library().ttc_lqr_solve_tv(self._h, *refs, tstride, qf, xx, int(H), ptr(K), ptr(P), ptr(x), ptr(u),
+                                               ptr(info), int(flags), self._stream(stream)))
 
     def solve_affine(self, A, B, Q, R, Qf, r, x0, H, tv=("A", "B", "Q", "R", "r"), K=None, kff=None, P=None, pvec=None,
                      x=None, u=None, info=None, flags=0, stream=None):
         """Enqueue ``ttc_lqr_solve_affine`` (linear control cost ``r_t'u_t``; Prop. A.1).  As :meth:`solve_tv`; ``r`` is
         ``[..batch.., H, m]`` when ``"r"`` is in ``tv``, else ``[..batch.., m]``.  ``kff [N, H, m]`` receives the
         feed-forward terms, ``pvec [N, H + 1, n]`` (``[N, n]`` with first-only) the linear value terms."""
-        ops, tstride = [], (ctypes.c_int64 * 4)()
-        for i, (name, t) in enumerate((("A", A), ("B", B), ("Q", Q), ("R", R))):
-            if name in tv:
-                if t.shape[-3] < H:
-                    raise ValueError("operand %s has %d time steps, H = %d" % (name, t.shape[-3], H))
-                ops.append(_operand(t[..., 0, :, :], 2, self.batch))
-                tstride[i] = t.stride(-3)
-            else:
-                ops.append(_operand(t, 2, self.batch))
-                tstride[i] = 0
+        ops = _Operands(7, self.batch)
+        refs, tstride = self._tv_ops(A, B, Q, R, H, tv, ops)
+        rst = 0
         if "r" in tv:
             if r.shape[-2] < H:
                 raise ValueError("operand r has %d time steps, H = %d" % (r.shape[-2], H))
-            orr, rst = _operand(r[..., 0, :], 1, self.batch), r.stride(-2)
-        else:
-            orr, rst = _operand(r, 1, self.batch), 0
-        oqf = _operand(Qf, 2, self.batch) if Qf is not None else None      # NULL: Q_f = Q (Q constant in time)
-        ox = _operand(x0, 1, self.batch)
-        ref = lambda o: ctypes.byref(o) if o is not None else None
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
-        _check(load_library().ttc_lqr_solve_affine(
-            self._h, ref(ops[0]), ref(ops[1]), ref(ops[2]), ref(ops[3]), tstride, ref(oqf), ref(orr), int(rst), ref(ox),
-            int(H), self._ptr(K), self._ptr(kff), self._ptr(P), self._ptr(pvec), self._ptr(x), self._ptr(u),
-            self._ptr(info), int(flags), ctypes.c_void_p(stream.cuda_stream)))
+            rst = r.stride(-2)
+            r = r.select(-2, 0)
+        qf, rr, xx = ops.put(Qf, 2), ops.put(r, 1), ops.put(x0, 1)             # Qf None: Q_f = Q (Q constant in time)
+        ptr = self._ptr
+        _check(load_library().ttc_lqr_solve_affine(self._h, *refs, tstride, qf, rr, int(rst), xx, int(H), ptr(K), ptr(kff), ptr(P),
+                                                   ptr(pvec), ptr(x), ptr(u), ptr(info), int(flags), self._stream(stream)))
 
     def grad(self, A, B, Q, R, Qf, x0, g, H, tv=("A", "B", "Q", "R"), dA=None, dB=None, dQ=None, dQf=None, dR=None,
              dx0=None, u0=None, info=None, stream=None):
@@ -297,46 +335,28 @@ class LqrSolver:
         (``[N, m]`` float32).  Operands as for :meth:`solve_tv`.  Outputs, each optional: ``dA [N, H, n, n]``,
         ``dB [N, H, n, m]``, ``dQ [N, H, n, n]``, ``dQf [N, n, n]``, ``dR [N, H, m, m]``, ``dx0 [N, n]``, ``u0 [N, m]``,
         ``info [N]`` (int32)."""
-        ops, tstride = [], (ctypes.c_int64 * 4)()
-        for i, (name, t) in enumerate((("A", A), ("B", B), ("Q", Q), ("R", R))):
-            if name in tv:
-                if t.shape[-3] < H:
-                    raise ValueError("operand %s has %d time steps, H = %d" % (name, t.shape[-3], H))
-                ops.append(_operand(t[..., 0, :, :], 2, self.batch))
-                tstride[i] = t.stride(-3)
-            else:
-                ops.append(_operand(t, 2, self.batch))
-                tstride[i] = 0
-        oqf = _operand(Qf, 2, self.batch) if Qf is not None else None      # NULL: Q_f = Q (Q constant in time)
-        ox = _operand(x0, 1, self.batch)
         if tuple(g.shape) != (self.N, self.m) or g.dtype != torch.float32 or not g.is_contiguous():
             raise ValueError("g must be a contiguous float32 tensor of shape (%d, %d)" % (self.N, self.m))
-        ref = lambda o: ctypes.byref(o) if o is not None else None
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
-        _check(load_library().ttc_lqr_grad(
-            self._h, ref(ops[0]), ref(ops[1]), ref(ops[2]), ref(ops[3]), tstride, ref(oqf), ref(ox), self._ptr(g), int(H),
-            self._ptr(dA), self._ptr(dB), self._ptr(dQ), self._ptr(dQf), self._ptr(dR), self._ptr(dx0), self._ptr(u0),
-            self._ptr(info), ctypes.c_void_p(stream.cuda_stream)))
+        ops = _Operands(6, self.batch)
+        refs, tstride = self._tv_ops(A, B, Q, R, H, tv, ops)
+        qf, xx = ops.put(Qf, 2), ops.put(x0, 1)                # Qf None: Q_f = Q (Q constant in time)
+        ptr = self._ptr
+        _check(load_library().ttc_lqr_grad(self._h, *refs, tstride, qf, xx, ptr(g), int(H), ptr(dA), ptr(dB), ptr(dQ), ptr(dQf),
+                                           ptr(dR), ptr(dx0), ptr(u0), ptr(info), self._stream(stream)))
 
     def _layer_inputs(self, tensors, host):
-        s_a, s_gamma_a, s_gamma_b, s_gamma_q, s_b, s_q, s_qf, r_inv, h0, B_basis, Q_basis = tensors
-        r = int(B_basis.shape[0])
+        r = int(tensors[9].shape[0])
         n, N = self.n, self.N
-        per_n = dict(s_a=s_a, s_gamma_a=s_gamma_a, s_gamma_b=s_gamma_b, s_gamma_q=s_gamma_q, r_inv=r_inv, h0=h0)
-        per_r = dict(s_b=s_b, s_q=s_q, s_qf=s_qf)
+        per_n, per_r, basis = (N, n), (N, r), (r, n, n)
         inp = ttc_layer_inputs()
-        for name, t in list(per_n.items()) + list(per_r.items()) + [("B_basis", B_basis), ("Q_basis", Q_basis)]:
-            want = (N, n) if name in per_n else (N, r) if name in per_r else (r, n, n)
-            if host:
-                placed = t.device.type == "cpu"
-            else:
-                placed = t.device.type == "cuda" and (t.device.index or 0) == self.device
-            if tuple(t.shape) != want or t.dtype != torch.float32 or not t.is_contiguous() or not placed:
+        ptrs = []
+        for t, want in zip(tensors, (per_n, per_n, per_n, per_n, per_r, per_r, per_r, per_n, per_n, basis, basis)):
+            placed = not t.is_cuda if host else t.is_cuda and t.get_device() == self.device
+            if t.shape != want or t.dtype != torch.float32 or not t.is_contiguous() or not placed:
                 raise ValueError("%s must be a contiguous float32 tensor of shape %s on %s" %
-                                 (name, want, "the host" if host else "cuda:%d" % self.device))
-            setattr(inp, name, t.data_ptr())
-        inp.r = r
+                                 (LAYER_GRAD_KEYS[len(ptrs)], want, "the host" if host else "cuda:%d" % self.device))
+            ptrs.append(t.data_ptr())
+        _LAYER_INPUTS.pack_into(inp, 0, *ptrs, r)
         return inp
 
     def solve_layer(self, s_a, s_gamma_a, s_gamma_b, s_gamma_q, s_b, s_q, s_qf, r_inv, h0, B_basis, Q_basis, T,
@@ -345,22 +365,18 @@ class LqrSolver:
         ``[N, n]`` (``s_b, s_q, s_qf``: ``[N, r]``), the bases ``[r, n, n]``; all float32, contiguous, on the
         solver's device.  ``u1 [N, n]``, ``P0 [N, n, n]``, ``info [N]`` (int32) are written if given."""
         inp = self._layer_inputs((s_a, s_gamma_a, s_gamma_b, s_gamma_q, s_b, s_q, s_qf, r_inv, h0, B_basis, Q_basis), False)
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
         _check(load_library().ttc_lqr_solve_layer(
             self._h, ctypes.byref(inp), int(T), self._ptr(u1), self._ptr(P0), self._ptr(info),
-            ctypes.c_void_p(stream.cuda_stream)))
+            self._stream(stream)))
 
     def solve_layer_sigma_baseline(self, s_a, s_gamma_a, s_gamma_b, s_gamma_q, s_b, s_q, s_qf, r_inv, h0, B_basis, Q_basis, T,
                                    u1=None, P0=None, info=None, stream=None):
         """``ttc_lqr_solve_layer_sigma_baseline``: the same layer evaluation by the row-normalised reverse symplectic
         product (a baseline whose float32 error grows with the horizon); arguments as :meth:`solve_layer`."""
         inp = self._layer_inputs((s_a, s_gamma_a, s_gamma_b, s_gamma_q, s_b, s_q, s_qf, r_inv, h0, B_basis, Q_basis), False)
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
         _check(load_library().ttc_lqr_solve_layer_sigma_baseline(
             self._h, ctypes.byref(inp), int(T), self._ptr(u1), self._ptr(P0), self._ptr(info),
-            ctypes.c_void_p(stream.cuda_stream)))
+            self._stream(stream)))
 
     def layer_grad(self, s_a, s_gamma_a, s_gamma_b, s_gamma_q, s_b, s_q, s_qf, r_inv, h0, B_basis, Q_basis, T, g,
                    grads, u1=None, info=None, stream=None):
@@ -376,11 +392,9 @@ class LqrSolver:
             setattr(out, k, None if t is None else t.data_ptr())
         if tuple(g.shape) != (self.N, self.n) or g.dtype != torch.float32 or not g.is_contiguous():
             raise ValueError("g must be a contiguous float32 tensor of shape (%d, %d)" % (self.N, self.n))
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
         _check(load_library().ttc_lqr_layer_grad(
             self._h, ctypes.byref(inp), int(T), self._ptr(g), ctypes.byref(out), self._ptr(u1), self._ptr(info),
-            ctypes.c_void_p(stream.cuda_stream)))
+            self._stream(stream)))
 
     def solve_layer_host(self, s_a, s_gamma_a, s_gamma_b, s_gamma_q, s_b, s_q, s_qf, r_inv, h0, B_basis, Q_basis, T,
                          u1=None, P0=None, info=None):
@@ -443,12 +457,11 @@ def solve_first_noalloc(A, B, Q, R, x0, H, batch, P0=None, u0=None, info=None, d
     batch = tuple(int(b) for b in batch)
     batch = (1,) * (3 - len(batch)) + batch
     n, m = B.shape[-2], B.shape[-1]
-    ops = [_operand(A, 2, batch), _operand(B, 2, batch), _operand(Q, 2, batch), _operand(R, 2, batch),
-           _operand(x0, 1, batch)]
-    refs = [ctypes.byref(o) if o is not None else None for o in ops]
+    ops = _Operands(5, batch)
+    refs = [ops.put(A, 2), ops.put(B, 2), ops.put(Q, 2), ops.put(R, 2), ops.put(x0, 1)]
     if stream is None:
         stream = torch.cuda.current_stream(device)
     barr = (ctypes.c_int64 * 3)(*batch)
     ptr = LqrSolver._ptr
     _check(lib.ttc_lqr_solve_first_noalloc(n, m, barr, device, *refs, int(H), ptr(P0), ptr(u0), ptr(info),
-                                           ctypes.c_void_p(stream.cuda_stream)))
+                                           stream.cuda_stream))
