@@ -62,10 +62,12 @@ extern "C" {
 #define TTC_MATH_AUTO  0  /* FP32 when every input is F32, TF32 when Q or x0 is BF16  */
 #define TTC_MATH_FP32  1  /* FFMA, fp32 throughout                                    */
 #define TTC_MATH_TF32  2  /* tcgen05 tensor cores, tf32 operands, fp32 accumulate (n = m = 64) */
-/* n = m = 64 is served by the tensor-core kernel only with TF32 math (AUTO picks it when Q or x0 is
- * BF16), per-head A, B, R and a time-invariant problem; FP32 math at n = m = 64, and every
- * time-varying / affine / gradient call at n = m = 64, run in the generic one-CTA-per-instance kernel
- * (TTC_KERNEL_RICCATI_CTA), which is one to two orders of magnitude slower. */
+/* n = m = 64 is served by the tensor-memory kernel only with TF32 math (AUTO picks it when Q or x0 is
+ * BF16), per-head A, B, R and a time-invariant problem.  Every other time-invariant request, and time-varying /
+ * affine ones up to 32 x 32, run with one warp per instance in float32 (three-pass tf32 products); time-varying and
+ * affine requests above 32 run in the generic one-CTA-per-instance kernel, one to two orders of magnitude slower.
+ * Above 48 states or controls the one-warp kernel keeps part of its matrices in local memory, for which the driver
+ * reserves up to 3.3 GB of device memory at the first such call. */
 
 /* ttc_lqr_solve flags */
 #define TTC_OUT_FIRST_ONLY  1u  /* P is [N][n][n] = P_0 and u is [N][m] = u_0          */
@@ -99,8 +101,8 @@ typedef struct ttc_lqr_handle ttc_lqr_handle; /* opaque; owned by the library */
  * is a DEVICE pointer (on the handle's device), for ttc_lqr_solve_host a HOST pointer.
  * It must be aligned to 16 bytes.  Strides are arbitrary non-negative element counts; vector
  * loads are used when every batch and time stride of an operand is a multiple of 16 bytes
- * (4 F32 or 8 BF16 elements).  Other strides are served with element-wise loads: somewhat
- * slower for n, m <= 16, much slower (the generic kernel) above. */
+ * (4 F32 or 8 BF16 elements).  Other strides are served with element-wise loads, somewhat
+ * slower. */
 typedef struct {
     const void* ptr;
     int32_t     dtype;       /* TTC_F32 or TTC_BF16 (BF16 only for Q and x0)            */

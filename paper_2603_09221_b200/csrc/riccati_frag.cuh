@@ -1,4 +1,4 @@
-// Riccati-backward + rollout kernel, float32, for n, m up to 32 (any request) or 48 (time-invariant): one WARP per
+// Riccati-backward + rollout kernel, float32, for n, m up to 32 (any request) or 64 (time-invariant): one WARP per
 // instance, every matrix of the step in registers in the mma.sync accumulator layout (frag.cuh), so that a step is a
 // chain of tensor-core products, one eight-column factorisation panel per block of controls and a few shuffles, without
 // barriers.  Other sizes than whole blocks are padded: R with the identity, everything else with zero.
@@ -10,12 +10,13 @@
 // What bounds it: at n = 16 a step is 87 tensor-core instructions (8 cycles on a scheduler's pipe, about 4 of its issue
 // slots) in about 830, and four or five warps per scheduler hide most of the chain of five products and sixteen pivots.
 // At n = 32 it is 670 tensor-core instructions, two warps per scheduler (all 255 registers); above, registers spill to
-// local memory (0.3 KB per lane at 40 x 16, 2.6 KB at 40 x 40), which the first-level cache absorbs.
+// local memory (0.3 KB per lane at 40 x 16, 2.7 KB at 40 x 40, which the first-level cache absorbs; 10.7 KB at 64 x 64,
+// which it does not: only twice as fast as one CTA per instance there).
 // The forms this replaced: rows broadcast from shared memory at n = 16 (load/store pipe at 88 %), products through shared
 // memory at n = 32 (74 %), one CTA per instance with two barriers per pivot elsewhere.  Measured before -> now:
 //   65536 instances n = 16, H = 32, operands from memory  4.26 -> 2.65 ms     4096, n = 16, H = 16, all outputs 188 -> 107 us
 //   16384 instances n = 32, H = 64, all outputs           14.2 -> 8.5 ms      1155, n = 40, m = 12, H = 20     2428 -> 232 us
-//   64 instances n = 8, H = 8, own dynamics               107 -> 23 us
+//   64 instances n = 8, H = 8, own dynamics               107 -> 11 us     1155, n = m = 60, H = 20            21.9 -> 10.3 ms
 #pragma once
 
 #include "common.cuh"
@@ -944,11 +945,10 @@ inline cudaError_t launch_one(const SolveParams& p, int sm_count, cudaStream_t s
     return cudaGetLastError();
 }
 
-// Sizes this kernel serves: up to 32 x 32 for every request, up to 48 x 48 for time-invariant ones.
+// Sizes this kernel serves: up to 32 x 32 for every request, all of them for time-invariant ones.
 inline bool riccati_frag_serves(int n, int m, bool time_varying)
 {
-    const int top = time_varying ? 32 : 48;
-    return n <= top && m <= top;
+    return !time_varying || (n <= 32 && m <= 32);
 }
 
 // `exact`: the strides keep the vector loads aligned (rows of Q, Qf, R and of K, A, B in the rollout).  The number of
@@ -984,6 +984,10 @@ inline cudaError_t launch_riccati_frag(const SolveParams& p, bool time_varying, 
         return mb == 1 ? launch_one<5, 1, false, false, true>(p, sm_count, st)
              : mb == 2 ? launch_one<5, 2, false, false, true>(p, sm_count, st)
              : mb == 3 ? launch_one<5, 3, false, false, true>(p, sm_count, st) : launch_one<5, 5, false, false, true>(p, sm_count, st);
+    case 7:
+    case 8:
+        return mb <= 2 ? launch_one<8, 2, false, false, true>(p, sm_count, st)
+             : mb <= 4 ? launch_one<8, 4, false, false, true>(p, sm_count, st) : launch_one<8, 8, false, false, true>(p, sm_count, st);
     default:
         return mb <= 2 ? launch_one<6, 2, false, false, true>(p, sm_count, st)
              : mb <= 4 ? launch_one<6, 4, false, false, true>(p, sm_count, st) : launch_one<6, 6, false, false, true>(p, sm_count, st);
