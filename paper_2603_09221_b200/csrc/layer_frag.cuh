@@ -18,7 +18,7 @@
 //
 // n = 16 is bound by the instructions it issues (about 690 per step, of which 220 are the sixteen pivots and 144 the
 // splitting of operands): 65536 instances, T = 32: 2.28 -> 1.87 ms against the broadcast-row form with two columns per
-// lane; 16 instances (one decoded token of 16 heads) are one dependent chain per SM: 98 -> 47 us.
+// lane; 16 instances (one decoded token of 16 heads) are one dependent chain per SM: 98 -> 41 us.
 // n = 32 needs all 255 registers for its eight 16 x 8 tiles per matrix and keeps two warps per scheduler: 16384
 // instances, T = 32: 5.45 -> 3.2 ms (products through shared memory before).
 #pragma once
@@ -152,7 +152,7 @@ __device__ __forceinline__ void prepare(Slot<NB>& sl, Mat<NB, NB>& nP, const Lay
 
 // The backward recursion of one instance.  nP comes in as -P_T and goes out as -P_0; `on_step(s, Zt, S, w)` is called
 // with what gains() needs after each factorisation.  Returns 0 or s n + j + 1 for the first bad pivot.
-template <int NB, typename F>
+template <int NB, bool PAIR, typename F>
 __device__ __forceinline__ int backward(Mat<NB, NB>& nP, Slot<NB>& sl, const Rates<NB>& rates, const float (&rd)[NB], int T, int lane,
                                         F&& on_step)
 {
@@ -234,7 +234,7 @@ __device__ __forceinline__ int backward(Mat<NB, NB>& nP, Slot<NB>& sl, const Rat
         }
         Split<NB, NB> zs;
         float w[NB][2];
-        const int bad = factor<NB, NB>(S, Zt, zs, w, lane);
+        const int bad = factor<NB, NB, PAIR>(S, Zt, zs, w, lane);
         if (bad && !fail)
             fail = s * N + bad;
         product_symmetric<NB, NB>(nP, zs);
@@ -244,7 +244,8 @@ __device__ __forceinline__ int backward(Mat<NB, NB>& nP, Slot<NB>& sl, const Rat
     return fail;
 }
 
-template <int NB>
+// FEW: at most four warps per SM, see chol8_inverse
+template <int NB, bool FEW>
 __global__ void __launch_bounds__(32 * MAX_WARPS, NB == 2 ? 5 : 2) layer_frag_kernel(LayerParams p)
 {
     constexpr int N = 8 * NB, MT = Mat<NB, NB>::MT;
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB == 2 ? 5 : 2) layer_frag_ke
 #pragma unroll
     for (int b = 0; b < NB; ++b)
         u[b][0] = u[b][1] = 0.f;
-    const int fail = backward<NB>(nP, sl, rates, rd, p.T, lane, [&](int s, Mat<NB, NB>& Zt, const Mat<NB, NB>& S, const float(&w)[NB][2]) {
+    const int fail = backward<NB, FEW>(nP, sl, rates, rd, p.T, lane, [&](int s, Mat<NB, NB>& Zt, const Mat<NB, NB>& S, const float(&w)[NB][2]) {
         if (s == 0 && p.u1) {                               // u_1* = K_1 h_0
             gains<NB, NB>(Zt, S, w, lane);
 #pragma unroll
@@ -311,13 +312,14 @@ template <int NB>
 inline cudaError_t launch_layer_frag(const LayerParams& p, int sm_count, cudaStream_t st)
 {
     const int warps = p.N <= 4ll * sm_count ? 1 : MAX_WARPS;
+    void (*kern)(LayerParams) = p.few ? layer_frag_kernel<NB, true> : layer_frag_kernel<NB, false>;
     const size_t smem = sizeof(Slot<NB>) * warps;
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(layer_frag_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
     }
-    layer_frag_kernel<NB><<<(unsigned)((p.N + warps - 1) / warps), 32 * warps, smem, st>>>(p);
+    kern<<<(unsigned)((p.N + warps - 1) / warps), 32 * warps, smem, st>>>(p);
     return cudaGetLastError();
 }
 

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(32 * lfrag::MAX_WARPS, NB == 2 ? 4 : 2) layer_
             rd[b] = 1.f / __ldg(p.r_inv + inst * N + 8 * b + g);
             k0[b][0] = k0[b][1] = 0.f;
         }
-        fail = lfrag::backward<NB>(nP, sl, rates, rd, T, lane, [&](int s, Mat<NB, NB>& Zt, const Mat<NB, NB>& S, const float(&w)[NB][2]) {
+        fail = lfrag::backward<NB, PART == 1>(nP, sl, rates, rd, T, lane, [&](int s, Mat<NB, NB>& Zt, const Mat<NB, NB>& S, const float(&w)[NB][2]) {
             if (s == 0) {
                 float gv[NB], zc[NB][2];
 #pragma unroll

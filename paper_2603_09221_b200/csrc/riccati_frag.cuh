@@ -483,7 +483,8 @@ __host__ __device__ constexpr size_t warp_bytes()
 // CH = one piece of the horizon of an instance (see SolveParams; time-invariant): it starts from the value matrix and the
 // state at the piece's ends, writes its part of the outputs and leaves failures to the caller.
 // GRAD = the gradients of the first control in the same kernel (n = m = 8 NB, float32 operands): see grad_tail().
-template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false, bool GRAD = false>
+// FEW = at most four warps per SM: the factorisation with the shorter chain (chol8_inverse).
+template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false, bool GRAD = false, bool FEW = false>
 __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 4) riccati_frag_kernel(SolveParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -689,7 +690,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
         }
         Split<NB, MB> zs;
         float w[MB][2];
-        const int bad = factor<NB, MB>(S, Zt, zs, w, lane);  // Zt becomes Z', S the blocks of L
+        const int bad = factor<NB, MB, FEW || (NB > 2)>(S, Zt, zs, w, lane);  // Zt becomes Z', S the blocks of L
         if (bad && !fail)
             fail = ts * m + bad;
         product<NB, MB, NB, true>(nP, &nP, zs, zs);                              // -P_t = -Q - A'PA + Z'Z
@@ -935,13 +936,17 @@ inline cudaError_t launch_one(const SolveParams& p, int sm_count, cudaStream_t s
     const long long nwin = p.b0 * p.b1 * p.tcount * (CH ? p.chunks : 1);
     const int warps = NB > 2 || nwin <= 4ll * sm_count ? 1 : MAX_WARPS;
     const size_t smem = warps * warp_bytes<NB, MB, TV, GRAD>();
+    // (above 16 states two warps per scheduler leave it idle at any batch: the shorter chain always)
+    constexpr bool CAN = NB <= 2 && !AFF && !CH && !GRAD;
+    // by the size of the whole batch: the windows of a sliced call have to give the same bits as one call
+    void (*kern)(SolveParams) = CAN && p.N <= 4ll * sm_count ? riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH, GRAD, CAN>
+                                                  : riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH, GRAD, false>;
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH, GRAD>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
     }
-    riccati_frag_kernel<NB, MB, TV, AFF, PAD, CH, GRAD><<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, smem, st>>>(p);
+    kern<<<(unsigned)((nwin + warps - 1) / warps), 32 * warps, smem, st>>>(p);
     return cudaGetLastError();
 }
 

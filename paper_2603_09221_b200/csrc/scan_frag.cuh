@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(32) scan_power_kernel(SolveParams p, int squar
         negate<NB>(G, B);
         Split<NB, NB> gs;
         float w[NB][2];
-        bad = factor<NB, NB>(S, G, gs, w, lane);            // G = B L_R^{-T}
+        bad = factor<NB, NB, true>(S, G, gs, w, lane);            // G = B L_R^{-T}
         Mat<NB, NB> Gt, C;
         transpose<NB>(Gt, G, lane);
         keep(mem.Gt, Gt, lane);
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(32) scan_power_kernel(SolveParams p, int squar
         }
         Split<2 * NB, NB> zs;
         float w[NB][2];
-        const int b = factor<2 * NB, NB>(S, rhs, zs, w, lane);
+        const int b = factor<2 * NB, NB, true>(S, rhs, zs, w, lane);
         if (b && !bad)
             bad = b;
         Split<NB, NB> us, z1;                               // U and Z'

@@ -7,6 +7,7 @@ namespace layer {
 
 struct LayerParams {
     long long N;                 // instances
+    bool few;                    // the whole batch (of which this may be a slice) has at most four instances per SM
     int T, r;
     const float *s_a, *s_ga, *s_gb, *s_gq;   // [N][n]
     const float *s_b, *s_q, *s_qf;           // [N][r]

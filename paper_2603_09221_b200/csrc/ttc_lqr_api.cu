@@ -52,6 +52,72 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
+// Workspaces of all handles of a device come from one pool, so that a program that makes handles for changing shapes does
+// not pay a cudaMalloc (0.2 to 2 ms above 1 MB) for each.  The pool keeps at most kPoolKeep bytes that no handle uses and
+// gives everything back when the last handle of the device goes.
+constexpr int kMaxPoolDevices = 64;
+constexpr unsigned long long kPoolKeep = 256ull << 20;
+struct DevicePool {
+    std::mutex lock;
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t stream = nullptr;       // orders allocations and releases; nothing else runs on it
+    long long handles = 0;
+};
+DevicePool g_pools[kMaxPoolDevices];
+
+// (the device is current)  A device whose driver has no pools keeps pool == nullptr: cudaMalloc is used.
+void pool_enter(int device)
+{
+    if (device >= kMaxPoolDevices)
+        return;
+    DevicePool& d = g_pools[device];
+    std::lock_guard<std::mutex> guard(d.lock);
+    ++d.handles;
+    if (d.pool)
+        return;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    unsigned long long keep = kPoolKeep;
+    if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess) {
+        d.pool = nullptr;
+    } else if (cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+               cudaStreamCreateWithFlags(&d.stream, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaMemPoolDestroy(d.pool);
+        d.pool = nullptr;
+    }
+    cudaGetLastError();
+}
+void pool_leave(int device)
+{
+    if (device >= kMaxPoolDevices)
+        return;
+    DevicePool& d = g_pools[device];
+    std::lock_guard<std::mutex> guard(d.lock);
+    if (--d.handles == 0 && d.pool) {
+        cudaStreamSynchronize(d.stream);
+        cudaMemPoolTrimTo(d.pool, 0);
+    }
+}
+cudaError_t device_alloc(int device, void** ptr, size_t bytes)
+{
+    DevicePool* d = device < kMaxPoolDevices ? &g_pools[device] : nullptr;
+    if (!d || !d->pool)
+        return cudaMalloc(ptr, bytes);
+    cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, d->pool, d->stream);
+    return e ? e : cudaStreamSynchronize(d->stream);
+}
+// (whatever used the memory has finished)
+void device_free(int device, void* ptr)
+{
+    DevicePool* d = device < kMaxPoolDevices ? &g_pools[device] : nullptr;
+    if (!d || !d->pool)
+        cudaFree(ptr);
+    else
+        cudaFreeAsync(ptr, d->stream);
+}
+
 } // namespace
 
 struct ttc_lqr_handle {
@@ -78,17 +144,20 @@ struct ttc_lqr_handle {
 
 namespace {
 
+// (the handle's device is current)
 int ensure(DevBuf& b, size_t bytes)
 {
     if (bytes <= b.bytes)
         return TTC_OK;
+    int device = 0;
+    TTC_CUDA(cudaGetDevice(&device));
     if (b.ptr) {
         cudaDeviceSynchronize();
-        cudaFree(b.ptr);
+        device_free(device, b.ptr);
         b.ptr = nullptr;
         b.bytes = 0;
     }
-    cudaError_t e = cudaMalloc(&b.ptr, bytes);
+    cudaError_t e = device_alloc(device, &b.ptr, bytes);
     if (e != cudaSuccess) {
         b.ptr = nullptr;
         cudaGetLastError();
@@ -98,10 +167,10 @@ int ensure(DevBuf& b, size_t bytes)
     return TTC_OK;
 }
 
-void release(DevBuf& b)
+void release(int device, DevBuf& b)
 {
     if (b.ptr)
-        cudaFree(b.ptr);
+        device_free(device, b.ptr);
     b.ptr = nullptr;
     b.bytes = 0;
 }
@@ -281,6 +350,7 @@ int ttc_lqr_create(const ttc_lqr_config* cfg, ttc_lqr_handle** out)
     h->host_pipeline_ready = false;
     h->last_launches = h->total_launches = 0;
     h->last_kernel = TTC_KERNEL_NONE;
+    pool_enter(cfg->device);
     *out = h;
     g_err[0] = 0;
     return TTC_OK;
@@ -292,20 +362,20 @@ int ttc_lqr_destroy(ttc_lqr_handle* h)
         return TTC_OK;
     cudaSetDevice(h->cfg.device);
     cudaDeviceSynchronize();
-    release(h->ws_K);
-    release(h->ws_P);
-    release(h->ws_E);
-    release(h->ws_elem);
-    release(h->ws_Q);
-    release(h->ws_info);
-    release(h->ws_G);
-    release(h->ws_k);
-    release(h->ws_vec);
+    release(h->cfg.device, h->ws_K);
+    release(h->cfg.device, h->ws_P);
+    release(h->cfg.device, h->ws_E);
+    release(h->cfg.device, h->ws_elem);
+    release(h->cfg.device, h->ws_Q);
+    release(h->cfg.device, h->ws_info);
+    release(h->cfg.device, h->ws_G);
+    release(h->cfg.device, h->ws_k);
+    release(h->cfg.device, h->ws_vec);
     for (int i = 0; i < 5; ++i) {
-        release(h->st_in[i]);
-        release(h->st_out[i]);
+        release(h->cfg.device, h->st_in[i]);
+        release(h->cfg.device, h->st_out[i]);
     }
-    release(h->st_layer);
+    release(h->cfg.device, h->st_layer);
     if (h->host_pipeline_ready) {
         for (int i = 0; i < kMaxSlices; ++i) {
             cudaEventDestroy(h->ev_in[i]);
@@ -316,6 +386,7 @@ int ttc_lqr_destroy(ttc_lqr_handle* h)
     }
     if (h->host_stream)
         cudaStreamDestroy(h->host_stream);
+    pool_leave(h->cfg.device);
     delete h;
     return TTC_OK;
 }
@@ -809,6 +880,7 @@ static int launch_layer(ttc_lqr_handle* h, const ttc_layer_inputs* in, int32_t T
     const int n = h->cfg.n;
     layer::LayerParams p;
     p.N = cnt < 0 ? h->N : cnt;
+    p.few = h->N <= 4ll * h->sm_count;
     p.T = T;
     p.r = in->r;
     const long long on = i0 * n, orr = i0 * in->r;
