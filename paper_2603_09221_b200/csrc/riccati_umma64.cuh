@@ -199,19 +199,15 @@ __device__ __forceinline__ void wg_barrier(int wg) { asm volatile("bar.sync %0, 
 
 // ---- blocked Cholesky of S fused with the forward substitution Z' = Y' L^{-T} --------------------------------------
 // In-thread Cholesky of an 8 x 8 SPD block: l (lower triangle) is overwritten by L, rinv[i] = 1 / L[i][i].
-// Right-looking; the chain from one pivot to the next is rsqrt -> multiply -> fma.
+// Right-looking; the chain from one pivot to the next is rsqrt -> multiply -> fma.  The signs of the pivots are looked at
+// when the chain is done (a non-positive one turns every later one into NaN or -inf): a test per pivot in the chain, together
+// with a look at misc.dead in every panel, cost 2 % of the step.
 // Returns 0 or 1 + the index of the first non-positive pivot.
 __device__ __forceinline__ int chol8(float (&l)[8][8], float (&rinv)[8])
 {
-    int bad = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        float d = l[j][j];
-        if (!(d > 0.f)) {
-            if (!bad)
-                bad = j + 1;
-            d = 1.f;
-        }
+        const float d = l[j][j];
         float rs;
         asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(d));
         rinv[j] = rs;
@@ -223,8 +219,12 @@ __device__ __forceinline__ int chol8(float (&l)[8][8], float (&rinv)[8])
 #pragma unroll
             for (int c = j + 1; c <= i; ++c)
                 l[i][c] = fmaf(-l[i][j], l[c][j], l[i][c]);
-        l[j][j] = d * rs;
     }
+    int bad = 0;                                            // l[j][j] is still the pivot itself
+#pragma unroll
+    for (int j = 7; j >= 0; --j)
+        if (!(l[j][j] > 0.f))
+            bad = j + 1;
     return bad;
 }
 // x (a row vector of 8) <- x L^{-T}  (forward substitution with the lower factor L)
@@ -415,8 +415,12 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
     long long offA_loaded = -1, offB_loaded = -1, offR_loaded = -1;
     bool dead = false;
 
+    // A thread that has waited in vain once does not wait again; everyone learns of it behind the next barrier that
+    // looks at misc.dead (twice a step: a look in every panel costs 40 cycles of the chain each).
+    bool gave_up = false;
     auto wait_mma = [&]() {
-        if (!mbar_wait(mbar, parity)) {
+        if (!mbar_wait(mbar, parity, gave_up ? 1 : SPIN_LIMIT)) {
+            gave_up = true;
             misc.dead = 1;
             atomicExch(error_flag, 1);
         }
@@ -492,7 +496,8 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                     // ordered after them by the pipe (measured: 7 % error in F when chained), so the issuing thread
                     // waits for W on a barrier of its own before it issues F
                     mma_commit(mbar_w);
-                    if (!mbar_wait(mbar_w, parity_w)) {
+                    if (!mbar_wait(mbar_w, parity_w, gave_up ? 1 : SPIN_LIMIT)) {
+                        gave_up = true;
                         misc.dead = 1;
                         atomicExch(error_flag, 1);
                     }
@@ -591,10 +596,6 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                     }
                     tc_fence_before();
                     wg_barrier(wg);
-                    if (misc.dead != 0) {
-                        dead = true;
-                        break;
-                    }
                     if (!GAINS && pnl == 7 && issuer) {
                         // every row has read its last columns of F: (4) DP = W A into the columns of F
                         // (with gains the columns of F still collect K_t': (4) follows their read-out)
@@ -691,6 +692,8 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                     wg_barrier(wg);
                     if (issuer) {                              // G -= panel * panel[0:64]'  (hi*hi + lo*hi + hi*lo)
                         tc_fence_after();
+                        // all 64 columns, though without gains only those to the right are read again: leaving the
+                        // others out (and the rows of L that are complete) measured 0.3 to 3 % slower
                         const uint32_t idn = instr_desc(64, 1);
                         const uint64_t dh = panel_desc(smem_u32(PH)), dl = panel_desc(smem_u32(PL));
                         mma_ss(RF, dh, dh, idn, 1u);
@@ -794,35 +797,23 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                     const long long Pidx = (inst * (long long)(p.first_only ? 1 : H + 1) + (p.first_only ? 0 : ts)) * N * N + (long long)j * N;
                     if (q_pref) {
 #pragma unroll
-                        for (int qt = 0; qt < 4; ++qt) {       // 16 columns at a time
-                            float q[16];
+                        for (int half = 0; half < 2; ++half) { // 32 columns at a time: two trips to tensor memory
+                            float hh[32];
+                            tmem_ld32(RF + lane_sel + 32 * half, hh);
 #pragma unroll
-                            for (int c = 0; c < 2; ++c) {
-                                const uint4 v4 = qraw[2 * qt + c];
+                            for (int c = 0; c < 4; ++c) {
+                                const uint4 v4 = qraw[4 * half + c];
                                 const uint32_t wd[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) {
-                                    q[8 * c + 2 * e] = __uint_as_float(wd[e] << 16);
-                                    q[8 * c + 2 * e + 1] = __uint_as_float(wd[e] & 0xffff0000u);
+                                    hh[8 * c + 2 * e] += __uint_as_float(wd[e] << 16);
+                                    hh[8 * c + 2 * e + 1] += __uint_as_float(wd[e] & 0xffff0000u);
                                 }
                             }
-                            uint32_t raw[16];
-                            tmem_ld16(RF + lane_sel + 16 * qt, raw);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int c = 0; c < 16; ++c)
-                                q[c] += __uint_as_float(raw[c]);
-                            if (ts > 0) {
-#pragma unroll
-                                for (int c = 0; c < 4; ++c)
-                                    *reinterpret_cast<float4*>(X0 + toff(j, 16 * qt + 4 * c)) =
-                                        make_float4(round_tf32(q[4 * c]), round_tf32(q[4 * c + 1]), round_tf32(q[4 * c + 2]), round_tf32(q[4 * c + 3]));
-                            }
-                            if (Pdst) {
-#pragma unroll
-                                for (int c = 0; c < 4; ++c)
-                                    store_out4(p.P, Pidx + 16 * qt + 4 * c, make_float4(q[4 * c], q[4 * c + 1], q[4 * c + 2], q[4 * c + 3]), obf);
-                            }
+                            if (ts > 0)
+                                store_half_tf32(X0, j, half, hh);
+                            if (Pdst)
+                                store_half_global(p.P, Pidx + 32 * half, hh, obf);
                         }
                     } else {
 #pragma unroll 1
