@@ -711,16 +711,14 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                     const int nn = wt - 64;
                     const long long ko = (inst * (long long)H + ts) * N * N + nn;
 #pragma unroll
-                    for (int qt = 0; qt < 4; ++qt) {
-                        uint32_t raw[16];
-                        tmem_ld16(RF + lane_sel + 16 * qt, raw);
-                        tmem_wait_ld();
+                    for (int half = 0; half < 2; ++half) {
+                        float kv[32];
+                        tmem_ld32(RF + lane_sel + 32 * half, kv);
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            const float kv = __uint_as_float(raw[c]);
-                            Kbase[ko + (long long)(16 * qt + c) * N] = kv;
+                        for (int c = 0; c < 32; ++c) {
+                            Kbase[ko + (long long)(32 * half + c) * N] = kv[c];
                             if (obf && p.K)
-                                store_out(p.K, ko + (long long)(16 * qt + c) * N, kv, 1);
+                                store_out(p.K, ko + (long long)(32 * half + c) * N, kv[c], 1);
                         }
                     }
                 }
@@ -738,10 +736,9 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                 }
                 if (dead)
                     break;
-                // Without gains nothing else runs between here and the read-out: the row of Q that the read-out adds
-                // travels while (5) is in flight (bf16: the whole row in 32 registers).
+                // The row of Q that the read-out adds travels while (5) is in flight (bf16: the whole row in 32 registers).
                 uint4 qraw[8];
-                const bool q_pref = !GAINS && p.Q.dtype == TTC_BF16;
+                const bool q_pref = p.Q.dtype == TTC_BF16;
                 if (q_pref && warp >= 2) {
                     const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.Q.ptr) + oq + (long long)(wt - 64) * N);
 #pragma unroll
