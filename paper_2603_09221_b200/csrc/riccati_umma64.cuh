@@ -529,17 +529,20 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                     // The rows of L^{-T} start from the upper triangle of S, the factorisation reads the lower one, and
                     // the two differ by the rounding of the tf32 contractions (and of a P that is only symmetrised now
                     // and then): at 1e-3 of |S| that would be the error of the gains.  Mirror the lower triangle into
-                    // the upper one first: every row through X1 (free here), element (r, c) at word 64 r + (c ^ r) so
-                    // that both the row stores and the column reads touch 32 banks.
+                    // the upper one first: every row through X1 (free here), the 16-byte chunks of row r at
+                    // position chunk ^ (r mod 16), so that both the row stores and the column reads touch 32 banks.
                     float* tr = reinterpret_cast<float*>(X1);
 #pragma unroll
                     for (int qt = 0; qt < 4; ++qt) {
+                        if (warp == 0 && qt >= 2)              // rows 0..31 end at column 31
+                            break;
                         uint32_t raw[16];
                         tmem_ld16(RF + lane_sel + 16 * qt, raw);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int c = 0; c < 16; ++c)
-                            tr[64 * wt + ((16 * qt + c) ^ wt)] = __uint_as_float(raw[c]);
+                        for (int c = 0; c < 4; ++c)
+                            *reinterpret_cast<uint4*>(tr + 64 * wt + 4 * ((4 * qt + c) ^ (wt & 15))) =
+                                make_uint4(raw[4 * c], raw[4 * c + 1], raw[4 * c + 2], raw[4 * c + 3]);
                     }
                     half_barrier(wg);
 #pragma unroll
@@ -551,7 +554,7 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                         for (int c = 0; c < 16; ++c) {
                             const int cc = 16 * qt + c;
                             if (cc > wt)
-                                raw[c] = __float_as_uint(tr[64 * cc + (wt ^ cc)]);
+                                raw[c] = __float_as_uint(tr[64 * cc + 4 * ((wt >> 2) ^ (cc & 15)) + (wt & 3)]);
                         }
                         tmem_st16(RF + lane_sel + 16 * qt, raw);
                     }
