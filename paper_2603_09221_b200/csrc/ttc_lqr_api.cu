@@ -10,6 +10,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "device_pool.h"
 #include "riccati_cta.cuh"
 #include "riccati_umma64.cuh"
 #include "riccati_frag.cuh"
@@ -24,6 +25,7 @@
 #include "peak_probe.cuh"
 
 using namespace ttc;
+using mem::DevBuf;
 
 namespace {
 
@@ -46,83 +48,6 @@ int fail(int status, const char* fmt, ...)
     } while (0)
 
 constexpr int kMaxSlices = 32;   // token slices of the pipelined host-buffer entry point
-
-struct DevBuf {
-    void* ptr = nullptr;
-    size_t bytes = 0;
-};
-
-// Workspaces of all handles of a device come from one pool, so that a program that makes handles for changing shapes does
-// not pay a cudaMalloc (0.2 to 2 ms above 1 MB) for each.  The pool keeps at most kPoolKeep bytes that no handle uses and
-// gives everything back when the last handle of the device goes.
-constexpr int kMaxPoolDevices = 64;
-constexpr unsigned long long kPoolKeep = 256ull << 20;
-constexpr size_t kPoolLargest = 64ull << 20;    // above, cudaMalloc: the pool maps gigabytes slower (21 against 13 ms)
-struct DevicePool {
-    std::mutex lock;
-    cudaMemPool_t pool = nullptr;
-    cudaStream_t stream = nullptr;       // orders allocations and releases; nothing else runs on it
-    long long handles = 0;
-};
-DevicePool g_pools[kMaxPoolDevices];
-
-// (the device is current)  A device whose driver has no pools keeps pool == nullptr: cudaMalloc is used.
-void pool_enter(int device)
-{
-    if (device >= kMaxPoolDevices)
-        return;
-    DevicePool& d = g_pools[device];
-    std::lock_guard<std::mutex> guard(d.lock);
-    ++d.handles;
-    if (d.pool)
-        return;
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = device;
-    unsigned long long keep = kPoolKeep;
-    if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess) {
-        d.pool = nullptr;
-    } else if (cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
-               cudaStreamCreateWithFlags(&d.stream, cudaStreamNonBlocking) != cudaSuccess) {
-        cudaMemPoolDestroy(d.pool);
-        d.pool = nullptr;
-    }
-    cudaGetLastError();
-}
-void pool_leave(int device)
-{
-    if (device >= kMaxPoolDevices)
-        return;
-    DevicePool& d = g_pools[device];
-    std::lock_guard<std::mutex> guard(d.lock);
-    if (--d.handles == 0 && d.pool) {
-        cudaStreamSynchronize(d.stream);
-        cudaMemPoolTrimTo(d.pool, 0);
-    }
-}
-DevicePool* pool_for(int device, size_t bytes)
-{
-    DevicePool* d = device < kMaxPoolDevices && bytes <= kPoolLargest ? &g_pools[device] : nullptr;
-    return d && d->pool ? d : nullptr;
-}
-cudaError_t device_alloc(int device, void** ptr, size_t bytes)
-{
-    DevicePool* d = pool_for(device, bytes);
-    if (!d)
-        return cudaMalloc(ptr, bytes);
-    cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, d->pool, d->stream);
-    return e ? e : cudaStreamSynchronize(d->stream);
-}
-// (whatever used the memory has finished)
-void device_free(int device, void* ptr, size_t bytes)
-{
-    DevicePool* d = pool_for(device, bytes);
-    if (!d)
-        cudaFree(ptr);
-    else
-        cudaFreeAsync(ptr, d->stream);
-}
 
 } // namespace
 
@@ -159,26 +84,14 @@ int ensure(DevBuf& b, size_t bytes)
     TTC_CUDA(cudaGetDevice(&device));
     if (b.ptr) {
         cudaDeviceSynchronize();
-        device_free(device, b.ptr, b.bytes);
-        b.ptr = nullptr;
-        b.bytes = 0;
+        mem::device_free(b);
     }
-    cudaError_t e = device_alloc(device, &b.ptr, bytes);
+    cudaError_t e = mem::device_alloc(device, b, bytes);
     if (e != cudaSuccess) {
-        b.ptr = nullptr;
         cudaGetLastError();
         return fail(TTC_STATUS_ALLOC_FAILED, "cudaMalloc(%zu bytes): %s", bytes, cudaGetErrorString(e));
     }
-    b.bytes = bytes;
     return TTC_OK;
-}
-
-void release(int device, DevBuf& b)
-{
-    if (b.ptr)
-        device_free(device, b.ptr, b.bytes);
-    b.ptr = nullptr;
-    b.bytes = 0;
 }
 
 size_t workspace_bytes(const ttc_lqr_handle* h)
@@ -356,7 +269,7 @@ int ttc_lqr_create(const ttc_lqr_config* cfg, ttc_lqr_handle** out)
     h->host_pipeline_ready = false;
     h->last_launches = h->total_launches = 0;
     h->last_kernel = TTC_KERNEL_NONE;
-    pool_enter(cfg->device);
+    mem::pool_enter(cfg->device);
     *out = h;
     g_err[0] = 0;
     return TTC_OK;
@@ -368,20 +281,20 @@ int ttc_lqr_destroy(ttc_lqr_handle* h)
         return TTC_OK;
     cudaSetDevice(h->cfg.device);
     cudaDeviceSynchronize();
-    release(h->cfg.device, h->ws_K);
-    release(h->cfg.device, h->ws_P);
-    release(h->cfg.device, h->ws_E);
-    release(h->cfg.device, h->ws_elem);
-    release(h->cfg.device, h->ws_Q);
-    release(h->cfg.device, h->ws_info);
-    release(h->cfg.device, h->ws_G);
-    release(h->cfg.device, h->ws_k);
-    release(h->cfg.device, h->ws_vec);
+    mem::device_free(h->ws_K);
+    mem::device_free(h->ws_P);
+    mem::device_free(h->ws_E);
+    mem::device_free(h->ws_elem);
+    mem::device_free(h->ws_Q);
+    mem::device_free(h->ws_info);
+    mem::device_free(h->ws_G);
+    mem::device_free(h->ws_k);
+    mem::device_free(h->ws_vec);
     for (int i = 0; i < 5; ++i) {
-        release(h->cfg.device, h->st_in[i]);
-        release(h->cfg.device, h->st_out[i]);
+        mem::device_free(h->st_in[i]);
+        mem::device_free(h->st_out[i]);
     }
-    release(h->cfg.device, h->st_layer);
+    mem::device_free(h->st_layer);
     if (h->host_pipeline_ready) {
         for (int i = 0; i < kMaxSlices; ++i) {
             cudaEventDestroy(h->ev_in[i]);
@@ -392,7 +305,7 @@ int ttc_lqr_destroy(ttc_lqr_handle* h)
     }
     if (h->host_stream)
         cudaStreamDestroy(h->host_stream);
-    pool_leave(h->cfg.device);
+    mem::pool_leave(h->cfg.device);
     delete h;
     return TTC_OK;
 }

@@ -1,0 +1,133 @@
+"""The workspace pool (``csrc/device_pool.h``) against a counting stand-in for the CUDA runtime, on the CPU: memory goes back
+to where it came from."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2603_09221_b200", "csrc")
+
+FAKE_RUNTIME = r"""
+#pragma once
+#include <cstddef>
+#include <cstdlib>
+#include <map>
+#include <mutex>
+enum cudaError_t { cudaSuccess = 0, cudaErrorInvalidValue = 1, cudaErrorMemoryAllocation = 2 };
+struct FakePool { int unused; };
+struct FakeStream { int unused; };
+typedef FakePool* cudaMemPool_t;
+typedef FakeStream* cudaStream_t;
+enum { cudaMemAllocationTypePinned = 1, cudaMemLocationTypeDevice = 1, cudaStreamNonBlocking = 1, cudaMemPoolAttrReleaseThreshold = 4 };
+struct cudaMemPoolProps { int allocType; struct { int type, id; } location; };
+namespace fake {
+inline std::mutex lock;
+inline std::map<void*, bool> live;               // allocation -> came from a pool
+inline int fail_pools = 0, pools = 0, streams = 0, wrong = 0;
+inline cudaError_t take(void** p, size_t n, bool pooled)
+{
+    std::lock_guard<std::mutex> g(lock);
+    *p = std::malloc(n < 64 ? n : 64);
+    live[*p] = pooled;
+    return cudaSuccess;
+}
+inline cudaError_t give(void* p, bool pooled)
+{
+    std::lock_guard<std::mutex> g(lock);
+    auto it = live.find(p);
+    if (it == live.end() || it->second != pooled) {
+        ++wrong;
+        return cudaErrorInvalidValue;
+    }
+    live.erase(it);
+    std::free(p);
+    return cudaSuccess;
+}
+} // namespace fake
+inline cudaError_t cudaMalloc(void** p, size_t n) { return fake::take(p, n, false); }
+inline cudaError_t cudaFree(void* p) { return fake::give(p, false); }
+inline cudaError_t cudaMemPoolCreate(cudaMemPool_t* p, const cudaMemPoolProps*)
+{
+    std::lock_guard<std::mutex> g(fake::lock);
+    if (fake::fail_pools > 0) {
+        --fake::fail_pools;
+        return cudaErrorMemoryAllocation;
+    }
+    ++fake::pools;
+    *p = new FakePool();
+    return cudaSuccess;
+}
+inline cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, int, void*) { return cudaSuccess; }
+inline cudaError_t cudaMemPoolTrimTo(cudaMemPool_t, size_t) { return cudaSuccess; }
+inline cudaError_t cudaMemPoolDestroy(cudaMemPool_t p)
+{
+    std::lock_guard<std::mutex> g(fake::lock);
+    --fake::pools;
+    delete p;
+    return cudaSuccess;
+}
+inline cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) { return fake::take(p, n, true); }
+inline cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return fake::give(p, true); }
+inline cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, int)
+{
+    std::lock_guard<std::mutex> g(fake::lock);
+    ++fake::streams;
+    *s = new FakeStream();
+    return cudaSuccess;
+}
+inline cudaError_t cudaStreamDestroy(cudaStream_t s)
+{
+    std::lock_guard<std::mutex> g(fake::lock);
+    --fake::streams;
+    delete s;
+    return cudaSuccess;
+}
+inline cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+inline cudaError_t cudaGetLastError() { return cudaSuccess; }
+"""
+
+DRIVER = r"""
+#include "device_pool.h"
+#include <cstdio>
+#include <cstring>
+using namespace ttc::mem;
+
+int main(int, char** argv)
+{
+    if (!std::strcmp(argv[1], "late_pool")) {            // the first handle gets no pool, the second one does
+        fake::fail_pools = 1;
+        pool_enter(0);
+        DevBuf a, b;
+        device_alloc(0, a, 1024);
+        pool_enter(0);
+        device_alloc(0, b, 1024);
+        device_free(a);
+        device_free(b);
+        pool_leave(0);
+        pool_leave(0);
+    }
+    std::printf("wrong=%d live=%d pools=%d streams=%d\n", fake::wrong, (int)fake::live.size(), fake::pools, fake::streams);
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def driver(tmp_path_factory):
+    if not shutil.which("g++"):
+        pytest.skip("no g++")
+    d = tmp_path_factory.mktemp("pool")
+    (d / "cuda_runtime.h").write_text(FAKE_RUNTIME)
+    (d / "driver.cpp").write_text(DRIVER)
+    cmd = ["g++", "-std=c++17", "-O1", "-pthread", "-I", str(d), "-I", CSRC, str(d / "driver.cpp"), "-o", str(d / "plain")]
+    subprocess.run(cmd, check=True)
+    return {"plain": str(d / "plain")}
+
+
+@pytest.mark.parametrize("scenario", ["late_pool"])
+def test_memory_goes_back_where_it_came_from(driver, scenario):
+    r = subprocess.run([driver["plain"], scenario], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stderr
+    assert r.stdout.startswith("wrong=0 live=0 ")
