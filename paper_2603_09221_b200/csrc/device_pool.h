@@ -2,7 +2,7 @@
 // for changing shapes does not pay a cudaMalloc (0.2 to 2 ms above 1 MB) for each.  Host code only.
 //
 // The pool keeps at most kPoolKeep bytes that no handle uses and gives everything back when the last handle of the device
-// goes.  A buffer belongs to one handle.
+// goes.  Every function may be called from any thread; a buffer belongs to one handle.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -18,7 +18,7 @@ constexpr unsigned long long kPoolKeep = 256ull << 20;
 constexpr size_t kPoolLargest = 64ull << 20;    // above, cudaMalloc: the pool maps gigabytes slower (21 against 13 ms)
 
 struct DevicePool {
-    std::mutex lock;
+    std::mutex lock;                     // guards everything below
     cudaMemPool_t pool = nullptr;
     cudaStream_t stream = nullptr;       // orders allocations and releases; nothing else runs on it
     long long handles = 0;
@@ -78,6 +78,7 @@ inline cudaError_t device_alloc(int device, DevBuf& b, size_t bytes)
     cudaStream_t stream = nullptr;
     if (device < kMaxPoolDevices && bytes <= kPoolLargest) {
         DevicePool& d = g_pools[device];
+        std::lock_guard<std::mutex> guard(d.lock);
         pool = d.pool;
         stream = d.stream;
     }

@@ -1,5 +1,6 @@
 """The workspace pool (``csrc/device_pool.h``) against a counting stand-in for the CUDA runtime, on the CPU: memory goes back
-to where it came from."""
+to where it came from
+and handles of several threads do not race."""
 import os
 import shutil
 import subprocess
@@ -92,7 +93,22 @@ DRIVER = r"""
 #include "device_pool.h"
 #include <cstdio>
 #include <cstring>
+#include <thread>
+#include <vector>
 using namespace ttc::mem;
+
+static void handle_life(int rounds)
+{
+    for (int r = 0; r < rounds; ++r) {
+        pool_enter(0);
+        DevBuf small, large;
+        device_alloc(0, small, 1024);
+        device_alloc(0, large, kPoolLargest + 1);
+        device_free(small);
+        device_free(large);
+        pool_leave(0);
+    }
+}
 
 int main(int, char** argv)
 {
@@ -107,6 +123,22 @@ int main(int, char** argv)
         device_free(b);
         pool_leave(0);
         pool_leave(0);
+    } else if (!std::strcmp(argv[1], "threads")) {
+        for (int round = 0; round < 200; ++round) {      // one handle works without a pool while another one makes it
+            fake::fail_pools = 1;
+            pool_enter(0);
+            std::thread worker([] {
+                for (int i = 0; i < 20; ++i) {
+                    DevBuf b;
+                    device_alloc(0, b, 1024);
+                    device_free(b);
+                }
+            });
+            std::thread other(handle_life, 3);
+            worker.join();
+            other.join();
+            pool_leave(0);
+        }
     }
     std::printf("wrong=%d live=%d pools=%d streams=%d\n", fake::wrong, (int)fake::live.size(), fake::pools, fake::streams);
     return 0;
@@ -121,13 +153,27 @@ def driver(tmp_path_factory):
     d = tmp_path_factory.mktemp("pool")
     (d / "cuda_runtime.h").write_text(FAKE_RUNTIME)
     (d / "driver.cpp").write_text(DRIVER)
-    cmd = ["g++", "-std=c++17", "-O1", "-pthread", "-I", str(d), "-I", CSRC, str(d / "driver.cpp"), "-o", str(d / "plain")]
-    subprocess.run(cmd, check=True)
-    return {"plain": str(d / "plain")}
+    out = {}
+    for name, flags in (("plain", []), ("tsan", ["-fsanitize=thread", "-g"])):
+        cmd = ["g++", "-std=c++17", "-O1", "-pthread", *flags, "-I", str(d), "-I", CSRC, str(d / "driver.cpp"), "-o", str(d / name)]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        assert r.returncode == 0 or name == "tsan", r.stderr
+        out[name] = str(d / name) if r.returncode == 0 else None
+    return out
 
 
-@pytest.mark.parametrize("scenario", ["late_pool"])
+@pytest.mark.parametrize("scenario", ["late_pool", "threads"])
 def test_memory_goes_back_where_it_came_from(driver, scenario):
     r = subprocess.run([driver["plain"], scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stderr
     assert r.stdout.startswith("wrong=0 live=0 ")
+
+
+def test_handles_of_several_threads_do_not_race(driver):
+    if not driver["tsan"]:
+        pytest.skip("g++ has no thread sanitizer")
+    r = subprocess.run([driver["tsan"], "threads"], capture_output=True, text=True, timeout=300)
+    if "ThreadSanitizer: unexpected memory mapping" in r.stderr:
+        pytest.skip("the thread sanitizer does not run on this kernel")
+    assert r.returncode == 0 and "WARNING" not in r.stderr, r.stderr[-2000:]
+    assert "wrong=0" in r.stdout
