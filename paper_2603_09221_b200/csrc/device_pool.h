@@ -1,8 +1,9 @@
 // Device memory of the handles' workspaces: one pool per device, shared by its handles, so that a program that makes handles
 // for changing shapes does not pay a cudaMalloc (0.2 to 2 ms above 1 MB) for each.  Host code only.
 //
-// The pool keeps at most kPoolKeep bytes that no handle uses and gives everything back when the last handle of the device
-// goes.  Every function may be called from any thread; a buffer belongs to one handle.
+// The pool keeps at most kPoolKeep bytes that no handle uses.  It lives as long as some handle of the device does: the
+// last one to go destroys the pool and its stream.  Every function may be called from any thread; a buffer belongs to
+// one handle, and between that handle's pool_enter and pool_leave the pool cannot go away.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -66,8 +67,11 @@ inline void pool_leave(int device)
     DevicePool& d = g_pools[device];
     std::lock_guard<std::mutex> guard(d.lock);
     if (--d.handles == 0 && d.pool) {
-        cudaStreamSynchronize(d.stream);
-        cudaMemPoolTrimTo(d.pool, 0);
+        cudaStreamSynchronize(d.stream);         // every release has happened: the memory goes back with the pool
+        cudaMemPoolDestroy(d.pool);
+        cudaStreamDestroy(d.stream);
+        d.pool = nullptr;
+        d.stream = nullptr;
     }
 }
 

@@ -1,6 +1,5 @@
 """The workspace pool (``csrc/device_pool.h``) against a counting stand-in for the CUDA runtime, on the CPU: memory goes back
-to where it came from
-and handles of several threads do not race."""
+to where it came from, nothing is left when the last handle goes, and handles of several threads do not race."""
 import os
 import shutil
 import subprocess
@@ -139,6 +138,8 @@ int main(int, char** argv)
             other.join();
             pool_leave(0);
         }
+    } else {                                             // the pool is made again after its last handle went
+        handle_life(2);
     }
     std::printf("wrong=%d live=%d pools=%d streams=%d\n", fake::wrong, (int)fake::live.size(), fake::pools, fake::streams);
     return 0;
@@ -162,11 +163,11 @@ def driver(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["late_pool", "threads"])
-def test_memory_goes_back_where_it_came_from(driver, scenario):
+@pytest.mark.parametrize("scenario", ["late_pool", "threads", "again"])
+def test_memory_goes_back_where_it_came_from_and_nothing_stays(driver, scenario):
     r = subprocess.run([driver["plain"], scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stderr
-    assert r.stdout.startswith("wrong=0 live=0 ")
+    assert r.stdout.strip() == "wrong=0 live=0 pools=0 streams=0"
 
 
 def test_handles_of_several_threads_do_not_race(driver):
