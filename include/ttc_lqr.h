@@ -125,8 +125,8 @@ typedef struct {
  * Definition A.1, fixes what a "problem" is: {A,B,Q,R}, h_0 and a horizon).
  * Validates cfg, selects the device, returns an opaque handle in *out.  The handle owns
  * only its device workspace, which is allocated on first need inside a solve call (such
- * a call synchronises the device once) and given up by ttc_lqr_destroy.  Workspaces of up to
- * 64 MB come from a pool that the handles of a device share: it keeps at most 256 MB that no
+ * a call synchronises the device once) and given up by ttc_lqr_destroy.  Workspaces of 64 KB
+ * to 64 MB come from a pool that the handles of a device share: it keeps at most 256 MB that no
  * handle uses, and goes with the last handle of the device.
  * Errors: INVALID_ARGUMENT (null pointers, sizes out of range), UNSUPPORTED (method/math
  * not available for this shape), CUDA_ERROR (no such device / not an sm_100 device).

@@ -1,9 +1,9 @@
 // Device memory of the handles' workspaces: one pool per device, shared by its handles, so that a program that makes handles
-// for changing shapes does not pay a cudaMalloc (0.2 to 2 ms above 1 MB) for each.  Host code only.
+// for changing shapes does not pay a cudaMalloc (0.35 ms from 2 MB on, and 0.3 ms for its release) for each.  Host code only.
 //
-// The pool keeps at most kPoolKeep bytes that no handle uses.  It lives as long as some handle of the device does: the
-// last one to go destroys the pool and its stream.  Every function may be called from any thread; a buffer belongs to
-// one handle, and between that handle's pool_enter and pool_leave the pool cannot go away.
+// The pool is made by the first buffer that goes into it and keeps at most kPoolKeep bytes that no handle uses.  When the
+// last handle of the device goes, the pool and its stream are destroyed.  Every function may be called from any thread; a
+// buffer belongs to one handle, and between that handle's pool_enter and pool_leave the pool cannot go away.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -16,7 +16,11 @@ namespace mem {
 
 constexpr int kMaxPoolDevices = 64;
 constexpr unsigned long long kPoolKeep = 256ull << 20;
-constexpr size_t kPoolLargest = 64ull << 20;    // above, cudaMalloc: the pool maps gigabytes slower (21 against 13 ms)
+// Outside these sizes cudaMalloc is the faster one.  Small buffers (the four status words of n = 64) find room in a block
+// that the driver has mapped already: 3 us, where the first buffer of a pool takes 0.22 ms, and making and destroying
+// pool and stream 0.25 ms.  Gigabytes are mapped slower by the pool (21 against 13 ms).
+constexpr size_t kPoolSmallest = 64ull << 10;
+constexpr size_t kPoolLargest = 64ull << 20;
 
 struct DevicePool {
     std::mutex lock;                     // guards everything below
@@ -32,8 +36,7 @@ struct DevBuf {
     cudaStream_t stream = nullptr;       // the pool's stream, or null for memory from cudaMalloc
 };
 
-// (the device is current, here and below)  Where the pool cannot be made, buffers come from cudaMalloc until a later
-// handle makes it; each buffer remembers where it came from.
+// (the device is current, here and below)
 inline void pool_enter(int device)
 {
     if (device >= kMaxPoolDevices)
@@ -41,8 +44,12 @@ inline void pool_enter(int device)
     DevicePool& d = g_pools[device];
     std::lock_guard<std::mutex> guard(d.lock);
     ++d.handles;
-    if (d.pool)
-        return;
+}
+
+// (d.lock is held)  Where the pool cannot be made, buffers come from cudaMalloc until a later one makes it; each buffer
+// remembers where it came from.
+inline void make_pool(DevicePool& d, int device)
+{
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -80,9 +87,11 @@ inline cudaError_t device_alloc(int device, DevBuf& b, size_t bytes)
 {
     cudaMemPool_t pool = nullptr;
     cudaStream_t stream = nullptr;
-    if (device < kMaxPoolDevices && bytes <= kPoolLargest) {
+    if (device < kMaxPoolDevices && bytes > kPoolSmallest && bytes <= kPoolLargest) {
         DevicePool& d = g_pools[device];
         std::lock_guard<std::mutex> guard(d.lock);
+        if (!d.pool)
+            make_pool(d, device);
         pool = d.pool;
         stream = d.stream;
     }

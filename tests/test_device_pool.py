@@ -100,10 +100,12 @@ static void handle_life(int rounds)
 {
     for (int r = 0; r < rounds; ++r) {
         pool_enter(0);
-        DevBuf small, large;
-        device_alloc(0, small, 1024);
+        DevBuf status, middle, large;
+        device_alloc(0, status, kPoolSmallest);
+        device_alloc(0, middle, kPoolSmallest + 1);
         device_alloc(0, large, kPoolLargest + 1);
-        device_free(small);
+        device_free(status);
+        device_free(middle);
         device_free(large);
         pool_leave(0);
     }
@@ -111,25 +113,25 @@ static void handle_life(int rounds)
 
 int main(int, char** argv)
 {
-    if (!std::strcmp(argv[1], "late_pool")) {            // the first handle gets no pool, the second one does
+    if (!std::strcmp(argv[1], "late_pool")) {            // the first buffer gets no pool, the second one does
         fake::fail_pools = 1;
         pool_enter(0);
         DevBuf a, b;
-        device_alloc(0, a, 1024);
+        device_alloc(0, a, 1 << 20);
         pool_enter(0);
-        device_alloc(0, b, 1024);
+        device_alloc(0, b, 1 << 20);
         device_free(a);
         device_free(b);
         pool_leave(0);
         pool_leave(0);
     } else if (!std::strcmp(argv[1], "threads")) {
-        for (int round = 0; round < 200; ++round) {      // one handle works without a pool while another one makes it
+        for (int round = 0; round < 200; ++round) {      // two handles, the first attempt at a pool fails
             fake::fail_pools = 1;
             pool_enter(0);
             std::thread worker([] {
                 for (int i = 0; i < 20; ++i) {
                     DevBuf b;
-                    device_alloc(0, b, 1024);
+                    device_alloc(0, b, 1 << 20);
                     device_free(b);
                 }
             });
@@ -138,6 +140,15 @@ int main(int, char** argv)
             other.join();
             pool_leave(0);
         }
+    } else if (!std::strcmp(argv[1], "no_pool")) {       // handles that need no pool do not make one
+        pool_enter(0);
+        DevBuf a, b;
+        device_alloc(0, a, 16);
+        device_alloc(0, b, kPoolLargest + 1);
+        std::printf("made=%d ", fake::pools);
+        device_free(a);
+        device_free(b);
+        pool_leave(0);
     } else {                                             // the pool is made again after its last handle went
         handle_life(2);
     }
@@ -168,6 +179,11 @@ def test_memory_goes_back_where_it_came_from_and_nothing_stays(driver, scenario)
     r = subprocess.run([driver["plain"], scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stderr
     assert r.stdout.strip() == "wrong=0 live=0 pools=0 streams=0"
+
+
+def test_a_pool_is_made_only_for_buffers_that_go_into_it(driver):
+    r = subprocess.run([driver["plain"], "no_pool"], capture_output=True, text=True, timeout=120)
+    assert r.stdout.strip() == "made=0 wrong=0 live=0 pools=0 streams=0"
 
 
 def test_handles_of_several_threads_do_not_race(driver):
