@@ -87,9 +87,8 @@ extern "C" {
 
 /* ids returned by TTC_QUERY_LAST_KERNEL */
 #define TTC_KERNEL_NONE           0
-#define TTC_KERNEL_RICCATI_CTA    1  /* recursion on any shape, any mix of strides     */
-#define TTC_KERNEL_RICCATI_WARP   2  /* recursion at n = m = 16 / 32, A, B, R all per head or all per
-                                        token, rows of Q and Qf on 16-byte boundaries      */
+#define TTC_KERNEL_RICCATI_CTA    1  /* recursion, one CTA per instance: time-varying / affine above 32 x 32 */
+#define TTC_KERNEL_RICCATI_WARP   2  /* recursion, one warp per instance: every other request but TF32 math's */
 #define TTC_KERNEL_SCAN           4  /* symplectic-pair scan + gain/rollout kernel     */
 #define TTC_KERNEL_RICCATI_UMMA   5  /* tcgen05 contractions (tensor memory), n = m = 64 */
 #define TTC_KERNEL_LAYER          6  /* contextualised layer: parameters synthesised in-kernel */
@@ -188,9 +187,8 @@ int ttc_lqr_solve_lowrank_q(ttc_lqr_handle* h,
  * at every t); the matrix of step t of instance i starts at the operand's batch offset + t * tstride.
  * Qf [n][n] (F32 or BF16, batch strides like any operand) is the terminal weight; it may be NULL only when
  * tstride[2] == 0, and then Q_f = Q.  Everything else (outputs, info, flags, stream, errors) as ttc_lqr_solve.
- * Served by the fp32 kernels (n = m = 16 / 32 warp kernel when A, B, R are all shared by the tokens of a head or all
- * per token, generic kernel otherwise); TTC_SCAN handles
- * time-invariant problems only and returns TTC_STATUS_UNSUPPORTED here.
+ * Served by the fp32 kernels (one warp per instance up to 32 x 32, the generic one-CTA-per-instance kernel above);
+ * TTC_SCAN handles time-invariant problems only and returns TTC_STATUS_UNSUPPORTED here.
  */
 int ttc_lqr_solve_tv(ttc_lqr_handle* h,
                      const ttc_operand* A, const ttc_operand* B, const ttc_operand* Q, const ttc_operand* R,

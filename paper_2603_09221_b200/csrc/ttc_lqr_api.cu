@@ -431,9 +431,9 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
         const bool bf16_in = (Q->dtype == TTC_BF16) || (x0 && x0->ptr && x0->dtype == TTC_BF16);
         const bool want_tf32 = h->cfg.math == TTC_MATH_TF32 || (h->cfg.math == TTC_MATH_AUTO && bf16_in);
         const bool head_shared = A->bstride[2] == 0 && B->bstride[2] == 0 && R->bstride[2] == 0;
-        // The tcgen05 and the warp kernels read the rows of Q and Qf with 16-byte loads: every batch and time stride
-        // of those operands must keep a row start on a 16-byte boundary (4 fp32 or 8 bf16 elements).  Other strides
-        // are served by the generic kernel, which loads element by element.
+        // The tcgen05 kernel and the unguarded variants of the one-warp kernel read the rows of Q and Qf with 16-byte
+        // loads: every batch and time stride of those operands must keep a row start on a 16-byte boundary (4 fp32 or 8
+        // bf16 elements).  Other strides go to the guarded variants, which load element by element.
         const bool q_rows_aligned = vector_rows_ok(p.Q) && (!p.Qf.ptr || vector_rows_ok(p.Qf));
         if (want_tf32 && n == 64 && m == 64 && head_shared && !time_varying && q_rows_aligned) {
             // tcgen05 kernel: persistent CTAs, four independent warpgroups each
@@ -467,7 +467,7 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
             h->last_kernel = TTC_KERNEL_RICCATI_UMMA;
             return TTC_OK;
         }
-        // A, B, R either all per head or all per token
+        // bfloat16 outputs are offered where A, B, R belong all to the head or all to the token
         const bool per_token = A->bstride[2] != 0 && B->bstride[2] != 0 && R->bstride[2] != 0;
         const bool uniform = (head_shared || per_token) && n == m && (n == 16 || n == 32) && q_rows_aligned;
         if (obf && !uniform)
@@ -481,7 +481,7 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
                 return fail(TTC_STATUS_CUDA_ERROR, "riccati_frag launch: %s", cudaGetErrorString(e));
             h->last_launches += 1;
             h->total_launches += 1;
-            h->last_kernel = uniform ? TTC_KERNEL_RICCATI_WARP : TTC_KERNEL_RICCATI_CTA;
+            h->last_kernel = TTC_KERNEL_RICCATI_WARP;
             return TTC_OK;
         }
         const size_t smem = riccati_cta_smem_bytes(n, m);
@@ -655,11 +655,9 @@ int ttc_lqr_grad(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
             const cudaError_t e = rfrag::launch_grad_frag(p, h->sm_count, st);
             if (e != cudaSuccess)
                 return fail(TTC_STATUS_CUDA_ERROR, "gradient launch: %s", cudaGetErrorString(e));
-            const bool head = A->bstride[2] == 0 && B->bstride[2] == 0 && R->bstride[2] == 0;
-            const bool token = A->bstride[2] != 0 && B->bstride[2] != 0 && R->bstride[2] != 0;
             h->last_launches = 1;
             h->total_launches += 1;
-            h->last_kernel = head || token ? TTC_KERNEL_RICCATI_WARP : TTC_KERNEL_RICCATI_CTA;
+            h->last_kernel = TTC_KERNEL_RICCATI_WARP;
             return TTC_OK;
         }
     }

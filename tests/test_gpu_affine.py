@@ -78,18 +78,19 @@ def check(out, ref, first_only, tol=1e-4):
     return errs
 
 
-@pytest.mark.parametrize("n,m,H", [(1, 1, 3), (5, 3, 6), (8, 8, 5), (16, 16, 12), (32, 32, 7), (12, 16, 4), (64, 64, 3)])
+@pytest.mark.parametrize("n,m,H", [(1, 1, 3), (5, 3, 6), (8, 8, 5), (16, 16, 12), (32, 32, 7), (12, 16, 4), (64, 64, 3),
+                                   (33, 33, 4), (40, 12, 6), (12, 36, 3)])
 def test_affine_all_outputs(n, m, H):
     w = affine_workload(n, m, H, (2, 3, 5), seed=900 + 7 * n + H)
     out, ref = run_both(w)
     errs = check(out, ref, False)
     print(n, m, H, out["kernel"], errs)
-    assert out["kernel"] == ("riccati_warp" if n == m and n in (16, 32) else "riccati_cta")
+    assert out["kernel"] == ("riccati_warp" if max(n, m) <= 32 else "riccati_cta")
     for k in ("K", "kff", "P", "pvec", "x", "u"):
         assert not torch.any(out[k] == 123456.0), "canary left in %s" % k
 
 
-@pytest.mark.parametrize("n", [8, 16, 32])
+@pytest.mark.parametrize("n", [8, 16, 32, 40])
 def test_affine_first_only_and_constant_linear_term(n):
     w = affine_workload(n, n, 9, (1, 2, 7), seed=60 + n, tv=("A", "Q"))       # r, B, R constant in time
     out, ref = run_both(w, first_only=True, want=("P", "pvec", "u", "info"))
@@ -122,10 +123,11 @@ def test_affine_warp_kernel_ragged_chunks_and_output_subsets(n, T):
         check(o, ref, first_only)
 
 
-def test_affine_failure_fills_every_output_with_nan():
-    w = affine_workload(16, 16, 5, (1, 2, 9), seed=77)
+@pytest.mark.parametrize("n", [16, 40])
+def test_affine_failure_fills_every_output_with_nan(n):
+    w = affine_workload(n, n, 5, (1, 2, 9), seed=77)
     w["R"] = w["R"].clone()
-    w["R"][0, 1, 0] = -50.0 * torch.eye(16, device=DEV)           # head 1: S_t loses positive definiteness
+    w["R"][0, 1, 0] = -50.0 * torch.eye(n, device=DEV)           # head 1: S_t loses positive definiteness
     out, _ = run_both(w, with_ref=False)
     info = out["info"].cpu().numpy().reshape(2, 9)
     assert (info[0] == 0).all() and (info[1] != 0).all()

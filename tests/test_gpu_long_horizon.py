@@ -12,7 +12,7 @@ from tests import parity_util as pu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("cfg,batch,kernel", [(0, (1, 1, 6), "riccati_cta"), (1, (1, 2, 20), "riccati_warp"),
+@pytest.mark.parametrize("cfg,batch,kernel", [(0, (1, 1, 6), "riccati_warp"), (1, (1, 2, 20), "riccati_warp"),
                                               (3, (1, 2, 10), "riccati_warp"), (4, (1, 2, 8), "riccati_umma"),
                                               (2, (1, 1, 8), "riccati_umma")])
 def test_unstable_dynamics_long_horizon(cfg, batch, kernel):
@@ -39,3 +39,25 @@ def test_unstable_dynamics_long_horizon(cfg, batch, kernel):
             P = gpu["P"].reshape((N, -1) + gpu["P"].shape[-2:])
             asym = float((P - P.transpose(-1, -2)).abs().max() / P.abs().max())
             assert asym <= (1e-6 if w["tol"] < 1e-3 else w["tol"] / 4), asym     # tf32 kernel: symmetrised every 8th step
+
+
+@pytest.mark.parametrize("n,kernel", [(16, "riccati_warp"), (40, "riccati_cta")])
+def test_unstable_dynamics_long_horizon_time_varying_kernels(n, kernel):
+    """The same through ttc_lqr_solve_tv (a terminal weight of its own), whose kernels symmetrise every step too."""
+    H, batch = 400, (1, 2, 6)
+    gen = torch.Generator(device="cuda:0")
+    gen.manual_seed(60 + n)
+    rn = lambda *shape: torch.randn(shape, generator=gen, device="cuda:0")
+    A = rn(1, 2, 1, n, n)
+    A = A * (1.15 / torch.linalg.eigvals(A).abs().amax(-1))[..., None, None]
+    psd = lambda *shape: (lambda L: 0.5 * (L @ L.mT + (L @ L.mT).mT) / n + 0.1 * torch.eye(n, device="cuda:0"))(rn(*shape, n, n))
+    w = dict(A=A.contiguous(), B=rn(1, 2, 1, n, n) / n ** 0.5, Q=psd(*batch), R=psd(1, 2, 1), Qf=psd(*batch), x0=rn(*batch, n),
+             n=n, m=n, H=H, batch=batch, tv=(), first_only=True)
+    s = lqr.LqrSolver(n, n, H, batch)
+    out = lqr.alloc_outputs(n, n, H, 12, "cuda:0", first_only=True, want=("P", "u", "info"))
+    s.solve_tv(w["A"], w["B"], w["Q"], w["R"], w["Qf"], w["x0"], H, tv=(), flags=lqr.TTC_OUT_FIRST_ONLY, **out)
+    torch.cuda.synchronize()
+    assert lqr.KERNEL_NAMES[s.query(lqr.TTC_QUERY_LAST_KERNEL)] == kernel
+    s.close()
+    pu.compare(out, pu.run_oracle_tv(w), np.arange(12), 1e-4, names=("P", "u"))
+    assert float((out["P"] - out["P"].mT).abs().max() / out["P"].abs().max()) <= 1e-6

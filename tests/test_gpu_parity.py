@@ -124,7 +124,7 @@ def test_per_instance_systems_and_strides():
 @pytest.mark.parametrize("method,n,bf16", [("riccati", 8, False), ("scan", 8, False), ("riccati", 16, False),
                                             ("riccati", 32, False), ("riccati", 64, True)])
 def test_not_positive_definite_instance_is_isolated(method, n, bf16):
-    # n = 8: generic kernel, 16 / 32: warp kernel, 64 with bf16 inputs: tcgen05 kernel
+    # up to 32: one-warp kernel (n = 8 with A, B, R per instance), 64 with bf16 inputs: tcgen05 kernel
     H = 6
     w = small_workload(n, n, H, (1, 1, 6), seed=9 + n, bf16=bf16)
     R_ok = w["R"].expand(1, 1, 6, n, n).clone()
@@ -132,14 +132,14 @@ def test_not_positive_definite_instance_is_isolated(method, n, bf16):
     R[0, 0, 2] = -10.0 * R[0, 0, 2]               # instance 2: R negative definite
     Q = w["Q"].clone()
     Q[0, 0, 4, 0, 0] = float("nan")               # instance 4: NaN input
-    per_instance = n == 8                          # per-token R needs the generic kernel; the others keep per-head R
+    per_instance = n == 8                          # R of the instance; the others keep per-head R
     if not per_instance:
         # keep A, B, R per head: break instance 2 through an indefinite Q instead (S loses definiteness)
         R = R_ok
         Q[0, 0, 2] = -50.0 * torch.eye(n, device=DEV, dtype=Q.dtype)
     w = dict(w, R=R.contiguous() if per_instance else w["R"], Q=Q)
     gpu = pu.run_gpu(w, method=METHODS[method])
-    expect = {8: "riccati_cta", 16: "riccati_warp", 32: "riccati_warp", 64: "riccati_umma"}[n] if method == "riccati" else "scan"
+    expect = {8: "riccati_warp", 16: "riccati_warp", 32: "riccati_warp", 64: "riccati_umma"}[n] if method == "riccati" else "scan"
     assert lqr.KERNEL_NAMES[gpu["kernel"]] == expect
     info = gpu["info"].cpu().numpy()
     assert info[2] > 0 and info[4] > 0 and np.all(info[[0, 1, 3, 5]] == 0), info
@@ -197,7 +197,7 @@ def test_first_control_request_on_a_batch_that_fills_the_machine():
 
 @pytest.mark.parametrize("first", [False, True])
 def test_tensor_core_kernel_on_float32_inputs_when_asked_for(first):
-    """float32 Q and x0 at n = m = 64 go to the generic kernel by default; with TTC_MATH_TF32 the tensor-core kernel takes
+    """float32 Q and x0 at n = m = 64 go to the one-warp kernel by default; with TTC_MATH_TF32 the tensor-core kernel takes
     them (the rows of Q are then read as float32).  Checked at the tf32 bounds of the bfloat16 configurations."""
     w = small_workload(64, 64, 6, (1, 2, 21), seed=640, bf16=False)
     N = 42
@@ -290,10 +290,10 @@ def test_tensor_core_kernel_ragged_work_items(tokens):
 
 
 @pytest.mark.parametrize("n,bf16,pad", [(16, False, 1), (32, False, 2), (64, True, 4), (16, False, 4)])
-def test_q_strides_that_break_16_byte_rows_go_to_the_generic_kernel(n, bf16, pad):
+def test_q_strides_that_break_16_byte_rows(n, bf16, pad):
     """Q with a batch stride of n*n + pad elements: when that is not a multiple of 16 bytes the rows of Q no longer
-    start on a 16-byte boundary and the request must be served by the generic kernel (scalar loads), never by a
-    kernel that reads rows with 16-byte loads; a padded stride that keeps the alignment stays on the fast kernel."""
+    start on a 16-byte boundary and must not be read with 16-byte loads (which would fault): the tcgen05 kernel leaves the
+    request to the one-warp kernel, which takes its guarded variant."""
     H, batch = 5, (1, 2, 9)
     w = small_workload(n, n, H, batch, seed=77 + n + pad, bf16=bf16)
     N = int(np.prod(batch))
@@ -304,7 +304,7 @@ def test_q_strides_that_break_16_byte_rows_go_to_the_generic_kernel(n, bf16, pad
     gpu = pu.run_gpu(w)
     aligned = (pad * (2 if bf16 else 4)) % 16 == 0
     fast = {16: "riccati_warp", 32: "riccati_warp", 64: "riccati_umma"}[n]
-    assert lqr.KERNEL_NAMES[gpu["kernel"]] == (fast if aligned else "riccati_cta")
+    assert lqr.KERNEL_NAMES[gpu["kernel"]] == (fast if aligned else "riccati_warp")
     ref = pu.run_oracle(w)
     pu.compare(gpu, ref, np.arange(N), w["tol"])
 

@@ -1,5 +1,5 @@
 """A, B, R that belong to the token instead of the head (the contextualised layer's situation, given as dense matrices):
-the fp32 warp kernel keeps a copy per instance.  Parity of every entry point that can receive such operands."""
+a warp (up to 32 x 32) or a CTA loads the operands of its own instance.  Parity of every entry point that can receive such operands."""
 import numpy as np
 import pytest
 import torch
@@ -87,15 +87,18 @@ def test_per_token_linear_cost():
     check(out, ref, True)
 
 
-def test_mixed_sharing_goes_to_the_generic_kernel():
-    """A per token but B, R per head: neither layout of the warp kernel applies."""
+@pytest.mark.parametrize("n,keys,expect", [(16, ("A",), "riccati_warp"), (32, ("B", "R"), "riccati_warp"),
+                                           (40, ("A",), "riccati_cta"), (36, ("R",), "riccati_cta"),
+                                           (36, ("A", "B", "R"), "riccati_cta")])
+def test_mixed_sharing(n, keys, expect):
+    """Some of A, B, R per token, the others per head."""
     H, batch = 5, (1, 2, 6)
-    w = per_token(tv_workload(16, 16, H, batch, seed=4), seed=1, keys=("A",))
-    s = lqr.LqrSolver(16, 16, H, batch)
-    out = lqr.alloc_outputs(16, 16, H, 12, DEV, first_only=False, want=("K", "P", "x", "u", "info"))
+    w = per_token(tv_workload(n, n, H, batch, seed=4), seed=1, keys=keys)
+    s = lqr.LqrSolver(n, n, H, batch)
+    out = lqr.alloc_outputs(n, n, H, 12, DEV, first_only=False, want=("K", "P", "x", "u", "info"))
     s.solve_tv(w["A"], w["B"], w["Q"], w["R"], w["Qf"], w["x0"], H, tv=w["tv"], K=out["K"], P=out["P"], x=out["x"], u=out["u"],
                info=out["info"])
     torch.cuda.synchronize()
-    assert lqr.KERNEL_NAMES[s.query(lqr.TTC_QUERY_LAST_KERNEL)] == "riccati_cta"
+    assert lqr.KERNEL_NAMES[s.query(lqr.TTC_QUERY_LAST_KERNEL)] == expect
     s.close()
     pu.compare(out, oracle_tv(w, H, False), np.arange(12), 1e-4)

@@ -56,8 +56,11 @@ def run_both(w, want=("K", "P", "x", "u", "info"), first_only=False, H=None):
     return out, ref
 
 
-@pytest.mark.parametrize("n,m,H,expect", [(1, 1, 3, "riccati_cta"), (5, 3, 6, "riccati_cta"), (16, 16, 12, "riccati_warp"),
-                                          (32, 32, 7, "riccati_warp"), (64, 64, 3, "riccati_cta"), (12, 16, 4, "riccati_cta")])
+# the generic one-CTA kernel serves what is above 32 x 32: sizes at the edges of its 4 x 4 register tiles, either side larger
+@pytest.mark.parametrize("n,m,H,expect", [(1, 1, 3, "riccati_warp"), (5, 3, 6, "riccati_warp"), (16, 16, 12, "riccati_warp"),
+                                          (32, 32, 7, "riccati_warp"), (64, 64, 3, "riccati_cta"), (12, 16, 4, "riccati_warp"),
+                                          (33, 33, 4, "riccati_cta"), (40, 12, 9, "riccati_cta"), (12, 40, 5, "riccati_cta"),
+                                          (64, 1, 4, "riccati_cta"), (1, 35, 3, "riccati_cta"), (47, 50, 3, "riccati_cta")])
 def test_time_varying_all_outputs(n, m, H, expect):
     w = tv_workload(n, m, H, (2, 3, 5), seed=500 + 7 * n + H)
     out, ref = run_both(w)
@@ -68,14 +71,14 @@ def test_time_varying_all_outputs(n, m, H, expect):
 
 
 @pytest.mark.parametrize("tv", [("A",), ("Q",), ("B", "R"), ()])
-@pytest.mark.parametrize("n", [8, 16])
+@pytest.mark.parametrize("n", [8, 16, 36])
 def test_partially_time_varying_and_terminal_weight_only(n, tv):
     w = tv_workload(n, n, 9, (1, 2, 9), seed=40 + n + len(tv), tv=tv)
     out, ref = run_both(w)
     pu.compare(out, ref, np.arange(18), 1e-4)
 
 
-@pytest.mark.parametrize("n", [16, 32])
+@pytest.mark.parametrize("n", [16, 32, 40])
 def test_time_varying_first_only_bf16_and_shorter_horizon(n):
     w = tv_workload(n, n, 10, (1, 2, 7), seed=77 + n, bf16=True)
     out, ref = run_both(w, want=("P", "u", "info"), first_only=True)
@@ -95,6 +98,45 @@ def test_time_varying_reduces_to_time_invariant_solve_bitwise():
     s.close()
     for k in o1:
         assert torch.equal(o1[k], o2[k]), k
+
+
+@pytest.mark.parametrize("n,expect", [(9, "riccati_warp"), (40, "riccati_cta")])
+def test_failed_instances_are_isolated(n, expect):
+    """R indefinite on one instance, NaN in Q of another: status and NaN there, the others untouched."""
+    H, batch = 5, (1, 1, 6)
+    w = tv_workload(n, n, H, batch, seed=21 + n)
+    w["R"] = w["R"].expand((1, 1, 6) + w["R"].shape[3:]).clone()
+    w["R"][0, 0, 2] = -10.0 * w["R"][0, 0, 2]
+    w["Q"] = w["Q"].clone()
+    w["Q"][0, 0, 4, 1, 0, 0] = float("nan")
+    good = np.array([0, 1, 3, 5])
+    s = lqr.LqrSolver(n, n, H, batch)
+    out = lqr.alloc_outputs(n, n, H, 6, DEV)
+    s.solve_tv(w["A"], w["B"], w["Q"], w["R"], w["Qf"], w["x0"], H, tv=w["tv"], **out)
+    torch.cuda.synchronize()
+    assert lqr.KERNEL_NAMES[s.query(lqr.TTC_QUERY_LAST_KERNEL)] == expect
+    s.close()
+    info = out["info"].cpu().numpy()
+    assert info[2] == (H - 1) * n + 1 and info[4] > 0 and not info[good].any(), info
+    for k in ("K", "P", "x", "u"):
+        assert torch.isnan(out[k][2]).all() and torch.isnan(out[k][4]).all(), k
+    ref = pu.run_oracle_tv(dict(w, first_only=False), idx=good)
+    pu.compare({k: out[k] for k in ("K", "P", "x", "u")}, ref, good, 1e-4)
+
+
+@pytest.mark.parametrize("n,expect", [(16, "riccati_warp"), (40, "riccati_cta")])
+def test_time_varying_strides_that_break_16_byte_rows(n, expect):
+    """Q_t and A_t further apart than their size by an odd number of elements: loaded element by element."""
+    H, batch = 4, (1, 2, 5)
+    w = tv_workload(n, n, H, batch, seed=3 + n)
+    for k, pad in (("Q", 1), ("A", 3)):
+        flat = torch.zeros(w[k].shape[:-2] + (n * n + pad,), device=DEV)
+        flat[..., :n * n] = w[k].reshape(w[k].shape[:-2] + (n * n,))
+        w[k] = flat[..., :n * n].unflatten(-1, (n, n))
+        assert w[k].stride(-3) == n * n + pad
+    out, ref = run_both(w)
+    assert lqr.KERNEL_NAMES[out["kernel"]] == expect
+    pu.compare(out, ref, np.arange(10), 1e-4)
 
 
 def test_scan_method_rejects_time_varying_requests():
