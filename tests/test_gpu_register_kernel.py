@@ -11,7 +11,8 @@ from tests.test_gpu_parity import small_workload
 
 pytestmark = pytest.mark.gpu
 SIZES = [(1, 1), (2, 7), (7, 8), (8, 7), (8, 9), (9, 8), (15, 1), (16, 8), (15, 16), (16, 15), (17, 5), (24, 24), (25, 8),
-         (31, 32), (32, 16), (20, 30), (33, 7), (40, 16), (39, 24), (33, 40), (41, 9), (48, 32), (47, 48), (49, 3), (57, 24), (64, 16), (55, 64), (64, 63)]
+         (31, 32), (32, 16), (20, 30), (33, 7), (40, 16), (39, 24), (33, 40), (41, 9), (48, 32), (47, 48), (49, 3), (57, 24), (64, 16), (55, 64), (64, 63),
+         (17, 9), (24, 16), (25, 17), (32, 24), (33, 25), (40, 32), (49, 33), (64, 48)]
 
 
 @pytest.mark.parametrize("n,m", SIZES)
