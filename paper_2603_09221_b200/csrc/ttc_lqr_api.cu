@@ -189,14 +189,15 @@ int clear_device_error(ttc_lqr_handle* h, cudaStream_t st)
 // of the GPU idle while it walks H dependent steps (4.4 us per step at n = 16, 12 us at n = 32), whereas the scan's
 // 2 log2(H) + 3 launches spread all N x H applications and gains over the machine (12 ns resp. 59 ns per instance
 // and step): the scan wins below about 300 (n = 16) and 180 (n = 32) instances.
-int pick_method(const ttc_lqr_handle* h, int H, bool time_varying, long long nwin)
+// The size that counts is the whole batch's: the slices of ttc_lqr_solve_host have to give the bits of one call.
+int pick_method(const ttc_lqr_handle* h, int H, bool time_varying)
 {
     if (h->cfg.method == TTC_SCAN)
         return TTC_SCAN;
     const int n = h->cfg.n;
     if (h->cfg.method == TTC_AUTO && !time_varying && n == h->cfg.m && (n == 16 || n == 32) && H >= 256) {
         const long long in_flight = (long long)h->sm_count * (n == 32 ? 12 : 32);   // instances the recursion keeps resident
-        if (nwin * (n == 32 ? 10 : 16) <= in_flight)
+        if (h->N * (n == 32 ? 10 : 16) <= in_flight)
             return TTC_SCAN;
     }
     return TTC_RICCATI;
@@ -373,7 +374,7 @@ int solve_window(ttc_lqr_handle* h, const ttc_operand* A, const ttc_operand* B, 
     p.out_bf16 = (flags & TTC_OUT_BF16) ? 1 : 0;
     const bool obf = p.out_bf16 != 0;
 
-    const int method = pick_method(h, H, time_varying, nwin);
+    const int method = pick_method(h, H, time_varying);
     if (method == TTC_SCAN && time_varying)
         return fail(TTC_STATUS_UNSUPPORTED, "the scan method handles time-invariant problems without a linear cost only");
     // The rollout reads every K_t in forward order after the backward pass produced them in

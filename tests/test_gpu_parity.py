@@ -348,6 +348,22 @@ def test_host_buffer_entry_point_slices_with_a_single_sequence_and_head():
         assert torch.equal(out[k], gpu[k].cpu()), k
 
 
+def test_host_buffer_entry_point_picks_the_method_of_the_whole_batch():
+    """TTC_AUTO over a long horizon: the batch is too large for the scan, its slices of 128 instances would not be."""
+    n, H, batch = 16, 256, (1, 1, 2048)
+    w = small_workload(n, n, H, batch, seed=516, rho=0.98)
+    gpu = pu.run_gpu(w, method=lqr.TTC_AUTO, want=("x", "u", "info"))
+    assert lqr.KERNEL_NAMES[gpu["kernel"]] == "riccati_warp"
+    s = lqr.LqrSolver(n, n, H, batch, method=lqr.TTC_AUTO)
+    host = {k: w[k].cpu().pin_memory() for k in ("A", "B", "Q", "R", "x0")}
+    out = lqr.alloc_outputs(n, n, H, 2048, "cpu", pin=True, want=("x", "u", "info"))
+    s.solve_host(host["A"], host["B"], host["Q"], host["R"], host["x0"], H, **out)
+    assert s.query(lqr.TTC_QUERY_LAST_LAUNCHES) > 1, "expected more than one slice"
+    s.close()
+    for k in ("x", "u", "info"):
+        assert torch.equal(out[k], gpu[k].cpu()), k
+
+
 def test_bounded_wait_gives_up_and_reports():
     """The give-up branch of the kernels' barrier wait, run on a barrier nothing ever arrives on (no MMA in flight): it
     must come back by itself with the error word set, and the context must stay usable afterwards."""
