@@ -143,7 +143,8 @@ int ttc_lqr_create(const ttc_lqr_config* cfg, ttc_lqr_handle** out);
  *                   x0 may be NULL when neither x nor u is requested.
  * Outputs (device, F32 -- BF16 with TTC_OUT_BF16 --, written completely, each may be NULL = not wanted):
  *     K    [N][H][m][n]
- *     P    [N][H+1][n][n]    (or [N][n][n] = P_0   with TTC_OUT_FIRST_ONLY)
+ *     P    [N][H+1][n][n]    (or [N][n][n] = P_0   with TTC_OUT_FIRST_ONLY);
+ *                            symmetric up to rounding (TF32 math: about 6e-4 of the largest entry)
  *     x    [N][H+1][n]
  *     u    [N][H][m]         (or [N][m]    = u_0   with TTC_OUT_FIRST_ONLY)
  *     info [N] int32: 0 = solved; t*m + j + 1 > 0 = pivot j (0-based) of R + B'P_{t+1}B at

@@ -355,9 +355,13 @@ __device__ __forceinline__ void store_half_global(float* base, long long idx, co
     for (int c = 0; c < 8; ++c)
         store_out4(base, idx + 4 * c, make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]), bf16);
 }
-// The thread's 32 values of a row of a symmetric matrix go to a column: the 32 lanes of a
-// request then share a line instead of touching 32 of them, which the load/store pipe takes one by one.  P_t by rows:
-// 17.0 instead of 15.9 ms on 65536 instances of 8 steps with every output.  (P_H = Q stays with rows: by columns 16.6 ms.)
+// The thread's 32 values of a row go to a column: the 32 lanes of a request then share a line instead of touching 32 of
+// them, which the load/store pipe takes one by one.  P_t by rows: 17.0 instead of 15.9 ms on 65536 instances of 8 steps with
+// every output.  (P_H = Q stays with rows: by columns 16.6 ms.)
+// What is written is the transpose of the accumulator C, that is the matrix which the next step multiplies: the rows of C
+// become the rows of the operand X0, and W = BA X0'.  C is symmetric only to the rounding of A'(P A) in tf32 (averaged every
+// eighth step): |C - C'| is at most 6e-4 of the largest entry, and by rows P_t differs from this one by that much, with the
+// same error against the oracle (4.0e-4).
 __device__ __forceinline__ void store_half_column(float* base, long long idx, const float (&v)[32], int bf16)
 {
     if (bf16) {
