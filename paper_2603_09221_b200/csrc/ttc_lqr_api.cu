@@ -184,11 +184,16 @@ int clear_device_error(ttc_lqr_handle* h, cudaStream_t st)
     return TTC_OK;
 }
 
-// Method of one call.  TTC_AUTO means the sequential recursion except where the scan is measured to be faster:
-// time-invariant problems with n = m = 16 / 32 over long horizons with few instances.  The recursion then leaves most
-// of the GPU idle while it walks H dependent steps (4.4 us per step at n = 16, 12 us at n = 32), whereas the scan's
-// 2 log2(H) + 3 launches spread all N x H applications and gains over the machine (12 ns resp. 59 ns per instance
-// and step): the scan wins below about 300 (n = 16) and 180 (n = 32) instances.
+// Method of one call.  TTC_AUTO means the sequential recursion except for time-invariant problems with n = m = 16 / 32 over
+// long horizons with few instances: there the recursion leaves most of the GPU idle while it walks H dependent steps (1.2 us
+// each at n = 16, 4.3 us at n = 32), where the scan's chain is about 2 sqrt(H) steps long and its work is 1.1 times the
+// recursion's.  Measured, recursion : scan in us, with every output / with P_0 and u_0 only:
+//   n = 16, H = 256    64 instances  442 : 115 / 314 : 90     296  499 : 204 / 314 : 91       1200  804 : 578 / 560 : 129
+//   n = 16, H = 1024   64 instances  1871 : 242 / 1207 : 141  296  2014 : 592 / 1213 : 144    1200  3167 : 2002 / 2174 : 211
+//   n = 32, H = 256    16 instances  1402 : 287 / 1100 : 236  177  1552 : 693 / 1130 : 249    592  1661 : 1616 / 1136 : 258
+// On its two lines (H = 256; two instances per SM at n = 16, six on five SMs at n = 32) the scan is still 2.2 to 4.5 times as
+// fast, and it is ahead beyond them: from H = 64 on below 128 instances (1.6 to 2.1 times) and, with P_0 and u_0 only, at any
+// number up to the 1200 that were measured.  Below H = 32 the recursion is as fast or faster.
 // The size that counts is the whole batch's: the slices of ttc_lqr_solve_host have to give the bits of one call.
 int pick_method(const ttc_lqr_handle* h, int H, bool time_varying)
 {
@@ -196,8 +201,8 @@ int pick_method(const ttc_lqr_handle* h, int H, bool time_varying)
         return TTC_SCAN;
     const int n = h->cfg.n;
     if (h->cfg.method == TTC_AUTO && !time_varying && n == h->cfg.m && (n == 16 || n == 32) && H >= 256) {
-        const long long in_flight = (long long)h->sm_count * (n == 32 ? 12 : 32);   // instances the recursion keeps resident
-        if (h->N * (n == 32 ? 10 : 16) <= in_flight)
+        const long long most = n == 32 ? 6ll * h->sm_count / 5 : 2ll * h->sm_count;          // 177 and 296 on 148 SMs
+        if (h->N <= most)
             return TTC_SCAN;
     }
     return TTC_RICCATI;
