@@ -45,7 +45,8 @@ class ttc_layer_inputs(ctypes.Structure):
                                                "r_inv", "h0", "B_basis", "Q_basis")] + [("r", ctypes.c_int32)]
 
 
-_LAYER_INPUTS = struct.Struct("11Pi")
+_LAYER_INPUTS = struct.Struct("11Pi")                       # (without the padding at the structure's end)
+assert _LAYER_INPUTS.size == ttc_layer_inputs.r.offset + ttc_layer_inputs.r.size
 
 LAYER_GRAD_KEYS = ("s_a", "s_gamma_a", "s_gamma_b", "s_gamma_q", "s_b", "s_q", "s_qf", "r_inv", "h0", "B_basis", "Q_basis")
 
