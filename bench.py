@@ -296,7 +296,9 @@ def run_grad(args):
     kernel_ms = statistics.median(per_step)
     ach = N * (bin_i + bout_i) / (kernel_ms * 1e-3) / 1e9
     roofline = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": ach / peaks["hbm_gbs"],
-                "traffic": None, "kernel": "whole step: backward pass + grad_vectors + grad_outer (3 launches)",
+                "traffic": None,
+                "kernel": ("riccati_frag_kernel<GRAD> (whole step)" if launches == args.steps
+                           else "whole step: backward pass + grad_vectors + grad_outer"),
                 "kernel_ms": kernel_ms, "peak_note": "copy bandwidth, of %s" % peaks["source"],
                 "algorithmic_bytes_per_launch": N * (bin_i + bout_i)}
     cpu = None

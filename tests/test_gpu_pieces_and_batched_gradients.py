@@ -1,5 +1,5 @@
 """Edges of the scan over the horizon (number, length and remainder of its pieces) and of the gradient kernels that batches
-of more than four instances per SM take (places in the workspace shared by the CTAs in flight)."""
+of more than four instances per SM take (one launch; a last CTA that is not full, more instances than are resident)."""
 import numpy as np
 import pytest
 import torch
@@ -29,7 +29,7 @@ def test_pieces_of_the_horizon(n, H):
     pu.compare(first, pu.run_oracle(w, first_only=True), idx, 1e-4, names=("P", "u"))
 
 
-# one instance more than the threshold (a ragged last CTA), and more instances than places in the workspace
+# one instance more than the threshold (a last CTA that is not full), and more instances than are resident at once
 @pytest.mark.parametrize("n,extra", [(16, 1), (16, 2600), (32, 1), (32, 1203)])
 def test_gradients_of_batches_that_fill_the_machine(n, extra):
     N = 4 * torch.cuda.get_device_properties(0).multi_processor_count + extra
@@ -47,7 +47,7 @@ def test_gradients_of_batches_that_fill_the_machine(n, extra):
 @pytest.mark.parametrize("key,extra,r", [("layer16", 3, 1), ("layer16", 1900, 15), ("layer32", 1, 17), ("layer32", 900, 5)])
 def test_layer_gradients_of_batches_that_fill_the_machine(key, extra, r):
     """Numbers of basis matrices that are no multiple of the sixteen a reduction block takes; twice, for the second call
-    finds the places of the workspace as the first one left them."""
+    finds the workspace as the first one left it."""
     N, T = 4 * torch.cuda.get_device_properties(0).multi_processor_count + extra, 4
     w = workloads.make_layer_workload(key, device=DEV, batch=(1, 1, N), seed=70 + extra)
     full = w["r"]
