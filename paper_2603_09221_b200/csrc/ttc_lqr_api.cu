@@ -192,8 +192,8 @@ int clear_device_error(ttc_lqr_handle* h, cudaStream_t st)
 //   n = 16, H = 1024   64 instances  1871 : 242 / 1207 : 141  296  2014 : 592 / 1213 : 144    1200  3167 : 2002 / 2174 : 211
 //   n = 32, H = 256    16 instances  1402 : 287 / 1100 : 236  177  1552 : 693 / 1130 : 249    592  1661 : 1616 / 1136 : 258
 // On its two lines (H = 256; two instances per SM at n = 16, six on five SMs at n = 32) the scan is still 2.2 to 4.5 times as
-// fast, and it is ahead beyond them: from H = 64 on below 128 instances (1.6 to 2.1 times) and, with P_0 and u_0 only, at any
-// number up to the 1200 that were measured.  Below H = 32 the recursion is as fast or faster.
+// fast, and it is ahead beyond them: from H = 64 on with at most 128 instances (1.4 to 2.1 times) and, with P_0 and u_0
+// only, with any number up to the 1200 that were measured.  At H = 16 the recursion is the faster one (up to 1.7 times).
 // The size that counts is the whole batch's: the slices of ttc_lqr_solve_host have to give the bits of one call.
 int pick_method(const ttc_lqr_handle* h, int H, bool time_varying)
 {
