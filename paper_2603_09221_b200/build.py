@@ -4,13 +4,14 @@ from __future__ import annotations
 import glob
 import os
 import subprocess
+import tempfile
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libttc_lqr.so")
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
-    "-Xcompiler", "-fPIC", "-shared",
+    "-Xcompiler", "-fPIC",
 ]
 
 
@@ -27,9 +28,17 @@ def _stale():
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile every ``csrc/*.cu`` into ``libttc_lqr.so`` (rebuilds when a source is newer)."""
+    """Compile every ``csrc/*.cu`` (side by side) into ``libttc_lqr.so``; rebuilds when a source is newer."""
     if force or _stale():
-        nvcc = os.environ.get("NVCC", "nvcc")
-        cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-o", LIB] + sources()
-        subprocess.run(cmd, check=True)
+        nvcc = [os.environ.get("NVCC", "nvcc")] + NVCC_FLAGS
+        with tempfile.TemporaryDirectory() as tmp:
+            objects, jobs = [], []
+            for src in sources():
+                objects.append(os.path.join(tmp, os.path.basename(src) + ".o"))
+                cmd = nvcc + (["-Xptxas", "-v"] if verbose else []) + ["-c", "-o", objects[-1], src]
+                jobs.append((cmd, subprocess.Popen(cmd)))
+            failed = [subprocess.CalledProcessError(job.returncode, cmd) for cmd, job in jobs if job.wait()]
+            if failed:
+                raise failed[0]
+            subprocess.run(nvcc + ["-shared", "-o", LIB] + objects, check=True)
     return LIB

@@ -1,0 +1,19 @@
+// One-warp recursion with five or six blocks of states (riccati_frag.cuh: time-invariant requests, any strides).
+#include "riccati_frag.cuh"
+
+namespace ttc {
+namespace rfrag {
+
+cudaError_t launch_blocks_5_6(const SolveParams& p, int kb, int mb, int sm_count, cudaStream_t st)
+{
+    if (kb == 5)
+        return mb == 1 ? launch_one<5, 1, false, false, true>(p, sm_count, st)
+             : mb == 2 ? launch_one<5, 2, false, false, true>(p, sm_count, st)
+             : mb == 3 ? launch_one<5, 3, false, false, true>(p, sm_count, st)
+             : mb == 4 ? launch_one<5, 4, false, false, true>(p, sm_count, st) : launch_one<5, 5, false, false, true>(p, sm_count, st);
+    return mb <= 2 ? launch_one<6, 2, false, false, true>(p, sm_count, st)
+         : mb <= 4 ? launch_one<6, 4, false, false, true>(p, sm_count, st) : launch_one<6, 6, false, false, true>(p, sm_count, st);
+}
+
+} // namespace rfrag
+} // namespace ttc

@@ -19,7 +19,7 @@
 // recursion's.  64 instances, n = 16, H = 1024: see the launcher.
 #pragma once
 
-#include "riccati_frag.cuh"
+#include "riccati_dispatch.cuh"
 
 namespace ttc {
 namespace scanf {

@@ -11,9 +11,10 @@
 
 #include "common.cuh"
 #include "device_pool.h"
+#include "lowrank_q.cuh"
 #include "riccati_cta.cuh"
 #include "riccati_umma64.cuh"
-#include "riccati_frag.cuh"
+#include "riccati_dispatch.cuh"
 #include "riccati_warp.cuh"
 #include "ttc_layer.cuh"
 #include "layer_frag.cuh"
