@@ -147,6 +147,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, int li
     }
     return false;
 }
+// true in one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t pred;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(pred));
+    return pred != 0;
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void async_proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -381,9 +388,14 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const int tid = threadIdx.x;
-    const int wg = tid / WG_THREADS;
+    // By way of a shuffle the compiler knows that these are the same in the whole warp, and with elect.sync around the issue
+    // (instead of a test of the thread index) it keeps descriptors and tensor-memory addresses in uniform registers.  From
+    // ordinary ones, the issue of a panel's three MMAs and the commit took 240 cycles of the chain, eight times a step:
+    // 131072 instances, H = 16, P_0 and u_0: 45.0 -> 41.9 ms; 65536, H = 8, every output: 15.9 -> 14.6 ms.
+    const int cwarp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int wg = cwarp >> 2;
     const int wt = tid % WG_THREADS;
-    const int warp = wt >> 5;                  // warp in warpgroup: owns tensor-memory lanes 32 warp .. 32 warp + 31
+    const int warp = cwarp & 3;                // warp in warpgroup: owns tensor-memory lanes 32 warp .. 32 warp + 31
     const int lane = wt & 31;
     unsigned char* BA = smem_raw;              // rows 0..63: B' (row j = column j of B), rows 64..127: A'; shared by the CTA
     float* Rs = reinterpret_cast<float*>(smem_raw + BUF_BYTES);   // R of the head, fp32, shared by the CTA
@@ -417,10 +429,10 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t RW = cta.tmem_base + 128u * wg, RF = RW + 64u;
+    const uint32_t RW = __shfl_sync(0xffffffffu, cta.tmem_base, 0) + 128u * wg, RF = RW + 64u;
     const uint32_t lane_sel = (uint32_t)(32 * warp) << 16;
     uint32_t parity = 0, parity_w = 0;
-    const bool issuer = wt == 96;              // one thread of warp 3 issues every MMA of the warpgroup
+    const bool issue_warp = warp == 3;         // one thread of warp 3 issues every MMA of the warpgroup
 
     const int H = p.H;
     const long long chunks_per_head = (p.tcount + CHUNK - 1) / CHUNK;
@@ -508,7 +520,7 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
 
             for (int ts = H - 1; ts >= 0 && !dead; --ts) {
                 // (1) W = BA P' -> R_W ; (2) F = W B -> R_F
-                if (issuer) {
+                if (issue_warp && elect_one()) {
                     tc_fence_after();
                     gemm_ss(RW, smem_u32(BA), smem_u32(X0), 64, 0, false);
                     // F reads W from tensor memory: an MMA whose A operand was written by the MMAs just before it is NOT
@@ -618,11 +630,15 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                     }
                     tc_fence_before();
                     wg_barrier(wg);
-                    if (!GAINS && pnl == 7 && issuer) {
+                    if (!GAINS && pnl == 7 && issue_warp && elect_one()) {
                         // every row has read its last columns of F: (4) DP = W A into the columns of F
                         // (with gains the columns of F still collect K_t': (4) follows their read-out)
                         tc_fence_after();
                         gemm_ts(RF, RW, smem_u32(BA) + MAT_BYTES, 64);
+                        const uint32_t idn = instr_desc(64, 1);   // and the k-steps of (5) whose columns of Z' are there (41.9 -> 41.1 ms)
+#pragma unroll
+                        for (int j = 0; j < 7; ++j)
+                            mma_ss(RF, smem_desc(smem_u32(X0) - MAT_BYTES + 2 * j * SC), smem_desc(smem_u32(X0) + 2 * j * SC), idn, 1u);
                     }
                     // GAINS: rows 0..63 carry X = L^{-T} behind L.  Row r of L ends in its diagonal block; from there on the
                     // same tensor-memory row (the unused upper triangle of S, which the trailing updates have brought to
@@ -712,7 +728,7 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                         break;
                     async_proxy_fence();
                     wg_barrier(wg);
-                    if (issuer) {                              // G -= panel * panel[0:64]'  (hi*hi + lo*hi + hi*lo)
+                    if (issue_warp && elect_one()) {                              // G -= panel * panel[0:64]'  (hi*hi + lo*hi + hi*lo)
                         tc_fence_after();
                         // all 64 columns, though without gains only those to the right are read again: leaving the
                         // others out (and the rows of L that are complete) measured 0.3 to 3 % slower
@@ -749,11 +765,14 @@ __global__ void __launch_bounds__(THREADS, 1) riccati_umma64_kernel(SolveParams 
                 wg_barrier(wg);
                 dead = dead || misc.dead != 0;
                 // (5) DP -= Z' Z : A operand rows 64..127 = Z' (rows 0..63 = X1, unused lanes)
-                if (issuer && !dead) {
+                if (issue_warp && !dead && elect_one()) {
                     tc_fence_after();
-                    if (GAINS)                                 // (4), once K_t' has been read out of the columns of F
+                    if (GAINS) {                               // (4), once K_t' has been read out of the columns of F
                         gemm_ts(RF, RW, smem_u32(BA) + MAT_BYTES, 64);
-                    gemm_ss(RF, smem_u32(X0) - MAT_BYTES, smem_u32(X0), 64, 1, true);
+                        gemm_ss(RF, smem_u32(X0) - MAT_BYTES, smem_u32(X0), 64, 1, true);
+                    } else {                                   // the last k-step
+                        mma_ss(RF, smem_desc(smem_u32(X0) - MAT_BYTES + 14 * SC), smem_desc(smem_u32(X0) + 14 * SC), instr_desc(64, 1), 1u);
+                    }
                     mma_commit(mbar);
                 }
                 if (dead)
