@@ -251,10 +251,11 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB == 2 ? 5 : 2) layer_frag_ke
     constexpr int N = 8 * NB, MT = Mat<NB, NB>::MT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const long long inst = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int warp = warp_index();
+    const long long inst = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
     if (inst >= p.N)
         return;
-    Slot<NB>& sl = reinterpret_cast<Slot<NB>*>(smem_raw)[threadIdx.x >> 5];
+    Slot<NB>& sl = reinterpret_cast<Slot<NB>*>(smem_raw)[warp];
     Mat<NB, NB> nP;
     prepare<NB>(sl, nP, p, inst, lane);
     Rates<NB> rates;

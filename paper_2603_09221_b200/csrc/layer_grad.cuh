@@ -79,10 +79,11 @@ __global__ void __launch_bounds__(32 * lfrag::MAX_WARPS, NB == 2 ? 4 : 2) layer_
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const layer::LayerParams& p = q.lp;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, T = p.T, r = p.r;
-    const long long inst = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int warp = warp_index();
+    const long long inst = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
     if (inst >= p.N)
         return;
-    unsigned char* const mem = smem_raw + (threadIdx.x >> 5) * warp_bytes<NB>();
+    unsigned char* const mem = smem_raw + warp * warp_bytes<NB>();
     float* const Kg = p.Kws + inst * (long long)T * N * N;
     float k0[NB][2];                                        // first control of the dual problem, column form
     int fail;

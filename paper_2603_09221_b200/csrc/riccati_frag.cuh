@@ -489,7 +489,8 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const long long widx = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int warp = warp_index();
+    const long long widx = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
     if (widx >= p.b0 * p.b1 * p.tcount * (CH ? p.chunks : 1))
         return;
     const int chunk = CH ? (int)(widx % p.chunks) : 0;
@@ -507,7 +508,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     using Ops = Operands<NB, MB>;
     constexpr bool TWO = TV && NB <= 2;
     using Mem = WarpMem<NB, MB, TWO>;
-    Mem& mem = *reinterpret_cast<Mem*>(smem_raw + (threadIdx.x >> 5) * warp_bytes<NB, MB, TV, GRAD>());
+    Mem& mem = *reinterpret_cast<Mem*>(smem_raw + warp * warp_bytes<NB, MB, TV, GRAD>());
     const long long oA = pl.off(p.A), oB = pl.off(p.B), oR = pl.off(p.R), oQ = pl.off(p.Q);
     Mat<NB, NB> nP;
     if constexpr (PAD) {                                    // what does not exist: R is the identity, the rest zero
