@@ -14,6 +14,7 @@
 // both about 2^-23 of the product.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 namespace ttc {
@@ -511,6 +512,129 @@ __device__ __forceinline__ void product_symmetric(Mat<NB, NB>& d, const Split<NB
             for (int e = 0; e < 4; ++e)
                 d.v[mt][cb][e] += e1[e] + e2[e];
         }
+}
+
+// ---- the same products on pairs of halves: an operand is split into two float16 numbers, each rounded to nearest, and one
+// instruction takes sixteen contraction indices at the price of eight in tf32 (8 cycles of a scheduler's pipe): half the
+// instructions, half the operand registers.  A float16 keeps the eleven bits of a tf32 number, so that the pair represents x
+// to 2^-22 |x| (tf32: 2^-21, the remainder is truncated) as long as its second half is no subnormal; below, to 2^-25.  What
+// that needs of the operands is in riccati_frag.cuh.  The tiles of two neighbouring column blocks are the instruction's A
+// operand as they stand, and the B operand of the transpose, as above.
+template <int RB, int CB>
+struct Halves {
+    static constexpr int MT = (RB + 1) / 2;
+    uint32_t h[MT][CB][2], l[MT][CB][2];                   // [..][0]: row g, columns 2 t and 2 t + 1; [..][1]: row g + 8
+};
+__device__ __forceinline__ void split_halves(float x0, float x1, uint32_t& h, uint32_t& l)
+{
+    const __half2 hh = __floats2half2_rn(x0, x1);
+    const float2 f = __half22float2(hh);
+    const __half2 ll = __floats2half2_rn(x0 - f.x, x1 - f.y);          // (the differences are exact)
+    h = *reinterpret_cast<const uint32_t*>(&hh);
+    l = *reinterpret_cast<const uint32_t*>(&ll);
+}
+template <int RB, int CB>
+__device__ __forceinline__ void split(Halves<RB, CB>& s, const Mat<RB, CB>& m)
+{
+#pragma unroll
+    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (e && 2 * mt + 1 >= RB)                  // rows that do not exist
+                    s.h[mt][cb][e] = s.l[mt][cb][e] = 0u;
+                else
+                    split_halves(m.v[mt][cb][2 * e], m.v[mt][cb][2 * e + 1], s.h[mt][cb][e], s.l[mt][cb][e]);
+            }
+}
+// d = c + X Y' over sixteen contraction indices, or over eight
+__device__ __forceinline__ void mma_halves(float (&d)[4], const float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                           uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
+}
+__device__ __forceinline__ void mma_halves(float (&d)[4], const float (&c)[4], uint32_t a0, uint32_t a1, uint32_t b0)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%7,%8,%9,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(b0), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
+}
+// split parts in shared memory, two column blocks to a 16-byte word (in the order of the instruction's A registers)
+template <int RB, int CB>
+struct StoredHalves {
+    static constexpr int MT = (RB + 1) / 2, CP = (CB + 1) / 2;
+    uint4 q[MT][CP][2][32];
+};
+template <int RB, int CB>
+__device__ __forceinline__ void keep(StoredHalves<RB, CB>& st, const Halves<RB, CB>& s, int lane)
+{
+#pragma unroll
+    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < CB; cb += 2) {
+            const int c1 = cb + 1 < CB ? cb + 1 : cb;       // (an odd last block: the second half of the word is not read)
+            st.q[mt][cb / 2][0][lane] = make_uint4(s.h[mt][cb][0], s.h[mt][cb][1], s.h[mt][c1][0], s.h[mt][c1][1]);
+            st.q[mt][cb / 2][1][lane] = make_uint4(s.l[mt][cb][0], s.l[mt][cb][1], s.l[mt][c1][0], s.l[mt][c1][1]);
+        }
+}
+// operand words of X for the column blocks kb, kb + 1: from registers, from shared memory
+template <int RB, int KB>
+__device__ __forceinline__ uint4 operand_word(const Halves<RB, KB>& x, int mt, int kb, int part, int)
+{
+    const int k1 = kb + 1 < KB ? kb + 1 : kb;
+    return part ? make_uint4(x.l[mt][kb][0], x.l[mt][kb][1], x.l[mt][k1][0], x.l[mt][k1][1])
+                : make_uint4(x.h[mt][kb][0], x.h[mt][kb][1], x.h[mt][k1][0], x.h[mt][k1][1]);
+}
+template <int RB, int KB>
+__device__ __forceinline__ uint4 operand_word(const StoredHalves<RB, KB>& x, int mt, int kb, int part, int lane)
+{
+    return x.q[mt][kb / 2][part][lane];
+}
+// d = c + X * Y', with the conventions of the products above
+template <int RB, int KB, int CB, bool LOWER = false, class X>
+__device__ __forceinline__ void product_halves(Mat<RB, CB>& d, const Mat<RB, CB>* c, const X& x, const Halves<CB, KB>& y, int lane)
+{
+    const float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int kb = 0; kb < KB; kb += 2) {
+        uint4 a[Mat<RB, CB>::MT][2];
+#pragma unroll
+        for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
+            a[mt][0] = operand_word(x, mt, kb, 0, lane);
+            a[mt][1] = operand_word(x, mt, kb, 1, lane);
+        }
+#pragma unroll
+        for (int pass = 0; pass < 3; ++pass)                // lo*hi, hi*lo, hi*hi
+#pragma unroll
+            for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+                for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
+                    if (LOWER && cb > 2 * mt + 1)
+                        continue;
+                    const uint4 v = a[mt][pass == 0];
+                    const uint32_t b0 = pass == 1 ? y.l[cb / 2][kb][cb & 1] : y.h[cb / 2][kb][cb & 1];
+                    float(&dd)[4] = d.v[mt][cb];
+                    if (kb + 1 < KB) {
+                        const uint32_t b1 = pass == 1 ? y.l[cb / 2][kb + 1][cb & 1] : y.h[cb / 2][kb + 1][cb & 1];
+                        if (kb || pass)
+                            mma_halves(dd, dd, v.x, v.y, v.z, v.w, b0, b1);
+                        else if (c)
+                            mma_halves(dd, c->v[mt][cb], v.x, v.y, v.z, v.w, b0, b1);
+                        else
+                            mma_halves(dd, z, v.x, v.y, v.z, v.w, b0, b1);
+                    } else {
+                        if (kb || pass)
+                            mma_halves(dd, dd, v.x, v.y, b0);
+                        else if (c)
+                            mma_halves(dd, c->v[mt][cb], v.x, v.y, b0);
+                        else
+                            mma_halves(dd, z, v.x, v.y, b0);
+                    }
+                }
+    }
 }
 
 // z = L^{-1} v and k = -L^{-T} z for a vector in row form, from the results of factor(): z in column form, k in column form

@@ -6,10 +6,12 @@
 // The recursion is carried in negated variables (nP = -P etc.): every update is then a plain accumulation.
 //   V = B' nP,  T = A' nP,  nS = -R + B' V',  nY' = A' V',  nP_t = -Q + A' T' + Z' Z     (Prop. 3.1; Alg. 1)
 // with S = L L', Z = L^{-1} Y and, when gains are wanted, K' = -Z' L^{-1} from the inverses of L's diagonal blocks.
+// The five products with A, B, P and Z'Z run on pairs of halves while the values permit it (below), otherwise and in the
+// factorisation in three passes of tf32.
 //
-// What bounds it: at n = 16 a step is 87 tensor-core instructions (8 cycles on a scheduler's pipe, about 4 of its issue
-// slots) in about 830, and four or five warps per scheduler hide most of the chain of five products and sixteen pivots.
-// At n = 32 it is 670 tensor-core instructions, two warps per scheduler (all 255 registers); above, registers spill to
+// What bounds it: at n = 16 a step is 60 tensor-core instructions (8 cycles on a scheduler's pipe, about 4 of its issue
+// slots; 96 in tf32) in about 780, and four or five warps per scheduler hide most of the chain of five products and sixteen
+// pivots.  At n = 32 it is 405 tensor-core instructions (657), two warps per scheduler (all 255 registers); above, registers spill to
 // local memory (0.3 KB per lane at 40 x 16, 2.7 KB at 40 x 40, which the first-level cache absorbs; 10.7 KB at 64 x 64,
 // which it does not: only twice as fast as one CTA per instance there).
 // The forms this replaced: rows broadcast from shared memory at n = 16 (load/store pipe at 88 %), products through shared
@@ -17,6 +19,9 @@
 //   65536 instances n = 16, H = 32, operands from memory  4.26 -> 2.65 ms     4096, n = 16, H = 16, all outputs 188 -> 107 us
 //   16384 instances n = 32, H = 64, all outputs           14.2 -> 8.5 ms      1155, n = 40, m = 12, H = 20     2428 -> 232 us
 //   64 instances n = 8, H = 8, own dynamics               107 -> 11 us     1155, n = m = 60, H = 20            21.9 -> 10.3 ms
+// and from three passes of tf32 throughout to pairs of halves, in the order of the first four: 2.50 -> 2.21 ms, 106 -> 92 us,
+// 8.39 -> 6.45 ms, 232 -> 184 us; error of P_t against float64 0.45e-6 -> 0.27e-6 at n = 16, 0.89e-6 -> 0.44e-6 at n = 32, K, x and u
+// 5 to 15 % smaller.  Problems outside the range (a control in other units): 107 -> 107, 8.4 -> 8.3 ms, at 40 x 12 236 -> 253 us.
 #pragma once
 
 #include "common.cuh"
@@ -72,6 +77,9 @@ struct WarpMem<NB, MB, false> {
     float Q[8 * NB * Ops::LQ], R[8 * MB * Ops::LR];
     __device__ __forceinline__ float* rawA() { return reinterpret_cast<float*>(&A); }
     __device__ __forceinline__ float* rawB() { return reinterpret_cast<float*>(&B); }
+    __device__ __forceinline__ StoredHalves<NB, NB>& halvesA() { return reinterpret_cast<StoredHalves<NB, NB>&>(A); }
+    __device__ __forceinline__ StoredHalves<MB, NB>& halvesB() { return reinterpret_cast<StoredHalves<MB, NB>&>(B); }
+    static_assert(sizeof(StoredHalves<NB, NB>) <= sizeof(Stored<NB, NB>) && sizeof(StoredHalves<MB, NB>) <= sizeof(Stored<MB, NB>), "halves");
     static_assert(sizeof(Stored<NB, NB>) >= sizeof(Ops::A) && sizeof(Stored<MB, NB>) >= sizeof(Ops::B), "raw operand does not fit");
 };
 
@@ -133,9 +141,9 @@ __device__ __forceinline__ void load_transposed(Mat<RB, CB>& x, const float* M, 
                     x.v[mt][cb][e] = PAD && !(i < ni && k < nk) ? 0.f : M[k * LD + i];
             }
 }
-// x = -M of a square matrix in shared memory
+// x = -c M of a square matrix in shared memory
 template <int RB, int LD>
-__device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const float* M, int lane)
+__device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const float* M, float c, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -147,8 +155,8 @@ __device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const float* M, int
                 float2 f = make_float2(0.f, 0.f);
                 if (h == 0 || 2 * mt + 1 < RB)
                     f = *reinterpret_cast<const float2*>(M + (16 * mt + 8 * h + g) * LD + 8 * cb + 2 * t);
-                x.v[mt][cb][2 * h] = -f.x;
-                x.v[mt][cb][2 * h + 1] = -f.y;
+                x.v[mt][cb][2 * h] = -c * f.x;
+                x.v[mt][cb][2 * h + 1] = -c * f.y;
             }
 }
 
@@ -161,7 +169,7 @@ __device__ __forceinline__ void store_pair(float* base, long long idx, float a, 
         *reinterpret_cast<float2*>(base + idx) = make_float2(a, b);
 }
 template <int RB, bool PAD>
-__device__ __forceinline__ void store_negated(float* base, long long off, const Mat<RB, RB>& x, int d, int bf16, int lane)
+__device__ __forceinline__ void store_negated(float* base, long long off, const Mat<RB, RB>& x, float c, int d, int bf16, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -173,7 +181,7 @@ __device__ __forceinline__ void store_negated(float* base, long long off, const 
                 if (h == 1 && 2 * mt + 1 >= RB)
                     continue;
                 const int i = 16 * mt + 8 * h + g, k = 8 * cb + 2 * t;
-                const float a = -x.v[mt][cb][2 * h], b = -x.v[mt][cb][2 * h + 1];
+                const float a = -c * x.v[mt][cb][2 * h], b = -c * x.v[mt][cb][2 * h + 1];
                 if (!PAD) {
                     store_pair(base, off + i * (8 * RB) + k, a, b, bf16);
                 } else if (i < d) {
@@ -201,6 +209,107 @@ __device__ __forceinline__ void store_gain(float* base, long long off, const Mat
                 if (!PAD || (i < n && j < m))
                     store_out(base, off + j * (PAD ? n : 8 * NB) + i, kt.v[mt][cb][e], bf16);
             }
+}
+
+// ---- when the five products with A, B and P and Z'Z run on pairs of halves (frag.cuh)
+// The pair's absolute error of 2^-25 takes the place of the relative one for small elements, and 65504 is the largest number.
+// A step runs on halves when
+//     every row of A' and of B' has its largest element in [2^-4, 8],
+//     every P_ii is at least 2^-4 and no |P_ij| is above 128, or P = 0
+// (rows of the padding aside), tested on the values in every step, for operands that do not change once; otherwise, and from
+// then on, the instance runs in tf32.  In this range the error of an operand is at most 2^-21 of the largest element of its row,
+// which is the bound of the tf32 split; V and T stay below 32 * 8 * 128 = 2^15 and |Z| below 2^13.
+// The rows are tested one by one because a control or a state in other units would otherwise lose its digits: with R_jj and
+// column j of B small together, row j of K is as large as 1 / |B_j|.
+template <bool V>
+struct OnHalves {
+    static constexpr bool value = V;
+};
+constexpr float HALF_LOW = 0.0625f, HALF_HIGH = 8.f, HALF_P_HIGH = 128.f;
+__device__ __forceinline__ __half2 as_half2(uint32_t x) { return *reinterpret_cast<const __half2*>(&x); }
+__device__ __forceinline__ __half2 max_xor(__half2 v, __half2 other, int lanes)
+{
+    return __hmax2(v, as_half2(__shfl_xor_sync(FULL, *reinterpret_cast<const uint32_t*>(&other), lanes)));
+}
+// largest elements of this lane's part of rows 16 mt + g (first half) and 16 mt + 8 + g (second)
+template <int RB, int CB>
+__device__ __forceinline__ __half2 row_top(const Halves<RB, CB>& x, int mt)
+{
+    __half2 m0 = __habs2(as_half2(x.h[mt][0][0])), m1 = __habs2(as_half2(x.h[mt][0][1]));
+#pragma unroll
+    for (int cb = 1; cb < CB; ++cb) {
+        m0 = __hmax2(m0, __habs2(as_half2(x.h[mt][cb][0])));
+        m1 = __hmax2(m1, __habs2(as_half2(x.h[mt][cb][1])));
+    }
+    return __hmax2(__lows2half2(m0, m1), __highs2half2(m0, m1));
+}
+// lower limits of those two rows: none for rows that do not exist (i >= d)
+template <bool PAD>
+__device__ __forceinline__ __half2 row_limit(int mt, int d, int g)
+{
+    return PAD ? __floats2half2_rn(16 * mt + g < d ? HALF_LOW : 0.f, 16 * mt + 8 + g < d ? HALF_LOW : 0.f) : __float2half2_rn(HALF_LOW);
+}
+template <int RB, int CB, bool PAD>
+__device__ __forceinline__ bool rows_fit(const Halves<RB, CB>& x, int d, int lane)
+{
+    bool ok = true;
+#pragma unroll
+    for (int mt = 0; mt < Halves<RB, CB>::MT; ++mt) {
+        __half2 v = row_top(x, mt);
+        v = max_xor(v, v, 1);
+        v = max_xor(v, v, 2);
+        ok = ok && __hbge2(v, row_limit<PAD || (RB % 2 != 0)>(mt, d, lane >> 2)) && __hble2(v, __float2half2_rn(HALF_HIGH));
+    }
+    return ok;
+}
+// the same for two operands of at most sixteen rows: of each pair of lanes the first one looks at A', the second one at B'
+template <int NB, int MB, bool PAD>
+__device__ __forceinline__ bool rows_fit(const Halves<NB, NB>& a, const Halves<MB, NB>& b, int n, int m, int lane)
+{
+    static_assert(NB <= 2 && MB <= 2, "one tile of rows each");
+    const bool second = lane & 1;
+    const __half2 ta = row_top(a, 0), tb = row_top(b, 0);
+    __half2 v = max_xor(second ? tb : ta, second ? ta : tb, 1);
+    v = max_xor(v, v, 2);
+    return __hbge2(v, row_limit<PAD || NB == 1 || MB == 1>(0, second ? m : n, lane >> 2)) && __hble2(v, __float2half2_rn(HALF_HIGH));
+}
+// the conditions on P, and `rows` of every lane (called by the whole warp); P = 0 (no terminal weight) fits as well
+template <int NB, bool PAD>
+__device__ __forceinline__ bool value_fits(const Halves<NB, NB>& x, bool rows, int n, int lane)
+{
+    const int g = lane >> 2, t = lane & 3;
+    __half2 top = __habs2(as_half2(x.h[0][0][0]));
+    bool ok = rows;
+#pragma unroll
+    for (int mt = 0; mt < Halves<NB, NB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < NB; ++cb)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (e && 2 * mt + 1 >= NB)
+                    continue;
+                const __half2 v = __habs2(as_half2(x.h[mt][cb][e]));
+                top = __hmax2(top, v);
+                if (cb == 2 * mt + e) {                     // diagonal block: the lane's element on the diagonal, if there is one
+                    const float low = !PAD || 8 * cb + g < n ? HALF_LOW : 0.f;
+                    ok = ok && __hbge2(v, __floats2half2_rn(g == 2 * t ? low : 0.f, g == 2 * t + 1 ? low : 0.f));
+                }
+            }
+    return __all_sync(FULL, ok && __hble2(top, __float2half2_rn(HALF_P_HIGH))) ||
+           __all_sync(FULL, rows && __hbeq2(top, __float2half2_rn(0.f)));
+}
+// power of four that brings the largest P_ii into [1, 4); 1 where there is none within 2^-60 .. 2^60
+template <int NB>
+__device__ __forceinline__ float value_scale(const Mat<NB, NB>& nP, int lane)
+{
+    const int g = lane >> 2, t = lane & 3;
+    float top = 0.f;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+        top = fmaxf(top, -((g & 1) ? nP.v[b / 2][b][2 * (b & 1) + 1] : nP.v[b / 2][b][2 * (b & 1)]));
+    const unsigned bits = __reduce_max_sync(FULL, t == (g >> 1) ? __float_as_uint(top) : 0u);
+    const int e = ((int)(bits >> 23) - 127) & ~1;
+    return e >= -60 && e <= 60 ? __int_as_float((127 - e) << 23) : 1.f;
 }
 
 // W consecutive elements of a row (16-byte loads), or with PAD element by element within [0, n)
@@ -528,7 +637,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
             if (p.Qf.ptr) {                                 // P_H = Q_f, by way of the second buffer
                 stage<NB, NB, Ops::LQ, PAD>(mem.op[1].Q, p.Qf, pl.off(p.Qf), n, n, lane);
                 copies_landed();
-                load_negated<NB, Ops::LQ>(nP, mem.op[1].Q, lane);
+                load_negated<NB, Ops::LQ>(nP, mem.op[1].Q, 1.f, lane);
                 __syncwarp();
             }
 #pragma unroll
@@ -540,7 +649,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
             }
             copies_landed();
             if (!p.Qf.ptr)
-                load_negated<NB, Ops::LQ>(nP, mem.op[0].Q, lane);
+                load_negated<NB, Ops::LQ>(nP, mem.op[0].Q, 1.f, lane);
         } else {
             OperandDev end = TV && p.Qf.ptr ? p.Qf : p.Q;   // P_H
             long long oend = TV && p.Qf.ptr ? pl.off(p.Qf) : oQ + last * p.Q.st;
@@ -555,7 +664,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
             stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + last * p.B.st, n, m, lane);
             stage<MB, MB, Ops::LR, PAD>(mem.R, p.R, oR + last * p.R.st, m, m, lane);
             copies_landed();
-            load_negated<NB, Ops::LQ>(nP, mem.Q, lane);
+            load_negated<NB, Ops::LQ>(nP, mem.Q, 1.f, lane);
             if ((TV && p.Qf.ptr) || inner) {
                 __syncwarp();
                 stage<NB, NB, Ops::LQ, PAD>(mem.Q, p.Q, oQ + last * p.Q.st, n, n, lane);
@@ -563,7 +672,24 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
         }
     }
     if (p.P && !p.first_only && last_piece)
-        store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, n, obf, lane);
+        store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, 1.f, n, obf, lane);
+
+    // (the affine recursion above n = 16 takes the float32 operands back from their tf32 parts, at n <= 8 nothing is gained)
+    constexpr bool HALF = (!AFF || TWO) && NB > 1;
+    // The recursion is homogeneous in (P, Q, R, p, r): it runs on their multiples by a power of four that brings the largest
+    // P_ii at the end of the horizon into [1, 4), which changes no digit and makes the range of the halves one of ratios.
+    float scale = 1.f, unscale = 1.f;
+    if constexpr (HALF) {
+        scale = value_scale<NB>(nP, lane);
+        unscale = 1.f / scale;
+#pragma unroll
+        for (int mt = 0; mt < Mat<NB, NB>::MT; ++mt)
+#pragma unroll
+            for (int cb = 0; cb < NB; ++cb)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    nP.v[mt][cb][e] *= scale;
+    }
 
     auto start_state = [&](int i) {
         if (CH && p.xc)
@@ -587,8 +713,50 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     }
 
     int fail = 0;
-#pragma unroll 1
-    for (int ts = H - 1; ts >= 0; --ts) {
+    // Raw A, B (staged in shared memory) -> split, in place.  On pairs of halves: false, and nothing done, when their rows are
+    // out of range.
+    auto install = [&](auto form, bool newA, bool newB) -> bool {
+        if constexpr (!TWO) {
+            Mat<NB, NB> At;
+            Mat<MB, NB> Bt;
+            if (newA)
+                load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
+            if (newB)
+                load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
+            if constexpr (decltype(form)::value) {
+                Halves<NB, NB> as;
+                Halves<MB, NB> bs;
+                bool ok = true;
+                if (newA) {
+                    split(as, At);
+                    ok = rows_fit<NB, NB, PAD>(as, n, lane);
+                }
+                if (newB) {
+                    split(bs, Bt);
+                    const bool okB = rows_fit<MB, NB, PAD>(bs, m, lane);
+                    ok = ok && okB;
+                }
+                if (!__all_sync(FULL, ok))
+                    return false;
+                __syncwarp();
+                if (newA)
+                    keep(mem.halvesA(), as, lane);
+                if (newB)
+                    keep(mem.halvesB(), bs, lane);
+            } else {
+                __syncwarp();
+                if (newA)
+                    keep(mem.A, At, lane);
+                if (newB)
+                    keep(mem.B, Bt, lane);
+            }
+            __syncwarp();
+        }
+        return true;
+    };
+    // One step.  On pairs of halves: false, and nothing done, when the operands are out of their range.
+    auto step = [&](auto form, const int ts) -> bool {
+        constexpr bool ON_HALVES = decltype(form)::value;
         Mat<NB, NB> At, T;
         Mat<MB, NB> Bt, V;
         Mat<NB, MB> Zt;
@@ -604,54 +772,86 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
                 if (p.R.st) stage<MB, MB, Ops::LR, PAD>(nx.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
                 if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(nx.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
             }
-            load_negated<MB, Ops::LR>(nR, op.R, lane);
+            load_negated<MB, Ops::LR>(nR, op.R, scale, lane);
             load_transposed<NB, NB, Ops::LA, false>(At, op.A, n, n, lane);
             load_transposed<MB, NB, Ops::LB, false>(Bt, op.B, n, m, lane);
-            Split<NB, NB> as, ps;
-            Split<MB, NB> bs, vs;
-            split(ps, nP);
-            split(as, At);
-            split(bs, Bt);
-            product<MB, NB, NB>(V, nullptr, bs, ps);        // V = B' nP
-            product<NB, NB, NB>(T, nullptr, as, ps);        // T = A' nP
-            split(vs, V);
-            product<MB, NB, MB, true>(S, &nR, bs, vs);      // -S = -R + B' V'
-            product<NB, NB, MB>(Zt, nullptr, as, vs);       // -Y' = A' V'
-            split(ps, T);
-            load_negated<NB, Ops::LQ>(nP, op.Q, lane);
-            product<NB, NB, NB, true>(nP, &nP, as, ps);     // -Q - A'P A
+            if constexpr (ON_HALVES) {
+                Halves<NB, NB> as, ps;
+                Halves<MB, NB> bs, vs;
+                split(ps, nP);
+                split(as, At);
+                split(bs, Bt);
+                const bool rows = rows_fit<NB, MB, PAD>(as, bs, n, m, lane);      // (shuffles: by every lane, whatever P is)
+                if (!value_fits<NB, PAD>(ps, rows, n, lane))
+                    return false;
+                product_halves<MB, NB, NB>(V, nullptr, bs, ps, lane);          // V = B' nP
+                product_halves<NB, NB, NB>(T, nullptr, as, ps, lane);          // T = A' nP
+                split(vs, V);
+                product_halves<MB, NB, MB, true>(S, &nR, bs, vs, lane);        // -S = -R + B' V'
+                product_halves<NB, NB, MB>(Zt, nullptr, as, vs, lane);         // -Y' = A' V'
+                split(ps, T);
+                load_negated<NB, Ops::LQ>(nP, op.Q, scale, lane);
+                product_halves<NB, NB, NB, true>(nP, &nP, as, ps, lane);       // -Q - A'P A
+            } else {
+                Split<NB, NB> as, ps;
+                Split<MB, NB> bs, vs;
+                split(ps, nP);
+                split(as, At);
+                split(bs, Bt);
+                product<MB, NB, NB>(V, nullptr, bs, ps);
+                product<NB, NB, NB>(T, nullptr, as, ps);
+                split(vs, V);
+                product<MB, NB, MB, true>(S, &nR, bs, vs);
+                product<NB, NB, MB>(Zt, nullptr, as, vs);
+                split(ps, T);
+                load_negated<NB, Ops::LQ>(nP, op.Q, scale, lane);
+                product<NB, NB, NB, true>(nP, &nP, as, ps);
+            }
         } else {
             if (TV || ts == H - 1)                          // (what CH stages for P_H is followed by Q)
                 copies_landed();
-            if (ts == H - 1 || (TV && p.A.st)) {            // raw -> split, in place
-                load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
-                __syncwarp();
-                keep(mem.A, At, lane);
-            }
-            if (ts == H - 1 || (TV && p.B.st)) {
-                load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
-                __syncwarp();
-                keep(mem.B, Bt, lane);
-            }
-            __syncwarp();
-            load_negated<MB, Ops::LR>(nR, mem.R, lane);
-            {
+            if (TV && !install(form, p.A.st != 0, p.B.st != 0))
+                return false;
+            if constexpr (ON_HALVES) {
+                Halves<NB, NB> ps;
+                split(ps, nP);
+                if (!value_fits<NB, PAD>(ps, true, n, lane))
+                    return false;
+                product_halves<MB, NB, NB>(V, nullptr, mem.halvesB(), ps, lane);
+                product_halves<NB, NB, NB>(T, nullptr, mem.halvesA(), ps, lane);
+            } else {
                 Split<NB, NB> ps;
                 split(ps, nP);
                 product<MB, NB, NB>(V, nullptr, mem.B, ps, lane);
                 product<NB, NB, NB>(T, nullptr, mem.A, ps, lane);
             }
-            {
-                Split<MB, NB> vs;
-                split(vs, V);
-                product<MB, NB, MB, true>(S, &nR, mem.B, vs, lane);
-                product<NB, NB, MB>(Zt, nullptr, mem.A, vs, lane);
-            }
-            load_negated<NB, Ops::LQ>(nP, mem.Q, lane);
-            {
-                Split<NB, NB> tsp;
-                split(tsp, T);
-                product<NB, NB, NB, true>(nP, &nP, mem.A, tsp, lane);
+            load_negated<MB, Ops::LR>(nR, mem.R, scale, lane);
+            if constexpr (ON_HALVES) {
+                {
+                    Halves<MB, NB> vs;
+                    split(vs, V);
+                    product_halves<MB, NB, MB, true>(S, &nR, mem.halvesB(), vs, lane);
+                    product_halves<NB, NB, MB>(Zt, nullptr, mem.halvesA(), vs, lane);
+                }
+                load_negated<NB, Ops::LQ>(nP, mem.Q, scale, lane);
+                {
+                    Halves<NB, NB> tsp;
+                    split(tsp, T);
+                    product_halves<NB, NB, NB, true>(nP, &nP, mem.halvesA(), tsp, lane);
+                }
+            } else {
+                {
+                    Split<MB, NB> vs;
+                    split(vs, V);
+                    product<MB, NB, MB, true>(S, &nR, mem.B, vs, lane);
+                    product<NB, NB, MB>(Zt, nullptr, mem.A, vs, lane);
+                }
+                load_negated<NB, Ops::LQ>(nP, mem.Q, scale, lane);
+                {
+                    Split<NB, NB> tsp;
+                    split(tsp, T);
+                    product<NB, NB, NB, true>(nP, &nP, mem.A, tsp, lane);
+                }
             }
             if (AFF && ts < p.r_count) {                    // the float32 operands once more, for the vector recursion
                 unkeep(At, mem.A, lane);
@@ -678,7 +878,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
 #pragma unroll
                 for (int k = 0; k < NB; ++k)
                     s = fmaf(Bt.v[b / 2][k][2 * (b & 1)], pc[k][0], fmaf(Bt.v[b / 2][k][2 * (b & 1) + 1], pc[k][1], s));
-                gr[b] = sum_over_t(s) + (8 * b + g < m ? load_elem(p.r, orv + 8 * b + g) : 0.f);
+                gr[b] = sum_over_t(s) + (8 * b + g < m ? scale * load_elem(p.r, orv + 8 * b + g) : 0.f);
             }
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
@@ -694,7 +894,13 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
         const int bad = factor<NB, MB, FEW || (NB > 2)>(S, Zt, zs, w, lane);  // Zt becomes Z', S the blocks of L
         if (bad && !fail)
             fail = ts * m + bad;
-        product<NB, MB, NB, true>(nP, &nP, zs, zs);                              // -P_t = -Q - A'PA + Z'Z
+        if constexpr (ON_HALVES) {                          // -P_t = -Q - A'PA + Z'Z
+            Halves<NB, MB> zh;
+            split(zh, Zt);
+            product_halves<NB, MB, NB, true>(nP, &nP, zh, zh, lane);
+        } else {
+            product<NB, MB, NB, true>(nP, &nP, zs, zs);
+        }
         const bool gain = need_K_all || need_k_all || (want_u0 && ts == 0);
         if (AFF) {
             // z = L^{-1}(B'p + r);  p_t = A'p - Z'z;  k_t = -L^{-T} z   (all zero while p and r are)
@@ -724,7 +930,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
 #pragma unroll
                 for (int b = 0; b < NB; ++b)
                     if (8 * b + g < n)
-                        p.pvec[(inst * (p.first_only ? 1 : H + 1) + (p.first_only ? 0 : ts)) * (long long)n + 8 * b + g] = pr[b];
+                        p.pvec[(inst * (p.first_only ? 1 : H + 1) + (p.first_only ? 0 : ts)) * (long long)n + 8 * b + g] = unscale * pr[b];
         }
         if (gain) {
             gains<NB, MB>(Zt, S, w, lane);                  // Zt = K_t'
@@ -756,8 +962,30 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
         // well the closed loop is damped.
         make_symmetric<NB>(nP, lane);
         if (p.P && first_ok && (!p.first_only || ts == 0))
-            store_negated<NB, PAD>(p.P, Poff + (long long)(p.first_only ? 0 : ts) * n * n, nP, n, obf, lane);
+            store_negated<NB, PAD>(p.P, Poff + (long long)(p.first_only ? 0 : ts) * n * n, nP, unscale, n, obf, lane);
+        return true;
+    };
+    int ts = H - 1;
+    const bool fixedA = !TV || !p.A.st, fixedB = !TV || !p.B.st;           // operands that are installed once
+    if constexpr (HALF) {
+        if (install(OnHalves<true>(), fixedA, fixedB))
+#pragma unroll 1
+            while (ts >= 0 && step(OnHalves<true>(), ts))
+                --ts;
+        if constexpr (!TWO)
+            if (ts >= 0) {                                  // an instance that has left the range: the raw operands once more
+                const long long now = TV ? ts : 0;
+                __syncwarp();
+                stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + now * p.A.st, n, n, lane);
+                stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + now * p.B.st, n, m, lane);
+                copies_landed();
+            }
     }
+    if (ts >= 0)
+        install(OnHalves<false>(), fixedA, fixedB);
+#pragma unroll 1
+    for (; ts >= 0; --ts)
+        step(OnHalves<false>(), ts);
     if (CH) {
         if (lane == 0)
             p.piece_info[widx] = fail;
