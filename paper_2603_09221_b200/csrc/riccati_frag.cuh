@@ -21,7 +21,9 @@
 //   64 instances n = 8, H = 8, own dynamics               107 -> 11 us     1155, n = m = 60, H = 20            21.9 -> 10.3 ms
 // and from three passes of tf32 throughout to pairs of halves, in the order of the first four: 2.50 -> 2.21 ms, 106 -> 92 us,
 // 8.39 -> 6.45 ms, 232 -> 184 us; error of P_t against float64 0.45e-6 -> 0.27e-6 at n = 16, 0.89e-6 -> 0.44e-6 at n = 32, K, x and u
-// 5 to 15 % smaller.  Problems outside the range (a control in other units): 107 -> 107, 8.4 -> 8.3 ms, at 40 x 12 236 -> 253 us.
+// 5 to 15 % smaller.  Time-varying n = 32, 2048 instances of 32 steps 0.55 -> 0.41 ms; gradients
+// of 65536 instances, n = 16, H = 32 5.4 -> 5.2 ms.  Problems outside the range (a control in other units) take 107, 253 us (40 x 12,
+// where tf32 alone took 236), 2.5 and 8.5 ms.
 #pragma once
 
 #include "common.cuh"
@@ -139,6 +141,21 @@ __device__ __forceinline__ void load_transposed(Mat<RB, CB>& x, const float* M, 
                     x.v[mt][cb][e] = 0.f;
                 else
                     x.v[mt][cb][e] = PAD && !(i < ni && k < nk) ? 0.f : M[k * LD + i];
+            }
+}
+// the same from a row-major operand in global memory (element by element), zero outside
+template <int RB, int CB>
+__device__ __forceinline__ void load_transposed_global(Mat<RB, CB>& x, const OperandDev& o, long long off, int ld, int nk, int ni, int lane)
+{
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = 16 * mt + g + ((e & 2) ? 8 : 0), k = 8 * cb + 2 * t + (e & 1);
+                x.v[mt][cb][e] = i < ni && k < nk ? load_elem(o, off + k * ld + i) : 0.f;
             }
 }
 // x = -c M of a square matrix in shared memory
@@ -341,7 +358,7 @@ __device__ __forceinline__ void load_part(float (&v)[W], const float* row, int c
 template <int N>
 struct GradRing {
     static constexpr int FWD = 3 * N * N, BWD = 2 * N * N + 4 * N;         // floats per stage: K, A, B / A, Q, four vectors
-    static constexpr int FS = N == 16 ? 4 : 2, BS = N == 16 ? 5 : 2;       // stages
+    static constexpr int FS = N == 16 ? 3 : 2, BS = N == 16 ? 4 : 2;       // stages (no more than the backward pass needs anyway)
     static constexpr int VEC = 8 * N;                                      // vectors in front of the stages
     static constexpr size_t BYTES = sizeof(float) * (VEC + (FS * FWD > BS * BWD ? FS * FWD : BS * BWD));
     static __device__ __forceinline__ int swizzle(int r) { return N == 16 ? (r >> 1) & 3 : r & 7; }
@@ -593,8 +610,11 @@ __host__ __device__ constexpr size_t warp_bytes()
 // state at the piece's ends, writes its part of the outputs and leaves failures to the caller.
 // GRAD = the gradients of the first control in the same kernel (n = m = 8 NB, float32 operands): see grad_tail().
 // FEW = at most four warps per SM: the factorisation with the shorter chain (chol8_inverse).
+// CTAs per SM at n <= 16: as many as shared memory (time-varying) or registers hold.  Time-invariant six of them, 80 registers (20 to
+// 30 bytes of them spilled at the end of the horizon): 32768 instances, H = 16, all outputs 0.667 -> 0.604 ms against four (five
+// 0.630, seven 0.608), 4096 instances 99.8 -> 96.2 us.  Launches that cannot fill that many (FEW, the pieces of a scan) keep four.
 template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false, bool GRAD = false, bool FEW = false>
-__global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 4) riccati_frag_kernel(SolveParams p)
+__global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 : TV ? 5 : CH || FEW ? 4 : 6) riccati_frag_kernel(SolveParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -674,8 +694,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     if (p.P && !p.first_only && last_piece)
         store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, 1.f, n, obf, lane);
 
-    // (the affine recursion above n = 16 takes the float32 operands back from their tf32 parts, at n <= 8 nothing is gained)
-    constexpr bool HALF = (!AFF || TWO) && NB > 1;
+    constexpr bool HALF = NB > 1;                           // (at n <= 8 nothing is gained)
     // The recursion is homogeneous in (P, Q, R, p, r): it runs on their multiples by a power of four that brings the largest
     // P_ii at the end of the horizon into [1, 4), which changes no digit and makes the range of the halves one of ratios.
     float scale = 1.f, unscale = 1.f;
@@ -713,52 +732,71 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     }
 
     int fail = 0;
-    // Raw A, B (staged in shared memory) -> split, in place.  On pairs of halves: false, and nothing done, when their rows are
-    // out of range.
+    // Raw A, B (staged in shared memory) -> split, in place, one after the other.  On pairs of halves: false in a lane whose
+    // rows are out of range (the caller stages the operands again then).
     auto install = [&](auto form, bool newA, bool newB) -> bool {
+        bool ok = true;
         if constexpr (!TWO) {
-            Mat<NB, NB> At;
-            Mat<MB, NB> Bt;
-            if (newA)
+            if (newA) {
+                Mat<NB, NB> At;
                 load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
-            if (newB)
-                load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
-            if constexpr (decltype(form)::value) {
-                Halves<NB, NB> as;
-                Halves<MB, NB> bs;
-                bool ok = true;
-                if (newA) {
+                __syncwarp();
+                if constexpr (decltype(form)::value) {
+                    Halves<NB, NB> as;
                     split(as, At);
                     ok = rows_fit<NB, NB, PAD>(as, n, lane);
+                    keep(mem.halvesA(), as, lane);
+                } else {
+                    keep(mem.A, At, lane);
                 }
-                if (newB) {
+            }
+            if (newB) {
+                Mat<MB, NB> Bt;
+                load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
+                __syncwarp();
+                if constexpr (decltype(form)::value) {
+                    Halves<MB, NB> bs;
                     split(bs, Bt);
                     const bool okB = rows_fit<MB, NB, PAD>(bs, m, lane);
                     ok = ok && okB;
-                }
-                if (!__all_sync(FULL, ok))
-                    return false;
-                __syncwarp();
-                if (newA)
-                    keep(mem.halvesA(), as, lane);
-                if (newB)
                     keep(mem.halvesB(), bs, lane);
-            } else {
-                __syncwarp();
-                if (newA)
-                    keep(mem.A, At, lane);
-                if (newB)
+                } else {
                     keep(mem.B, Bt, lane);
+                }
             }
             __syncwarp();
         }
-        return true;
+        return ok;
     };
-    // One step.  On pairs of halves: false, and nothing done, when the operands are out of their range.
+    float gr[MB], ap[NB];                                   // affine: B'p + r and A'p in row form
+    auto affine_part = [&](const Mat<NB, NB>& At, const Mat<MB, NB>& Bt, const int ts) {
+        float pc[NB][2];
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+            row_to_col(pc[b][0], pc[b][1], pr[b], lane);
+        const long long orv = pl.off(p.r) + ts * p.r.st;
+#pragma unroll
+        for (int b = 0; b < MB; ++b) {
+            float s = 0.f;
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+                s = fmaf(Bt.v[b / 2][k][2 * (b & 1)], pc[k][0], fmaf(Bt.v[b / 2][k][2 * (b & 1) + 1], pc[k][1], s));
+            gr[b] = sum_over_t(s) + (8 * b + g < m ? scale * load_elem(p.r, orv + 8 * b + g) : 0.f);
+        }
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            float s = 0.f;
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+                s = fmaf(At.v[b / 2][k][2 * (b & 1)], pc[k][0], fmaf(At.v[b / 2][k][2 * (b & 1) + 1], pc[k][1], s));
+            ap[b] = sum_over_t(s);
+        }
+    };
+    // One step.  On pairs of halves: false, and nothing else done, when an operand is out of its range.
     auto step = [&](auto form, const int ts) -> bool {
         constexpr bool ON_HALVES = decltype(form)::value;
-        Mat<NB, NB> At, T;
-        Mat<MB, NB> Bt, V;
+        Mat<NB, NB> T;
+        Mat<MB, NB> V;
         Mat<NB, MB> Zt;
         Mat<MB, MB> S, nR;
         if constexpr (TWO) {
@@ -773,8 +811,12 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
                 if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(nx.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
             }
             load_negated<MB, Ops::LR>(nR, op.R, scale, lane);
+            Mat<NB, NB> At;
+            Mat<MB, NB> Bt;
             load_transposed<NB, NB, Ops::LA, false>(At, op.A, n, n, lane);
             load_transposed<MB, NB, Ops::LB, false>(Bt, op.B, n, m, lane);
+            if (AFF && ts < p.r_count)
+                affine_part(At, Bt, ts);
             if constexpr (ON_HALVES) {
                 Halves<NB, NB> as, ps;
                 Halves<MB, NB> bs, vs;
@@ -810,12 +852,24 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
         } else {
             if (TV || ts == H - 1)                          // (what CH stages for P_H is followed by Q)
                 copies_landed();
-            if (TV && !install(form, p.A.st != 0, p.B.st != 0))
-                return false;
+            if (AFF && ts < p.r_count) {                    // from the float32 operands, before they are split in place
+                Mat<NB, NB> At;
+                Mat<MB, NB> Bt;
+                if (p.A.st)
+                    load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
+                else
+                    load_transposed_global<NB, NB>(At, p.A, oA, n, n, n, lane);
+                if (p.B.st)
+                    load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
+                else
+                    load_transposed_global<MB, NB>(Bt, p.B, oB, m, n, m, lane);
+                affine_part(At, Bt, ts);
+            }
+            const bool rows = TV ? install(form, p.A.st != 0, p.B.st != 0) : true;
             if constexpr (ON_HALVES) {
                 Halves<NB, NB> ps;
                 split(ps, nP);
-                if (!value_fits<NB, PAD>(ps, true, n, lane))
+                if (!value_fits<NB, PAD>(ps, rows, n, lane))
                     return false;
                 product_halves<MB, NB, NB>(V, nullptr, mem.halvesB(), ps, lane);
                 product_halves<NB, NB, NB>(T, nullptr, mem.halvesA(), ps, lane);
@@ -853,40 +907,12 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
                     product<NB, NB, NB, true>(nP, &nP, mem.A, tsp, lane);
                 }
             }
-            if (AFF && ts < p.r_count) {                    // the float32 operands once more, for the vector recursion
-                unkeep(At, mem.A, lane);
-                unkeep(Bt, mem.B, lane);
-            }
             if (TV && ts > 0) {                             // operands of the next step, in flight while this one is factored
                 __syncwarp();
                 if (p.A.st) stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + (ts - 1) * p.A.st, n, n, lane);
                 if (p.B.st) stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + (ts - 1) * p.B.st, n, m, lane);
                 if (p.R.st) stage<MB, MB, Ops::LR, PAD>(mem.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
                 if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(mem.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
-            }
-        }
-        float gr[MB], ap[NB];                               // affine: B'p + r and A'p in row form
-        if (AFF && ts < p.r_count) {
-            float pc[NB][2];
-#pragma unroll
-            for (int b = 0; b < NB; ++b)
-                row_to_col(pc[b][0], pc[b][1], pr[b], lane);
-            const long long orv = pl.off(p.r) + ts * p.r.st;
-#pragma unroll
-            for (int b = 0; b < MB; ++b) {
-                float s = 0.f;
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    s = fmaf(Bt.v[b / 2][k][2 * (b & 1)], pc[k][0], fmaf(Bt.v[b / 2][k][2 * (b & 1) + 1], pc[k][1], s));
-                gr[b] = sum_over_t(s) + (8 * b + g < m ? scale * load_elem(p.r, orv + 8 * b + g) : 0.f);
-            }
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                float s = 0.f;
-#pragma unroll
-                for (int k = 0; k < NB; ++k)
-                    s = fmaf(At.v[b / 2][k][2 * (b & 1)], pc[k][0], fmaf(At.v[b / 2][k][2 * (b & 1) + 1], pc[k][1], s));
-                ap[b] = sum_over_t(s);
             }
         }
         Split<NB, MB> zs;
@@ -968,7 +994,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : TV && !AFF ? 5 : 
     int ts = H - 1;
     const bool fixedA = !TV || !p.A.st, fixedB = !TV || !p.B.st;           // operands that are installed once
     if constexpr (HALF) {
-        if (install(OnHalves<true>(), fixedA, fixedB))
+        if (__all_sync(FULL, install(OnHalves<true>(), fixedA, fixedB)))
 #pragma unroll 1
             while (ts >= 0 && step(OnHalves<true>(), ts))
                 --ts;
