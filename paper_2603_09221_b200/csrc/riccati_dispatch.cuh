@@ -12,9 +12,13 @@ inline bool riccati_frag_serves(int n, int m, bool time_varying)
     return !time_varying || (n <= 32 && m <= 32);
 }
 
-// The variants of five, six and eight blocks of states take half of the build time: they are instantiated in sources of their
-// own (riccati_frag_5_6.cu, riccati_frag_8.cu), which compile beside the rest.
-cudaError_t launch_blocks_5_6(const SolveParams& p, int kb, int mb, int sm_count, cudaStream_t st);
+// Most variants are instantiated in sources of their own (riccati_frag_*.cu), which compile beside the rest.
+cudaError_t launch_affine(const SolveParams& p, int kb, bool full16, bool full32, int sm_count, cudaStream_t st);
+cudaError_t launch_time_varying(const SolveParams& p, int kb, bool full16, bool full32, int sm_count, cudaStream_t st);
+cudaError_t launch_blocks_3_4(const SolveParams& p, int kb, int mb, bool full32, int sm_count, cudaStream_t st);
+cudaError_t launch_blocks_5(const SolveParams& p, int mb, int sm_count, cudaStream_t st);
+cudaError_t launch_blocks_6(const SolveParams& p, int mb, int sm_count, cudaStream_t st);
+cudaError_t launch_blocks_8_wide(const SolveParams& p, int mb, int sm_count, cudaStream_t st);
 cudaError_t launch_blocks_8(const SolveParams& p, int mb, int sm_count, cudaStream_t st);
 
 // `exact`: the strides keep the vector loads aligned (rows of Q, Qf, R and of K, A, B in the rollout).
@@ -27,16 +31,10 @@ inline cudaError_t launch_riccati_frag(const SolveParams& p, bool time_varying, 
 {
     const int nb = (p.n + 7) / 8, mb = (p.m + 7) / 8, kb = nb > mb ? nb : mb;
     const bool full16 = exact && p.n == 16 && p.m == 16, full32 = exact && p.n == 32 && p.m == 32;
-    if (affine) {
-        if (kb <= 2)
-            return full16 ? launch_one<2, 2, true, true, false>(p, sm_count, st) : launch_one<2, 2, true, true, true>(p, sm_count, st);
-        return full32 ? launch_one<4, 4, true, true, false>(p, sm_count, st) : launch_one<4, 4, true, true, true>(p, sm_count, st);
-    }
-    if (time_varying) {
-        if (kb <= 2)
-            return full16 ? launch_one<2, 2, true, false, false>(p, sm_count, st) : launch_one<2, 2, true, false, true>(p, sm_count, st);
-        return full32 ? launch_one<4, 4, true, false, false>(p, sm_count, st) : launch_one<4, 4, true, false, true>(p, sm_count, st);
-    }
+    if (affine)
+        return launch_affine(p, kb, full16, full32, sm_count, st);
+    if (time_varying)
+        return launch_time_varying(p, kb, full16, full32, sm_count, st);
     switch (kb) {
     case 1:
         return exact && p.n == 8 && p.m == 8 ? launch_one<1, 1, false, false, false>(p, sm_count, st)
@@ -45,27 +43,19 @@ inline cudaError_t launch_riccati_frag(const SolveParams& p, bool time_varying, 
         return full16 ? launch_one<2, 2, false, false, false>(p, sm_count, st)
              : mb == 1 ? launch_one<2, 1, false, false, true>(p, sm_count, st) : launch_one<2, 2, false, false, true>(p, sm_count, st);
     case 3:
-        return mb == 1 ? launch_one<3, 1, false, false, true>(p, sm_count, st)
-             : mb == 2 ? launch_one<3, 2, false, false, true>(p, sm_count, st) : launch_one<3, 3, false, false, true>(p, sm_count, st);
     case 4:
-        return full32 ? launch_one<4, 4, false, false, false>(p, sm_count, st)
-             : mb == 1 ? launch_one<4, 1, false, false, true>(p, sm_count, st)
-             : mb == 2 ? launch_one<4, 2, false, false, true>(p, sm_count, st)
-             : mb == 3 ? launch_one<4, 3, false, false, true>(p, sm_count, st) : launch_one<4, 4, false, false, true>(p, sm_count, st);
+        return launch_blocks_3_4(p, kb, mb, full32, sm_count, st);
     case 5:
+        return launch_blocks_5(p, mb, sm_count, st);
     case 6:
-        return launch_blocks_5_6(p, kb, mb, sm_count, st);
+        return launch_blocks_6(p, mb, sm_count, st);
     default:
-        return launch_blocks_8(p, mb, sm_count, st);
+        return mb <= 4 ? launch_blocks_8(p, mb, sm_count, st) : launch_blocks_8_wide(p, mb, sm_count, st);
     }
 }
 
 // Gradients of the first control, everything in one kernel: n = m = 16 / 32, float32 operands with aligned strides.
-inline cudaError_t launch_grad_frag(const SolveParams& p, int sm_count, cudaStream_t st)
-{
-    return p.n == 16 ? launch_one<2, 2, true, true, false, false, true>(p, sm_count, st)
-                     : launch_one<4, 4, true, true, false, false, true>(p, sm_count, st);
-}
+cudaError_t launch_grad_frag(const SolveParams& p, int sm_count, cudaStream_t st);
 
 } // namespace rfrag
 } // namespace ttc

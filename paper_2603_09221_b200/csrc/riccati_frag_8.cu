@@ -1,4 +1,4 @@
-// One-warp recursion with seven or eight blocks of states (riccati_frag.cuh: time-invariant requests, any strides).
+// One-warp recursion with seven or eight blocks of states and at most four of controls (riccati_frag.cuh: time-invariant requests).
 #include "riccati_frag.cuh"
 
 namespace ttc {
@@ -6,9 +6,7 @@ namespace rfrag {
 
 cudaError_t launch_blocks_8(const SolveParams& p, int mb, int sm_count, cudaStream_t st)
 {
-    return mb <= 2 ? launch_one<8, 2, false, false, true>(p, sm_count, st)
-         : mb <= 4 ? launch_one<8, 4, false, false, true>(p, sm_count, st)
-         : mb <= 6 ? launch_one<8, 6, false, false, true>(p, sm_count, st) : launch_one<8, 8, false, false, true>(p, sm_count, st);
+    return mb <= 2 ? launch_one<8, 2, false, false, true>(p, sm_count, st) : launch_one<8, 4, false, false, true>(p, sm_count, st);
 }
 
 } // namespace rfrag
