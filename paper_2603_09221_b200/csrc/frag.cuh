@@ -528,9 +528,12 @@ struct Halves {
 __device__ __forceinline__ void split_halves(float x0, float x1, uint32_t& h, uint32_t& l)
 {
     const __half2 hh = __floats2half2_rn(x0, x1);
-    const float2 f = __half22float2(hh);
-    const __half2 ll = __floats2half2_rn(x0 - f.x, x1 - f.y);          // (the differences are exact)
     h = *reinterpret_cast<const uint32_t*>(&hh);
+    float l0, l1;                                           // x - h, exact; the mixed fma saves converting h back (n = 32 6.44 -> 6.19 ms)
+    asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\t"
+        "fma.rn.f32.f16 %0, a, %5, %3;\n\tfma.rn.f32.f16 %1, b, %5, %4;\n\t}"
+        : "=f"(l0), "=f"(l1) : "r"(h), "f"(x0), "f"(x1), "h"((unsigned short)0xbc00));
+    const __half2 ll = __floats2half2_rn(l0, l1);
     l = *reinterpret_cast<const uint32_t*>(&ll);
 }
 template <int RB, int CB>
