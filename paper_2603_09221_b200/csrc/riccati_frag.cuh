@@ -10,7 +10,7 @@
 // factorisation in three passes of tf32.
 //
 // What bounds it: at n = 16 a step is 60 tensor-core instructions (8 cycles on a scheduler's pipe, about 4 of its issue
-// slots; 96 in tf32) in about 780, and four or five warps per scheduler hide most of the chain of five products and sixteen
+// slots; 96 in tf32) in about 820, and five or six warps per scheduler hide most of the chain of five products and sixteen
 // pivots.  At n = 32 it is 405 tensor-core instructions (657), two warps per scheduler (all 255 registers); above, registers spill to
 // local memory (0.3 KB per lane at 40 x 16, 2.7 KB at 40 x 40, which the first-level cache absorbs; 10.7 KB at 64 x 64,
 // which it does not: only twice as fast as one CTA per instance there).
@@ -19,8 +19,8 @@
 //   65536 instances n = 16, H = 32, operands from memory  4.26 -> 2.65 ms     4096, n = 16, H = 16, all outputs 188 -> 107 us
 //   16384 instances n = 32, H = 64, all outputs           14.2 -> 8.5 ms      1155, n = 40, m = 12, H = 20     2428 -> 232 us
 //   64 instances n = 8, H = 8, own dynamics               107 -> 11 us     1155, n = m = 60, H = 20            21.9 -> 10.3 ms
-// and from three passes of tf32 throughout to pairs of halves, in the order of the first four: 2.50 -> 2.21 ms, 106 -> 92 us,
-// 8.39 -> 6.45 ms, 232 -> 184 us; error of P_t against float64 0.45e-6 -> 0.27e-6 at n = 16, 0.89e-6 -> 0.44e-6 at n = 32, K, x and u
+// and from three passes of tf32 throughout to pairs of halves, in the order of the first four: 2.50 -> 2.19 ms, 106 -> 88 us,
+// 8.39 -> 6.22 ms, 232 -> 181 us; error of P_t against float64 0.45e-6 -> 0.27e-6 at n = 16, 0.89e-6 -> 0.44e-6 at n = 32, K, x and u
 // 5 to 15 % smaller.  Time-varying n = 32, 2048 instances of 32 steps 0.55 -> 0.41 ms; gradients
 // of 65536 instances, n = 16, H = 32 5.4 -> 5.2 ms.  Problems outside the range (a control in other units) take 107, 253 us (40 x 12,
 // where tf32 alone took 236), 2.5 and 8.5 ms.
