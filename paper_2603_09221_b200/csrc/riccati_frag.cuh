@@ -290,9 +290,24 @@ __device__ __forceinline__ bool rows_fit(const Halves<NB, NB>& a, const Halves<M
     v = max_xor(v, v, 2);
     return __hbge2(v, row_limit<PAD || NB == 1 || MB == 1>(0, second ? m : n, lane >> 2)) && __hble2(v, __float2half2_rn(HALF_HIGH));
 }
-// the conditions on P, and `rows` of every lane (called by the whole warp); P = 0 (no terminal weight) fits as well
+// every element is zero (in float32: a half rounds to zero from 2^-25 downwards)
+template <int RB, int CB>
+__device__ __forceinline__ bool is_zero(const Mat<RB, CB>& x)
+{
+    unsigned any = 0u;
+#pragma unroll
+    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                any |= __float_as_uint(x.v[mt][cb][e]);
+    return !(any & 0x7fffffffu);
+}
+// the conditions on P (x: the halves of nP), and `rows` of every lane (called by the whole warp); P = 0 (no terminal weight)
+// fits as well
 template <int NB, bool PAD>
-__device__ __forceinline__ bool value_fits(const Halves<NB, NB>& x, bool rows, int n, int lane)
+__device__ __forceinline__ bool value_fits(const Halves<NB, NB>& x, const Mat<NB, NB>& nP, bool rows, int n, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
     __half2 top = __habs2(as_half2(x.h[0][0][0]));
@@ -313,7 +328,7 @@ __device__ __forceinline__ bool value_fits(const Halves<NB, NB>& x, bool rows, i
                 }
             }
     return __all_sync(FULL, ok && __hble2(top, __float2half2_rn(HALF_P_HIGH))) ||
-           __all_sync(FULL, rows && __hbeq2(top, __float2half2_rn(0.f)));
+           __all_sync(FULL, rows && is_zero(nP));
 }
 // power of four that brings the largest P_ii into [1, 4); 1 where there is none within 2^-60 .. 2^60
 template <int NB>
@@ -824,7 +839,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
                 split(as, At);
                 split(bs, Bt);
                 const bool rows = rows_fit<NB, MB, PAD>(as, bs, n, m, lane);      // (shuffles: by every lane, whatever P is)
-                if (!value_fits<NB, PAD>(ps, rows, n, lane))
+                if (!value_fits<NB, PAD>(ps, nP, rows, n, lane))
                     return false;
                 product_halves<MB, NB, NB>(V, nullptr, bs, ps, lane);          // V = B' nP
                 product_halves<NB, NB, NB>(T, nullptr, as, ps, lane);          // T = A' nP
@@ -869,7 +884,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
             if constexpr (ON_HALVES) {
                 Halves<NB, NB> ps;
                 split(ps, nP);
-                if (!value_fits<NB, PAD>(ps, rows, n, lane))
+                if (!value_fits<NB, PAD>(ps, nP, rows, n, lane))
                     return false;
                 product_halves<MB, NB, NB>(V, nullptr, mem.halvesB(), ps, lane);
                 product_halves<NB, NB, NB>(T, nullptr, mem.halvesA(), ps, lane);

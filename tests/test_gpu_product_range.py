@@ -1,0 +1,53 @@
+"""Costs, units and couplings at which the matrix products of the one-warp kernel could lose digits or leave their range.
+Everything is compared with the float64 oracles."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2603_09221_b200 import lqr
+from tests import parity_util as pu
+from tests import test_gpu_affine as aff
+from tests import test_gpu_grad as grad
+from tests.test_gpu_parity import small_workload
+from tests.test_gpu_time_varying import run_both, tv_workload
+
+pytestmark = pytest.mark.gpu
+
+
+def scale_costs(w, e):
+    for k in ("Q", "Qf", "R"):
+        if k in w:
+            w[k] = w[k] * 2.0 ** e
+    return w
+
+
+@pytest.mark.parametrize("e", [-24, -27, -30, -50])
+@pytest.mark.parametrize("n,m", [(5, 5), (16, 16), (20, 12), (32, 32)])
+def test_small_costs_without_terminal_weight(n, m, e):
+    """The value matrix is zero at the end of the horizon and small, not zero, from then on."""
+    w = scale_costs(tv_workload(n, m, 6, (1, 2, 4), seed=50 + n), e)
+    w["Qf"].zero_()
+    out, ref = run_both(w)
+    pu.compare(out, ref, np.arange(8), 1e-4)
+
+
+@pytest.mark.parametrize("n", [16, 32])
+def test_small_costs_affine_and_gradients(n):
+    w = scale_costs(aff.affine_workload(n, n, 6, (1, 2, 4), seed=70 + n), -30)
+    w["r"] = w["r"] * 2.0 ** -30
+    w["Qf"].zero_()
+    out, ref = aff.run_both(w)
+    aff.check(out, ref, False)
+    w = scale_costs(tv_workload(n, n, 6, (1, 2, 4), seed=90 + n), -30)
+    w["Qf"].zero_()
+    g = grad.draw_g(8, n, 3)
+    out = grad.run_gpu(w, g)
+    errs = grad.errors(out, grad.run_oracle(w, g))
+    assert int(out["info"].abs().max()) == 0 and all(v <= 1e-4 for v in errs.values()), errs
+
+
+@pytest.mark.parametrize("e", [-63, -70, 63])
+@pytest.mark.parametrize("n,m", [(9, 9), (16, 16), (32, 32), (40, 12)])
+def test_costs_far_from_one_time_invariant(n, m, e):
+    w = scale_costs(small_workload(n, m, 6, (1, 2, 4), seed=110 + n), e)
+    pu.compare(pu.run_gpu(w), pu.run_oracle(w), np.arange(8), 1e-4)
