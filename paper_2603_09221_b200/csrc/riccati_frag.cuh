@@ -232,17 +232,18 @@ __device__ __forceinline__ void store_gain(float* base, long long off, const Mat
 // The pair's absolute error of 2^-25 takes the place of the relative one for small elements, and 65504 is the largest number.
 // A step runs on halves when
 //     every row of A' and of B' has its largest element in [2^-4, 8],
-//     every P_ii is at least 2^-4 and no |P_ij| is above 128, or P = 0
+//     every P_ii is at least 2^-4 and no |P_ij| is above 128 (64 above 32 states), or P = 0
 // (rows of the padding aside), tested on the values in every step, for operands that do not change once; otherwise, and from
 // then on, the instance runs in tf32.  In this range the error of an operand is at most 2^-21 of the largest element of its row,
-// which is the bound of the tf32 split; V and T stay below 32 * 8 * 128 = 2^15 and |Z| below 2^13.
+// which is the bound of the tf32 split; V and T stay below 32 * 8 * 128 = 64 * 8 * 64 = 2^15 and |Z| below 2^13.
 // The rows are tested one by one because a control or a state in other units would otherwise lose its digits: with R_jj and
 // column j of B small together, row j of K is as large as 1 / |B_j|.
 template <bool V>
 struct OnHalves {
     static constexpr bool value = V;
 };
-constexpr float HALF_LOW = 0.0625f, HALF_HIGH = 8.f, HALF_P_HIGH = 128.f;
+constexpr float HALF_LOW = 0.0625f, HALF_HIGH = 8.f;
+__host__ __device__ constexpr float half_p_high(int blocks) { return blocks > 4 ? 64.f : 128.f; }
 __device__ __forceinline__ __half2 as_half2(uint32_t x) { return *reinterpret_cast<const __half2*>(&x); }
 __device__ __forceinline__ __half2 max_xor(__half2 v, __half2 other, int lanes)
 {
@@ -327,7 +328,7 @@ __device__ __forceinline__ bool value_fits(const Halves<NB, NB>& x, const Mat<NB
                     ok = ok && __hbge2(v, __floats2half2_rn(g == 2 * t ? low : 0.f, g == 2 * t + 1 ? low : 0.f));
                 }
             }
-    return __all_sync(FULL, ok && __hble2(top, __float2half2_rn(HALF_P_HIGH))) ||
+    return __all_sync(FULL, ok && __hble2(top, __float2half2_rn(half_p_high(NB)))) ||
            __all_sync(FULL, rows && is_zero(nP));
 }
 // power of four that brings the largest P_ii into [1, 4); 1 where there is none within 2^-60 .. 2^60

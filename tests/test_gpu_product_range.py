@@ -51,3 +51,21 @@ def test_small_costs_affine_and_gradients(n):
 def test_costs_far_from_one_time_invariant(n, m, e):
     w = scale_costs(small_workload(n, m, 6, (1, 2, 4), seed=110 + n), e)
     pu.compare(pu.run_gpu(w), pu.run_oracle(w), np.arange(8), 1e-4)
+
+
+def test_sixty_four_equal_contributions():
+    """Every contraction index contributes 8 * 128 to a row of A'P: 64 * 8 * 128 is above the largest float16.  P_1 =
+    1 + 8^2 64^2 R / (R + 64^2) passes through 128 over the heads.  It is what is left of 262144 after a cancellation by 2^11,
+    so float32 products (2^-20 each) give it to 2^-9, K (no cancellation) to the usual bound; P_0 cancels once more by the
+    same and is only finite."""
+    heads = 24
+    w = small_workload(64, 1, 2, (1, heads, 1), seed=1)
+    w["A"].fill_(8.0)
+    w["B"].fill_(1.0)
+    w["Q"].fill_(1.0)
+    w["R"].copy_(torch.linspace(1.983, 1.987, heads).reshape(w["R"].shape))
+    gpu, ref = pu.run_gpu(w, want=("K", "P", "info")), pu.run_oracle(w)
+    assert 127.8 < ref["P"][0, 1].max() and ref["P"][-1, 1].max() < 128.2
+    assert int(gpu["info"].abs().max()) == 0 and bool(torch.isfinite(gpu["P"]).all())
+    assert pu.block_rel_err(gpu["K"][:, 1:].cpu(), ref["K"][:, 1:], 2) <= 1e-4
+    assert pu.block_rel_err(gpu["P"][:, 1:].cpu(), ref["P"][:, 1:], 2) <= 2.0 ** -9
