@@ -331,7 +331,8 @@ __device__ __forceinline__ bool value_fits(const Halves<NB, NB>& x, const Mat<NB
     return __all_sync(FULL, ok && __hble2(top, __float2half2_rn(half_p_high(NB)))) ||
            __all_sync(FULL, rows && is_zero(nP));
 }
-// power of four that brings the largest P_ii into [1, 4); 1 where there is none within 2^-60 .. 2^60
+// power of four, at most 1, that brings the largest P_ii into [1, 4); 1 where it is below or above 2^60.  (Never above 1: the
+// weights are multiplied by it too, and one of 2^70 beside a small value matrix would leave float32.)
 template <int NB>
 __device__ __forceinline__ float value_scale(const Mat<NB, NB>& nP, int lane)
 {
@@ -342,7 +343,7 @@ __device__ __forceinline__ float value_scale(const Mat<NB, NB>& nP, int lane)
         top = fmaxf(top, -((g & 1) ? nP.v[b / 2][b][2 * (b & 1) + 1] : nP.v[b / 2][b][2 * (b & 1)]));
     const unsigned bits = __reduce_max_sync(FULL, t == (g >> 1) ? __float_as_uint(top) : 0u);
     const int e = ((int)(bits >> 23) - 127) & ~1;
-    return e >= -60 && e <= 60 ? __int_as_float((127 - e) << 23) : 1.f;
+    return e >= 0 && e <= 60 ? __int_as_float((127 - e) << 23) : 1.f;
 }
 
 // W consecutive elements of a row (16-byte loads), or with PAD element by element within [0, n)
@@ -711,8 +712,10 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
         store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, 1.f, n, obf, lane);
 
     constexpr bool HALF = NB > 1;                           // (at n <= 8 nothing is gained)
-    // The recursion is homogeneous in (P, Q, R, p, r): it runs on their multiples by a power of four that brings the largest
-    // P_ii at the end of the horizon into [1, 4), which changes no digit and makes the range of the halves one of ratios.
+    // The recursion is homogeneous in (P, Q, R, p, r): on halves it runs on their multiples by a power of four that brings the
+    // largest P_ii at the end of the horizon into [1, 4), which makes the range of the halves one of ratios.  In tf32 it runs
+    // on the weights as they are: a small R_jj would become subnormal beside a control without effect (the reciprocals of
+    // the factorisation flush those to zero).
     float scale = 1.f, unscale = 1.f;
     if constexpr (HALF) {
         scale = value_scale<NB>(nP, lane);
@@ -1023,8 +1026,23 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
                 copies_landed();
             }
     }
-    if (ts >= 0)
+    if (ts >= 0) {
+        if constexpr (HALF) {                               // (what is scaled back are results that the horizon may keep)
+#pragma unroll
+            for (int mt = 0; mt < Mat<NB, NB>::MT; ++mt)
+#pragma unroll
+                for (int cb = 0; cb < NB; ++cb)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        nP.v[mt][cb][e] *= unscale;
+            if (AFF)
+#pragma unroll
+                for (int b = 0; b < NB; ++b)
+                    pr[b] *= unscale;
+            scale = unscale = 1.f;
+        }
         install(OnHalves<false>(), fixedA, fixedB);
+    }
 #pragma unroll 1
     for (; ts >= 0; --ts)
         step(OnHalves<false>(), ts);

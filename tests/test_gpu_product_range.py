@@ -69,3 +69,24 @@ def test_sixty_four_equal_contributions():
     assert int(gpu["info"].abs().max()) == 0 and bool(torch.isfinite(gpu["P"]).all())
     assert pu.block_rel_err(gpu["K"][:, 1:].cpu(), ref["K"][:, 1:], 2) <= 1e-4
     assert pu.block_rel_err(gpu["P"][:, 1:].cpu(), ref["P"][:, 1:], 2) <= 2.0 ** -9
+
+
+@pytest.mark.parametrize("n,m", [(16, 16), (32, 32)])
+def test_weights_far_from_the_terminal_weight(n, m):
+    w = tv_workload(n, m, 6, (1, 2, 4), seed=130 + n)
+    w["Qf"] *= 2.0 ** -58
+    w["Q"] *= 2.0 ** 73
+    w["R"] *= 2.0 ** 73
+    out, ref = run_both(w)
+    pu.compare(out, ref, np.arange(8), 1e-4)
+
+
+@pytest.mark.parametrize("n,m", [(16, 5), (32, 12), (40, 12)])
+def test_small_control_weight_of_a_control_without_effect(n, m):
+    """R_22 = 2^-70 beside P = 2^60, and column 2 of B is zero: S_22 = R_22, row 2 of K is zero."""
+    w = small_workload(n, m, 6, (1, 2, 4), seed=150 + n)
+    w["Q"] *= 2.0 ** 59
+    w["R"] = torch.diag_embed(torch.full((1, 2, 1, m), 2.0 ** -70, device=w["R"].device)).contiguous()
+    w["R"][..., torch.arange(m) != 2, torch.arange(m) != 2] = 2.0 ** 55
+    w["B"][..., 2] = 0.0
+    pu.compare(pu.run_gpu(w), pu.run_oracle(w), np.arange(8), 1e-4)
