@@ -11,7 +11,8 @@
 //     V = B'P = (B')(P)',  T = A'P,  S = R + (B')(V)',  Y' = (A')(V)',  A'PA = (A')(T)',  Z'Z = (Z')(Z')'
 // Every product keeps float32-grade accuracy: operands are split into a tf32 part rounded to nearest and the remainder,
 // three passes (lo*hi + hi*lo + hi*hi) accumulate in float32.  The dropped term and the truncation of the remainder are
-// both about 2^-23 of the product.
+// both about 2^-23 of the product on average, 2^-20 at most.  (A second set of products takes pairs of float16 numbers, for
+// operands whose values permit it.)
 #pragma once
 
 #include <cuda_fp16.h>
@@ -514,30 +515,43 @@ __device__ __forceinline__ void product_symmetric(Mat<NB, NB>& d, const Split<NB
         }
 }
 
-// ---- the same products on pairs of halves: an operand is split into two float16 numbers, each rounded to nearest, and one
-// instruction takes sixteen contraction indices at the price of eight in tf32 (8 cycles of a scheduler's pipe): half the
-// instructions, half the operand registers.  A float16 keeps the eleven bits of a tf32 number, so that the pair represents x
-// to 2^-22 |x| (tf32: 2^-21, the remainder is truncated) as long as its second half is no subnormal; below, to 2^-25.  What
-// that needs of the operands is in riccati_frag.cuh.  The tiles of two neighbouring column blocks are the instruction's A
+// ---- the same products on pairs of halves: one instruction takes sixteen contraction indices at the price of eight in tf32
+// (8 cycles of a scheduler's pipe): half the instructions, half the operand registers.  An operand is split into
+//     s x = h + 2^-11 l,    h = half(s x),  l = half(2^11 (s x - h)),    s a power of two,
+// so that the remainder has the exponent of the number itself (Ootomo and Yokota, 2022) and l*h + h*l are summed first, from
+// zero, and multiplied by 2^-11 before h*h goes on top.  A float16 keeps the eleven bits of a tf32 number: the pair represents
+// s x to 2^-22 |s x| (tf32: 2^-21, the remainder is truncated) above 2^-14 and to 2^-36 below, which is 2^-21 |s x| down to
+// 2^-15.  Who may use them, and when: riccati_frag.cuh.  The tiles of two neighbouring column blocks are the instruction's A
 // operand as they stand, and the B operand of the transpose, as above.
 template <int RB, int CB>
 struct Halves {
     static constexpr int MT = (RB + 1) / 2;
     uint32_t h[MT][CB][2], l[MT][CB][2];                   // [..][0]: row g, columns 2 t and 2 t + 1; [..][1]: row g + 8
 };
-__device__ __forceinline__ void split_halves(float x0, float x1, uint32_t& h, uint32_t& l)
+constexpr float HALF_LOW = 0x1p-15f, HALF_HIGH = 65504.f, REMAINDER = 2048.f;
+__device__ __forceinline__ __half2 as_half2(uint32_t x) { return *reinterpret_cast<const __half2*>(&x); }
+// (a, b) <- (c a, c b)
+__device__ __forceinline__ void scale_pair(float& a, float& b, float c)
 {
-    const __half2 hh = __floats2half2_rn(x0, x1);
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %2};\n\tmul.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "+f"(a), "+f"(b) : "f"(c));
+}
+__device__ __forceinline__ void split_halves(float x0, float x1, float s, uint32_t& h, uint32_t& l)
+{
+    float y0 = x0, y1 = x1;
+    scale_pair(y0, y1, s);
+    const __half2 hh = __floats2half2_rn(y0, y1);
     h = *reinterpret_cast<const uint32_t*>(&hh);
-    float l0, l1;                                           // x - h, exact; the mixed fma saves converting h back (n = 32 6.44 -> 6.19 ms)
+    scale_pair(y0, y1, REMAINDER);
+    float l0, l1;                                           // 2^11 (s x - h), exact; the mixed fma saves converting h back
     asm("{\n\t.reg .b16 a, b;\n\tmov.b32 {a, b}, %2;\n\t"
         "fma.rn.f32.f16 %0, a, %5, %3;\n\tfma.rn.f32.f16 %1, b, %5, %4;\n\t}"
-        : "=f"(l0), "=f"(l1) : "r"(h), "f"(x0), "f"(x1), "h"((unsigned short)0xbc00));
+        : "=f"(l0), "=f"(l1) : "r"(h), "f"(y0), "f"(y1), "h"((unsigned short)0xe800));     // -2048
     const __half2 ll = __floats2half2_rn(l0, l1);
     l = *reinterpret_cast<const uint32_t*>(&ll);
 }
 template <int RB, int CB>
-__device__ __forceinline__ void split(Halves<RB, CB>& s, const Mat<RB, CB>& m)
+__device__ __forceinline__ void split(Halves<RB, CB>& x, const Mat<RB, CB>& m, float s)
 {
 #pragma unroll
     for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
@@ -546,12 +560,32 @@ __device__ __forceinline__ void split(Halves<RB, CB>& s, const Mat<RB, CB>& m)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 if (e && 2 * mt + 1 >= RB)                  // rows that do not exist
-                    s.h[mt][cb][e] = s.l[mt][cb][e] = 0u;
+                    x.h[mt][cb][e] = x.l[mt][cb][e] = 0u;
                 else
-                    split_halves(m.v[mt][cb][2 * e], m.v[mt][cb][2 * e + 1], s.h[mt][cb][e], s.l[mt][cb][e]);
+                    split_halves(m.v[mt][cb][2 * e], m.v[mt][cb][2 * e + 1], s, x.h[mt][cb][e], x.l[mt][cb][e]);
             }
 }
-// d = c + X Y' over sixteen contraction indices, or over eight
+// true in the whole warp when at least `elements` of X are not below LOW and none is above the largest float16 or a NaN
+template <int RB, int CB>
+__device__ __forceinline__ bool in_range(const Halves<RB, CB>& x, float low, int elements)
+{
+    __half2 count = __float2half2_rn(0.f), top = __float2half2_rn(0.f);
+#pragma unroll
+    for (int mt = 0; mt < Halves<RB, CB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (e && 2 * mt + 1 >= RB)
+                    continue;
+                const __half2 v = __habs2(as_half2(x.h[mt][cb][e]));
+                count = __hadd2(count, __hge2(v, __float2half2_rn(low)));
+                top = __hmax2_nan(top, v);
+            }
+    const float2 c = __half22float2(count);
+    return __reduce_add_sync(FULL, __hble2(top, __float2half2_rn(HALF_HIGH)) ? (int)(c.x + c.y) : -65536) >= elements;
+}
+// d = X Y' over sixteen contraction indices, or over eight
 __device__ __forceinline__ void mma_halves(float (&d)[4], const float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                            uint32_t b0, uint32_t b1)
 {
@@ -583,60 +617,49 @@ __device__ __forceinline__ void keep(StoredHalves<RB, CB>& st, const Halves<RB, 
             st.q[mt][cb / 2][1][lane] = make_uint4(s.l[mt][cb][0], s.l[mt][cb][1], s.l[mt][c1][0], s.l[mt][c1][1]);
         }
 }
-// operand words of X for the column blocks kb, kb + 1: from registers, from shared memory
-template <int RB, int KB>
-__device__ __forceinline__ uint4 operand_word(const Halves<RB, KB>& x, int mt, int kb, int part, int)
+// d = X Y' with X stored, scaled by the scales of both operands; LOWER as above
+template <int RB, int KB, int CB, bool LOWER = false>
+__device__ __forceinline__ void product_halves(Mat<RB, CB>& d, const StoredHalves<RB, KB>& x, const Halves<CB, KB>& y, int lane)
 {
-    const int k1 = kb + 1 < KB ? kb + 1 : kb;
-    return part ? make_uint4(x.l[mt][kb][0], x.l[mt][kb][1], x.l[mt][k1][0], x.l[mt][k1][1])
-                : make_uint4(x.h[mt][kb][0], x.h[mt][kb][1], x.h[mt][k1][0], x.h[mt][k1][1]);
-}
-template <int RB, int KB>
-__device__ __forceinline__ uint4 operand_word(const StoredHalves<RB, KB>& x, int mt, int kb, int part, int lane)
-{
-    return x.q[mt][kb / 2][part][lane];
-}
-// d = c + X * Y', with the conventions of the products above
-template <int RB, int KB, int CB, bool LOWER = false, class X>
-__device__ __forceinline__ void product_halves(Mat<RB, CB>& d, const Mat<RB, CB>* c, const X& x, const Halves<CB, KB>& y, int lane)
-{
-    const float z[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int kb = 0; kb < KB; kb += 2) {
-        uint4 a[Mat<RB, CB>::MT][2];
+    for (int main = 0; main < 2; ++main) {                  // lo*hi + hi*lo, then hi*hi
 #pragma unroll
-        for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
-            a[mt][0] = operand_word(x, mt, kb, 0, lane);
-            a[mt][1] = operand_word(x, mt, kb, 1, lane);
+        for (int kb = 0; kb < KB; kb += 2) {
+#pragma unroll
+            for (int pass = main ? 2 : 0; pass < (main ? 3 : 2); ++pass) {
+                uint4 a[Mat<RB, CB>::MT];
+#pragma unroll
+                for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+                    a[mt] = x.q[mt][kb / 2][pass == 0][lane];
+#pragma unroll
+                for (int cb = 0; cb < CB; ++cb)
+#pragma unroll
+                    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
+                        if (LOWER && cb > 2 * mt + 1)
+                            continue;
+                        float(&dd)[4] = d.v[mt][cb];
+                        if (!kb && !pass)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                dd[e] = 0.f;
+                        const uint32_t b0 = pass == 1 ? y.l[cb / 2][kb][cb & 1] : y.h[cb / 2][kb][cb & 1];
+                        if (kb + 1 < KB)
+                            mma_halves(dd, dd, a[mt].x, a[mt].y, a[mt].z, a[mt].w, b0,
+                                       pass == 1 ? y.l[cb / 2][kb + 1][cb & 1] : y.h[cb / 2][kb + 1][cb & 1]);
+                        else
+                            mma_halves(dd, dd, a[mt].x, a[mt].y, b0);
+                    }
+            }
         }
-#pragma unroll
-        for (int pass = 0; pass < 3; ++pass)                // lo*hi, hi*lo, hi*hi
+        if (!main)
 #pragma unroll
             for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-                for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt) {
-                    if (LOWER && cb > 2 * mt + 1)
-                        continue;
-                    const uint4 v = a[mt][pass == 0];
-                    const uint32_t b0 = pass == 1 ? y.l[cb / 2][kb][cb & 1] : y.h[cb / 2][kb][cb & 1];
-                    float(&dd)[4] = d.v[mt][cb];
-                    if (kb + 1 < KB) {
-                        const uint32_t b1 = pass == 1 ? y.l[cb / 2][kb + 1][cb & 1] : y.h[cb / 2][kb + 1][cb & 1];
-                        if (kb || pass)
-                            mma_halves(dd, dd, v.x, v.y, v.z, v.w, b0, b1);
-                        else if (c)
-                            mma_halves(dd, c->v[mt][cb], v.x, v.y, v.z, v.w, b0, b1);
-                        else
-                            mma_halves(dd, z, v.x, v.y, v.z, v.w, b0, b1);
-                    } else {
-                        if (kb || pass)
-                            mma_halves(dd, dd, v.x, v.y, b0);
-                        else if (c)
-                            mma_halves(dd, c->v[mt][cb], v.x, v.y, b0);
-                        else
-                            mma_halves(dd, z, v.x, v.y, b0);
+                for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+                    if (!(LOWER && cb > 2 * mt + 1)) {
+                        scale_pair(d.v[mt][cb][0], d.v[mt][cb][1], 1.f / REMAINDER);
+                        scale_pair(d.v[mt][cb][2], d.v[mt][cb][3], 1.f / REMAINDER);
                     }
-                }
     }
 }
 

@@ -6,24 +6,22 @@
 // The recursion is carried in negated variables (nP = -P etc.): every update is then a plain accumulation.
 //   V = B' nP,  T = A' nP,  nS = -R + B' V',  nY' = A' V',  nP_t = -Q + A' T' + Z' Z     (Prop. 3.1; Alg. 1)
 // with S = L L', Z = L^{-1} Y and, when gains are wanted, K' = -Z' L^{-1} from the inverses of L's diagonal blocks.
-// The five products with A, B, P and Z'Z run on pairs of halves while the values permit it (below), otherwise and in the
-// factorisation in three passes of tf32.
+// Above 16 states or controls the five products with A, B and P run on pairs of halves while the values permit it (below); Z'Z,
+// the factorisation and everything up to 16 in three passes of tf32.
 //
-// What bounds it: at n = 16 a step is 60 tensor-core instructions (8 cycles on a scheduler's pipe, about 4 of its issue
-// slots; 96 in tf32) in about 820, and five or six warps per scheduler hide most of the chain of five products and sixteen
-// pivots.  At n = 32 it is 405 tensor-core instructions (657), two warps per scheduler (all 255 registers); above, registers spill to
-// local memory (0.3 KB per lane at 40 x 16, 2.7 KB at 40 x 40, which the first-level cache absorbs; 10.7 KB at 64 x 64,
+// What bounds it: at n = 16 a step is 96 tensor-core instructions (8 cycles on a scheduler's pipe, about 4 of its issue
+// slots) in about 830, and five or six warps per scheduler hide most of the chain of five products and sixteen
+// pivots.  At n = 32 it is 441 tensor-core instructions (657 in tf32), two warps per scheduler (all 255 registers); above, registers spill
+// to local memory (0.2 KB per lane at 40 x 16, 1.6 KB at 40 x 40, which the first-level cache absorbs; 10.7 KB at 64 x 64,
 // which it does not: only twice as fast as one CTA per instance there).
 // The forms this replaced: rows broadcast from shared memory at n = 16 (load/store pipe at 88 %), products through shared
 // memory at n = 32 (74 %), one CTA per instance with two barriers per pivot elsewhere.  Measured before -> now:
-//   65536 instances n = 16, H = 32, operands from memory  4.26 -> 2.65 ms     4096, n = 16, H = 16, all outputs 188 -> 107 us
-//   16384 instances n = 32, H = 64, all outputs           14.2 -> 8.5 ms      1155, n = 40, m = 12, H = 20     2428 -> 232 us
+//   65536 instances n = 16, H = 32, operands from memory  4.26 -> 2.50 ms     4096, n = 16, H = 16, all outputs 188 -> 106 us
+//   16384 instances n = 32, H = 64, all outputs           14.2 -> 6.87 ms     1155, n = 40, m = 12, H = 20     2428 -> 198 us
 //   64 instances n = 8, H = 8, own dynamics               107 -> 11 us     1155, n = m = 60, H = 20            21.9 -> 10.3 ms
-// and from three passes of tf32 throughout to pairs of halves, in the order of the first four: 2.50 -> 2.19 ms, 106 -> 88 us,
-// 8.39 -> 6.22 ms, 232 -> 181 us; error of P_t against float64 0.45e-6 -> 0.27e-6 at n = 16, 0.89e-6 -> 0.44e-6 at n = 32, K, x and u
-// 5 to 15 % smaller.  Time-varying n = 32, 2048 instances of 32 steps 0.55 -> 0.41 ms; gradients
-// of 65536 instances, n = 16, H = 32 5.4 -> 5.2 ms.  Problems outside the range (a control in other units) take 107, 253 us (40 x 12,
-// where tf32 alone took 236), 2.5 and 8.5 ms.
+// The halves' part in that, against three passes of tf32 throughout: n = 32 8.41 -> 6.87 ms, 40 x 12 235 -> 198 us, time-varying
+// n = 32, 2048 instances of 32 steps 0.54 -> 0.49 ms.  Problems outside the range take 235 us at 40 x 12, and at n = 32 what
+// they took (1.10 ms on 4096 instances of 32 steps, 0.91 inside).
 #pragma once
 
 #include "common.cuh"
@@ -158,9 +156,9 @@ __device__ __forceinline__ void load_transposed_global(Mat<RB, CB>& x, const Ope
                 x.v[mt][cb][e] = i < ni && k < nk ? load_elem(o, off + k * ld + i) : 0.f;
             }
 }
-// x = -c M of a square matrix in shared memory
+// x = -M of a square matrix in shared memory
 template <int RB, int LD>
-__device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const float* M, float c, int lane)
+__device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const float* M, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -172,9 +170,30 @@ __device__ __forceinline__ void load_negated(Mat<RB, RB>& x, const float* M, flo
                 float2 f = make_float2(0.f, 0.f);
                 if (h == 0 || 2 * mt + 1 < RB)
                     f = *reinterpret_cast<const float2*>(M + (16 * mt + 8 * h + g) * LD + 8 * cb + 2 * t);
-                x.v[mt][cb][2 * h] = -c * f.x;
-                x.v[mt][cb][2 * h + 1] = -c * f.y;
+                x.v[mt][cb][2 * h] = -f.x;
+                x.v[mt][cb][2 * h + 1] = -f.y;
             }
+}
+// x = c x - M
+template <int RB, int LD, bool LOWER>
+__device__ __forceinline__ void scale_and_subtract(Mat<RB, RB>& x, float c, const float* M, int lane)
+{
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int mt = 0; mt < Mat<RB, RB>::MT; ++mt)
+#pragma unroll
+        for (int cb = 0; cb < RB; ++cb) {
+            if (LOWER && cb > 2 * mt + 1)
+                continue;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float2 f = make_float2(0.f, 0.f);
+                if (h == 0 || 2 * mt + 1 < RB)
+                    f = *reinterpret_cast<const float2*>(M + (16 * mt + 8 * h + g) * LD + 8 * cb + 2 * t);
+                x.v[mt][cb][2 * h] = fmaf(c, x.v[mt][cb][2 * h], -f.x);
+                x.v[mt][cb][2 * h + 1] = fmaf(c, x.v[mt][cb][2 * h + 1], -f.y);
+            }
+        }
 }
 
 // element pair (row i, columns k, k + 1) of a row-major output with row length ld
@@ -186,7 +205,7 @@ __device__ __forceinline__ void store_pair(float* base, long long idx, float a, 
         *reinterpret_cast<float2*>(base + idx) = make_float2(a, b);
 }
 template <int RB, bool PAD>
-__device__ __forceinline__ void store_negated(float* base, long long off, const Mat<RB, RB>& x, float c, int d, int bf16, int lane)
+__device__ __forceinline__ void store_negated(float* base, long long off, const Mat<RB, RB>& x, int d, int bf16, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -198,7 +217,7 @@ __device__ __forceinline__ void store_negated(float* base, long long off, const 
                 if (h == 1 && 2 * mt + 1 >= RB)
                     continue;
                 const int i = 16 * mt + 8 * h + g, k = 8 * cb + 2 * t;
-                const float a = -c * x.v[mt][cb][2 * h], b = -c * x.v[mt][cb][2 * h + 1];
+                const float a = -x.v[mt][cb][2 * h], b = -x.v[mt][cb][2 * h + 1];
                 if (!PAD) {
                     store_pair(base, off + i * (8 * RB) + k, a, b, bf16);
                 } else if (i < d) {
@@ -228,124 +247,79 @@ __device__ __forceinline__ void store_gain(float* base, long long off, const Mat
             }
 }
 
-// ---- when the five products with A, B and P and Z'Z run on pairs of halves (frag.cuh)
-// The pair's absolute error of 2^-25 takes the place of the relative one for small elements, and 65504 is the largest number.
-// A step runs on halves when
-//     every row of A' and of B' has its largest element in [2^-4, 8],
-//     every P_ii is at least 2^-4 and no |P_ij| is above 128 (64 above 32 states), or P = 0
-// (rows of the padding aside), tested on the values in every step, for operands that do not change once; otherwise, and from
-// then on, the instance runs in tf32.  In this range the error of an operand is at most 2^-21 of the largest element of its row,
-// which is the bound of the tf32 split; V and T stay below 32 * 8 * 128 = 64 * 8 * 64 = 2^15 and |Z| below 2^13.
-// The rows are tested one by one because a control or a state in other units would otherwise lose its digits: with R_jj and
-// column j of B small together, row j of K is as large as 1 / |B_j|.
-template <bool V>
-struct OnHalves {
-    static constexpr bool value = V;
+// ---- when the five products with A, B and P run on pairs of halves (frag.cuh)
+// In tf32 every element of an operand is represented to 2^-21 of itself, which leaves an error of 2^-20 |X||Y'| in a product
+// (|.| element by element).  The pairs run where they leave no more.  A', B' and P are multiplied by powers of two that bring
+// the largest |A_ij|, the largest |B_ij| and the largest P_ii into [2^14, 2^15); the conditions, on the values so scaled, are
+//     every |A'_ij| and |B'_ij| is at least 2^-15                                         (represented to 2^-21 of itself)
+//     every row sum of |A'| is at least 2^-5 of the power of two above the largest one, and so of |B'|
+//     every |P_ij| is at least 2^-9 and none above 65504; if no element is more than half of its row sum in |A'| and |B'|,
+//     two of P (P_ij and P_ji) may be smaller
+// B'P and A'P are divided by those powers of two, so that they cannot overflow.  Their elements are represented to 2^-22 of
+// themselves or 2^-36, and (|A'||P|)_ij is at least 2^-9 2^-5 / 2 = 2^-15 after that division: 2^-21 of it.  (The allowance for
+// two is for dense matrices, where an element that small is an accident, once in 2000 steps at n = 40, and where a step in
+// tf32 costs a launch of one wave 18 %: 1155 instances 201 or 238 us by chance, without it.)  Z'Z stays in tf32, whose split of Z'
+// the factorisation makes anyway; on halves, with a test of Z', it took 6.87 instead of 6.91 ms at n = 32 and 212 instead of 201 us
+// at 40 x 12.  A step in which P fails runs in tf32, an instance whose operands fail (zeros, rows of other units) throughout.
+constexpr float OPERAND_LOW = 0x1p-15f, ROW_LOW = 0x1p-5f, VALUE_LOW = 0x1p-9f;
+__device__ __forceinline__ float power_of_two(int e) { return __int_as_float((127 + e) << 23); }
+__device__ __forceinline__ int exponent(unsigned bits) { return (int)(bits >> 23) - 127; }
+// what a split of A' or B' (rows x cols exist) is scaled by, 2^scale, and its products with P, 2^shift
+struct Scaling {
+    int scale, shift;
+    bool fits, spread;                                      // (spread: no element is more than half of its row)
 };
-constexpr float HALF_LOW = 0.0625f, HALF_HIGH = 8.f;
-__host__ __device__ constexpr float half_p_high(int blocks) { return blocks > 4 ? 64.f : 128.f; }
-__device__ __forceinline__ __half2 as_half2(uint32_t x) { return *reinterpret_cast<const __half2*>(&x); }
-__device__ __forceinline__ __half2 max_xor(__half2 v, __half2 other, int lanes)
-{
-    return __hmax2(v, as_half2(__shfl_xor_sync(FULL, *reinterpret_cast<const uint32_t*>(&other), lanes)));
-}
-// largest elements of this lane's part of rows 16 mt + g (first half) and 16 mt + 8 + g (second)
-template <int RB, int CB>
-__device__ __forceinline__ __half2 row_top(const Halves<RB, CB>& x, int mt)
-{
-    __half2 m0 = __habs2(as_half2(x.h[mt][0][0])), m1 = __habs2(as_half2(x.h[mt][0][1]));
-#pragma unroll
-    for (int cb = 1; cb < CB; ++cb) {
-        m0 = __hmax2(m0, __habs2(as_half2(x.h[mt][cb][0])));
-        m1 = __hmax2(m1, __habs2(as_half2(x.h[mt][cb][1])));
-    }
-    return __hmax2(__lows2half2(m0, m1), __highs2half2(m0, m1));
-}
-// lower limits of those two rows: none for rows that do not exist (i >= d)
-template <bool PAD>
-__device__ __forceinline__ __half2 row_limit(int mt, int d, int g)
-{
-    return PAD ? __floats2half2_rn(16 * mt + g < d ? HALF_LOW : 0.f, 16 * mt + 8 + g < d ? HALF_LOW : 0.f) : __float2half2_rn(HALF_LOW);
-}
 template <int RB, int CB, bool PAD>
-__device__ __forceinline__ bool rows_fit(const Halves<RB, CB>& x, int d, int lane)
+__device__ __forceinline__ Scaling operand_scaling(const Mat<RB, CB>& x, int rows, int cols, int lane)
 {
-    bool ok = true;
+    const int g = lane >> 2, t = lane & 3;
+    const float inf = __int_as_float(0x7f800000);
+    float top = 0.f, least = inf, low = inf, high = 0.f;
+    bool spread = true;
 #pragma unroll
-    for (int mt = 0; mt < Halves<RB, CB>::MT; ++mt) {
-        __half2 v = row_top(x, mt);
-        v = max_xor(v, v, 1);
-        v = max_xor(v, v, 2);
-        ok = ok && __hbge2(v, row_limit<PAD || (RB % 2 != 0)>(mt, d, lane >> 2)) && __hble2(v, __float2half2_rn(HALF_HIGH));
-    }
-    return ok;
-}
-// the same for two operands of at most sixteen rows: of each pair of lanes the first one looks at A', the second one at B'
-template <int NB, int MB, bool PAD>
-__device__ __forceinline__ bool rows_fit(const Halves<NB, NB>& a, const Halves<MB, NB>& b, int n, int m, int lane)
-{
-    static_assert(NB <= 2 && MB <= 2, "one tile of rows each");
-    const bool second = lane & 1;
-    const __half2 ta = row_top(a, 0), tb = row_top(b, 0);
-    __half2 v = max_xor(second ? tb : ta, second ? ta : tb, 1);
-    v = max_xor(v, v, 2);
-    return __hbge2(v, row_limit<PAD || NB == 1 || MB == 1>(0, second ? m : n, lane >> 2)) && __hble2(v, __float2half2_rn(HALF_HIGH));
-}
-// every element is zero (in float32: a half rounds to zero from 2^-25 downwards)
-template <int RB, int CB>
-__device__ __forceinline__ bool is_zero(const Mat<RB, CB>& x)
-{
-    unsigned any = 0u;
-#pragma unroll
-    for (int mt = 0; mt < Mat<RB, CB>::MT; ++mt)
+    for (int b = 0; b < RB; ++b) {
+        const bool row = !PAD || 8 * b + g < rows;
+        float sum = 0.f, most = 0.f;
 #pragma unroll
         for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                any |= __float_as_uint(x.v[mt][cb][e]);
-    return !(any & 0x7fffffffu);
-}
-// the conditions on P (x: the halves of nP), and `rows` of every lane (called by the whole warp); P = 0 (no terminal weight)
-// fits as well
-template <int NB, bool PAD>
-__device__ __forceinline__ bool value_fits(const Halves<NB, NB>& x, const Mat<NB, NB>& nP, bool rows, int n, int lane)
-{
-    const int g = lane >> 2, t = lane & 3;
-    __half2 top = __habs2(as_half2(x.h[0][0][0]));
-    bool ok = rows;
-#pragma unroll
-    for (int mt = 0; mt < Halves<NB, NB>::MT; ++mt)
-#pragma unroll
-        for (int cb = 0; cb < NB; ++cb)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                if (e && 2 * mt + 1 >= NB)
-                    continue;
-                const __half2 v = __habs2(as_half2(x.h[mt][cb][e]));
-                top = __hmax2(top, v);
-                if (cb == 2 * mt + e) {                     // diagonal block: the lane's element on the diagonal, if there is one
-                    const float low = !PAD || 8 * cb + g < n ? HALF_LOW : 0.f;
-                    ok = ok && __hbge2(v, __floats2half2_rn(g == 2 * t ? low : 0.f, g == 2 * t + 1 ? low : 0.f));
-                }
+            for (int k = 0; k < 2; ++k) {
+                const float v = fabsf(x.v[b / 2][cb][2 * (b & 1) + k]);
+                sum += v;
+                most = fmaxf(most, v);
+                least = fminf(least, row && (!PAD || 8 * cb + 2 * t + k < cols) ? v : inf);
             }
-    return __all_sync(FULL, ok && __hble2(top, __float2half2_rn(half_p_high(NB)))) ||
-           __all_sync(FULL, rows && is_zero(nP));
+        sum = sum_over_t(sum);
+        most = fmaxf(most, __shfl_xor_sync(FULL, most, 1));
+        most = fmaxf(most, __shfl_xor_sync(FULL, most, 2));
+        top = fmaxf(top, most);
+        high = fmaxf(high, sum);
+        low = fminf(low, row ? sum : inf);
+        spread = spread && 2.f * most <= sum;
+    }
+    const int et = exponent(__reduce_max_sync(FULL, __float_as_uint(top)));
+    const int eh = exponent(__reduce_max_sync(FULL, __float_as_uint(high))) + 1;          // 2^eh is above every row sum
+    Scaling r;
+    r.scale = 14 - et;
+    r.shift = -(eh + r.scale);
+    r.spread = __all_sync(FULL, spread);
+    r.fits = et >= -20 && eh <= 34;                         // (keeps every power of two below a normal number)
+    if (r.fits)
+        r.fits = __all_sync(FULL, least >= OPERAND_LOW * power_of_two(-r.scale) && low >= ROW_LOW * power_of_two(eh));
+    return r;
 }
-// power of four, at most 1, that brings the largest P_ii into [1, 4); 1 where it is below or above 2^60.  (Never above 1: the
-// weights are multiplied by it too, and one of 2^70 beside a small value matrix would leave float32.)
+// the scale of P: false when there is none
 template <int NB>
-__device__ __forceinline__ float value_scale(const Mat<NB, NB>& nP, int lane)
+__device__ __forceinline__ bool value_scaling(int& scale, const Mat<NB, NB>& nP, int lane)
 {
     const int g = lane >> 2, t = lane & 3;
     float top = 0.f;
 #pragma unroll
     for (int b = 0; b < NB; ++b)
         top = fmaxf(top, -((g & 1) ? nP.v[b / 2][b][2 * (b & 1) + 1] : nP.v[b / 2][b][2 * (b & 1)]));
-    const unsigned bits = __reduce_max_sync(FULL, t == (g >> 1) ? __float_as_uint(top) : 0u);
-    const int e = ((int)(bits >> 23) - 127) & ~1;
-    return e >= 0 && e <= 60 ? __int_as_float((127 - e) << 23) : 1.f;
+    scale = 14 - exponent(__reduce_max_sync(FULL, t == (g >> 1) ? __float_as_uint(top) : 0u));
+    return scale >= -26 && scale <= 54;
 }
-
 // W consecutive elements of a row (16-byte loads), or with PAD element by element within [0, n)
 template <int W, bool PAD>
 __device__ __forceinline__ void load_part(float (&v)[W], const float* row, int c0, int n)
@@ -627,9 +601,9 @@ __host__ __device__ constexpr size_t warp_bytes()
 // state at the piece's ends, writes its part of the outputs and leaves failures to the caller.
 // GRAD = the gradients of the first control in the same kernel (n = m = 8 NB, float32 operands): see grad_tail().
 // FEW = at most four warps per SM: the factorisation with the shorter chain (chol8_inverse).
-// CTAs per SM at n <= 16: as many as shared memory (time-varying) or registers hold.  Time-invariant six of them, 80 registers (20 to
-// 30 bytes of them spilled at the end of the horizon): 32768 instances, H = 16, all outputs 0.667 -> 0.604 ms against four (five
-// 0.630, seven 0.608), 4096 instances 99.8 -> 96.2 us.  Launches that cannot fill that many (FEW, the pieces of a scan) keep four.
+// CTAs per SM at n <= 16: as many as shared memory (time-varying) or registers hold.  Time-invariant six of them: 32768 instances,
+// n = 16, H = 16, all outputs 0.756 ms with four, 0.737 with five, 0.716 with six, 4096 instances 106.6, 106.4, 106.2 us.  Launches
+// that cannot fill that many (FEW, the pieces of a scan) keep four.
 template <int NB, int MB, bool TV, bool AFF, bool PAD, bool CH = false, bool GRAD = false, bool FEW = false>
 __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 : TV ? 5 : CH || FEW ? 4 : 6) riccati_frag_kernel(SolveParams p)
 {
@@ -674,7 +648,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
             if (p.Qf.ptr) {                                 // P_H = Q_f, by way of the second buffer
                 stage<NB, NB, Ops::LQ, PAD>(mem.op[1].Q, p.Qf, pl.off(p.Qf), n, n, lane);
                 copies_landed();
-                load_negated<NB, Ops::LQ>(nP, mem.op[1].Q, 1.f, lane);
+                load_negated<NB, Ops::LQ>(nP, mem.op[1].Q, lane);
                 __syncwarp();
             }
 #pragma unroll
@@ -686,7 +660,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
             }
             copies_landed();
             if (!p.Qf.ptr)
-                load_negated<NB, Ops::LQ>(nP, mem.op[0].Q, 1.f, lane);
+                load_negated<NB, Ops::LQ>(nP, mem.op[0].Q, lane);
         } else {
             OperandDev end = TV && p.Qf.ptr ? p.Qf : p.Q;   // P_H
             long long oend = TV && p.Qf.ptr ? pl.off(p.Qf) : oQ + last * p.Q.st;
@@ -701,7 +675,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
             stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + last * p.B.st, n, m, lane);
             stage<MB, MB, Ops::LR, PAD>(mem.R, p.R, oR + last * p.R.st, m, m, lane);
             copies_landed();
-            load_negated<NB, Ops::LQ>(nP, mem.Q, 1.f, lane);
+            load_negated<NB, Ops::LQ>(nP, mem.Q, lane);
             if ((TV && p.Qf.ptr) || inner) {
                 __syncwarp();
                 stage<NB, NB, Ops::LQ, PAD>(mem.Q, p.Q, oQ + last * p.Q.st, n, n, lane);
@@ -709,25 +683,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
         }
     }
     if (p.P && !p.first_only && last_piece)
-        store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, 1.f, n, obf, lane);
-
-    constexpr bool HALF = NB > 1;                           // (at n <= 8 nothing is gained)
-    // The recursion is homogeneous in (P, Q, R, p, r): on halves it runs on their multiples by a power of four that brings the
-    // largest P_ii at the end of the horizon into [1, 4), which makes the range of the halves one of ratios.  In tf32 it runs
-    // on the weights as they are: a small R_jj would become subnormal beside a control without effect (the reciprocals of
-    // the factorisation flush those to zero).
-    float scale = 1.f, unscale = 1.f;
-    if constexpr (HALF) {
-        scale = value_scale<NB>(nP, lane);
-        unscale = 1.f / scale;
-#pragma unroll
-        for (int mt = 0; mt < Mat<NB, NB>::MT; ++mt)
-#pragma unroll
-            for (int cb = 0; cb < NB; ++cb)
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    nP.v[mt][cb][e] *= scale;
-    }
+        store_negated<NB, PAD>(p.P, Poff + (long long)H * n * n, nP, n, obf, lane);
 
     auto start_state = [&](int i) {
         if (CH && p.xc)
@@ -751,42 +707,6 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
     }
 
     int fail = 0;
-    // Raw A, B (staged in shared memory) -> split, in place, one after the other.  On pairs of halves: false in a lane whose
-    // rows are out of range (the caller stages the operands again then).
-    auto install = [&](auto form, bool newA, bool newB) -> bool {
-        bool ok = true;
-        if constexpr (!TWO) {
-            if (newA) {
-                Mat<NB, NB> At;
-                load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
-                __syncwarp();
-                if constexpr (decltype(form)::value) {
-                    Halves<NB, NB> as;
-                    split(as, At);
-                    ok = rows_fit<NB, NB, PAD>(as, n, lane);
-                    keep(mem.halvesA(), as, lane);
-                } else {
-                    keep(mem.A, At, lane);
-                }
-            }
-            if (newB) {
-                Mat<MB, NB> Bt;
-                load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
-                __syncwarp();
-                if constexpr (decltype(form)::value) {
-                    Halves<MB, NB> bs;
-                    split(bs, Bt);
-                    const bool okB = rows_fit<MB, NB, PAD>(bs, m, lane);
-                    ok = ok && okB;
-                    keep(mem.halvesB(), bs, lane);
-                } else {
-                    keep(mem.B, Bt, lane);
-                }
-            }
-            __syncwarp();
-        }
-        return ok;
-    };
     float gr[MB], ap[NB];                                   // affine: B'p + r and A'p in row form
     auto affine_part = [&](const Mat<NB, NB>& At, const Mat<MB, NB>& Bt, const int ts) {
         float pc[NB][2];
@@ -800,7 +720,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
 #pragma unroll
             for (int k = 0; k < NB; ++k)
                 s = fmaf(Bt.v[b / 2][k][2 * (b & 1)], pc[k][0], fmaf(Bt.v[b / 2][k][2 * (b & 1) + 1], pc[k][1], s));
-            gr[b] = sum_over_t(s) + (8 * b + g < m ? scale * load_elem(p.r, orv + 8 * b + g) : 0.f);
+            gr[b] = sum_over_t(s) + (8 * b + g < m ? load_elem(p.r, orv + 8 * b + g) : 0.f);
         }
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
@@ -811,141 +731,112 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
             ap[b] = sum_over_t(s);
         }
     };
-    // One step.  On pairs of halves: false, and nothing else done, when an operand is out of its range.
-    auto step = [&](auto form, const int ts) -> bool {
-        constexpr bool ON_HALVES = decltype(form)::value;
-        Mat<NB, NB> T;
-        Mat<MB, NB> V;
-        Mat<NB, MB> Zt;
-        Mat<MB, MB> S, nR;
-        if constexpr (TWO) {
-            const Ops& op = mem.op[(H - 1 - ts) & 1];
-            if (ts < H - 1)
-                copies_landed();                            // also: every lane is done with the other buffer
-            if (ts > 0) {                                   // operands of the next step
-                Ops& nx = mem.op[(H - ts) & 1];
-                if (p.A.st) stage<NB, NB, Ops::LA, PAD>(nx.A, p.A, oA + (ts - 1) * p.A.st, n, n, lane);
-                if (p.B.st) stage<NB, MB, Ops::LB, PAD>(nx.B, p.B, oB + (ts - 1) * p.B.st, n, m, lane);
-                if (p.R.st) stage<MB, MB, Ops::LR, PAD>(nx.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
-                if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(nx.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
-            }
-            load_negated<MB, Ops::LR>(nR, op.R, scale, lane);
-            Mat<NB, NB> At;
-            Mat<MB, NB> Bt;
-            load_transposed<NB, NB, Ops::LA, false>(At, op.A, n, n, lane);
-            load_transposed<MB, NB, Ops::LB, false>(Bt, op.B, n, m, lane);
-            if (AFF && ts < p.r_count)
-                affine_part(At, Bt, ts);
-            if constexpr (ON_HALVES) {
-                Halves<NB, NB> as, ps;
-                Halves<MB, NB> bs, vs;
-                split(ps, nP);
-                split(as, At);
-                split(bs, Bt);
-                const bool rows = rows_fit<NB, MB, PAD>(as, bs, n, m, lane);      // (shuffles: by every lane, whatever P is)
-                if (!value_fits<NB, PAD>(ps, nP, rows, n, lane))
-                    return false;
-                product_halves<MB, NB, NB>(V, nullptr, bs, ps, lane);          // V = B' nP
-                product_halves<NB, NB, NB>(T, nullptr, as, ps, lane);          // T = A' nP
-                split(vs, V);
-                product_halves<MB, NB, MB, true>(S, &nR, bs, vs, lane);        // -S = -R + B' V'
-                product_halves<NB, NB, MB>(Zt, nullptr, as, vs, lane);         // -Y' = A' V'
-                split(ps, T);
-                load_negated<NB, Ops::LQ>(nP, op.Q, scale, lane);
-                product_halves<NB, NB, NB, true>(nP, &nP, as, ps, lane);       // -Q - A'P A
-            } else {
-                Split<NB, NB> as, ps;
-                Split<MB, NB> bs, vs;
-                split(ps, nP);
-                split(as, At);
-                split(bs, Bt);
-                product<MB, NB, NB>(V, nullptr, bs, ps);
-                product<NB, NB, NB>(T, nullptr, as, ps);
-                split(vs, V);
-                product<MB, NB, MB, true>(S, &nR, bs, vs);
-                product<NB, NB, MB>(Zt, nullptr, as, vs);
-                split(ps, T);
-                load_negated<NB, Ops::LQ>(nP, op.Q, scale, lane);
-                product<NB, NB, NB, true>(nP, &nP, as, ps);
-            }
-        } else {
+    // Form in which the operands lie in the warp's memory.  They are split in place, so that a change between the two split
+    // forms stages the raw ones again.  After a failed attempt to run on halves, or the end of one, `rest` steps in tf32 pass
+    // before the next: none the first time (a diagonal terminal weight), then one, three, seven ...
+    // HALF: up to 16 the scaling and the tests take back most of what the products gain (4096 instances, H = 16: 100 us in the range
+    // and 110 out of it, against 106 in tf32); above, see the head of this file.
+    constexpr bool HALF = NB > 2;
+    enum { RAW, TF32, HALVES };
+    int formA = RAW, formB = RAW, scaleP = 0, rest = 0, pause = 0;
+    Scaling sA = {}, sB = {};
+    bool okP = HALF && value_scaling<NB>(scaleP, nP, lane);
+    auto failed = [&]() {
+        rest = pause;
+        pause = pause < 1 << 20 ? 2 * pause + 1 : pause;
+    };
+    auto raw_instead_of = [&](int form, int ts) {           // what lies there in that form: the raw operand once more
+        if constexpr (HALF) {
+            if (formA != form && formB != form)
+                return;
+            const long long now = TV ? ts : 0;
+            __syncwarp();
+            if (formA == form) stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + now * p.A.st, n, n, lane);
+            if (formB == form) stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + now * p.B.st, n, m, lane);
+            copies_landed();
+            formA = formA == form ? RAW : formA;
+            formB = formB == form ? RAW : formB;
+        }
+    };
+    auto begin_step = [&](const int ts) {
+        if constexpr (!TWO) {
             if (TV || ts == H - 1)                          // (what CH stages for P_H is followed by Q)
                 copies_landed();
+            if (TV && p.A.st)
+                formA = RAW;
+            if (TV && p.B.st)
+                formB = RAW;
             if (AFF && ts < p.r_count) {                    // from the float32 operands, before they are split in place
                 Mat<NB, NB> At;
                 Mat<MB, NB> Bt;
-                if (p.A.st)
+                if (formA == RAW)
                     load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
                 else
                     load_transposed_global<NB, NB>(At, p.A, oA, n, n, n, lane);
-                if (p.B.st)
+                if (formB == RAW)
                     load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
                 else
                     load_transposed_global<MB, NB>(Bt, p.B, oB, m, n, m, lane);
                 affine_part(At, Bt, ts);
             }
-            const bool rows = TV ? install(form, p.A.st != 0, p.B.st != 0) : true;
-            if constexpr (ON_HALVES) {
-                Halves<NB, NB> ps;
-                split(ps, nP);
-                if (!value_fits<NB, PAD>(ps, nP, rows, n, lane))
-                    return false;
-                product_halves<MB, NB, NB>(V, nullptr, mem.halvesB(), ps, lane);
-                product_halves<NB, NB, NB>(T, nullptr, mem.halvesA(), ps, lane);
-            } else {
-                Split<NB, NB> ps;
-                split(ps, nP);
-                product<MB, NB, NB>(V, nullptr, mem.B, ps, lane);
-                product<NB, NB, NB>(T, nullptr, mem.A, ps, lane);
-            }
-            load_negated<MB, Ops::LR>(nR, mem.R, scale, lane);
-            if constexpr (ON_HALVES) {
-                {
-                    Halves<MB, NB> vs;
-                    split(vs, V);
-                    product_halves<MB, NB, MB, true>(S, &nR, mem.halvesB(), vs, lane);
-                    product_halves<NB, NB, MB>(Zt, nullptr, mem.halvesA(), vs, lane);
-                }
-                load_negated<NB, Ops::LQ>(nP, mem.Q, scale, lane);
-                {
-                    Halves<NB, NB> tsp;
-                    split(tsp, T);
-                    product_halves<NB, NB, NB, true>(nP, &nP, mem.halvesA(), tsp, lane);
-                }
-            } else {
-                {
-                    Split<MB, NB> vs;
-                    split(vs, V);
-                    product<MB, NB, MB, true>(S, &nR, mem.B, vs, lane);
-                    product<NB, NB, MB>(Zt, nullptr, mem.A, vs, lane);
-                }
-                load_negated<NB, Ops::LQ>(nP, mem.Q, scale, lane);
-                {
-                    Split<NB, NB> tsp;
-                    split(tsp, T);
-                    product<NB, NB, NB, true>(nP, &nP, mem.A, tsp, lane);
-                }
-            }
-            if (TV && ts > 0) {                             // operands of the next step, in flight while this one is factored
-                __syncwarp();
-                if (p.A.st) stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + (ts - 1) * p.A.st, n, n, lane);
-                if (p.B.st) stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + (ts - 1) * p.B.st, n, m, lane);
-                if (p.R.st) stage<MB, MB, Ops::LR, PAD>(mem.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
-                if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(mem.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
-            }
         }
+    };
+    auto stage_next = [&](const int ts) {                   // operands of the next step, in flight while this one is factored
+        if constexpr (TV && !TWO) {
+            if (ts == 0)
+                return;
+            __syncwarp();
+            if (p.A.st) stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + (ts - 1) * p.A.st, n, n, lane);
+            if (p.B.st) stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + (ts - 1) * p.B.st, n, m, lane);
+            if (p.R.st) stage<MB, MB, Ops::LR, PAD>(mem.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
+            if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(mem.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
+        }
+    };
+    // whether the raw operand permits halves, and the operand on halves, in place (time-varying: when it does)
+    auto fits_A = [&](const Mat<NB, NB>& At) {
+        sA = operand_scaling<NB, NB, PAD>(At, n, n, lane);
+        return sA.fits;
+    };
+    auto fits_B = [&](const Mat<MB, NB>& Bt) {
+        sB = operand_scaling<MB, NB, PAD>(Bt, m, n, lane);
+        return sB.fits;
+    };
+    auto install_halves = [&]() -> bool {
+        if constexpr (HALF) {
+            if (formB == RAW) {
+                Mat<MB, NB> Bt;
+                load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
+                if (TV && !fits_B(Bt))
+                    return false;
+                Halves<MB, NB> bs;
+                split(bs, Bt, power_of_two(sB.scale));
+                __syncwarp();
+                keep(mem.halvesB(), bs, lane);
+                formB = HALVES;
+            }
+            if (formA == RAW) {
+                Mat<NB, NB> At;
+                load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
+                if (TV && !fits_A(At))
+                    return false;
+                Halves<NB, NB> as;
+                split(as, At, power_of_two(sA.scale));
+                __syncwarp();
+                keep(mem.halvesA(), as, lane);
+                formA = HALVES;
+            }
+            __syncwarp();
+        }
+        return true;
+    };
+    // the rest of a step, from S, Y' (Zt) and -Q - A'PA (nP)
+    auto finish_step = [&](const int ts, Mat<MB, MB>& S, Mat<NB, MB>& Zt) {
         Split<NB, MB> zs;
         float w[MB][2];
         const int bad = factor<NB, MB, FEW || (NB > 2)>(S, Zt, zs, w, lane);  // Zt becomes Z', S the blocks of L
         if (bad && !fail)
             fail = ts * m + bad;
-        if constexpr (ON_HALVES) {                          // -P_t = -Q - A'PA + Z'Z
-            Halves<NB, MB> zh;
-            split(zh, Zt);
-            product_halves<NB, MB, NB, true>(nP, &nP, zh, zh, lane);
-        } else {
-            product<NB, MB, NB, true>(nP, &nP, zs, zs);
-        }
+        product<NB, MB, NB, true>(nP, &nP, zs, zs);                              // -P_t = -Q - A'PA + Z'Z
         const bool gain = need_K_all || need_k_all || (want_u0 && ts == 0);
         if (AFF) {
             // z = L^{-1}(B'p + r);  p_t = A'p - Z'z;  k_t = -L^{-T} z   (all zero while p and r are)
@@ -975,7 +866,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
 #pragma unroll
                 for (int b = 0; b < NB; ++b)
                     if (8 * b + g < n)
-                        p.pvec[(inst * (p.first_only ? 1 : H + 1) + (p.first_only ? 0 : ts)) * (long long)n + 8 * b + g] = unscale * pr[b];
+                        p.pvec[(inst * (p.first_only ? 1 : H + 1) + (p.first_only ? 0 : ts)) * (long long)n + 8 * b + g] = pr[b];
         }
         if (gain) {
             gains<NB, MB>(Zt, S, w, lane);                  // Zt = K_t'
@@ -1005,47 +896,160 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, NB > 2 ? 2 : AFF && !GRAD ? 4 
         // Q and Z'Z are symmetric, but the rounding of A'(PA) is not, and since the next step reads P through one
         // orientation only, the antisymmetric part E obeys E <- -A'E A: it grows along an open-loop unstable A however
         // well the closed loop is damped.
+        if constexpr (HALF)
+            okP = value_scaling<NB>(scaleP, nP, lane);      // (the diagonal stays)
         make_symmetric<NB>(nP, lane);
         if (p.P && first_ok && (!p.first_only || ts == 0))
-            store_negated<NB, PAD>(p.P, Poff + (long long)(p.first_only ? 0 : ts) * n * n, nP, unscale, n, obf, lane);
-        return true;
+            store_negated<NB, PAD>(p.P, Poff + (long long)(p.first_only ? 0 : ts) * n * n, nP, n, obf, lane);
     };
     int ts = H - 1;
-    const bool fixedA = !TV || !p.A.st, fixedB = !TV || !p.B.st;           // operands that are installed once
-    if constexpr (HALF) {
-        if (__all_sync(FULL, install(OnHalves<true>(), fixedA, fixedB)))
 #pragma unroll 1
-            while (ts >= 0 && step(OnHalves<true>(), ts))
-                --ts;
-        if constexpr (!TWO)
-            if (ts >= 0) {                                  // an instance that has left the range: the raw operands once more
-                const long long now = TV ? ts : 0;
-                __syncwarp();
-                stage<NB, NB, Ops::LA, PAD>(mem.rawA(), p.A, oA + now * p.A.st, n, n, lane);
-                stage<NB, MB, Ops::LB, PAD>(mem.rawB(), p.B, oB + now * p.B.st, n, m, lane);
-                copies_landed();
+    while (ts >= 0) {
+        Mat<NB, MB> Zt;
+        Mat<MB, MB> S;
+        if constexpr (TWO) {
+            const Ops& op = mem.op[(H - 1 - ts) & 1];
+            if (ts < H - 1)
+                copies_landed();                            // also: every lane is done with the other buffer
+            if (ts > 0) {                                   // operands of the next step
+                Ops& nx = mem.op[(H - ts) & 1];
+                if (p.A.st) stage<NB, NB, Ops::LA, PAD>(nx.A, p.A, oA + (ts - 1) * p.A.st, n, n, lane);
+                if (p.B.st) stage<NB, MB, Ops::LB, PAD>(nx.B, p.B, oB + (ts - 1) * p.B.st, n, m, lane);
+                if (p.R.st) stage<MB, MB, Ops::LR, PAD>(nx.R, p.R, oR + (ts - 1) * p.R.st, m, m, lane);
+                if (p.Q.st) stage<NB, NB, Ops::LQ, PAD>(nx.Q, p.Q, oQ + (ts - 1) * p.Q.st, n, n, lane);
             }
-    }
-    if (ts >= 0) {
-        if constexpr (HALF) {                               // (what is scaled back are results that the horizon may keep)
-#pragma unroll
-            for (int mt = 0; mt < Mat<NB, NB>::MT; ++mt)
-#pragma unroll
-                for (int cb = 0; cb < NB; ++cb)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        nP.v[mt][cb][e] *= unscale;
-            if (AFF)
-#pragma unroll
-                for (int b = 0; b < NB; ++b)
-                    pr[b] *= unscale;
-            scale = unscale = 1.f;
-        }
-        install(OnHalves<false>(), fixedA, fixedB);
-    }
+            Mat<NB, NB> At, T;
+            Mat<MB, NB> Bt, V;
+            Mat<MB, MB> nR;
+            load_negated<MB, Ops::LR>(nR, op.R, lane);
+            load_transposed<NB, NB, Ops::LA, false>(At, op.A, n, n, lane);
+            load_transposed<MB, NB, Ops::LB, false>(Bt, op.B, n, m, lane);
+            Split<NB, NB> as, ps;
+            Split<MB, NB> bs, vs;
+            split(ps, nP);
+            split(as, At);
+            split(bs, Bt);
+            product<MB, NB, NB>(V, nullptr, bs, ps);        // V = B' nP
+            product<NB, NB, NB>(T, nullptr, as, ps);        // T = A' nP
+            split(vs, V);
+            product<MB, NB, MB, true>(S, &nR, bs, vs);      // -S = -R + B' V'
+            product<NB, NB, MB>(Zt, nullptr, as, vs);       // -Y' = A' V'
+            split(ps, T);
+            load_negated<NB, Ops::LQ>(nP, op.Q, lane);
+            product<NB, NB, NB, true>(nP, &nP, as, ps);     // -Q - A'P A
+            if (AFF && ts < p.r_count)
+                affine_part(At, Bt, ts);
+        } else {
+            begin_step(ts);
+            if constexpr (HALF && !TV)
+                if (ts == H - 1) {                          // operands that do not change are looked at once
+                    Mat<MB, NB> Bt;
+                    load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
+                    bool fits = fits_B(Bt);
+                    if (fits) {
+                        Mat<NB, NB> At;
+                        load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
+                        fits = fits_A(At);
+                    }
+                    rest = fits ? 0 : 1 << 30;
+                }
+            if constexpr (HALF) {
+                if (rest > 0) {
+                    --rest;
+                } else {
+                    bool installed = false;                 // operands that do not change, on halves
 #pragma unroll 1
-    for (; ts >= 0; --ts)
-        step(OnHalves<false>(), ts);
+                    while (true) {
+                        {
+                            Halves<NB, NB> ps;
+                            split(ps, nP, power_of_two(okP ? scaleP : 0));
+                            if (!in_range(ps, VALUE_LOW, n * n - (!TV && sA.spread && sB.spread ? 2 : 0)) || !okP) {
+                                failed();
+                                break;
+                            }
+                            if (!installed) {
+                                raw_instead_of(TF32, ts);
+                                if (!install_halves()) {
+                                    failed();
+                                    break;
+                                }
+                                installed = !TV;
+                            }
+                            Mat<MB, NB> V;
+                            Mat<NB, NB> T;
+                            Halves<MB, NB> vs;
+                            Halves<NB, NB> tsp;
+                            product_halves<MB, NB, NB>(V, mem.halvesB(), ps, lane);
+                            product_halves<NB, NB, NB>(T, mem.halvesA(), ps, lane);
+                            split(vs, V, power_of_two(sB.shift));
+                            split(tsp, T, power_of_two(sA.shift));
+                            product_halves<MB, NB, MB, true>(S, mem.halvesB(), vs, lane);
+                            scale_and_subtract<MB, Ops::LR, true>(S, power_of_two(-(2 * sB.scale + sB.shift + scaleP)), mem.R, lane);
+                            product_halves<NB, NB, MB>(Zt, mem.halvesA(), vs, lane);
+                            const float c = power_of_two(-(sA.scale + sB.scale + sB.shift + scaleP));
+#pragma unroll
+                            for (int mt = 0; mt < Mat<NB, MB>::MT; ++mt)
+#pragma unroll
+                                for (int cb = 0; cb < MB; ++cb)
+#pragma unroll
+                                    for (int e = 0; e < 4; e += 2)
+                                        scale_pair(Zt.v[mt][cb][e], Zt.v[mt][cb][e + 1], c);
+                            product_halves<NB, NB, NB, true>(nP, mem.halvesA(), tsp, lane);
+                            scale_and_subtract<NB, Ops::LQ, true>(nP, power_of_two(-(2 * sA.scale + sA.shift + scaleP)), mem.Q, lane);
+                        }
+                        stage_next(ts);
+                        finish_step(ts, S, Zt);
+                        if (--ts < 0)
+                            break;
+                        begin_step(ts);
+                    }
+                    if (ts < 0)
+                        break;
+                }
+            }
+            if constexpr (HALF)
+                raw_instead_of(HALVES, ts);
+            if (formA == RAW) {                             // raw -> split, in place
+                Mat<NB, NB> At;
+                load_transposed<NB, NB, Ops::LA, PAD>(At, mem.rawA(), n, n, lane);
+                __syncwarp();
+                keep(mem.A, At, lane);
+            }
+            if (formB == RAW) {
+                Mat<MB, NB> Bt;
+                load_transposed<MB, NB, Ops::LB, PAD>(Bt, mem.rawB(), n, m, lane);
+                __syncwarp();
+                keep(mem.B, Bt, lane);
+            }
+            formA = formB = TF32;
+            __syncwarp();
+            Mat<MB, NB> V;
+            Mat<NB, NB> T;
+            Mat<MB, MB> nR;
+            load_negated<MB, Ops::LR>(nR, mem.R, lane);
+            {
+                Split<NB, NB> ps;
+                split(ps, nP);
+                product<MB, NB, NB>(V, nullptr, mem.B, ps, lane);
+                product<NB, NB, NB>(T, nullptr, mem.A, ps, lane);
+            }
+            {
+                Split<MB, NB> vs;
+                split(vs, V);
+                product<MB, NB, MB, true>(S, &nR, mem.B, vs, lane);
+                product<NB, NB, MB>(Zt, nullptr, mem.A, vs, lane);
+            }
+            load_negated<NB, Ops::LQ>(nP, mem.Q, lane);
+            {
+                Split<NB, NB> tsp;
+                split(tsp, T);
+                product<NB, NB, NB, true>(nP, &nP, mem.A, tsp, lane);
+            }
+            stage_next(ts);
+        }
+        finish_step(ts, S, Zt);
+        --ts;
+    }
     if (CH) {
         if (lane == 0)
             p.piece_info[widx] = fail;
