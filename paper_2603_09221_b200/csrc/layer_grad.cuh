@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(32 * lfrag::MAX_WARPS, NB > 2 ? 2 : PART == 0 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const layer::LayerParams& p = q.lp;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, T = p.T, r = p.r;
-    const int warp = warp_index();
+    const int warp = NB > 2 ? (int)(threadIdx.x >> 5) : warp_index();       // (as in layer_frag_kernel)
     const long long inst = (long long)blockIdx.x * (blockDim.x >> 5) + warp;
     if (inst >= p.N)
         return;
