@@ -35,6 +35,12 @@ FP32_LANES_PER_SM = 128
 TF32_TO_BF16_RATIO = 0.5     # nominal dense tensor ratio tf32 : bf16 on B200 (1.1 : 2.25 PFLOP/s)
 
 
+def mma_sync_peak(halves, mhz):
+    """TFLOP/s of float32-grade products in the one-warp kernels: three passes of mma.sync m16n8k8 (tf32) or m16n8k16 (pairs
+    of halves, above 16 states), 8 cycles each on the tensor pipe of one of an SM's four schedulers."""
+    return SM_COUNT * 4 * (2 * 16 * 8 * (16 if halves else 8) / 8) / 3 * mhz * 1e6 / 1e12
+
+
 def measured_peaks():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(path):
@@ -495,11 +501,12 @@ def run_layer(args):
         return
     flops_i, bin_i, bout_i = layer_counts(c)
     kernel_ms = statistics.median(per_step)
-    fp32_peak = SM_COUNT * FP32_LANES_PER_SM * 2 * peaks["sm_max_mhz"] * 1e6 / 1e12
+    peak = mma_sync_peak(False, peaks["sm_max_mhz"])
     ach = N * flops_i / (kernel_ms * 1e-3) / 1e12
-    roofline = {"bound": "alu", "achieved": ach, "peak": fp32_peak, "unit": "TFLOP/s", "frac": ach / fp32_peak,
+    roofline = {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                 "traffic": None, "kernel": "ttc_layer", "kernel_ms": kernel_ms,
-                "peak_note": "148 SMs x 128 FP32 lanes x 2 x %.0f MHz (derived)" % peaks["sm_max_mhz"],
+                "peak_note": "mma.sync in three passes of tf32, 8 cycles each on 148 x 4 schedulers, %.0f MHz (derived)"
+                             % peaks["sm_max_mhz"],
                 "algorithmic_flops_per_launch": N * flops_i, "algorithmic_bytes_per_launch": N * (bin_i + bout_i),
                 "hbm_frac": (N * (bin_i + bout_i) / (kernel_ms * 1e-3) / 1e9) / peaks["hbm_gbs"]}
     cpu = None
@@ -737,10 +744,17 @@ def run_solve(args, workload, method_name, ctx, light=False):
         peak_note = "copy bandwidth, of %s (the tensor-core time at the measured tf32 peak is shorter)" % peaks["source"]
         extra = {"tensor_frac": (alg_flops / (kernel_ms * 1e-3) / 1e12) / tf32_peak, "tf32_peak_tflops": tf32_peak}
     else:
-        t_alu = alg_flops / (fp32_peak * 1e12)
-        if t_hbm >= t_alu:
+        one_warp = kname in ("riccati_warp", "scan")
+        halves = max(n, m) > 16
+        pipe_peak = mma_sync_peak(halves, peaks["sm_max_mhz"]) if one_warp else fp32_peak
+        if t_hbm >= alg_flops / (pipe_peak * 1e12):
             bound, peak, unit, ach = "hbm", peaks["hbm_gbs"], "GB/s", alg_bytes / (kernel_ms * 1e-3) / 1e9
             peak_note = "copy bandwidth, of %s" % peaks["source"]
+        elif one_warp:
+            bound, peak, unit, ach = "tensor", pipe_peak, "TFLOP/s", alg_flops / (kernel_ms * 1e-3) / 1e12
+            peak_note = ("mma.sync in three passes of %s, 8 cycles each on 148 x 4 schedulers, %.0f MHz (derived)"
+                         % ("pairs of halves" if halves else "tf32", peaks["sm_max_mhz"]))
+            extra = {"frac_of_fp32_fma_peak": ach / fp32_peak, "fp32_fma_peak_tflops": fp32_peak}
         else:
             bound, peak, unit, ach = "alu", fp32_peak, "TFLOP/s", alg_flops / (kernel_ms * 1e-3) / 1e12
             peak_note = ("FMA-chain micro-kernel measured in this run" if run_peaks else

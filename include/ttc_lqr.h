@@ -60,11 +60,13 @@ extern "C" {
 
 /* ttc_lqr_config.math : arithmetic of the n x n contractions */
 #define TTC_MATH_AUTO  0  /* FP32 when every input is F32, TF32 when Q or x0 is BF16  */
-#define TTC_MATH_FP32  1  /* FFMA, fp32 throughout                                    */
+#define TTC_MATH_FP32  1  /* fp32 accuracy: split operands on the tensor cores        */
 #define TTC_MATH_TF32  2  /* tcgen05 tensor cores, tf32 operands, fp32 accumulate (n = m = 64) */
 /* n = m = 64 is served by the tensor-memory kernel only with TF32 math (AUTO picks it when Q or x0 is
  * BF16), per-head A, B, R and a time-invariant problem.  Every other time-invariant request, and time-varying /
- * affine ones up to 32 x 32, run with one warp per instance in float32 (three-pass products of split operands); time-varying and
+ * affine ones up to 32 x 32, run with one warp per instance in float32 (three-pass products of operands split into
+ * two tf32 numbers, 2^-21 of each element, or, above 16 states or controls and where the values at hand lose no more by it,
+ * into two float16 numbers; sums in float32); time-varying and
  * affine requests above 32 run in the generic one-CTA-per-instance kernel, one to two orders of magnitude slower than the
  * tensor-memory kernel.  Above 32 states or controls the one-warp kernel keeps part of its matrices in local memory, for
  * which the driver reserves device memory at the first such call: up to 1 GB, above 48 up to 3.3 GB. */
