@@ -20,7 +20,7 @@
 //   16384 instances n = 32, H = 64, all outputs           14.2 -> 6.87 ms     1155, n = 40, m = 12, H = 20     2428 -> 198 us
 //   64 instances n = 8, H = 8, own dynamics               107 -> 11 us     1155, n = m = 60, H = 20            21.9 -> 10.3 ms
 // The halves' part in that, against three passes of tf32 throughout: n = 32 8.41 -> 6.87 ms, 40 x 12 235 -> 198 us, time-varying
-// n = 32, 2048 instances of 32 steps 0.54 -> 0.49 ms.  Problems outside the range take 235 us at 40 x 12, and at n = 32 what
+// n = 32, 2048 instances of 32 steps 0.54 -> 0.47 ms.  Problems outside the range take 235 us at 40 x 12, and at n = 32 what
 // they took (1.10 ms on 4096 instances of 32 steps, 0.91 inside).
 #pragma once
 

@@ -4,7 +4,6 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2603_09221_b200 import lqr
 from tests import parity_util as pu
 from tests import test_gpu_affine as aff
 from tests import test_gpu_grad as grad
